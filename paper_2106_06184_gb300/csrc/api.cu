@@ -338,12 +338,16 @@ static std::vector<int> repeated_objects(const HostMesh& h, const sldm_material*
 // only, so two pairs whose objects have the same shapes at the same relative
 // displacement have equal blocks; in a layered background G depends on the
 // horizontal part of r - r' and on z and z' apart, so the pairs must also share
-// the objects' heights.  `reps` lists one pair per distinct block (filled), the
-// copies send each representative block to its repeats.  Objects of one shape
-// class and their translations: cls[o], shift[o] (from the class's first object).
+// the objects' heights.  The kernel and the 6 x 6 rule are symmetric (reciprocity; in
+// a stack the tabulated kernel's two components that trade places under it are
+// equal up to sign), so the block of (j, i) is the transpose of that of (i, j):
+// `reps` lists one pair per distinct block and its transpose (filled), transA/P
+// send them to the transposed blocks' first places, and then copyA/P send each
+// distinct block to its repeats.  Objects of one shape class and their
+// translations: cls[o], shift[o] (from the class's first object).
 struct GlobalReuse {
   std::vector<std::pair<int, int>> reps;
-  std::vector<BlockCopy> copyA, copyP;
+  std::vector<BlockCopy> transA, transP, copyA, copyP;
 };
 static GlobalReuse global_reuse(const HostMesh& h, bool layered) {
   const int nobj = int(h.nobj);
@@ -373,8 +377,11 @@ static GlobalReuse global_reuse(const HostMesh& h, bool layered) {
   struct Rep {
     int i, j;
     double d[3], zi;
+    int id;
   };
   std::map<std::pair<int, int>, std::vector<Rep>> by_cls;
+  std::vector<std::pair<int, int>> first;             // the first pair of every distinct block
+  std::vector<int> group(size_t(nobj) * nobj);        // distinct block of each pair
   for (int i = 0; i < nobj; ++i)
     for (int j = 0; j < nobj; ++j) {
       double d[3];
@@ -389,17 +396,41 @@ static GlobalReuse global_reuse(const HostMesh& h, bool layered) {
           break;
         }
       if (!hit) {
-        list.push_back({i, j, {d[0], d[1], d[2]}, zi});
-        g.reps.push_back({i, j});
+        group[size_t(i) * nobj + j] = int(first.size());
+        list.push_back({i, j, {d[0], d[1], d[2]}, zi, int(first.size())});
+        first.push_back({i, j});
         continue;
       }
+      group[size_t(i) * nobj + j] = hit->id;
       const int ri = hit->i, rj = hit->j;
       g.copyA.push_back({h.edge_begin[ri], h.edge_begin[rj], h.edge_begin[i], h.edge_begin[j],
                          h.edge_begin[i + 1] - h.edge_begin[i], h.edge_begin[j + 1] - h.edge_begin[j]});
       g.copyP.push_back({h.tri_begin[ri], h.tri_begin[rj], h.tri_begin[i], h.tri_begin[j],
                          h.tri_begin[i + 1] - h.tri_begin[i], h.tri_begin[j + 1] - h.tri_begin[j]});
     }
+  for (size_t k = 0; k < first.size(); ++k) {
+    const int i = first[k].first, j = first[k].second;
+    const int kt = group[size_t(j) * nobj + i];  // the transposed pair's block
+    if (kt >= int(k)) {
+      g.reps.push_back({i, j});
+      continue;
+    }
+    // block k = transpose of block kt, filled before it
+    const int ri = first[kt].first, rj = first[kt].second;
+    g.transA.push_back({h.edge_begin[ri], h.edge_begin[rj], h.edge_begin[i], h.edge_begin[j],
+                        h.edge_begin[ri + 1] - h.edge_begin[ri], h.edge_begin[rj + 1] - h.edge_begin[rj]});
+    g.transP.push_back({h.tri_begin[ri], h.tri_begin[rj], h.tri_begin[i], h.tri_begin[j],
+                        h.tri_begin[ri + 1] - h.tri_begin[ri], h.tri_begin[rj + 1] - h.tri_begin[rj]});
+  }
   return g;
+}
+
+// the transposed and the repeated global blocks from the filled ones
+static void reuse_blocks(sldm_op* op, const GlobalReuse& g, size_t es, cudaStream_t s) {
+  copy_blocks(g.transA, es, op->LAm.p, op->ne, s, true);
+  copy_blocks(g.transP, es, op->LPm.p, op->nt, s, true);
+  copy_blocks(g.copyA, es, op->LAm.p, op->ne, s);
+  copy_blocks(g.copyP, es, op->LPm.p, op->nt, s);
 }
 
 // Sommerfeld remainder tables of the objects' layer over the objects' extent:
@@ -452,7 +483,8 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
     // distinct relative placement; a background that splits sources (a good
     // conductor) keeps the single task, whose far-pair cut spans the whole fill
     if (op->nobj > 1 && !split_rules_L(h, t).split) gr = global_reuse(h, op->layered);
-    if (!gr.copyA.empty()) {
+    if (gr.copyA.empty()) gr = GlobalReuse();  // nothing repeats: one symmetric task
+    if (!gr.reps.empty()) {
       std::vector<LTask> tasks;
       for (auto& pr : gr.reps) {
         LTask u = t;
@@ -465,10 +497,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
       }
       fill_L<R>(m, tasks, s);
       // in a stack the repeats are copied once the reflected part is in
-      if (!op->layered) {
-        copy_blocks(gr.copyA, es, op->LAm.p, op->ne, s);
-        copy_blocks(gr.copyP, es, op->LPm.p, op->nt, s);
-      }
+      if (!op->layered) reuse_blocks(op, gr, es, s);
     } else {
       fill_L<R>(m, {t}, s);
       rtasks.push_back({0, int32_t(op->nt), 0, int32_t(op->nt)});
@@ -646,8 +675,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
   if (op->layered) {
     layered_tables(op, s);
     mgf_fill_reflected<C>(m, op->H, omega, op->T, rtasks, op->LAm.p, op->ne, op->LPm.p, op->nt, s);
-    copy_blocks(gr.copyA, es, op->LAm.p, op->ne, s);
-    copy_blocks(gr.copyP, es, op->LPm.p, op->nt, s);
+    reuse_blocks(op, gr, es, s);
     SLDM_CUDA(cudaStreamSynchronize(s));
   }
   if (!finish) return;

@@ -1597,13 +1597,38 @@ __global__ void __launch_bounds__(256) copy_blocks_kernel(const BlockCopy* __res
   for (int j = lane; j < c.nc; j += 32) dst[j] = __ldcs(src + j);
 }
 
-void copy_blocks(const std::vector<BlockCopy>& copies, size_t esz, void* M, int64_t ld, cudaStream_t s) {
+// One CTA per 32 x 32 tile of a transposed copy, through shared memory (both
+// sides in whole 32-entry rows); tiles of every copy in order, split by an
+// exclusive prefix sum.
+template <class C>
+__global__ void __launch_bounds__(256) copy_blocks_t_kernel(const BlockCopy* __restrict__ cp, const int64_t* __restrict__ ts,
+                                                            int ncp, C* M, int64_t ld) {
+  __shared__ C buf[32][33];
+  const int64_t w = blockIdx.x;
+  int lo = 0, hi = ncp - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (ts[mid] <= w) lo = mid;
+    else hi = mid - 1;
+  }
+  const BlockCopy c = cp[lo];
+  const int tc = (c.nc + 31) / 32;
+  const int r0 = int((w - ts[lo]) / tc) * 32, c0 = int((w - ts[lo]) % tc) * 32;
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  for (int i = row; i < 32; i += 8)
+    if (r0 + i < c.nr && c0 + lane < c.nc) buf[i][lane] = M[(c.sr + r0 + i) * ld + c.sc + c0 + lane];
+  __syncthreads();
+  for (int i = row; i < 32; i += 8)
+    if (c0 + i < c.nc && r0 + lane < c.nr) M[(c.dr + c0 + i) * ld + c.dc + r0 + lane] = buf[lane][i];
+}
+
+void copy_blocks(const std::vector<BlockCopy>& copies, size_t esz, void* M, int64_t ld, cudaStream_t s, bool transpose) {
   if (copies.empty()) return;
   std::vector<int64_t> rs(copies.size());
   int64_t acc = 0;
   for (size_t i = 0; i < copies.size(); ++i) {
     rs[i] = acc;
-    acc += copies[i].nr;
+    acc += transpose ? int64_t((copies[i].nr + 31) / 32) * ((copies[i].nc + 31) / 32) : copies[i].nr;
   }
   DBuf<BlockCopy> dc;
   DBuf<int64_t> drs;
@@ -1611,7 +1636,11 @@ void copy_blocks(const std::vector<BlockCopy>& copies, size_t esz, void* M, int6
   drs.upload(rs, s);
   const unsigned blocks = unsigned((acc * 32 + 255) / 256);
   ScopedTimer tm("copy_blocks", s);
-  if (esz == sizeof(double2))
+  if (transpose && esz == sizeof(double2))
+    copy_blocks_t_kernel<double2><<<unsigned(acc), 256, 0, s>>>(dc.p, drs.p, int(copies.size()), (double2*)M, ld);
+  else if (transpose)
+    copy_blocks_t_kernel<float2><<<unsigned(acc), 256, 0, s>>>(dc.p, drs.p, int(copies.size()), (float2*)M, ld);
+  else if (esz == sizeof(double2))
     copy_blocks_kernel<double2><<<blocks, 256, 0, s>>>(dc.p, drs.p, int(copies.size()), acc, (double2*)M, ld);
   else
     copy_blocks_kernel<float2><<<blocks, 256, 0, s>>>(dc.p, drs.p, int(copies.size()), acc, (float2*)M, ld);

@@ -57,7 +57,8 @@ __device__ void write_geo(double* g, const double* p0, const double* p1, const d
 
 __global__ void geometry_kernel(int nt, const double* __restrict__ xyz, const int32_t* __restrict__ tri,
                                 const int32_t* __restrict__ tri_edge, const int8_t* __restrict__ tri_sign,
-                                const int8_t* __restrict__ btri_sign, int64_t nv, double* geo, double* bgeo) {
+                                const int8_t* __restrict__ btri_sign, int64_t nv, double* geo, double* bgeo, double* rad,
+                                double* brad) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nt) return;
   const double* a = xyz + 3 * tri[3 * t];
@@ -65,6 +66,7 @@ __global__ void geometry_kernel(int nt, const double* __restrict__ xyz, const in
   const double* c = xyz + 3 * tri[3 * t + 2];
   double s[3] = {double(tri_sign[3 * t]), double(tri_sign[3 * t + 1]), double(tri_sign[3 * t + 2])};
   write_geo(geo + size_t(t) * GEO_STRIDE, a, b, c, s);
+  rad[t] = bound_radius(geo + size_t(t) * GEO_STRIDE + GEO_C, a, b, c);
   double mab[3], mbc[3], mca[3], g[3];
   for (int d = 0; d < 3; ++d) {
     mab[d] = 0.5 * (a[d] + b[d]);
@@ -78,21 +80,25 @@ __global__ void geometry_kernel(int nt, const double* __restrict__ xyz, const in
     int cc = 6 * t + k;
     double sb[3] = {double(btri_sign[3 * cc]), double(btri_sign[3 * cc + 1]), double(btri_sign[3 * cc + 2])};
     write_geo(bgeo + size_t(cc) * GEO_STRIDE, ch[k][0], ch[k][1], ch[k][2], sb);
+    brad[cc] = bound_radius(bgeo + size_t(cc) * GEO_STRIDE + GEO_C, ch[k][0], ch[k][1], ch[k][2]);
   }
 }
 
 void geometry(const HostMesh& hm, DevMesh& dm, cudaStream_t s) {
   dm.geo.alloc(size_t(hm.nt) * GEO_STRIDE);
   dm.bgeo.alloc(size_t(hm.nt) * 6 * GEO_STRIDE);
+  dm.rad.alloc(size_t(hm.nt));
+  dm.brad.alloc(size_t(hm.nt) * 6);
   int nt = int(hm.nt);
   geometry_kernel<<<(nt + 127) / 128, 128, 0, s>>>(nt, dm.xyz.p, dm.tri.p, dm.tri_edge.p, dm.tri_sign.p,
-                                                   dm.btri_sign.p, hm.nv, dm.geo.p, dm.bgeo.p), ::sldm::count_launch();
+                                                   dm.btri_sign.p, hm.nv, dm.geo.p, dm.bgeo.p, dm.rad.p,
+                                                   dm.brad.p), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
 
-// ---------------------------------------------------------------- bulk L kernel
+// ---------------------------------------------------------------- bulk fill: nodal moments of a pair
 constexpr int TILE_SRC = 128;  // source triangles per CTA (one per thread)
-constexpr int TILE_TEST = 8;   // test triangles per CTA (FP64 fills)
+constexpr int TILE_TEST = 8;   // test triangles per CTA, at most (FP64 fills)
 // Test triangles per CTA: each thread converts its source record to the fill's
 // precision once per CTA, so the FP32 fills take 32 test triangles to keep those
 // conversions (on the narrow FP64 pipe of this part) off the per-pair cost.
@@ -101,8 +107,9 @@ constexpr int tile_test() {
   return sizeof(R) == 4 ? 32 : TILE_TEST;
 }
 
+// One CTA's share of a task: test triangles [test0, test0 + ntest) x TILE_SRC sources from src0
 struct TileRef {
-  int32_t task, test0, src0, pad;
+  int32_t task, test0, src0, ntest;
 };
 
 // Centroids as hi + lo in the fill's precision (for FP32: two floats, c to ~2^-48),
@@ -110,9 +117,8 @@ struct TileRef {
 // fill's precision relative to the distance without FP64 operations in the loop.
 template <class R>
 struct TestRec {
-  R rho[18], W[6], av[9], sig[3];
+  R rho[18], av[9], sgn[3];  // quadrature points and c - v_i (centroid-local), +-1/2 per edge
   R chi[3], clo[3];
-  R invA;
   int32_t v[3], e[3];
 };
 template <class R>
@@ -120,59 +126,170 @@ __device__ __forceinline__ void split_hl(double v, R& hi, R& lo) {
   hi = R(v);
   lo = R(v - double(hi));
 }
-
 template <class R>
-__global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 5 : 1) fill_L_bulk(const LTask* __restrict__ tasks, const TileRef* __restrict__ tiles,
+__device__ __forceinline__ void load_test_tile(TestRec<R>* T, const TileRef& tile, int t0, const double* __restrict__ geo,
+                                               const int32_t* __restrict__ tri, const int32_t* __restrict__ tri_edge) {
+  for (int idx = threadIdx.x; idx < tile.ntest; idx += blockDim.x) {
+    const int tg = t0 + tile.test0 + idx;
+    const double* g = geo + size_t(tg) * GEO_STRIDE;
+    for (int d = 0; d < 18; ++d) T[idx].rho[d] = R(g[GEO_RHO + d]);
+    for (int d = 0; d < 9; ++d) T[idx].av[d] = R(g[GEO_AV + d]);
+    for (int d = 0; d < 3; ++d) {
+      T[idx].sgn[d] = half_sign<R>(g[GEO_SIG + d]);
+      split_hl(g[GEO_C + d], T[idx].chi[d], T[idx].clo[d]);
+      T[idx].v[d] = tri[3 * tg + d];
+      T[idx].e[d] = tri_edge[3 * tg + d];
+    }
+  }
+}
+
+// The kernels of L (G without 1/(4 pi)) and Kbar (g1 without 1/(4 pi), grad G = (r - r') g1)
+// at squared distance r2, in the fill's precision.
+struct NoTab {};
+template <class R>
+struct PairKernel;
+template <>
+struct PairKernel<double> {
+  typedef WaveTab Tab;
+  const WaveTab& tab;
+  double kr, ki, ys, ye;  // k, and k.r, k.i in steps of the tables
+  __device__ PairKernel(const WaveTab& t, double kr_, double ki_)
+      : tab(t), kr(kr_), ki(ki_), ys(kr_ * (WAVE_N / (2.0 * PI))), ye(ki_ * (WAVE_N * 1.4426950408889634074)) {}
+  template <bool LOSSY>
+  __device__ __forceinline__ void green(double r2, double& gr, double& gi) const {
+    const double ir = rsqrt_pos(r2), Rr = r2 * ir;
+    double c, s;
+    wave_cis(tab, ys * Rr, c, s);
+    const double a = LOSSY ? ir * wave_exp2(tab, ye * Rr) : ir;
+    gr = a * c;
+    gi = -a * s;
+  }
+  // g1 = -(1 + j k R) exp(-j k R) / R^3
+  template <bool LOSSY>
+  __device__ __forceinline__ void grad(double r2, double& gr, double& gi) const {
+    const double ir = rsqrt_pos(r2), Rr = r2 * ir;
+    double c, s;
+    wave_cis(tab, ys * Rr, c, s);
+    double a = -(ir * ir) * ir;
+    if (LOSSY) a *= wave_exp2(tab, ye * Rr);
+    const double ai = kr * Rr, ar = LOSSY ? fma(-ki, Rr, 1.0) : 1.0;
+    gr = a * fma(ai, s, LOSSY ? ar * c : c);
+    gi = a * fma(ai, c, LOSSY ? -ar * s : -s);
+  }
+};
+template <>
+struct PairKernel<float> {
+  typedef NoTab Tab;
+  float kr, ki;
+  __device__ PairKernel(const NoTab&, double kr_, double ki_) : kr(float(kr_)), ki(float(ki_)) {}
+  template <bool LOSSY>
+  __device__ __forceinline__ void green(float r2, float& gr, float& gi) const {
+    const float ir = M<float>::rsqrt_(r2), Rr = r2 * ir;
+    float c, s;
+    M<float>::sincos_(kr * Rr, &s, &c);
+    const float a = LOSSY ? ir * M<float>::exp_(ki * Rr) : ir;
+    gr = a * c;
+    gi = -a * s;
+  }
+  template <bool LOSSY>
+  __device__ __forceinline__ void grad(float r2, float& gr, float& gi) const {
+    const float ir = M<float>::rsqrt_(r2), Rr = r2 * ir;
+    float c, s;
+    M<float>::sincos_(kr * Rr, &s, &c);
+    float a = -(ir * ir) * ir;
+    if (LOSSY) a *= M<float>::exp_(ki * Rr);
+    const float ai = kr * Rr, ar = LOSSY ? 1.0f - ki * Rr : 1.0f;
+    gr = a * (ai * s + ar * c);
+    gi = a * (ai * c - ar * s);
+  }
+};
+__device__ __forceinline__ void wave_tab_init(NoTab&, bool) {}
+__device__ __forceinline__ void wave_tab_init(WaveTab& t, bool lossy) { wave_tab_fill(t, lossy); }
+
+// N[u][v] = sum over the 6 x 6 points of w_q w_k lambda_u(q) lambda_v(k) g(q, k):
+// every 3 x 3 block of a pair is a contraction of these nine moments with the
+// triangles' vertices (lambda: barycentric coordinates; areas and 1/(4 pi) left out).
+// The rule's points are two orbits of one vertex each (weight w1, coordinates a1, b1,
+// b1; w2, a2, b2, b2), so the source side takes sums of the two orbits and one
+// FMA per vertex: 4 operations per evaluation instead of the 8 of moments of r'.
+template <class R, bool GRAD, bool LOSSY>
+__device__ __forceinline__ void pair_moments(const PairKernel<R>& G, const TestRec<R>& X, const R (&rs)[18], R dc0, R dc1,
+                                             R dc2, R (&Nr)[9], R (&Ni)[9]) {
+  constexpr double A1 = 0.108103018168070, B1 = 0.445948490915965, W1 = 0.223381589678011;
+  constexpr double A2 = 0.816847572980459, B2 = 0.091576213509771, W2 = 0.109951743655322;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) Nr[i] = Ni[i] = R(0);
+#pragma unroll 1
+  for (int q = 0; q < 6; ++q) {
+    const R px = dc0 + X.rho[3 * q], py = dc1 + X.rho[3 * q + 1], pz = dc2 + X.rho[3 * q + 2];
+    R gr[6], gi[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const R dx = px - rs[3 * k], dy = py - rs[3 * k + 1], dz = pz - rs[3 * k + 2];
+      const R r2 = dx * dx + dy * dy + dz * dz;
+      if (GRAD) G.template grad<LOSSY>(r2, gr[k], gi[k]);
+      else G.template green<LOSSY>(r2, gr[k], gi[k]);
+    }
+    const R tr = R(W1 * B1) * (gr[0] + gr[1] + gr[2]) + R(W2 * B2) * (gr[3] + gr[4] + gr[5]);
+    const R ti = R(W1 * B1) * (gi[0] + gi[1] + gi[2]) + R(W2 * B2) * (gi[3] + gi[4] + gi[5]);
+    const R wa = q < 3 ? R(W1 * A1) : R(W2 * A2), wb = q < 3 ? R(W1 * B1) : R(W2 * B2);
+    const int qv = q < 3 ? q : q - 3;
+    const R w0 = qv == 0 ? wa : wb, w1 = qv == 1 ? wa : wb, w2 = qv == 2 ? wa : wb;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      const R lr = R(W1 * (A1 - B1)) * gr[v] + (R(W2 * (A2 - B2)) * gr[v + 3] + tr);
+      const R li = R(W1 * (A1 - B1)) * gi[v] + (R(W2 * (A2 - B2)) * gi[v + 3] + ti);
+      Nr[v] += w0 * lr;
+      Ni[v] += w0 * li;
+      Nr[3 + v] += w1 * lr;
+      Ni[3 + v] += w1 * li;
+      Nr[6 + v] += w2 * lr;
+      Ni[6 + v] += w2 * li;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- bulk L kernel
+// A task whose test and source triangles are the same set is symmetric (the
+// 6 x 6 rule and the Galerkin product are): only pairs s > t are integrated, and
+// each is scattered to both places (tk.sym).
+// FP64: bound by the FP64 pipe, ~45 operations per evaluation.  320-triangle sphere:
+// 0.71 ms (every pair, moments of r', general sincos) -> 0.24 ms; the distinct
+// blocks of 5 x 5 cylinders 20.0 -> 7.4 ms.
+template <class R>
+__global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 4 : 2) fill_L_bulk(const LTask* __restrict__ tasks, const TileRef* __restrict__ tiles,
                                                         const double* __restrict__ geo, const int32_t* __restrict__ tri,
                                                         const int32_t* __restrict__ tri_edge) {
   __shared__ TestRec<R> T[tile_test<R>()];
+  __shared__ typename PairKernel<R>::Tab tab;
   const TileRef tile = tiles[blockIdx.x];
   const LTask tk = tasks[tile.task];
-  // load the test tile
-  for (int idx = threadIdx.x; idx < tile_test<R>(); idx += blockDim.x) {
-    int t = tile.test0 + idx;
-    if (t < tk.ntest) {
-      int tg = tk.t0 + t;
-      const double* g = geo + size_t(tg) * GEO_STRIDE;
-      for (int d = 0; d < 18; ++d) T[idx].rho[d] = R(g[GEO_RHO + d]);
-      for (int d = 0; d < 6; ++d) T[idx].W[d] = R(g[GEO_W + d]);
-      for (int d = 0; d < 9; ++d) T[idx].av[d] = R(g[GEO_AV + d]);
-      for (int d = 0; d < 3; ++d) {
-        T[idx].sig[d] = R(g[GEO_SIG + d]);
-        split_hl(g[GEO_C + d], T[idx].chi[d], T[idx].clo[d]);
-        T[idx].v[d] = tri[3 * tg + d];
-        T[idx].e[d] = tri_edge[3 * tg + d];
-      }
-      T[idx].invA = R(1.0 / g[GEO_A]);
-    }
-  }
+  load_test_tile(T, tile, tk.t0, geo, tri, tri_edge);
+  wave_tab_init(tab, tk.ki != 0.0);
   __syncthreads();
   const int s = tile.src0 + threadIdx.x;
   if (s >= tk.nsrc) return;
   const int sg = tk.s0 + s;
   const double* gs = geo + size_t(sg) * GEO_STRIDE;
-  R rs[18], Ws[6], bv[9], sg_[3], cshi[3], cslo[3];
+  R rs[18], cshi[3], cslo[3];
 #pragma unroll
   for (int d = 0; d < 18; ++d) rs[d] = R(gs[GEO_RHO + d]);
 #pragma unroll
-  for (int d = 0; d < 6; ++d) Ws[d] = R(gs[GEO_W + d]);
-#pragma unroll
-  for (int d = 0; d < 9; ++d) bv[d] = R(gs[GEO_AV + d]);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    sg_[d] = R(gs[GEO_SIG + d]);
-    split_hl(gs[GEO_C + d], cshi[d], cslo[d]);
-  }
-  const R invAs = R(1.0 / gs[GEO_A]);
+  for (int d = 0; d < 3; ++d) split_hl(gs[GEO_C + d], cshi[d], cslo[d]);
   const int32_t sv0 = tri[3 * sg], sv1 = tri[3 * sg + 1], sv2 = tri[3 * sg + 2];
-  const int32_t se[3] = {tri_edge[3 * sg], tri_edge[3 * sg + 1], tri_edge[3 * sg + 2]};
-  const R kr = R(tk.kr), ki = R(tk.ki);
+  const PairKernel<R> G(tab, tk.kr, tk.ki);
+  const bool lossy = tk.ki != 0.0;
+  const R sAr = R(tk.sAr * INV4PI), sAi = R(tk.sAi * INV4PI), sPr = R(tk.sPr * INV4PI), sPi = R(tk.sPi * INV4PI);
+  // the source's vertices: kept by FP32 fills, whose conversions they are; FP64 fills reload them per pair (registers)
+  constexpr bool KEEP = sizeof(R) == 4;
+  R bk[KEEP ? 9 : 1];
+  if constexpr (KEEP)
 #pragma unroll
-  for (int k = 0; k < 6; ++k) Ws[k] *= R(INV4PI);  // 1/(4 pi) of G folded into the source weights
-  const R sAr = R(tk.sAr), sAi = R(tk.sAi), sPr = R(tk.sPr), sPi = R(tk.sPi);
+    for (int d = 0; d < 9; ++d) bk[d] = R(gs[GEO_AV + d]);
 
-  for (int tt = 0; tt < tile_test<R>(); ++tt) {
-    if (tile.test0 + tt >= tk.ntest) break;
+  for (int tt = 0; tt < tile.ntest; ++tt) {
+    const int t = tile.test0 + tt;
+    if (tk.sym && s <= t) continue;
     const TestRec<R>& X = T[tt];
     // touching pairs (sharing a vertex) are computed by the FP64 extraction kernel
     bool touch = false;
@@ -182,74 +299,33 @@ __global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 5 : 1) fill_L_bulk(
     const R dc0 = (X.chi[0] - cshi[0]) + (X.clo[0] - cslo[0]);
     const R dc1 = (X.chi[1] - cshi[1]) + (X.clo[1] - cslo[1]);
     const R dc2 = (X.chi[2] - cshi[2]) + (X.clo[2] - cslo[2]);
-    R m0r = 0, m0i = 0, mqr[3] = {0, 0, 0}, mqi[3] = {0, 0, 0}, msr[3] = {0, 0, 0}, msi[3] = {0, 0, 0};
-    R mqsr = 0, mqsi = 0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const R px = dc0 + X.rho[3 * q], py = dc1 + X.rho[3 * q + 1], pz = dc2 + X.rho[3 * q + 2];
-      R ar = 0, ai = 0, br[3] = {0, 0, 0}, bi[3] = {0, 0, 0};
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const R dx = px - rs[3 * k], dy = py - rs[3 * k + 1], dz = pz - rs[3 * k + 2];
-        const R r2 = dx * dx + dy * dy + dz * dz;
-        const R ir = M<R>::rsqrt_(r2);
-        const R Rr = r2 * ir;
-        R sn, cn;
-        M<R>::sincos_(kr * Rr, &sn, &cn);
-        const R amp = (ki != R(0) ? M<R>::exp_(ki * Rr) : R(1)) * ir * Ws[k];
-        const R gr = amp * cn, gi = -amp * sn;
-        ar += gr;
-        ai += gi;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          br[d] += gr * rs[3 * k + d];
-          bi[d] += gi * rs[3 * k + d];
-        }
-      }
-      const R w = X.W[q];
-      m0r += w * ar;
-      m0i += w * ai;
-      R dotr = 0, doti = 0;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const R rq = X.rho[3 * q + d];
-        mqr[d] += w * ar * rq;
-        mqi[d] += w * ai * rq;
-        msr[d] += w * br[d];
-        msi[d] += w * bi[d];
-        dotr += rq * br[d];
-        doti += rq * bi[d];
-      }
-      mqsr += w * dotr;
-      mqsi += w * doti;
-    }
-    // local RWG x RWG: sig_i sig_j [Mqs + a_i.Ms + b_j.Mq + (a_i.b_j) M0]
+    R Nr[9], Ni[9];
+    if (lossy) pair_moments<R, false, true>(G, X, rs, dc0, dc1, dc2, Nr, Ni);
+    else pair_moments<R, false, false>(G, X, rs, dc0, dc1, dc2, Nr, Ni);
+    const R Sr = sum9(Nr), Si = sum9(Ni);
     if (tk.A) {
+      R bv[9];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const R ax = X.av[3 * i], ay = X.av[3 * i + 1], az = X.av[3 * i + 2];
-        const R ams_r = ax * msr[0] + ay * msr[1] + az * msr[2];
-        const R ams_i = ax * msi[0] + ay * msi[1] + az * msi[2];
-        const int64_t row = int64_t(X.e[i] - tk.e_row0) * tk.ldA;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const R bx = bv[3 * j], by = bv[3 * j + 1], bz = bv[3 * j + 2];
-          const R ab = ax * bx + ay * by + az * bz;
-          R vr = mqsr + ams_r + bx * mqr[0] + by * mqr[1] + bz * mqr[2] + ab * m0r;
-          R vi = mqsi + ams_i + bx * mqi[0] + by * mqi[1] + bz * mqi[2] + ab * m0i;
-          const R sc = X.sig[i] * sg_[j];
-          vr *= sc;
-          vi *= sc;
-          M<R>::add(tk.A, row + (se[j] - tk.e_col0), vr * sAr - vi * sAi, vr * sAi + vi * sAr);
-        }
+      for (int d = 0; d < 9; ++d) {
+        if constexpr (KEEP) bv[d] = bk[d];
+        else bv[d] = gs[GEO_AV + d];
       }
+      const int32_t se[3] = {tri_edge[3 * sg], tri_edge[3 * sg + 1], tri_edge[3 * sg + 2]};
+      contract_L(Nr, Ni, Sr, Si, X.av, bv, [&](int i, int j, R vr, R vi) {
+        const R sc = X.sgn[i] * half_sign<R>(gs[GEO_SIG + j]);
+        vr *= sc;
+        vi *= sc;
+        const R orr = vr * sAr - vi * sAi, oi = vr * sAi + vi * sAr;
+        const int64_t row = X.e[i] - tk.e_row0, col = se[j] - tk.e_col0;
+        M<R>::add(tk.A, row * tk.ldA + col, orr, oi);
+        if (tk.sym) M<R>::add(tk.A, col * tk.ldA + row, orr, oi);
+      });
     }
-    if (tk.P) {
-      const R sc = X.invA * invAs;
-      const R vr = m0r * sc, vi = m0i * sc;
-      const int t = tile.test0 + tt;
-      M<R>::store_r(tk.P, int64_t(t + tk.t0 - tk.t_row0) * tk.ldP + (sg - tk.t_col0), vr * sPr - vi * sPi,
-                    vr * sPi + vi * sPr);
+    if (tk.P) {  // 1/(A A') against the areas of the two integrals
+      const R vr = Sr * sPr - Si * sPi, vi = Sr * sPi + Si * sPr;
+      const int64_t row = t + tk.t0 - tk.t_row0, col = sg - tk.t_col0;
+      M<R>::store_r(tk.P, row * tk.ldP + col, vr, vi);
+      if (tk.sym) M<R>::store_r(tk.P, col * tk.ldP + row, vr, vi);
     }
   }
 }
@@ -361,30 +437,20 @@ __global__ void fill_L_touch(const LTask* __restrict__ tasks, const int32_t* __r
 }
 
 // ---------------------------------------------------------------- bulk Kbar kernel (primal test x child source)
+// FP64: bound by the FP64 pipe (ncu: 87% busy), 56 operations per evaluation for a real
+// wavenumber, 69 for a complex one.  320-triangle sphere: 3.47 ms (cross products and
+// four vector moments per evaluation, general sincos) -> 2.25 ms (real), 2.9 ms (complex).
 template <class R>
-__global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 5 : 1) fill_K_bulk(const KTask* __restrict__ tasks, const TileRef* __restrict__ tiles,
+__global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 4 : 2) fill_K_bulk(const KTask* __restrict__ tasks, const TileRef* __restrict__ tiles,
                                                         const double* __restrict__ geo, const double* __restrict__ bgeo,
                                                         const int32_t* __restrict__ tri, const int32_t* __restrict__ tri_edge,
                                                         const int32_t* __restrict__ btri_edge) {
   __shared__ TestRec<R> T[tile_test<R>()];
+  __shared__ typename PairKernel<R>::Tab tab;
   const TileRef tile = tiles[blockIdx.x];
   const KTask tk = tasks[tile.task];
-  for (int idx = threadIdx.x; idx < tile_test<R>(); idx += blockDim.x) {
-    int t = tile.test0 + idx;
-    if (t < tk.ntest) {
-      int tg = tk.t0 + t;
-      const double* g = geo + size_t(tg) * GEO_STRIDE;
-      for (int d = 0; d < 18; ++d) T[idx].rho[d] = R(g[GEO_RHO + d]);
-      for (int d = 0; d < 6; ++d) T[idx].W[d] = R(g[GEO_W + d]);
-      for (int d = 0; d < 9; ++d) T[idx].av[d] = R(g[GEO_AV + d]);
-      for (int d = 0; d < 3; ++d) {
-        T[idx].sig[d] = R(g[GEO_SIG + d]);
-        split_hl(g[GEO_C + d], T[idx].chi[d], T[idx].clo[d]);
-        T[idx].v[d] = tri[3 * tg + d];
-        T[idx].e[d] = tri_edge[3 * tg + d];
-      }
-    }
-  }
+  load_test_tile(T, tile, tk.t0, geo, tri, tri_edge);
+  wave_tab_init(tab, tk.ki != 0.0);
   __syncthreads();
   const int s = tile.src0 + threadIdx.x;
   if (s >= tk.nsrc) return;
@@ -393,100 +459,44 @@ __global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 5 : 1) fill_K_bulk(
   const int32_t cv = tri[3 * par + ((kk & 1) ? (pp + 1) % 3 : pp)];  // child's primal vertex
   const int32_t ce = tri_edge[3 * par + (pp + 2) % 3];                // edge of the child's midpoint
   const double* gs = bgeo + size_t(cg) * GEO_STRIDE;
-  R rs[18], Ws[6], bv[9], sg_[3], cshi[3], cslo[3];
+  R rs[18], cshi[3], cslo[3];
 #pragma unroll
   for (int d = 0; d < 18; ++d) rs[d] = R(gs[GEO_RHO + d]);
 #pragma unroll
-  for (int d = 0; d < 6; ++d) Ws[d] = R(gs[GEO_W + d]);
+  for (int d = 0; d < 3; ++d) split_hl(gs[GEO_C + d], cshi[d], cslo[d]);
+  const PairKernel<R> G(tab, tk.kr, tk.ki);
+  const bool lossy = tk.ki != 0.0;
+  constexpr bool KEEP = sizeof(R) == 4;  // as fill_L_bulk
+  R bk[KEEP ? 9 : 1];
+  if constexpr (KEEP)
 #pragma unroll
-  for (int d = 0; d < 9; ++d) bv[d] = R(gs[GEO_AV + d]);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    sg_[d] = R(gs[GEO_SIG + d]);
-    split_hl(gs[GEO_C + d], cshi[d], cslo[d]);
-  }
-  const int32_t be[3] = {btri_edge[3 * cg], btri_edge[3 * cg + 1], btri_edge[3 * cg + 2]};
-  const R kr = R(tk.kr), ki = R(tk.ki);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) Ws[k] *= R(INV4PI);  // 1/(4 pi) of grad G folded into the source weights
+    for (int d = 0; d < 9; ++d) bk[d] = R(gs[GEO_AV + d]);
 
-  for (int tt = 0; tt < tile_test<R>(); ++tt) {
+  for (int tt = 0; tt < tile.ntest; ++tt) {
     const int t = tile.test0 + tt;
-    if (t >= tk.ntest) break;
     const TestRec<R>& X = T[tt];
     if (tk.t0 + t == par) continue;  // child of the test triangle: coplanar, Kbar = 0
     bool touch = false;
 #pragma unroll
     for (int i = 0; i < 3; ++i) touch |= (X.v[i] == cv) | (X.e[i] == ce);
     if (touch) continue;  // FP64 extraction kernel
-    const R dc0 = (X.chi[0] - cshi[0]) + (X.clo[0] - cslo[0]);
-    const R dc1 = (X.chi[1] - cshi[1]) + (X.clo[1] - cslo[1]);
-    const R dc2 = (X.chi[2] - cshi[2]) + (X.clo[2] - cslo[2]);
-    R p1r = 0, p1i = 0, p2r[3] = {0, 0, 0}, p2i[3] = {0, 0, 0}, xr[3] = {0, 0, 0}, xi[3] = {0, 0, 0};
-    R sr[3] = {0, 0, 0}, si[3] = {0, 0, 0};
+    R dc[3];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const R rqx = X.rho[3 * q], rqy = X.rho[3 * q + 1], rqz = X.rho[3 * q + 2];
-      const R px = dc0 + rqx, py = dc1 + rqy, pz = dc2 + rqz;
-      R ur[3] = {0, 0, 0}, ui[3] = {0, 0, 0}, vr[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
+    for (int d = 0; d < 3; ++d) dc[d] = (X.chi[d] - cshi[d]) + (X.clo[d] - cslo[d]);
+    R Nr[9], Ni[9];
+    if (lossy) pair_moments<R, true, true>(G, X, rs, dc[0], dc[1], dc[2], Nr, Ni);
+    else pair_moments<R, true, false>(G, X, rs, dc[0], dc[1], dc[2], Nr, Ni);
+    R bv[9];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const R dx = px - rs[3 * k], dy = py - rs[3 * k + 1], dz = pz - rs[3 * k + 2];
-        const R r2 = dx * dx + dy * dy + dz * dz;
-        const R ir = M<R>::rsqrt_(r2);
-        const R Rr = r2 * ir;
-        R sn, cn;
-        M<R>::sincos_(kr * Rr, &sn, &cn);
-        const R amp = (ki != R(0) ? M<R>::exp_(ki * Rr) : R(1)) * ir * ir * ir * Ws[k];
-        // g1 = -(1 + j k R) exp(-j k R) / (4 pi R^3)
-        const R er = amp * cn, ei = -amp * sn;
-        const R ar = R(1) - ki * Rr, ai = kr * Rr;
-        const R g1r = -(ar * er - ai * ei), g1i = -(ar * ei + ai * er);
-        // D x rho'
-        const R cx = dy * rs[3 * k + 2] - dz * rs[3 * k + 1];
-        const R cy = dz * rs[3 * k] - dx * rs[3 * k + 2];
-        const R cz = dx * rs[3 * k + 1] - dy * rs[3 * k];
-        ur[0] += g1r * cx; ui[0] += g1i * cx;
-        ur[1] += g1r * cy; ui[1] += g1i * cy;
-        ur[2] += g1r * cz; ui[2] += g1i * cz;
-        vr[0] += g1r * dx; vi[0] += g1i * dx;
-        vr[1] += g1r * dy; vi[1] += g1i * dy;
-        vr[2] += g1r * dz; vi[2] += g1i * dz;
-      }
-      const R w = X.W[q];
-      p1r += w * (rqx * ur[0] + rqy * ur[1] + rqz * ur[2]);
-      p1i += w * (rqx * ui[0] + rqy * ui[1] + rqz * ui[2]);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        p2r[d] += w * ur[d];
-        p2i[d] += w * ui[d];
-        sr[d] += w * vr[d];
-        si[d] += w * vi[d];
-      }
-      // rho_q x V
-      xr[0] += w * (rqy * vr[2] - rqz * vr[1]); xi[0] += w * (rqy * vi[2] - rqz * vi[1]);
-      xr[1] += w * (rqz * vr[0] - rqx * vr[2]); xi[1] += w * (rqz * vi[0] - rqx * vi[2]);
-      xr[2] += w * (rqx * vr[1] - rqy * vr[0]); xi[2] += w * (rqx * vi[1] - rqy * vi[0]);
+    for (int d = 0; d < 9; ++d) {
+      if constexpr (KEEP) bv[d] = bk[d];
+      else bv[d] = gs[GEO_AV + d];
     }
-    // local: sig_i sig'_j [P1 + a_i.P2 + b_j.X + b_j.(a_i x S)]
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const R ax = X.av[3 * i], ay = X.av[3 * i + 1], az = X.av[3 * i + 2];
-      const R baser = p1r + ax * p2r[0] + ay * p2r[1] + az * p2r[2];
-      const R basei = p1i + ax * p2i[0] + ay * p2i[1] + az * p2i[2];
-      // a_i x S
-      const R csr0 = ay * sr[2] - az * sr[1], csr1 = az * sr[0] - ax * sr[2], csr2 = ax * sr[1] - ay * sr[0];
-      const R csi0 = ay * si[2] - az * si[1], csi1 = az * si[0] - ax * si[2], csi2 = ax * si[1] - ay * si[0];
-      const int64_t row = int64_t(X.e[i] - tk.e_row0) * tk.ld;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const R bx = bv[3 * j], by = bv[3 * j + 1], bz = bv[3 * j + 2];
-        R vr_ = baser + bx * (xr[0] + csr0) + by * (xr[1] + csr1) + bz * (xr[2] + csr2);
-        R vi_ = basei + bx * (xi[0] + csi0) + by * (xi[1] + csi1) + bz * (xi[2] + csi2);
-        const R sc = X.sig[i] * sg_[j];
-        M<R>::add(tk.Kb, row + (be[j] - tk.b_col0), vr_ * sc, vi_ * sc);
-      }
-    }
+    const int32_t be[3] = {btri_edge[3 * cg], btri_edge[3 * cg + 1], btri_edge[3 * cg + 2]};
+    contract_K(Nr, Ni, X.av, bv, dc, [&](int i, int j, R vr, R vi) {
+      const R sc = X.sgn[i] * (half_sign<R>(gs[GEO_SIG + j]) * R(INV4PI));
+      M<R>::add(tk.Kb, int64_t(X.e[i] - tk.e_row0) * tk.ld + (be[j] - tk.b_col0), vr * sc, vi * sc);
+    });
   }
 }
 
@@ -643,8 +653,34 @@ static std::vector<int32_t> unsplit_object_tasks(const HostMesh& h, const std::v
   return ot;
 }
 
+// Tiles of the unsplit tasks.  Few pairs leave SMs without a CTA, so the test
+// triangles of a tile are halved until there are TILES_WANTED tiles (four per
+// SM slot of two CTAs) or one test triangle each; FP32 tiles stay at 8 or more, whose
+// source conversions cost as much as two pairs.
+constexpr size_t TILES_WANTED = 152 * 8;
+static bool is_sym(const LTask& t) { return t.sym != 0; }
+static bool is_sym(const KTask&) { return false; }
+template <class R, class T>
+static std::vector<TileRef> bulk_tiles(const std::vector<T>& tasks, const std::vector<char>& split) {
+  std::vector<TileRef> tiles;
+  const int least = sizeof(R) == 4 ? 8 : 1;
+  for (int tt = tile_test<R>();; tt /= 2) {
+    tiles.clear();
+    for (size_t i = 0; i < tasks.size(); ++i) {
+      if (split[i]) continue;
+      const T& k = tasks[i];
+      for (int t0 = 0; t0 < k.ntest; t0 += tt)
+        for (int s0 = 0; s0 < k.nsrc; s0 += TILE_SRC) {
+          if (is_sym(k) && s0 + TILE_SRC <= t0 + 1) continue;  // every s <= t
+          tiles.push_back({int32_t(i), t0, s0, std::min(tt, k.ntest - t0)});
+        }
+    }
+    if (tiles.size() >= TILES_WANTED || tt / 2 < least) return tiles;
+  }
+}
+
 template <class R>
-void fill_L(const sldm_mesh* m, const std::vector<LTask>& tasks, cudaStream_t s) {
+void fill_L(const sldm_mesh* m, std::vector<LTask> tasks, cudaStream_t s) {
   if (tasks.empty()) return;
   std::vector<SplitRules> rules(tasks.size());
   std::vector<char> split(tasks.size(), 0);
@@ -652,12 +688,9 @@ void fill_L(const sldm_mesh* m, const std::vector<LTask>& tasks, cudaStream_t s)
     rules[i] = split_rules_L(m->h, tasks[i]);
     split[i] = rules[i].split;
   }
-  std::vector<TileRef> tiles;
-  for (size_t i = 0; i < tasks.size(); ++i) {
-    if (split[i]) continue;
-    for (int t0 = 0; t0 < tasks[i].ntest; t0 += tile_test<R>())
-      for (int s0 = 0; s0 < tasks[i].nsrc; s0 += TILE_SRC) tiles.push_back({int32_t(i), t0, s0, 0});
-  }
+  for (LTask& t : tasks)
+    t.sym = t.t0 == t.s0 && t.ntest == t.nsrc && t.e_row0 == t.e_col0 && t.t_row0 == t.t_col0;
+  const std::vector<TileRef> tiles = bulk_tiles<R>(tasks, split);
   DBuf<LTask> dt;
   DBuf<TileRef> dtl;
   dt.upload(tasks, s);
@@ -701,12 +734,7 @@ void fill_K(const sldm_mesh* m, const std::vector<KTask>& tasks, cudaStream_t s)
     rules[i] = split_rules_K(m->h, tasks[i]);
     split[i] = rules[i].split;
   }
-  std::vector<TileRef> tiles;
-  for (size_t i = 0; i < tasks.size(); ++i) {
-    if (split[i]) continue;
-    for (int t0 = 0; t0 < tasks[i].ntest; t0 += tile_test<R>())
-      for (int s0 = 0; s0 < tasks[i].nsrc; s0 += TILE_SRC) tiles.push_back({int32_t(i), t0, s0, 0});
-  }
+  const std::vector<TileRef> tiles = bulk_tiles<R>(tasks, split);
   DBuf<KTask> dt;
   DBuf<TileRef> dtl;
   dt.upload(tasks, s);
@@ -1076,8 +1104,8 @@ void farfield_layered(const sldm_mesh* m, const double2* jd, int64_t ldj, int nr
   SLDM_CUDA(cudaGetLastError());
 }
 
-template void fill_L<float>(const sldm_mesh*, const std::vector<LTask>&, cudaStream_t);
-template void fill_L<double>(const sldm_mesh*, const std::vector<LTask>&, cudaStream_t);
+template void fill_L<float>(const sldm_mesh*, std::vector<LTask>, cudaStream_t);
+template void fill_L<double>(const sldm_mesh*, std::vector<LTask>, cudaStream_t);
 template void fill_K<float>(const sldm_mesh*, const std::vector<KTask>&, cudaStream_t);
 template void fill_K<double>(const sldm_mesh*, const std::vector<KTask>&, cudaStream_t);
 template void contract_bc<float>(const sldm_mesh*, int, const void*, int64_t, void*, int64_t, cudaStream_t);
@@ -1228,10 +1256,13 @@ static void* noalloc_scratch(int dev) {
 }
 
 // Writes the task record and the tile list of one object into the scratch.
-__global__ void noalloc_setup_kernel(KTask task, int ntile_t, int ntile_s, KTask* dtask, TileRef* dtiles) {
+__global__ void noalloc_setup_kernel(KTask task, int tt, int ntile_t, int ntile_s, KTask* dtask, TileRef* dtiles) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) *dtask = task;
-  if (i < ntile_t * ntile_s) dtiles[i] = TileRef{0, (i / ntile_s) * TILE_TEST, (i % ntile_s) * TILE_SRC, 0};
+  if (i < ntile_t * ntile_s) {
+    const int t0 = (i / ntile_s) * tt;
+    dtiles[i] = TileRef{0, t0, (i % ntile_s) * TILE_SRC, min(tt, task.ntest - t0)};
+  }
 }
 
 }  // namespace sldm
@@ -1249,7 +1280,12 @@ extern "C" int sldm_kbar_noalloc(const sldm_mesh* m, int32_t obj, double k_re, d
     const int t0 = h.tri_begin[obj], nt_o = h.tri_begin[obj + 1] - t0;
     const int e0 = h.edge_begin[obj], ne_o = h.edge_begin[obj + 1] - e0;
     const int b0 = h.bedge_begin[obj], nbe_o = h.bedge_begin[obj + 1] - b0;
-    const int ntile_t = (nt_o + TILE_TEST - 1) / TILE_TEST, ntile_s = (6 * nt_o + TILE_SRC - 1) / TILE_SRC;
+    // test triangles per tile: halved while the tiles are few (as bulk_tiles) and fit the list
+    const int ntile_s = (6 * nt_o + TILE_SRC - 1) / TILE_SRC;
+    int tt = TILE_TEST;
+    auto ntiles = [&](int w) { return size_t((nt_o + w - 1) / w) * ntile_s; };
+    while (tt > 1 && ntiles(tt) < TILES_WANTED && ntiles(tt / 2) <= NOALLOC_MAX_TILES) tt /= 2;
+    const int ntile_t = (nt_o + tt - 1) / tt;
     const size_t nkb = size_t(ne_o) * size_t(nbe_o);
     SLDM_REQUIRE(nkb <= NOALLOC_MAX_KB && size_t(ntile_t) * ntile_s <= NOALLOC_MAX_TILES, SLDM_EINVAL,
                  "kbar_noalloc: object too large for the fixed scratch (edges x barycentric edges = " +
@@ -1270,7 +1306,7 @@ extern "C" int sldm_kbar_noalloc(const sldm_mesh* m, int32_t obj, double k_re, d
     // the block accumulates atomically: it must start at zero on every call
     SLDM_CUDA(cudaMemsetAsync(Kb, 0, nkb * sizeof(double2), s));
     const int nset = ntile_t * ntile_s;
-    noalloc_setup_kernel<<<(nset + 127) / 128, 128, 0, s>>>(t, ntile_t, ntile_s, dtask, dtiles), ::sldm::count_launch();
+    noalloc_setup_kernel<<<(nset + 127) / 128, 128, 0, s>>>(t, tt, ntile_t, ntile_s, dtask, dtiles), ::sldm::count_launch();
     SLDM_CUDA(cudaGetLastError());
     const DevMesh& d = m->d;
     fill_K_bulk<double><<<unsigned(nset), TILE_SRC, 0, s>>>(dtask, dtiles, d.geo.p, d.bgeo.p, d.tri.p, d.tri_edge.p,

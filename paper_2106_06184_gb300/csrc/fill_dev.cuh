@@ -75,6 +75,190 @@ __device__ __forceinline__ void add_d(void* base, int64_t idx, double re, double
   M<R>::add(base, idx, R(re), R(im));
 }
 
+// ---------------------------------------------------------------- FP64 kernel evaluations
+// This part issues two FP64 operations per SM and clock (a warp instruction every
+// 16 clocks) beside 128 FP32 or integer ones, so an FP64 fill costs what its FP64
+// instructions cost.  exp(-j k R) therefore takes its argument in steps of a
+// table, y = R (k 256 / 2 pi): the nearest step n and the remainder f = y - n come
+// from adding and subtracting 1.5 2^52 (exact for |y| < 2^51), the table of the 256
+// roots of unity lies in shared memory, and the remainder (an angle below
+// pi / 256) needs three Taylor terms of sin and cos each to 1e-17:
+// 14 FP64 operations, against ~35 of the general sincos, whose argument may have
+// any size.  exp(Im k R) the same way from 256 powers of two (9 operations).
+constexpr int WAVE_N = 256;
+struct WaveTab {
+  double2 cs[WAVE_N];  // (cos, sin)(2 pi i / 256)
+  double ex[WAVE_N];   // 2^(i / 256)
+};
+// Fills the tables of a CTA (call with every thread, then __syncthreads).  The
+// roots of one octant are computed, the others are their reflections.
+__device__ __forceinline__ void wave_tab_fill(WaveTab& T, bool lossy) {
+  for (int i = threadIdx.x; i <= WAVE_N / 8; i += blockDim.x) {
+    double sn, cn;
+    sincospi(double(i) / (WAVE_N / 2), &sn, &cn);
+    T.cs[i] = make_double2(cn, sn);
+    T.cs[64 - i] = make_double2(sn, cn);
+    T.cs[64 + i] = make_double2(-sn, cn);
+    T.cs[128 - i] = make_double2(-cn, sn);
+    T.cs[128 + i] = make_double2(-cn, -sn);
+    T.cs[192 - i] = make_double2(-sn, -cn);
+    T.cs[192 + i] = make_double2(sn, -cn);
+    T.cs[(WAVE_N - i) & (WAVE_N - 1)] = make_double2(cn, -sn);
+  }
+  if (lossy)
+    for (int i = threadIdx.x; i < WAVE_N; i += blockDim.x) T.ex[i] = exp2(double(i) / WAVE_N);
+}
+static_assert(WAVE_N == 256, "octant reflections above");
+// (cos, sin) of y steps of 2 pi / 256
+__device__ __forceinline__ void wave_cis(const WaveTab& T, double y, double& c, double& s) {
+  constexpr double H = 2.0 * PI / WAVE_N, H2 = H * H;
+  const double t = __dadd_rn(y, 6755399441055744.0);
+  const double f = __dsub_rn(y, __dsub_rn(t, 6755399441055744.0));
+  const double2 w = T.cs[__double2loint(t) & (WAVE_N - 1)];
+  const double f2 = f * f;
+  const double sf = f * fma(f2, fma(f2, H * H2 * H2 / 120.0, -H * H2 / 6.0), H);
+  const double cf = f2 * fma(f2, fma(f2, -H2 * H2 * H2 / 720.0, H2 * H2 / 24.0), -H2 / 2.0);  // cos - 1
+  c = fma(-w.y, sf, fma(w.x, cf, w.x));
+  s = fma(w.x, sf, fma(w.y, cf, w.y));
+}
+// 2^(y / 256); 0 or infinity where that leaves the normal range
+__device__ __forceinline__ double wave_exp2(const WaveTab& T, double y) {
+  constexpr double L = 0.69314718055994530942 / WAVE_N;
+  const double t = __dadd_rn(y, 6755399441055744.0);
+  const double f = __dsub_rn(y, __dsub_rn(t, 6755399441055744.0));
+  const int n = __double2loint(t), yh = __double2hiint(y);
+  const double w = T.ex[n & (WAVE_N - 1)];
+  const double p = f * fma(f, fma(f, fma(f, L * L * L * L / 24.0, L * L * L / 6.0), L * L / 2.0), L);
+  const double v = fma(w, p, w);
+  int hi = __double2hiint(v) + ((n >> 8) << 20), lo = __double2loint(v);
+  if ((yh & 0x7fffffff) >= 0x410fe800) {  // |y| >= 1021 x 256
+    hi = yh < 0 ? 0 : 0x7ff00000;
+    lo = 0;
+  }
+  return __hiloint2double(hi, lo);
+}
+// 1 / sqrt(x), x > 0: the special-function unit's 2^-20 estimate and one step of
+// Householder's third-order iteration (error cubed: below the rounding)
+__device__ __forceinline__ double rsqrt_pos(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(fma(e, 0.375, 0.5) * e, y, y);
+}
+
+__device__ __forceinline__ double bound_radius(const double* c, const double* p0, const double* p1, const double* p2) {
+  double r = 0.0;
+  const double* P[3] = {p0, p1, p2};
+  for (int i = 0; i < 3; ++i) {
+    const double dx = P[i][0] - c[0], dy = P[i][1] - c[1], dz = P[i][2] - c[2];
+    r = fmax(r, sqrt(dx * dx + dy * dy + dz * dz));
+  }
+  return r;
+}
+
+// ---------------------------------------------------------------- contraction of a pair's moments
+// N[u][v] = int int lambda_u lambda'_v kernel / (A A') holds all a pair needs: the local
+// RWGs are s_i (r - V_i) / (2 A) with r = sum_u lambda_u V_u, so the areas cancel
+// (factors s_i s_j / 4 remain: half_sign).  Vertices enter as a_i = c - V_i (GEO_AV).
+template <class R>
+__device__ __forceinline__ R half_sign(double sig) {  // on the sign bit: no FP64 compare
+  return __double2hiint(sig) < 0 ? R(-0.5) : R(0.5);
+}
+template <class R>
+__device__ __forceinline__ R sum9(const R (&n)[9]) {
+  return ((n[0] + n[1]) + (n[2] + n[3])) + ((n[4] + n[5]) + (n[6] + n[7])) + n[8];
+}
+// put(i, j, value): sum_uv N_uv (V_u - V_i).(V'_v - V'_j) = T - P_i - Q_j + S D_ij, D_uv = V_u . V'_v,
+// P_i = sum_v (sum_u N_uv) D_iv, Q_j = sum_u (sum_v N_uv) D_uj, T = sum N D
+template <class R, class Put>
+__device__ __forceinline__ void contract_L(const R (&Nr)[9], const R (&Ni)[9], R Sr, R Si, const R* av, const R* bv, Put put) {
+  R D[9], Pr[3], Pi[3], Qr[3], Qi[3], Tr = 0, Ti = 0;
+#pragma unroll
+  for (int v = 0; v < 3; ++v)
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      D[3 * u + v] = av[3 * u] * bv[3 * v] + av[3 * u + 1] * bv[3 * v + 1] + av[3 * u + 2] * bv[3 * v + 2];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    Pr[i] = Pi[i] = Qr[i] = Qi[i] = R(0);
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      Pr[i] += (Nr[w] + Nr[3 + w] + Nr[6 + w]) * D[3 * i + w];
+      Pi[i] += (Ni[w] + Ni[3 + w] + Ni[6 + w]) * D[3 * i + w];
+      Qr[i] += (Nr[3 * w] + Nr[3 * w + 1] + Nr[3 * w + 2]) * D[3 * w + i];
+      Qi[i] += (Ni[3 * w] + Ni[3 * w + 1] + Ni[3 * w + 2]) * D[3 * w + i];
+      Tr += Nr[3 * i + w] * D[3 * i + w];
+      Ti += Ni[3 * i + w] * D[3 * i + w];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      put(i, j, (Tr - Pr[i]) - (Qr[j] - Sr * D[3 * i + j]), (Ti - Pi[i]) - (Qi[j] - Si * D[3 * i + j]));
+}
+// put(i, j, value): sum_uv N_uv (V_i - V'_j).((V'_v - V'_j) x (V_u - V_i)), the moments N of g1, from
+// (r - V_i).((r - r') x (r' - V'_j)) = (V_i - V'_j).((r' - V'_j) x (r - V_i)).  With local vertices,
+// dc = c - c', A = sum N V'_v, B = sum N V_u, X = sum N V'_v x V_u, S = sum N, q_ij = V_i x V'_j it is
+// dc.X + V_i.X - V'_j.X - B.(dc x V'_j) - A.(V_i x dc) + (A - B - S dc).q_ij
+template <class R, class Put>
+__device__ __forceinline__ void contract_K(const R (&Nr)[9], const R (&Ni)[9], const R* av, const R* bv, const R* dc, Put put) {
+  R Ar[3] = {0, 0, 0}, Ai[3] = {0, 0, 0}, Br[3] = {0, 0, 0}, Bi[3] = {0, 0, 0}, Xr[3] = {0, 0, 0}, Xi[3] = {0, 0, 0};
+  R Sr = 0, Si = 0;
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    R cr[3], ci[3];  // sum_v N_uv b_v
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      cr[d] = Nr[3 * u] * bv[d] + Nr[3 * u + 1] * bv[3 + d] + Nr[3 * u + 2] * bv[6 + d];
+      ci[d] = Ni[3 * u] * bv[d] + Ni[3 * u + 1] * bv[3 + d] + Ni[3 * u + 2] * bv[6 + d];
+      Ar[d] += cr[d];
+      Ai[d] += ci[d];
+    }
+    const R rr = Nr[3 * u] + Nr[3 * u + 1] + Nr[3 * u + 2], ri = Ni[3 * u] + Ni[3 * u + 1] + Ni[3 * u + 2];
+    Sr += rr;
+    Si += ri;
+    const R* a = av + 3 * u;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int d1 = (d + 1) % 3, d2 = (d + 2) % 3;
+      Br[d] += rr * a[d];
+      Bi[d] += ri * a[d];
+      Xr[d] += cr[d1] * a[d2] - cr[d2] * a[d1];
+      Xi[d] += ci[d1] * a[d2] - ci[d2] * a[d1];
+    }
+  }
+  // a, b have the opposite sign of V, V': A and B above hold -A and -B, X and q are even
+  R Fr[3], Fi[3];  // A - B - S dc
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Fr[d] = (Br[d] - Ar[d]) - Sr * dc[d];
+    Fi[d] = (Bi[d] - Ai[d]) - Si * dc[d];
+  }
+  const R cxr = dc[0] * Xr[0] + dc[1] * Xr[1] + dc[2] * Xr[2], cxi = dc[0] * Xi[0] + dc[1] * Xi[1] + dc[2] * Xi[2];
+  R hr[3], hi[3];  // the source's part
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const R bx = bv[3 * j], by = bv[3 * j + 1], bz = bv[3 * j + 2];
+    const R px = dc[1] * bz - dc[2] * by, py = dc[2] * bx - dc[0] * bz, pz = dc[0] * by - dc[1] * bx;
+    hr[j] = (bx * Xr[0] + by * Xr[1] + bz * Xr[2]) - (Br[0] * px + Br[1] * py + Br[2] * pz);
+    hi[j] = (bx * Xi[0] + by * Xi[1] + bz * Xi[2]) - (Bi[0] * px + Bi[1] * py + Bi[2] * pz);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const R ax = av[3 * i], ay = av[3 * i + 1], az = av[3 * i + 2];
+    const R px = ay * dc[2] - az * dc[1], py = az * dc[0] - ax * dc[2], pz = ax * dc[1] - ay * dc[0];
+    const R tr = cxr - (ax * Xr[0] + ay * Xr[1] + az * Xr[2]) - (Ar[0] * px + Ar[1] * py + Ar[2] * pz);
+    const R ti = cxi - (ax * Xi[0] + ay * Xi[1] + az * Xi[2]) - (Ai[0] * px + Ai[1] * py + Ai[2] * pz);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const R bx = bv[3 * j], by = bv[3 * j + 1], bz = bv[3 * j + 2];
+      const R qx = ay * bz - az * by, qy = az * bx - ax * bz, qz = ax * by - ay * bx;
+      put(i, j, tr + hr[j] + (Fr[0] * qx + Fr[1] * qy + Fr[2] * qz), ti + hi[j] + (Fi[0] * qx + Fi[1] * qy + Fi[2] * qz));
+    }
+  }
+}
+
 // ---------------------------------------------------------------- FP64 closed forms
 // Integrals over the flat triangle (p1, p2, p3) seen from r: each surface
 // integral is reduced to a sum over the three edges with the surface divergence

@@ -76,16 +76,6 @@ __device__ __forceinline__ void src_point(const SrcPoint& b, const double ev[3][
   for (int d = 0; d < 3; ++d) rp[d] = b.x * ev[0][d] + b.y * ev[1][d] + b.z * ev[2][d];
 }
 
-__device__ __forceinline__ double bound_radius(const double* c, const double* p0, const double* p1, const double* p2) {
-  double r = 0.0;
-  const double* P[3] = {p0, p1, p2};
-  for (int i = 0; i < 3; ++i) {
-    const double dx = P[i][0] - c[0], dy = P[i][1] - c[1], dz = P[i][2] - c[2];
-    r = fmax(r, sqrt(dx * dx + dy * dy + dz * dz));
-  }
-  return r;
-}
-
 // ---------------------------------------------------------------- L^A, L^phi
 template <class R>
 __global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __restrict__ soff,

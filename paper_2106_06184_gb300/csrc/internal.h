@@ -145,6 +145,7 @@ struct DevMesh {
   // geometry computed on the device (see fill.cu: geometry_kernel)
   DBuf<double> geo;   // per triangle: GEO_STRIDE doubles
   DBuf<double> bgeo;  // per child: BGEO_STRIDE doubles
+  DBuf<double> rad, brad;  // largest distance of a vertex from the centroid, per triangle and per child
 };
 
 // Per-triangle geometry record (doubles): centroid(3) area(1) normal(3)
@@ -196,6 +197,7 @@ struct LTask {
   void* P;                    // L^phi destination or null
   double kr, ki;              // wavenumber
   double sAr, sAi, sPr, sPi;  // complex scale of L^A and L^phi
+  int32_t sym, pad;           // same test and source set (set by fill_L): half the pairs, scattered twice
 };
 struct KTask {
   int32_t t0, ntest;          // primal test triangles
@@ -207,7 +209,7 @@ struct KTask {
 };
 
 template <class R>
-void fill_L(const sldm_mesh* m, const std::vector<LTask>& tasks, cudaStream_t s);
+void fill_L(const sldm_mesh* m, std::vector<LTask> tasks, cudaStream_t s);
 template <class R>
 void fill_K(const sldm_mesh* m, const std::vector<KTask>& tasks, cudaStream_t s);
 
