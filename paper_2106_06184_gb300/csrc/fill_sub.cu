@@ -8,11 +8,12 @@
 // Kbar the static grad 1/(4 pi R) is extracted as always.  Pairs whose bounding
 // spheres are farther apart than 40/|Im k| are dropped (G has decayed below e^-40).
 //
-// One warp per (test, source) pair: the lanes stride over the 6 x (points of
-// the source's rule) (test point, source point) pairs, the lanes 0..5 add the closed forms
-// of test point q = lane on touching pairs, the moments are summed with
-// shuffles, and lane 0 scatters the 3x3 local block as the unsplit kernels do.
-// Everything is FP64; the destination precision is R.
+// Pairs that do not touch (all but ~15 per triangle): fill_split_bulk, FP64-pipe
+// bound like the unsplit bulk fill and built from the same moments (fill_dev.cuh).
+// Touching pairs: one warp per pair, the lanes stride over the 6 x (points of the
+// source's rule) (test point, source point) pairs, lanes 0..5 add the closed
+// forms of test point q = lane, the moments are summed with shuffles, and lane 0
+// scatters the 3x3 local block.  Everything is FP64; the destination precision is R.
 #include <algorithm>
 #include <string>
 #include <vector>
@@ -53,54 +54,208 @@ __device__ cd green_smooth1(cd k, double R) {
   return {(ex * cn - 1.0) * INV4PI / R, -ex * sn * INV4PI / R};
 }
 
-// G = exp(-j k R)/(4 pi R), from R and 1/R (no division on the FP64 pipe)
-__device__ __forceinline__ cd green_full(cd k, double R, double iR) {
-  double sn, cn;
-  sincos(k.r * R, &sn, &cn);
-  const double a = exp(k.i * R) * INV4PI * iR;
-  return {a * cn, -a * sn};
-}
-
-// g1 of grad G = (r - r') g1 = -(1 + j k R) exp(-j k R)/(4 pi R^3)
-__device__ __forceinline__ cd grad_full(cd k, double R, double iR) {
-  double sn, cn;
-  sincos(k.r * R, &sn, &cn);
-  const double a = exp(k.i * R) * INV4PI * (iR * iR * iR);
-  const cd e = {a * cn, -a * sn};
-  const cd f = {1.0 - k.i * R, k.r * R};  // 1 + j k R
-  const cd p = cmul(f, e);
-  return {-p.r, -p.i};
-}
-
 __device__ __forceinline__ void src_point(const SrcPoint& b, const double ev[3][3], double rp[3]) {
   for (int d = 0; d < 3; ++d) rp[d] = b.x * ev[0][d] + b.y * ev[1][d] + b.z * ev[2][d];
 }
 
-// ---------------------------------------------------------------- L^A, L^phi
+// ---------------------------------------------------------------- pairs that do not touch
+// A CTA takes one block of SB sources against TB test triangles, one test after the
+// other.  Sources are listed by the size of their rule, so the groups of 8 lanes
+// of a warp, one per pair, run alike; a pair beyond the cutoff or touching is left
+// out before it is given a group.  A lane takes every 8th point of the source's
+// rule against all 6 test points; the 9 moments are summed over the group by a
+// transposing exchange (21 additions) and left in shared memory, and then one lane
+// per pair contracts and scatters them, so that those ~450 (Kbar) operations run
+// with full warps.  Bound by the FP64 pipe, ~70 operations per evaluation.  Against one
+// warp per pair (20 moments of r and r', 36 units on 32 lanes, bounding radii and the
+// contraction per pair), the 2,048-triangle copper wire at 3 GHz: Kbar 851 -> 166 ms,
+// L 239 -> 73 ms.
+constexpr int SPLIT_THREADS = 128, SPLIT_SB = 64, SPLIT_TB = 8;
+
+struct SplitTab {
+  const int32_t* order;  // sources by rule size
+  const int32_t* off;    // a source's points: pts[off[s] .. off[s + 1])
+  const SrcPoint* pts;
+};
+
+// sum over groups of 8 lanes: lane l & 7 receives the totals of v[3 (l & 7) .. + 2]
+template <int O, int N>
+__device__ __forceinline__ void grp_fold(double (&v)[24], int lane) {
+  const bool up = lane & O;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const double send = up ? v[i] : v[i + N];
+    const double keep = up ? v[i + N] : v[i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+  }
+}
+__device__ __forceinline__ void grp_tsum8(double (&v)[24], int lane) {
+  grp_fold<4, 12>(v, lane);
+  grp_fold<2, 6>(v, lane);
+  grp_fold<1, 3>(v, lane);
+}
+
+// GRAD: Kbar (sources: children), else L.  TASK: KTask or LTask.
+template <class R, bool GRAD, class TASK>
+__global__ void __launch_bounds__(SPLIT_THREADS, 3) fill_split_bulk(TASK tk, SplitTab rules, const double* __restrict__ geo,
+                                                                    const double* __restrict__ sgeo, const double* __restrict__ rad,
+                                                                    const double* __restrict__ srad, const int32_t* __restrict__ tri,
+                                                                    const int32_t* __restrict__ tri_edge,
+                                                                    const int32_t* __restrict__ src_edge) {
+  constexpr double A1 = 0.108103018168070, B1 = 0.445948490915965, W1 = 0.223381589678011;
+  constexpr double A2 = 0.816847572980459, B2 = 0.091576213509771, W2 = 0.109951743655322;
+  __shared__ WaveTab tab;
+  __shared__ double mom[SPLIT_SB][25];  // 18 used; odd stride
+  __shared__ int32_t act[SPLIT_SB];
+  __shared__ int nact;
+  wave_tab_fill(tab, true);
+  const int lane = threadIdx.x & 31, g8 = threadIdx.x & 7;
+  const int sb = blockIdx.y * SPLIT_SB;
+  int src0, nsrc;
+  if constexpr (GRAD) src0 = tk.c0, nsrc = tk.nsrc;
+  else src0 = tk.s0, nsrc = tk.nsrc;
+  const double kr = tk.kr, ki = tk.ki;
+  const double ys = kr * (WAVE_N / (2.0 * PI)), ye = ki * (WAVE_N * 1.4426950408889634074);
+  for (int tt = 0; tt < SPLIT_TB; ++tt) {
+    const int tl = blockIdx.x * SPLIT_TB + tt;
+    if (tl >= tk.ntest) break;
+    const int t = tk.t0 + tl;
+    const double* gt = geo + size_t(t) * GEO_STRIDE;
+    if (threadIdx.x == 0) nact = 0;
+    __syncthreads();  // tables, and the last test's moments are consumed
+    if (threadIdx.x < SPLIT_SB && sb + int(threadIdx.x) < nsrc) {
+      const int s = src0 + rules.order[sb + threadIdx.x];
+      bool use = true;
+      if constexpr (GRAD) {
+        const int par = s / 6, kk = s % 6, pp = kk / 2;
+        const int32_t cv = tri[3 * par + ((kk & 1) ? (pp + 1) % 3 : pp)], ce = tri_edge[3 * par + (pp + 2) % 3];
+        use = par != t;  // a child of the test triangle is coplanar: Kbar = 0
+        for (int i = 0; i < 3; ++i) use &= tri[3 * t + i] != cv && tri_edge[3 * t + i] != ce;
+      } else {
+        for (int i = 0; i < 3; ++i)
+          for (int j = 0; j < 3; ++j) use &= tri[3 * t + i] != tri[3 * s + j];
+      }
+      const double* gs = sgeo + size_t(s) * GEO_STRIDE;
+      const double dx = gt[GEO_C] - gs[GEO_C], dy = gt[GEO_C + 1] - gs[GEO_C + 1], dz = gt[GEO_C + 2] - gs[GEO_C + 2];
+      if (fabs(ki) * (sqrt(dx * dx + dy * dy + dz * dz) - rad[t] - srad[s]) > R8_CUTOFF) use = false;
+      if (use) act[atomicAdd(&nact, 1)] = s;
+    }
+    __syncthreads();
+    const int na = nact;
+    for (int a0 = 0; a0 < na; a0 += SPLIT_THREADS / 8) {
+      const int a = a0 + int(threadIdx.x) / 8;
+      double v[24];
+#pragma unroll
+      for (int i = 0; i < 24; ++i) v[i] = 0.0;
+      if (a < na) {
+        const int s = act[a], sl = s - src0;
+        const double* gs = sgeo + size_t(s) * GEO_STRIDE;
+        const double d0 = gt[GEO_C] - gs[GEO_C], d1 = gt[GEO_C + 1] - gs[GEO_C + 1], d2 = gt[GEO_C + 2] - gs[GEO_C + 2];
+        double av[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) av[i] = gs[GEO_AV + i];
+        const int p1 = rules.off[sl + 1];
+        for (int p = rules.off[sl] + g8; p < p1; p += 8) {
+          const SrcPoint sp = rules.pts[p];
+          // r - r' = dc + rho_q - r'_local, r'_local = - sum lambda_v a_v
+          const double x = fma(sp.x, av[0], fma(sp.y, av[3], fma(sp.z, av[6], d0)));
+          const double y = fma(sp.x, av[1], fma(sp.y, av[4], fma(sp.z, av[7], d1)));
+          const double z = fma(sp.x, av[2], fma(sp.y, av[5], fma(sp.z, av[8], d2)));
+          double gr[6], gi[6];
+#pragma unroll
+          for (int q = 0; q < 6; ++q) {
+            const double dx = x + gt[GEO_RHO + 3 * q], dy = y + gt[GEO_RHO + 3 * q + 1], dz = z + gt[GEO_RHO + 3 * q + 2];
+            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            const double ir = rsqrt_pos(r2), Rr = r2 * ir;
+            double c, sn;
+            wave_cis(tab, ys * Rr, c, sn);
+            const double e = wave_exp2(tab, ye * Rr);
+            if constexpr (GRAD) {
+              const double am = -(ir * ir) * (ir * e), ai = kr * Rr, ar = fma(-ki, Rr, 1.0);
+              gr[q] = am * fma(ai, sn, ar * c);
+              gi[q] = am * fma(ai, c, -ar * sn);
+            } else {
+              const double am = ir * e;
+              gr[q] = am * c;
+              gi[q] = -am * sn;
+            }
+          }
+          const double tr = W1 * B1 * (gr[0] + gr[1] + gr[2]) + W2 * B2 * (gr[3] + gr[4] + gr[5]);
+          const double ti = W1 * B1 * (gi[0] + gi[1] + gi[2]) + W2 * B2 * (gi[3] + gi[4] + gi[5]);
+          const double wx = sp.w * sp.x, wy = sp.w * sp.y, wz = sp.w * sp.z;
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const double lr = fma(W1 * (A1 - B1), gr[u], fma(W2 * (A2 - B2), gr[u + 3], tr));
+            const double li = fma(W1 * (A1 - B1), gi[u], fma(W2 * (A2 - B2), gi[u + 3], ti));
+            v[3 * u] = fma(wx, lr, v[3 * u]);
+            v[3 * u + 1] = fma(wy, lr, v[3 * u + 1]);
+            v[3 * u + 2] = fma(wz, lr, v[3 * u + 2]);
+            v[9 + 3 * u] = fma(wx, li, v[9 + 3 * u]);
+            v[10 + 3 * u] = fma(wy, li, v[10 + 3 * u]);
+            v[11 + 3 * u] = fma(wz, li, v[11 + 3 * u]);
+          }
+        }
+      }
+      __syncwarp();
+      grp_tsum8(v, lane);
+      if (a < na)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) mom[a][3 * g8 + i] = v[i];
+    }
+    __syncthreads();
+    // one lane per pair
+    if (int(threadIdx.x) < na) {
+      const int s = act[threadIdx.x];
+      const double* gs = sgeo + size_t(s) * GEO_STRIDE;
+      double Nr[9], Ni[9], av[9], bv[9], dc[3];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        Nr[i] = mom[threadIdx.x][i];
+        Ni[i] = mom[threadIdx.x][9 + i];
+        av[i] = gt[GEO_AV + i];
+        bv[i] = gs[GEO_AV + i];
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) dc[d] = gt[GEO_C + d] - gs[GEO_C + d];
+      if constexpr (GRAD) {
+        contract_K(Nr, Ni, av, bv, dc, [&](int i, int j, double vr, double vi) {
+          const double sc = half_sign<double>(gt[GEO_SIG + i]) * (half_sign<double>(gs[GEO_SIG + j]) * INV4PI);
+          add_d<R>(tk.Kb, int64_t(tri_edge[3 * t + i] - tk.e_row0) * tk.ld + (src_edge[3 * s + j] - tk.b_col0), vr * sc, vi * sc);
+        });
+      } else {
+        const double Sr = sum9(Nr), Si = sum9(Ni);
+        if (tk.A)
+          contract_L(Nr, Ni, Sr, Si, av, bv, [&](int i, int j, double vr, double vi) {
+            const double sc = half_sign<double>(gt[GEO_SIG + i]) * (half_sign<double>(gs[GEO_SIG + j]) * INV4PI);
+            const cd out = cmul({vr * sc, vi * sc}, {tk.sAr, tk.sAi});
+            add_d<R>(tk.A, int64_t(tri_edge[3 * t + i] - tk.e_row0) * tk.ldA + (src_edge[3 * s + j] - tk.e_col0), out.r, out.i);
+          });
+        if (tk.P) {  // 1/(A A') against the areas of the two integrals
+          const cd out = cmul({Sr * INV4PI, Si * INV4PI}, {tk.sPr, tk.sPi});
+          M<R>::store(tk.P, int64_t(t - tk.t_row0) * tk.ldP + (s - tk.t_col0), out.r, out.i);
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------- L^A, L^phi, touching pairs
 template <class R>
-__global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __restrict__ soff,
+__global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __restrict__ pa, const int32_t* __restrict__ pb,
+                                                    int npairs, const int32_t* __restrict__ soff,
                                                     const SrcPoint* __restrict__ spts,
                                                     const double* __restrict__ geo, const double* __restrict__ xyz,
                                                     const int32_t* __restrict__ tri, const int32_t* __restrict__ tri_edge) {
   const int64_t pair = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (pair >= int64_t(tk.ntest) * tk.nsrc) return;  // whole warps
-  const int t = tk.t0 + int(pair / tk.nsrc), s = tk.s0 + int(pair % tk.nsrc);
+  if (pair >= npairs) return;  // whole warps
+  const int t = pa[pair], s = pb[pair];
+  if (t < tk.t0 || t >= tk.t0 + tk.ntest || s < tk.s0 || s >= tk.s0 + tk.nsrc) return;
   const double* gt = geo + size_t(t) * GEO_STRIDE;
   const double* gs = geo + size_t(s) * GEO_STRIDE;
   const int32_t sv[3] = {tri[3 * s], tri[3 * s + 1], tri[3 * s + 2]};
-  bool touch = false;
-  for (int i = 0; i < 3; ++i) {
-    const int32_t tv = tri[3 * t + i];
-    touch |= (tv == sv[0]) | (tv == sv[1]) | (tv == sv[2]);
-  }
   const double* ps[3] = {xyz + 3 * sv[0], xyz + 3 * sv[1], xyz + 3 * sv[2]};
-  if (!touch) {
-    const double rt = bound_radius(gt + GEO_C, xyz + 3 * tri[3 * t], xyz + 3 * tri[3 * t + 1], xyz + 3 * tri[3 * t + 2]);
-    const double rs = bound_radius(gs + GEO_C, ps[0], ps[1], ps[2]);
-    const double dx = gt[GEO_C] - gs[GEO_C], dy = gt[GEO_C + 1] - gs[GEO_C + 1], dz = gt[GEO_C + 2] - gs[GEO_C + 2];
-    if (fabs(tk.ki) * (sqrt(dx * dx + dy * dy + dz * dz) - rt - rs) > R8_CUTOFF) return;
-  }
   const SrcPoint* rule = spts + soff[s - tk.s0];
   const int nu = soff[s - tk.s0 + 1] - soff[s - tk.s0];
   const bool split = nu > 6;
@@ -124,8 +279,7 @@ __global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __r
     const double* rq = gt + GEO_RHO + 3 * q;
     const double D0 = dc[0] + rq[0] - rp[0], D1 = dc[1] + rq[1] - rp[1], D2 = dc[2] + rq[2] - rp[2];
     const double r2 = D0 * D0 + D1 * D1 + D2 * D2;
-    const double iR = rsqrt(r2), Rr = r2 * iR;
-    cd g = touch ? (split ? green_smooth1(k, sqrt(r2)) : green_smooth(k, sqrt(r2))) : green_full(k, Rr, iR);
+    cd g = split ? green_smooth1(k, sqrt(r2)) : green_smooth(k, sqrt(r2));
     const double w = gt[GEO_W + q] * ws;
     g.r *= w;
     g.i *= w;
@@ -141,7 +295,7 @@ __global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __r
     m[14] += g.r * qs;
     m[15] += g.i * qs;
   }
-  if (touch && lane < 6) {
+  if (lane < 6) {
     const int q = lane;
     const double* rq = gt + GEO_RHO + 3 * q;
     double r[3];
@@ -205,9 +359,10 @@ __global__ void __launch_bounds__(256) fill_L_split(LTask tk, const int32_t* __r
   }
 }
 
-// ---------------------------------------------------------------- Kbar (primal test x barycentric child)
+// ---------------------------------------------------------------- Kbar (primal test x barycentric child), touching pairs
 template <class R>
-__global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __restrict__ soff,
+__global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __restrict__ pa, const int32_t* __restrict__ pc,
+                                                    int npairs, const int32_t* __restrict__ soff,
                                                     const SrcPoint* __restrict__ spts,
                                                     const double* __restrict__ geo,
                                                     const double* __restrict__ bgeo, const double* __restrict__ xyz,
@@ -215,14 +370,10 @@ __global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __r
                                                     const int32_t* __restrict__ btri_edge) {
   const int64_t pair = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (pair >= int64_t(tk.ntest) * tk.nsrc) return;
-  const int t = tk.t0 + int(pair / tk.nsrc), cg = tk.c0 + int(pair % tk.nsrc);
-  const int par = cg / 6, kk = cg % 6, pp = kk / 2;
-  if (par == t) return;  // child of the test triangle: coplanar, Kbar = 0
-  const int32_t cvx = tri[3 * par + ((kk & 1) ? (pp + 1) % 3 : pp)];  // child's primal vertex
-  const int32_t ce = tri_edge[3 * par + (pp + 2) % 3];                 // edge of the child's midpoint
-  bool touch = false;
-  for (int i = 0; i < 3; ++i) touch |= (tri[3 * t + i] == cvx) | (tri_edge[3 * t + i] == ce);
+  if (pair >= npairs) return;
+  const int t = pa[pair], cg = pc[pair];
+  if (t < tk.t0 || t >= tk.t0 + tk.ntest || cg < tk.c0 || cg >= tk.c0 + tk.nsrc) return;
+  const int par = cg / 6, kk = cg % 6;
   const double* gt = geo + size_t(t) * GEO_STRIDE;
   const double* gs = bgeo + size_t(cg) * GEO_STRIDE;
   // child vertices rebuilt from the parent: (a, m_ab, g) (m_ab, b, g) (b, m_bc, g) (m_bc, c, g) (c, m_ca, g) (m_ca, a, g)
@@ -237,12 +388,6 @@ __global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __r
   }
   const int cvt[6][3] = {{0, 3, 6}, {3, 1, 6}, {1, 4, 6}, {4, 2, 6}, {2, 5, 6}, {5, 0, 6}};
   const double* ps[3] = {V[cvt[kk][0]], V[cvt[kk][1]], V[cvt[kk][2]]};
-  if (!touch) {
-    const double rt = bound_radius(gt + GEO_C, xyz + 3 * tri[3 * t], xyz + 3 * tri[3 * t + 1], xyz + 3 * tri[3 * t + 2]);
-    const double rs = bound_radius(gs + GEO_C, ps[0], ps[1], ps[2]);
-    const double dx = gt[GEO_C] - gs[GEO_C], dy = gt[GEO_C + 1] - gs[GEO_C + 1], dz = gt[GEO_C + 2] - gs[GEO_C + 2];
-    if (fabs(tk.ki) * (sqrt(dx * dx + dy * dy + dz * dz) - rt - rs) > R8_CUTOFF) return;
-  }
   const SrcPoint* rule = spts + soff[cg - tk.c0];
   const int nu = soff[cg - tk.c0 + 1] - soff[cg - tk.c0];
   const double As = gs[GEO_A];
@@ -265,8 +410,7 @@ __global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __r
     const double* rq = gt + GEO_RHO + 3 * q;
     const double D[3] = {dc[0] + rq[0] - rp[0], dc[1] + rq[1] - rp[1], dc[2] + rq[2] - rp[2]};
     const double r2 = D[0] * D[0] + D[1] * D[1] + D[2] * D[2];
-    const double iR = rsqrt(r2), Rr = r2 * iR;
-    cd g1 = touch ? grad_smooth(k, sqrt(r2)) : grad_full(k, Rr, iR);
+    cd g1 = grad_smooth(k, sqrt(r2));
     const double w = gt[GEO_W + q] * ws;
     g1.r *= w;
     g1.i *= w;
@@ -284,7 +428,7 @@ __global__ void __launch_bounds__(256) fill_K_split(KTask tk, const int32_t* __r
       m[15 + 2 * d] += g1.i * D[d];
     }
   }
-  if (touch && lane < 6) {
+  if (lane < 6) {
     // static part: V_s = int grad 1/(4 pi R) dS', U_s = V_s x (r - c')
     const int q = lane;
     const double* rq = gt + GEO_RHO + 3 * q;
@@ -460,18 +604,33 @@ SplitRules split_rules_K(const HostMesh& h, const KTask& tk) {
   });
 }
 
+// sources of a task by rule size, largest first (mesh order among equals)
+static std::vector<int32_t> by_rule_size(const SplitRules& rules) {
+  std::vector<int32_t> o(rules.off.size() - 1);
+  for (size_t i = 0; i < o.size(); ++i) o[i] = int32_t(i);
+  std::stable_sort(o.begin(), o.end(), [&](int32_t a, int32_t b) {
+    return rules.off[a + 1] - rules.off[a] > rules.off[b + 1] - rules.off[b];
+  });
+  return o;
+}
+
 template <class R>
 void fill_L_split_task(const sldm_mesh* m, const LTask& tk, const SplitRules& rules, cudaStream_t s) {
-  DBuf<int32_t> doff;
+  DBuf<int32_t> doff, dord;
   DBuf<SrcPoint> dpts;
   doff.upload(rules.off, s);
   dpts.upload(rules.pts, s);
-  const int64_t threads = int64_t(tk.ntest) * tk.nsrc * 32;
+  dord.upload(by_rule_size(rules), s);
   const DevMesh& d = m->d;
+  const int np = int(m->h.touchL_a.size());
   {
     ScopedTimer tm("fill_L_split", s);
-    fill_L_split<R><<<unsigned((threads + 255) / 256), 256, 0, s>>>(tk, doff.p, dpts.p, d.geo.p, d.xyz.p, d.tri.p,
-                                                                   d.tri_edge.p), ::sldm::count_launch();
+    fill_split_bulk<R, false><<<dim3((tk.ntest + SPLIT_TB - 1) / SPLIT_TB, (tk.nsrc + SPLIT_SB - 1) / SPLIT_SB), SPLIT_THREADS, 0,
+                                s>>>(tk, SplitTab{dord.p, doff.p, dpts.p}, d.geo.p, d.geo.p, d.rad.p, d.rad.p, d.tri.p,
+                                     d.tri_edge.p, d.tri_edge.p), ::sldm::count_launch();
+    fill_L_split<R><<<unsigned((int64_t(np) * 32 + 255) / 256), 256, 0, s>>>(tk, d.touchL_a.p, d.touchL_b.p, np, doff.p, dpts.p,
+                                                                            d.geo.p, d.xyz.p, d.tri.p, d.tri_edge.p),
+        ::sldm::count_launch();
   }
   SLDM_CUDA(cudaGetLastError());
   SLDM_CUDA(cudaStreamSynchronize(s));
@@ -479,16 +638,21 @@ void fill_L_split_task(const sldm_mesh* m, const LTask& tk, const SplitRules& ru
 
 template <class R>
 void fill_K_split_task(const sldm_mesh* m, const KTask& tk, const SplitRules& rules, cudaStream_t s) {
-  DBuf<int32_t> doff;
+  DBuf<int32_t> doff, dord;
   DBuf<SrcPoint> dpts;
   doff.upload(rules.off, s);
   dpts.upload(rules.pts, s);
-  const int64_t threads = int64_t(tk.ntest) * tk.nsrc * 32;
+  dord.upload(by_rule_size(rules), s);
   const DevMesh& d = m->d;
+  const int np = int(m->h.touchK_a.size());
   {
     ScopedTimer tm("fill_K_split", s);
-    fill_K_split<R><<<unsigned((threads + 255) / 256), 256, 0, s>>>(tk, doff.p, dpts.p, d.geo.p, d.bgeo.p, d.xyz.p, d.tri.p,
-                                                                   d.tri_edge.p, d.btri_edge.p), ::sldm::count_launch();
+    fill_split_bulk<R, true><<<dim3((tk.ntest + SPLIT_TB - 1) / SPLIT_TB, (tk.nsrc + SPLIT_SB - 1) / SPLIT_SB), SPLIT_THREADS, 0,
+                               s>>>(tk, SplitTab{dord.p, doff.p, dpts.p}, d.geo.p, d.bgeo.p, d.rad.p, d.brad.p, d.tri.p,
+                                    d.tri_edge.p, d.btri_edge.p), ::sldm::count_launch();
+    fill_K_split<R><<<unsigned((int64_t(np) * 32 + 255) / 256), 256, 0, s>>>(tk, d.touchK_a.p, d.touchK_c.p, np, doff.p, dpts.p,
+                                                                            d.geo.p, d.bgeo.p, d.xyz.p, d.tri.p, d.tri_edge.p,
+                                                                            d.btri_edge.p), ::sldm::count_launch();
   }
   SLDM_CUDA(cudaGetLastError());
   SLDM_CUDA(cudaStreamSynchronize(s));
