@@ -199,7 +199,7 @@ __device__ void spectral_rem(const DevStack& S, const MgfStatic& Q, cx kr, int p
     out[0] = out[0] - (mur * (guh * E1 + gdh * E2)) * g;
     out[1] = out[1] - ((gue * E1 + gde * E2) * g) / epsl;
     out[2] = out[2] - (mur * ((guh - 2.0 * gue) * E1 + (gdh - 2.0 * gde) * E2)) * g;
-    // z-rho / rho-z: the static single reflections exp(-k_rho zeta) (closed form in space: static_zr)
+    // z-rho / rho-z: the static single reflections exp(-k_rho zeta) (closed form in space)
     const cx X1 = S.top ? cexp_(-(kr * mk(2 * S.zu - arg))) : zero;
     const cx X2 = S.bot ? cexp_(-(kr * mk(arg - 2 * S.zb))) : zero;
     const cx cu = gue - guh, cdn = gde - gdh;
@@ -467,44 +467,89 @@ void mgf_build_tables(const MgfStackHost& H, double omega, double rho_min, doubl
 }
 
 // ---------------------------------------------------------------- reflected fill of L^A_m, L^phi_m
-struct TabView {
-  const double2* A;
-  const double2* B;
+// The tables as bilinear cells: cell (i, j) holds, for the four components the fill
+// needs (xx, phi, zz, rho-z: the z-rho component is -(rho-z) in A and equal to it in
+// B), a = f_00, b = f_10 - f_00, c = f_01 - f_00, d = f_11 - f_10 - f_01 + f_00, so a
+// value costs three FMAs per real part and its 16 operands are 256 contiguous bytes.
+constexpr int CELL_C = 4;
+__global__ void mgf_cells_kernel(const double2* __restrict__ t, int nr, int ny, double2* __restrict__ cells) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (nr - 1) * ny * CELL_C) return;
+  const int comp = idx % CELL_C, ij = idx / CELL_C, i = ij / ny, j = ij % ny, j1 = min(j + 1, ny - 1);
+  const double2* f = t + int64_t(comp == 3 ? 4 : comp) * nr * ny;
+  const double2 f00 = f[int64_t(i) * ny + j], f10 = f[int64_t(i + 1) * ny + j], f01 = f[int64_t(i) * ny + j1],
+                f11 = f[int64_t(i + 1) * ny + j1];
+  double2* o = cells + int64_t(idx) * 4;
+  o[0] = f00;
+  o[1] = make_double2(f10.x - f00.x, f10.y - f00.y);
+  o[2] = make_double2(f01.x - f00.x, f01.y - f00.y);
+  o[3] = make_double2((f11.x - f10.x) - (f01.x - f00.x), (f11.y - f10.y) - (f01.y - f00.y));
+}
+
+// Cell index and offset of a fractional index f in [0, n - 1] (clamped there):
+// round f - 1/2 by adding and subtracting 1.5 2^52, no conversion on the FP64 pipe.
+__device__ __forceinline__ int cell_of(double f, int last, double& t) {
+  if (__double2hiint(f) < 0) f = 0.0;
+  const double h = f - 0.5, m = __dadd_rn(h, 6755399441055744.0);
+  int i = __double2loint(m);
+  t = f - __dsub_rn(m, 6755399441055744.0);
+  if (i > last) {  // the table's edge, up to rounding
+    i = last;
+    t = 1.0;
+  }
+  return i;
+}
+__device__ __forceinline__ cx cell_value(const double2* __restrict__ c, double tx, double ty) {
+  const double2 a = c[0], b = c[1], g = c[2], d = c[3];
+  return {fma(tx, fma(ty, d.x, b.x), fma(ty, g.x, a.x)), fma(tx, fma(ty, d.y, b.y), fma(ty, g.y, a.y))};
+}
+
+// log2 of positive normal x from 128 values of log2 of the mantissa's leading bits and
+// the series of the rest (|r| < 2^-7): ~11 FP64 operations, error a few 1e-17 + rounding
+constexpr int LOG_N = 128;
+struct LogTab {
+  double2 t[LOG_N];  // (1 / c, log2 c), c the middle of [1 + i / 128, 1 + (i + 1) / 128)
+};
+__device__ __forceinline__ void log_tab_fill(LogTab& T) {
+  for (int i = threadIdx.x; i < LOG_N; i += blockDim.x) {
+    const double inv = 1.0 / (1.0 + (i + 0.5) / LOG_N);
+    T.t[i] = make_double2(inv, -log2(inv));
+  }
+}
+__device__ __forceinline__ double log2_pos(const LogTab& T, double x) {
+  constexpr double L = 1.44269504088896340736;
+  const int hi = __double2hiint(x);
+  const double2 w = T.t[(hi >> 13) & (LOG_N - 1)];
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+  const double r = fma(m, w.x, -1.0);
+  const double p = r * fma(r, fma(r, fma(r, fma(r, fma(r, fma(r, L / 7.0, -L / 6.0), L / 5.0), -L / 4.0), L / 3.0), -L / 2.0), L);
+  // the exponent as a double: 2^52 + 2^31 + e built from bits
+  const double e = __dsub_rn(__hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ int(0x80000000)), 4503601774854144.0);
+  return (e + w.y) + p;
+}
+// 1 / x, x > 0: the hardware estimate and one third-order step
+__device__ __forceinline__ double recip_pos(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(fma(e, e, e), y, y);
+}
+
+// What the fill needs of the stack, worked out on the host.
+struct ReflArgs {
+  cx k;                        // of the objects' layer
+  double ys, ye;               // k.r, k.i in steps of the wave tables
+  double zu2, zb2;             // 2 zu, 2 zb
+  double kxx_u, kxx_d;         // image coefficients: xx mu_r g_h, phi g_e / eps_r, zz mu_r (g_h - 2 g_e)
+  cx kph_u, kph_d, kzz_u, kzz_d;
+  cx kzr_u, kzr_d;             // mu_r (g_e - g_h) of the static rho-z images
+  const double2 *ca, *cb;      // cells of the two tables
   int nr, ns, nd;
-  double lr0, lr1, s0, s1, d1;
-  int hasB;
-  double rmin, inv_rmin;  // exp(lr0), exp(-lr0)
-  double sx, ss, sd;      // index scales (nr - 1)/(lr1 - lr0), (ns - 1)/(s1 - s0), (nd - 1)/d1 (0 if d1 = 0)
+  double fx1, fx0;             // cell index of rho: fx1 log2(rho^2) + fx0
+  double s0, ss, sd;           // (z + z' - s0) ss, |z - z'| sd
+  double rmin2, inv_rmin;
 };
 
-// Bilinear cell of a table at fractional indices (fx, fy), clamped as bilin does.
-struct Cell {
-  int64_t i00, i10, i01, i11;
-  double w00, w10, w01, w11;
-};
-__device__ __forceinline__ Cell cell(int nr, int ny, double fx, double fy) {
-  fx = fmin(fmax(fx, 0.0), nr - 1 - 1e-9);
-  fy = ny > 1 ? fmin(fmax(fy, 0.0), ny - 1 - 1e-9) : 0.0;
-  const int ix = int(fx), iy = int(fy);
-  const double tx = fx - ix, ty = fy - iy;
-  const int iy1 = min(iy + 1, ny - 1);
-  return {int64_t(ix) * ny + iy, int64_t(ix + 1) * ny + iy, int64_t(ix) * ny + iy1, int64_t(ix + 1) * ny + iy1,
-          (1 - tx) * (1 - ty), tx * (1 - ty), (1 - tx) * ty, tx * ty};
-}
-__device__ __forceinline__ cx at(const double2* t, int64_t plane, const Cell& c, int comp) {
-  const double2* b = t + comp * plane;
-  const double2 a00 = b[c.i00], a10 = b[c.i10], a01 = b[c.i01], a11 = b[c.i11];
-  return {c.w00 * a00.x + c.w10 * a10.x + c.w01 * a01.x + c.w11 * a11.x,
-          c.w00 * a00.y + c.w10 * a10.y + c.w01 * a01.y + c.w11 * a11.y};
-}
-
-
-// Static z-rho image in space: rho / (4 pi R (R + zeta)), R = |(rho, zeta)|, zeta >= 0; 0 at R = 0.
-__device__ __forceinline__ double static_zr(double rho, double zeta) {
-  const double R = sqrt(rho * rho + zeta * zeta);
-  const double den = R * (R + zeta);
-  return den > 0 ? (0.25 / 3.14159265358979323846) * rho / den : 0.0;
-}
 
 // Pair (t, s) touches through an interface when the triangles share a vertex on
 // it: bits 0-2 (bottom) and 4-6 (top) of onmask flag vertices on the interfaces.
@@ -518,156 +563,212 @@ __device__ __forceinline__ bool touch_through(const int32_t* tri, int t, int s, 
   return false;
 }
 
+// acc += s b for a real s
+__device__ __forceinline__ void fmac(cx& acc, double s, cx b) {
+  acc.r = fma(s, b.r, acc.r);
+  acc.i = fma(s, b.i, acc.i);
+}
+// acc += a b
+__device__ __forceinline__ void cmac(cx& acc, cx a, cx b) {
+  acc.r = fma(-a.i, b.i, fma(a.r, b.r, acc.r));
+  acc.i = fma(a.i, b.r, fma(a.r, b.i, acc.i));
+}
+
 // One thread per (test, source) triangle pair of a block task, 6 x 6 points: the
 // images (spherical waves and static z-rho / rho-z) and the tabulated remainder.
 // An interface's images are left out for pairs touching through it (they are
 // integrated apart by fill_reflected_touch); a coincident image point adds 0.
-template <class C>
-__global__ void __launch_bounds__(128) fill_reflected_kernel(const RTask* __restrict__ tasks, const double* __restrict__ geo,
-                                                             const int32_t* __restrict__ tri_edge, const int32_t* __restrict__ tri,
-                                                             const int32_t* __restrict__ onmask, DevStack S, MgfStatic Q, TabView T,
-                                                             C* LA, int64_t ldA, C* LP, int64_t ldP) {
+// The dyadic kernel (xx, zz, and with rhohat = (hx, hy) the vectors R = grz rhohat, Z =
+// gzr rhohat) meets f_i(r) = s_i (r - V_i) / (2 A) and f'_j alike, so the sums over
+// source points of kernel x (1, r') and then over test points of those x (1, r) give
+// the 3x3 block at the end of the pair.  A task of one triangle set against itself is
+// symmetric (gzr(r, r') = -grz(r', r) in the images and the A table, and with the sign of
+// z - z' in the B table): pairs s >= t, scattered to both places.
+// Bound by the FP64 pipe.  5 x 5 cylinders on glass (one interface): 95 ms (every pair,
+// ~300 operations per evaluation, the dyadic products and 3x3 block per test point) -> 48 ms
+// with half the pairs -> 26 ms; 2,048-triangle wire between two interfaces: 119 -> 38 ms.
+template <class C, bool TOP, bool BOT>
+__global__ void __launch_bounds__(128, 2) fill_reflected_kernel(const RTask* __restrict__ tasks, const double* __restrict__ geo,
+                                                                const int32_t* __restrict__ tri_edge,
+                                                                const int32_t* __restrict__ tri,
+                                                                const int32_t* __restrict__ onmask, const ReflArgs P, C* LA,
+                                                                int64_t ldA, C* LP, int64_t ldP) {
+  constexpr bool HASB = TOP && BOT;
+  __shared__ WaveTab wt;
+  __shared__ LogTab lt;
   const RTask tk = tasks[blockIdx.y];
+  const int64_t total = int64_t(tk.ntest) * tk.nsrc;
+  if (int64_t(blockIdx.x) * blockDim.x >= total) return;
+  wave_tab_fill(wt, P.k.i != 0.0);
+  log_tab_fill(lt);
+  __syncthreads();
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= int64_t(tk.ntest) * tk.nsrc) return;
+  if (p >= total) return;
   const int t = tk.t0 + int(p / tk.nsrc), sidx = tk.s0 + int(p % tk.nsrc);
+  const bool sym = tk.t0 == tk.s0 && tk.ntest == tk.nsrc;
+  if (sym && sidx < t) return;
   const double* gt = geo + size_t(t) * GEO_STRIDE;
   const double* gs = geo + size_t(sidx) * GEO_STRIDE;
-  const double k0 = S.omega / C0_;
-  const cx epsl = S.eps[S.l];
-  const double mur = S.mu[S.l];
-  const cx k = k0 * csqrt_(mur * epsl);
+  const bool lossy = P.k.i != 0.0;
   const int mt = onmask[t], ms = onmask[sidx];
-  const double use_bot = touch_through(tri, t, sidx, mt, ms, 0) ? 0.0 : 1.0;
-  const double use_top = touch_through(tri, t, sidx, mt, ms, 4) ? 0.0 : 1.0;
-  const cx gue = {Q.gue.r, Q.gue.i}, guh = {Q.guh.r, Q.guh.i}, gde = {Q.gde.r, Q.gde.i}, gdh = {Q.gdh.r, Q.gdh.i};
-  const cx cu = gue - guh, cdn = gde - gdh;
-  // image coefficients: xx mu_r g_h, phi g_e / eps_r, zz mu_r (g_h - 2 g_e), up and down
-  const cx kxx_u = mur * guh, kxx_d = mur * gdh, kph_u = gue / epsl, kph_d = gde / epsl;
-  const cx kzz_u = mur * (guh - 2.0 * gue), kzz_d = mur * (gdh - 2.0 * gde);
-  cx loc[9];
-  for (int i = 0; i < 9; ++i) loc[i] = mk(0);
-  cx lp = mk(0);
-  const double inv4pi = 0.25 / 3.14159265358979323846;
+  const double img_b = touch_through(tri, t, sidx, mt, ms, 0) ? 0.0 : INV4PI;
+  const double img_t = touch_through(tri, t, sidx, mt, ms, 4) ? 0.0 : INV4PI;
+  const double dcx = gt[GEO_C] - gs[GEO_C], dcy = gt[GEO_C + 1] - gs[GEO_C + 1];
+  const cx zero = mk(0);
+  cx xS = zero, xMx = zero, xMy = zero, xRx = zero, xRy = zero, x0 = zero;  // xx: r.r', r', r, 1
+  cx zS = zero, zM = zero, zR = zero, z0 = zero;                            // zz: z z', z', z, 1
+  cx rS = zero, rMx = zero, rMy = zero, rR = zero, r0x = zero, r0y = zero;  // R: r.R z', R z', r.R, R
+  cx cS = zero, cM = zero, cRx = zero, cRy = zero, c0x = zero, c0y = zero;  // Z: z Z.r', Z.r', z Z, Z
+  cx lp = zero;
+#pragma unroll 1
   for (int q = 0; q < 6; ++q) {
-    double r[3], f[3][3];
-    for (int d = 0; d < 3; ++d) r[d] = gt[GEO_C + d] + gt[GEO_RHO + 3 * q + d];
-    for (int i = 0; i < 3; ++i)
-      for (int d = 0; d < 3; ++d) f[i][d] = gt[GEO_SIG + i] * (gt[GEO_RHO + 3 * q + d] + gt[GEO_AV + 3 * i + d]);
-    // Moments of the dyadic kernel T over the source points (weights w, offsets
-    // rho_s from the source centre, rhohat = (hx, hy)): with f_j(r_s) = sig_j (rho_s + av_j),
-    // sum_s w T . f_j = sig_j (M1 + M0 . av_j), T . u = (gxx u_x + grz hx u_z,
-    // gxx u_y + grz hy u_z, gzz u_z + gzr (hx u_x + hy u_y)).
-    cx a0 = mk(0), az = mk(0), bx = mk(0), by = mk(0), cxm = mk(0), cym = mk(0);      // M0
-    cx a0x = mk(0), a0y = mk(0), bxz = mk(0), byz = mk(0), azz = mk(0), cr = mk(0);  // M1
-    cx sphi = mk(0);
+    const double tx = gt[GEO_RHO + 3 * q], ty = gt[GEO_RHO + 3 * q + 1], tz = gt[GEO_RHO + 3 * q + 2];
+    const double zz = gt[GEO_C + 2] + tz;
+    cx a0 = zero, ax = zero, ay = zero, az0 = zero, azz = zero, bx = zero, by = zero, bxz = zero, byz = zero;
+    cx dx0 = zero, dy0 = zero, dr = zero, sphi = zero;
+#pragma unroll 1
     for (int sq = 0; sq < 6; ++sq) {
-      double rs[3];
-      for (int d = 0; d < 3; ++d) rs[d] = gs[GEO_C + d] + gs[GEO_RHO + 3 * sq + d];
-      const double dx = r[0] - rs[0], dy = r[1] - rs[1];
-      const double rho2 = dx * dx + dy * dy;
-      const double irho = rho2 > 0 ? rsqrt(rho2) : 0.0;
-      const double rho = rho2 * irho;
-      const double zz = r[2], zp = rs[2];
-      // quasistatic images: spherical waves exp(-j k R)/(4 pi R) and the static
-      // z-rho image rho / (4 pi R (R + zeta)) from the image points
-      cx G1 = mk(0), G2 = mk(0);
-      double F1 = 0, F2 = 0;
-      if (S.top) {
-        const double zeta = 2 * S.zu - zz - zp;
-        const double R2 = rho2 + zeta * zeta;
-        if (R2 > 0) {
-          const double r1 = rsqrt(R2), R = R2 * r1;
-          const double iR = use_top * inv4pi * r1;
-          G1 = iR * eikr(k, R);
-          F1 = iR * rho / (R + zeta);
-        }
-      }
-      if (S.bot) {
-        const double zeta = zz + zp - 2 * S.zb;
-        const double R2 = rho2 + zeta * zeta;
-        if (R2 > 0) {
-          const double r1 = rsqrt(R2), R = R2 * r1;
-          const double iR = use_bot * inv4pi * r1;
-          G2 = iR * eikr(k, R);
-          F2 = iR * rho / (R + zeta);
-        }
-      }
-      cx gxx = kxx_u * G1 + kxx_d * G2;
-      cx gphi = kph_u * G1 + kph_d * G2;
-      cx gzz = kzz_u * G1 + kzz_d * G2;
-      // tabulated remainder (one bilinear cell for the five components)
-      const double lr = log(fmax(rho, T.rmin));
-      const double fx = (lr - T.lr0) * T.sx;
-      const double fs = (zz + zp - T.s0) * T.ss;
-      const Cell ca = cell(T.nr, T.ns, fx, fs);
-      const int64_t pa = int64_t(T.nr) * T.ns;
-      gxx = gxx + at(T.A, pa, ca, 0);
-      gphi = gphi + at(T.A, pa, ca, 1);
-      gzz = gzz + at(T.A, pa, ca, 2);
-      cx bzr = at(T.A, pa, ca, 3), brz = at(T.A, pa, ca, 4);
-      const double dd = zz - zp;
-      const double sg = dd > 0 ? 1.0 : (dd < 0 ? -1.0 : 0.0);
-      if (T.hasB) {
-        const double fd = fabs(dd) * T.sd;
-        const Cell cb = cell(T.nr, T.nd, fx, fd);
-        const int64_t pb = int64_t(T.nr) * T.nd;
-        gxx = gxx + at(T.B, pb, cb, 0);
-        gphi = gphi + at(T.B, pb, cb, 1);
-        gzz = gzz + at(T.B, pb, cb, 2);
-        bzr = bzr + sg * at(T.B, pb, cb, 3);
-        brz = brz + sg * at(T.B, pb, cb, 4);
-      }
-      // the S1 (z-rho, rho-z) remainders vanish linearly at rho = 0: below rho_min scale by rho / rho_min
-      const double lin = fmin(rho * T.inv_rmin, 1.0);
-      const cx gzr = lin * bzr + mur * (cdn * F2 - cu * F1);
-      const cx grz = lin * brz + mur * (cu * F1 - cdn * F2);
-      const double hx = dx * irho, hy = dy * irho;
-      const double w = gs[GEO_W + sq];
       const double px = gs[GEO_RHO + 3 * sq], py = gs[GEO_RHO + 3 * sq + 1], pz = gs[GEO_RHO + 3 * sq + 2];
-      const cx wxx = w * gxx, wzz = w * gzz, wrx = (w * hx) * grz, wry = (w * hy) * grz;
-      const cx wzx = (w * hx) * gzr, wzy = (w * hy) * gzr;
+      const double w = gs[GEO_W + sq];
+      const double zp = gs[GEO_C + 2] + pz;
+      const double dx = dcx + (tx - px), dy = dcy + (ty - py);
+      const double rho2 = fma(dx, dx, dy * dy);
+      const double irho = rho2 > 0 ? rsqrt_pos(rho2) : 0.0;
+      const double rho = rho2 * irho;
+      const double zs = zz + zp;
+      cx gxx = zero, gphi = zero, gzz = zero, grz = zero;
+      // quasistatic images: spherical waves exp(-j k R)/(4 pi R) and the static
+      // rho-z image rho / (4 pi R (R + zeta)) from the image points
+      auto image = [&](double zeta, double img, double kxx, cx kph, cx kzz, cx krz) {
+        const double R2 = fma(zeta, zeta, rho2);
+        if (!(R2 > 0)) return;
+        const double r1 = rsqrt_pos(R2), R = R2 * r1, iR = img * r1;
+        double c, sn;
+        wave_cis(wt, P.ys * R, c, sn);
+        const double am = lossy ? iR * wave_exp2(wt, P.ye * R) : iR;
+        const cx G = {am * c, -am * sn};
+        const double F = iR * rho * recip_pos(R + zeta);
+        fmac(gxx, kxx, G);
+        cmac(gphi, kph, G);
+        cmac(gzz, kzz, G);
+        fmac(grz, F, krz);
+      };
+      if (TOP) image(P.zu2 - zs, img_t, P.kxx_u, P.kph_u, P.kzz_u, P.kzr_u);
+      if (BOT) image(zs - P.zb2, img_b, P.kxx_d, P.kph_d, P.kzz_d, -P.kzr_d);
+      // tabulated remainder (one bilinear cell for the components of a table)
+      const double rc2 = __double_as_longlong(rho2) > __double_as_longlong(P.rmin2) ? rho2 : P.rmin2;
+      double fx, fy;
+      const int ix = cell_of(fma(P.fx1, log2_pos(lt, rc2), P.fx0), P.nr - 2, fx);
+      const int iy = cell_of((zs - P.s0) * P.ss, P.ns - 2, fy);
+      const double2* ca = P.ca + (int64_t(ix) * P.ns + iy) * (4 * CELL_C);
+      gxx = gxx + cell_value(ca, fx, fy);
+      gphi = gphi + cell_value(ca + 4, fx, fy);
+      gzz = gzz + cell_value(ca + 8, fx, fy);
+      // the S1 (z-rho, rho-z) remainders vanish linearly at rho = 0: below rho_min scale by rho / rho_min
+      const double lin = rc2 == rho2 ? 1.0 : rho * P.inv_rmin;
+      fmac(grz, lin, cell_value(ca + 12, fx, fy));
+      cx gzr = -grz;
+      if (HASB) {
+        const double dd = zz - zp;
+        const int iyb = cell_of(fabs(dd) * P.sd, P.nd - 2, fy);
+        const double2* cb = P.cb + (int64_t(ix) * P.nd + iyb) * (4 * CELL_C);
+        gxx = gxx + cell_value(cb, fx, fy);
+        gphi = gphi + cell_value(cb + 4, fx, fy);
+        gzz = gzz + cell_value(cb + 8, fx, fy);
+        const double ls = dd > 0 ? lin : (dd < 0 ? -lin : 0.0);
+        const cx b = cell_value(cb + 12, fx, fy);
+        fmac(grz, ls, b);
+        fmac(gzr, ls, b);
+      }
+      const double whx = w * (dx * irho), why = w * (dy * irho);
+      const cx wxx = w * gxx, wzz = w * gzz;
       a0 = a0 + wxx;
-      az = az + wzz;
+      fmac(ax, px, wxx);
+      fmac(ay, py, wxx);
+      az0 = az0 + wzz;
+      fmac(azz, pz, wzz);
+      fmac(sphi, w, gphi);
+      const cx wrx = whx * grz, wry = why * grz;
       bx = bx + wrx;
       by = by + wry;
-      cxm = cxm + wzx;
-      cym = cym + wzy;
-      a0x = a0x + px * wxx;
-      a0y = a0y + py * wxx;
-      bxz = bxz + pz * wrx;
-      byz = byz + pz * wry;
-      azz = azz + pz * wzz;
-      cr = cr + (px * wzx + py * wzy);
-      sphi = sphi + w * gphi;
-    }
-    cx V[3][3];  // sum_s W' T . f_j(r'_s)
-    for (int j = 0; j < 3; ++j) {
-      const double sj = gs[GEO_SIG + j];
-      const double ux = gs[GEO_AV + 3 * j], uy = gs[GEO_AV + 3 * j + 1], uz = gs[GEO_AV + 3 * j + 2];
-      V[j][0] = sj * (a0x + ux * a0 + bxz + uz * bx);
-      V[j][1] = sj * (a0y + uy * a0 + byz + uz * by);
-      V[j][2] = sj * (azz + uz * az + cr + ux * cxm + uy * cym);
-    }
-    const double wq = gt[GEO_W + q];
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) loc[3 * i + j] = loc[3 * i + j] + wq * (f[i][0] * V[j][0] + f[i][1] * V[j][1] + f[i][2] * V[j][2]);
-    lp = lp + wq * sphi;
-  }
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      C* dst = LA + int64_t(tri_edge[3 * t + i]) * ldA + tri_edge[3 * sidx + j];
-      if (sizeof(dst->x) == 4) {
-        atomicAdd(reinterpret_cast<float2*>(dst), make_float2(float(loc[3 * i + j].r), float(loc[3 * i + j].i)));
-      } else {
-        atomicAdd(reinterpret_cast<double*>(dst), loc[3 * i + j].r);
-        atomicAdd(reinterpret_cast<double*>(dst) + 1, loc[3 * i + j].i);
+      fmac(bxz, pz, wrx);
+      fmac(byz, pz, wry);
+      if (HASB) {
+        const cx wzx = whx * gzr, wzy = why * gzr;
+        dx0 = dx0 + wzx;
+        dy0 = dy0 + wzy;
+        fmac(dr, px, wzx);
+        fmac(dr, py, wzy);
+      } else {  // gzr = -grz
+        fmac(dr, -px, wrx);
+        fmac(dr, -py, wry);
       }
     }
+    if (!HASB) {
+      dx0 = -bx;
+      dy0 = -by;
+    }
+    const double wq = gt[GEO_W + q], wx = wq * tx, wy = wq * ty, wz = wq * tz;
+    fmac(xS, wx, ax);
+    fmac(xS, wy, ay);
+    fmac(xMx, wq, ax);
+    fmac(xMy, wq, ay);
+    fmac(xRx, wx, a0);
+    fmac(xRy, wy, a0);
+    fmac(x0, wq, a0);
+    fmac(zS, wz, azz);
+    fmac(zM, wq, azz);
+    fmac(zR, wz, az0);
+    fmac(z0, wq, az0);
+    fmac(rS, wx, bxz);
+    fmac(rS, wy, byz);
+    fmac(rMx, wq, bxz);
+    fmac(rMy, wq, byz);
+    fmac(rR, wx, bx);
+    fmac(rR, wy, by);
+    fmac(r0x, wq, bx);
+    fmac(r0y, wq, by);
+    fmac(cS, wz, dr);
+    fmac(cM, wq, dr);
+    fmac(cRx, wz, dx0);
+    fmac(cRy, wz, dy0);
+    fmac(c0x, wq, dx0);
+    fmac(c0y, wq, dy0);
+    fmac(lp, wq, sphi);
+  }
+  // (r + a_i).T.(r' + b_j) from the sums (a = c - V, GEO_AV)
+  const cx base = (xS + zS) + (rS + cS);
+  for (int i = 0; i < 3; ++i) {
+    const double ax = gt[GEO_AV + 3 * i], ay = gt[GEO_AV + 3 * i + 1], az = gt[GEO_AV + 3 * i + 2];
+    cx bi = base;  // terms without b_j
+    fmac(bi, ax, xMx + rMx);
+    fmac(bi, ay, xMy + rMy);
+    fmac(bi, az, zM + cM);
+    for (int j = 0; j < 3; ++j) {
+      const double ux = gs[GEO_AV + 3 * j], uy = gs[GEO_AV + 3 * j + 1], uz = gs[GEO_AV + 3 * j + 2];
+      cx v = bi;
+      fmac(v, ux, xRx + cRx);
+      fmac(v, uy, xRy + cRy);
+      fmac(v, uz, zR + rR);
+      fmac(v, fma(ax, ux, ay * uy), x0);
+      fmac(v, az * uz, z0);
+      fmac(v, ax * uz, r0x);
+      fmac(v, ay * uz, r0y);
+      fmac(v, az * ux, c0x);
+      fmac(v, az * uy, c0y);
+      v = (gt[GEO_SIG + i] * gs[GEO_SIG + j]) * v;
+      const int64_t row = tri_edge[3 * t + i], col = tri_edge[3 * sidx + j];
+      M<decltype(LA->x)>::add(LA, row * ldA + col, v.r, v.i);
+      if (sym && sidx != t) M<decltype(LA->x)>::add(LA, col * ldA + row, v.r, v.i);
+    }
+  }
   const double sc = 1.0 / (gt[GEO_A] * gs[GEO_A]);
-  C* dp = LP + int64_t(t) * ldP + sidx;
-  dp->x = decltype(dp->x)(double(dp->x) + sc * lp.r);
-  dp->y = decltype(dp->y)(double(dp->y) + sc * lp.i);
+  auto addp = [&](C* dp) {
+    dp->x = decltype(dp->x)(double(dp->x) + sc * lp.r);
+    dp->y = decltype(dp->y)(double(dp->y) + sc * lp.i);
+  };
+  addp(LP + int64_t(t) * ldP + sidx);
+  if (sym && sidx != t) addp(LP + int64_t(sidx) * ldP + t);
 }
 
 // ---------------------------------------------------------------- pairs touching through an interface
@@ -933,9 +1034,51 @@ void mgf_fill_reflected(const sldm_mesh* m, const MgfStackHost& H, double omega,
                         const std::vector<RTask>& tasks, void* LA, int64_t ldA, void* LP, int64_t ldP, cudaStream_t s) {
   if (tasks.empty()) return;
   const DevStack S = dev_stack(H, omega);
-  TabView tv{T.A.p, T.B.p, T.nr, T.ns, T.nd, T.lr0, T.lr1, T.s0, T.s1, T.d1, T.hasB ? 1 : 0, std::exp(T.lr0), std::exp(-T.lr0),
-             (T.nr - 1) / (T.lr1 - T.lr0), T.s1 > T.s0 ? (T.ns - 1) / (T.s1 - T.s0) : 0.0, T.d1 > 0 ? (T.nd - 1) / T.d1 : 0.0};
   ScopedTimer tm("fill_reflected", s);
+  ReflArgs P{};
+  {
+    const std::complex<double> el = H.eps[H.l];
+    const double mur = H.mu[H.l], k0 = omega / C0_;
+    const std::complex<double> k = k0 * std::sqrt(mur * el);
+    auto put = [](std::complex<double> z) { return cx{z.real(), z.imag()}; };
+    const std::complex<double> gue(T.Q.gue.r, T.Q.gue.i), gde(T.Q.gde.r, T.Q.gde.i);
+    const double guh = T.Q.guh.r, gdh = T.Q.gdh.r;  // real: permeabilities are
+    P.k = put(k);
+    P.ys = k.real() * (WAVE_N / (2.0 * PI));
+    P.ye = k.imag() * (WAVE_N * 1.4426950408889634074);
+    P.zu2 = 2 * H.zu;
+    P.zb2 = 2 * H.zb;
+    P.kxx_u = mur * guh;
+    P.kxx_d = mur * gdh;
+    P.kph_u = put(gue / el);
+    P.kph_d = put(gde / el);
+    P.kzz_u = put(mur * (guh - 2.0 * gue));
+    P.kzz_d = put(mur * (gdh - 2.0 * gde));
+    P.kzr_u = put(mur * (gue - guh));
+    P.kzr_d = put(mur * (gde - gdh));
+    P.nr = T.nr;
+    P.ns = T.ns;
+    P.nd = T.nd;
+    // (log rho - lr0) (nr - 1) / (lr1 - lr0) with log rho = log2(rho^2) log(2) / 2
+    const double sx = (T.nr - 1) / (T.lr1 - T.lr0);
+    P.fx1 = 0.5 * std::log(2.0) * sx;
+    P.fx0 = -T.lr0 * sx;
+    P.s0 = T.s0;
+    P.ss = T.s1 > T.s0 ? (T.ns - 1) / (T.s1 - T.s0) : 0.0;
+    P.sd = T.d1 > 0 ? (T.nd - 1) / T.d1 : 0.0;
+    P.rmin2 = std::exp(2 * T.lr0);
+    P.inv_rmin = std::exp(-T.lr0);
+  }
+  DBuf<double2> ca, cb;
+  auto cells = [&](const DBuf<double2>& t, int ny, DBuf<double2>& c) {
+    const int n = (T.nr - 1) * ny * CELL_C;
+    c.alloc(size_t(n) * 4);
+    mgf_cells_kernel<<<(n + 255) / 256, 256, 0, s>>>(t.p, T.nr, ny, c.p), ::sldm::count_launch();
+  };
+  cells(T.A, T.ns, ca);
+  if (T.hasB) cells(T.B, T.nd, cb);
+  P.ca = ca.p;
+  P.cb = cb.p;
   std::vector<int32_t> onmask, pairs;
   mgf_touch_setup(m->h, H, tasks, onmask, pairs);
   DBuf<RTask> dt;
@@ -946,13 +1089,20 @@ void mgf_fill_reflected(const sldm_mesh* m, const MgfStackHost& H, double omega,
   double pairs_total = 0;
   for (const RTask& k : tasks) {
     most = std::max(most, int64_t(k.ntest) * k.nsrc);
-    pairs_total += double(k.ntest) * k.nsrc;
+    const bool sym = k.t0 == k.s0 && k.ntest == k.nsrc;
+    pairs_total += sym ? 0.5 * k.ntest * (k.ntest + 1.0) : double(k.ntest) * k.nsrc;
   }
   {
     ScopedTimer tb("fill_reflected_bulk", s);
     timer_units("fill_reflected_bulk", 36.0 * pairs_total);
-    fill_reflected_kernel<C><<<dim3(unsigned((most + 127) / 128), unsigned(tasks.size())), 128, 0, s>>>(
-        dt.p, m->d.geo.p, m->d.tri_edge.p, m->d.tri.p, dm.p, S, T.Q, tv, (C*)LA, ldA, (C*)LP, ldP), ::sldm::count_launch();
+    const dim3 grid(unsigned((most + 127) / 128), unsigned(tasks.size()));
+    auto go = [&](auto kernel) {
+      kernel<<<grid, 128, 0, s>>>(dt.p, m->d.geo.p, m->d.tri_edge.p, m->d.tri.p, dm.p, P, (C*)LA, ldA, (C*)LP, ldP),
+          ::sldm::count_launch();
+    };
+    if (H.top && H.bot) go(fill_reflected_kernel<C, true, true>);
+    else if (H.top) go(fill_reflected_kernel<C, true, false>);
+    else go(fill_reflected_kernel<C, false, true>);
     SLDM_CUDA(cudaGetLastError());
   }
   const int np = int(pairs.size() / 3);
