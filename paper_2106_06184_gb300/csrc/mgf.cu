@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <complex>
+#include <type_traits>
 
 #include "dense.h"
 #include "fill_dev.cuh"
@@ -148,9 +149,19 @@ __device__ void reflections(const DevStack& S, cx kr, int te, cx* Gu, cx* Gd) {
   *Gd = down;
 }
 
-// Remainder spectral kernels at one node: part 0 = single reflections minus the
-// quasistatic images (argument s = z + z'), part 1 = double reflections (argument d = z - z').
-__device__ void spectral_rem(const DevStack& S, const MgfStatic& Q, cx kr, int part, double arg, cx out[5]) {
+// What the remainder's spectral kernels need at one node.  They are linear in the
+// exponentials of the vertical argument: part 0 (argument s = z + z') single
+// reflections minus the quasistatic images, in E1 = exp(-j k_z (2 zu - s)) and E2 =
+// exp(-j k_z (s - 2 zb)), X1, X2 the static ones exp(-k_rho ..); part 1 (argument d = z - z')
+// double reflections, in E3 = exp(-j k_z (2 dl + d)) and E4 = exp(-j k_z (2 dl - d)).  The
+// reflections seen from layer l cost ~10^3 FP64 operations and depend on the node
+// alone, so they are worked out once per node, not per (node, argument).
+struct SpecNode {
+  cx kz, kr;
+  cx a[4], b[4];  // weight included: factors of E1 (E3) and E2 (E4) for xx, phi, zz, rho-z
+  cx x1, x2;      // part 0: factors of X1 and X2 in rho-z
+};
+__device__ void spectral_node(const DevStack& S, const MgfStatic& Q, cx kr, cx f, int part, SpecNode& o) {
   const double k0 = S.omega / C0_;
   const cx epsl = S.eps[S.l];
   const double mur = S.mu[S.l];
@@ -163,137 +174,191 @@ __device__ void spectral_rem(const DevStack& S, const MgfStatic& Q, cx kr, int p
   reflections(S, kr, 1, &Guh, &Gdh);
   const double dl = S.zu - S.zb;
   const cx zero = mk(0);
-  cx E1 = zero, E2 = zero, E3 = zero, E4 = zero;
-  const cx mj = mk(0, -1);
-  if (part == 0) {
-    if (S.top) E1 = cexp_(mj * kz * mk(2 * S.zu - arg));
-    if (S.bot) E2 = cexp_(mj * kz * mk(arg - 2 * S.zb));
-  } else if (S.top && S.bot) {
-    E3 = cexp_(mj * kz * mk(2 * dl + arg));
-    E4 = cexp_(mj * kz * mk(2 * dl - arg));
-  }
   const cx e2d = (S.top && S.bot) ? cexp_(mk(0, -2.0) * kz * mk(dl)) : zero;
   const cx De = mk(1) - Gue * Gde * e2d, Dh = mk(1) - Guh * Gdh * e2d;
-  // reflected parts of the line functions
-  auto Vi = [&](cx Z, cx Gu, cx Gd, cx D) { return (0.5 * Z) * ((Gu * E1 + Gd * E2 + Gu * Gd * (E3 + E4)) / D); };
-  auto Iv = [&](cx Z, cx Gu, cx Gd, cx D) {
-    return (mk(0.5) / Z) * ((-(Gu * E1) - Gd * E2 + Gu * Gd * (E3 + E4)) / D);
-  };
-  auto Ii = [&](cx Gu, cx Gd, cx D) { return 0.5 * ((-(Gu * E1) + Gd * E2 + Gu * Gd * (E3 - E4)) / D); };
-  auto Vv = [&](cx Gu, cx Gd, cx D) { return 0.5 * ((Gu * E1 - Gd * E2 + Gu * Gd * (E3 - E4)) / D); };
-  const cx Vie = Vi(Ze, Gue, Gde, De), Vih = Vi(Zh, Guh, Gdh, Dh);
-  const cx Ive = Iv(Ze, Gue, Gde, De), Ivh = Iv(Zh, Guh, Gdh, Dh);
-  const cx Iie = Ii(Gue, Gde, De), Iih = Ii(Guh, Gdh, Dh);
-  const cx Vve = Vv(Gue, Gde, De), Vvh = Vv(Guh, Gdh, Dh);
-  const cx jw = mk(0, S.omega);
-  const cx kr2 = kr * kr;
+  // reflected parts of the line functions at unit amplitude of each exponential
+  auto Vi = [&](cx Z, cx g, cx D) { return (0.5 * Z) * (g / D); };
+  auto Iv = [&](cx Z, cx g, cx D) { return (mk(0.5) / Z) * (g / D); };
+  auto Ch = [&](cx g, cx D) { return 0.5 * (g / D); };
+  const cx jw = mk(0, S.omega), kr2 = kr * kr;
+  const cx cxx = mk(1) / (jw * mk(MU0_)), cph = EPS0_ * (jw / kr2);
+  const cx czv = (mur * ((kr2 - kz * kz) / (EPS0_ * epsl * kr2))) / jw;
+  const cx czh = ((S.omega * S.omega * MU0_ * mur * mur) * (mk(1) / kr2)) / jw;
+  const cx crz = mk(0, mur) / kr;
   const cx gue = {Q.gue.r, Q.gue.i}, guh = {Q.guh.r, Q.guh.i}, gde = {Q.gde.r, Q.gde.i}, gdh = {Q.gdh.r, Q.gdh.i};
-  out[0] = Vih / (jw * mk(MU0_));                                                    // xx
-  out[1] = (EPS0_ * (jw / kr2)) * (Vie - Vih);                                        // phi
-  out[2] = ((mur * ((kr2 - kz * kz) / (EPS0_ * epsl * kr2))) * Ive +
-            ((S.omega * S.omega * MU0_ * mur * mur) * (mk(1) / kr2)) * Ivh) / jw;     // zz
-  out[3] = (mk(0, mur) / kr) * (Iie - Iih);                                           // z-rho
-  out[4] = (mk(0, mur) / kr) * (Vve - Vvh);                                           // rho-z
-  if (part == 0) {
-    const cx g = mk(1) / (mk(0, 2) * kz);
-    out[0] = out[0] - (mur * (guh * E1 + gdh * E2)) * g;
-    out[1] = out[1] - ((gue * E1 + gde * E2) * g) / epsl;
-    out[2] = out[2] - (mur * ((guh - 2.0 * gue) * E1 + (gdh - 2.0 * gde) * E2)) * g;
-    // z-rho / rho-z: the static single reflections exp(-k_rho zeta) (closed form in space)
-    const cx X1 = S.top ? cexp_(-(kr * mk(2 * S.zu - arg))) : zero;
-    const cx X2 = S.bot ? cexp_(-(kr * mk(arg - 2 * S.zb))) : zero;
-    const cx cu = gue - guh, cdn = gde - gdh;
-    const cx c = mk(0, 0.5 * mur) / kr;
-    out[3] = out[3] - c * (cdn * X2 - cu * X1);
-    out[4] = out[4] - c * (cu * X1 - cdn * X2);
+  o.kz = kz;
+  o.kr = kr;
+  o.x1 = o.x2 = zero;
+  for (int side = 0; side < 2; ++side) {  // 0: E1 or E3, 1: E2 or E4
+    // signs of the line functions: Vi (Gu, Gd, GuGd, GuGd), Iv (-Gu, -Gd, +, +), Vv (Gu, -Gd, GuGd, -GuGd)
+    const cx ge = part == 0 ? (side == 0 ? Gue : Gde) : Gue * Gde;
+    const cx gh = part == 0 ? (side == 0 ? Guh : Gdh) : Guh * Gdh;
+    const double sIv = part == 0 ? -1.0 : 1.0, sVv = side == 0 ? 1.0 : -1.0;
+    cx out[4];
+    out[0] = Vi(Zh, gh, Dh) * cxx;
+    out[1] = cph * (Vi(Ze, ge, De) - Vi(Zh, gh, Dh));
+    out[2] = sIv * (czv * Iv(Ze, ge, De) + czh * Iv(Zh, gh, Dh));
+    out[3] = sVv * (crz * (Ch(ge, De) - Ch(gh, Dh)));
+    if (part == 0) {
+      const cx g = mk(1) / (mk(0, 2) * kz);
+      const cx se = side == 0 ? gue : gde, sh = side == 0 ? guh : gdh;
+      out[0] = out[0] - (mur * sh) * g;
+      out[1] = out[1] - (se * g) / epsl;
+      out[2] = out[2] - (mur * (sh - 2.0 * se)) * g;
+      // rho-z: the static single reflections exp(-k_rho zeta) (closed form in space)
+      const cx c = f * ((mk(0, 0.5 * mur) / kr) * (se - sh));
+      if (side == 0) o.x1 = -c;
+      else o.x2 = c;
+    }
+    for (int c = 0; c < 4; ++c) (side == 0 ? o.a[c] : o.b[c]) = f * out[c];
   }
 }
 
-// F[c][node][j] = w_node k_node g_c(k_node; arg_j) / (2 pi)
-__global__ void mgf_spectral_kernel(DevStack S, MgfStatic Q, const double2* __restrict__ nodes,
-                                    const double2* __restrict__ weights, int nnodes, const double* __restrict__ args,
-                                    int nargs, int part, double2* F) {
+__global__ void mgf_nodes_kernel(DevStack S, MgfStatic Q, const double2* __restrict__ nodes, const double2* __restrict__ weights,
+                                 int nnodes, int part, SpecNode* __restrict__ out) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= nnodes) return;
+  const cx kr = {nodes[n].x, nodes[n].y};
+  const cx f = (0.5 / 3.14159265358979323846) * (cx{weights[n].x, weights[n].y} * kr);
+  SpecNode o;
+  spectral_node(S, Q, kr, f, part, o);
+  out[n] = o;
+}
+// exp(-x): no sine and cosine for a real exponent (the tail of a lossless stack)
+__device__ __forceinline__ cx cexp_neg(cx x) {
+  const double e = exp(-x.r);
+  if (x.i == 0.0) return {e, 0.0};
+  double s, c;
+  sincos(x.i, &s, &c);
+  return {e * c, -e * s};
+}
+
+// F[c][node][j] = w_node k_node g_c(k_node; arg_j) / (2 pi) for xx, phi, zz, rho-z; zero from
+// the column group's last node on (group_end, see build_one)
+constexpr int CT_J = 32;  // columns (arguments) of a group
+__global__ void mgf_spectral_kernel(DevStack S, const SpecNode* __restrict__ sn, int nnodes, const double* __restrict__ args,
+                                    int nargs, int part, const int* __restrict__ group_end, double2* F) {
   const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= int64_t(nnodes) * nargs) return;
   const int n = int(idx / nargs), j = int(idx % nargs);
-  const cx kr = {nodes[n].x, nodes[n].y};
-  const cx w = {weights[n].x, weights[n].y};
-  cx g[5];
-  spectral_rem(S, Q, kr, part, args[j], g);
-  const cx f = (0.5 / 3.14159265358979323846) * (w * kr);
-  for (int c = 0; c < 5; ++c) {
-    const cx v = f * g[c];
-    F[(int64_t(c) * nnodes + n) * nargs + j] = make_double2(v.r, v.i);
+  if (n >= group_end[j / CT_J]) return;  // not read either
+  const SpecNode& o = sn[n];
+  const double arg = args[j], dl = S.zu - S.zb;
+  cx out[4] = {mk(0), mk(0), mk(0), mk(0)};
+  auto add = [&](const cx* c, double zeta) {
+    const cx E = cexp_neg(mk(0, 1) * o.kz * mk(zeta));
+    for (int m = 0; m < 4; ++m) out[m] = out[m] + c[m] * E;
+  };
+  if (part == 0) {
+    if (S.top) {
+      add(o.a, 2 * S.zu - arg);
+      out[3] = out[3] + o.x1 * cexp_neg(o.kr * mk(2 * S.zu - arg));
+    }
+    if (S.bot) {
+      add(o.b, arg - 2 * S.zb);
+      out[3] = out[3] + o.x2 * cexp_neg(o.kr * mk(arg - 2 * S.zb));
+    }
+  } else if (S.top && S.bot) {
+    add(o.a, 2 * dl + arg);
+    add(o.b, 2 * dl - arg);
   }
+  for (int c = 0; c < 4; ++c) F[(int64_t(c) * nnodes + n) * nargs + j] = make_double2(out[c].r, out[c].i);
 }
 
-// Jm[order][i][n] = J_order(k_n rho_i)
-__global__ void mgf_bessel_kernel(const double2* __restrict__ nodes, int nnodes, const double* __restrict__ rho, int nr,
-                                  double2* Jm) {
+// J[order][i][n] = J_order(k_n rho_i): the real part for every node, the imaginary part
+// Jc[order][i][n] for the ncomplex first nodes (the arc; the real-axis nodes have none)
+__global__ void mgf_bessel_kernel(const double2* __restrict__ nodes, int nnodes, int ncomplex, const double* __restrict__ rho,
+                                  int nr, double* __restrict__ J, double* __restrict__ Jc) {
   const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= int64_t(nnodes) * nr) return;
   const int i = int(idx / nnodes), n = int(idx % nnodes);
   const double2 k = nodes[n];
-  cx j0, j1;
-  if (k.y == 0.0) {
+  if (n >= ncomplex) {
     // real axis (the tail panels, arguments up to ~1e4): the math library's J0, J1
-    j0 = mk(::j0(k.x * rho[i]));
-    j1 = mk(::j1(k.x * rho[i]));
-  } else {
-    // the elliptic arc (|z| below ~1e2): the periodic trapezoid rule is accurate to
-    // rounding once it has 2(|z| + 40) points
-    bessel01_complex(mk(k.x * rho[i], k.y * rho[i]), &j0, &j1);
+    J[int64_t(i) * nnodes + n] = ::j0(k.x * rho[i]);
+    J[int64_t(nr) * nnodes + int64_t(i) * nnodes + n] = ::j1(k.x * rho[i]);
+    return;
   }
-  Jm[int64_t(i) * nnodes + n] = make_double2(j0.r, j0.i);
-  Jm[int64_t(nr) * nnodes + int64_t(i) * nnodes + n] = make_double2(j1.r, j1.i);
+  // the elliptic arc (|z| below ~1e2): the periodic trapezoid rule is accurate to
+  // rounding once it has 2(|z| + 40) points
+  cx j0, j1;
+  bessel01_complex(mk(k.x * rho[i], k.y * rho[i]), &j0, &j1);
+  J[int64_t(i) * nnodes + n] = j0.r;
+  J[int64_t(nr) * nnodes + int64_t(i) * nnodes + n] = j1.r;
+  Jc[int64_t(i) * ncomplex + n] = j0.i;
+  Jc[int64_t(nr) * ncomplex + int64_t(i) * ncomplex + n] = j1.i;
 }
 
-// part[split][c][i][j] = sum over the split's nodes n of J_{order(c)}[i][n] F[c][n][j]:
-// a complex product (rows i: rho, columns j: arguments) blocked as CT_I rows x 128
-// columns per CTA, CT_N nodes of J staged in shared memory per step, the nodes
-// split over gridDim.z / 5 CTAs (summed in a fixed order by mgf_sum_splits).
+// part[split][c][i][j] = sum over the split's nodes n of J_{order(c)}[i][n] F[c][n][j].
+// Rows i: rho, columns j: arguments; a CTA takes 32 rows (8 per warp) x 32 columns of
+// one component, CT_N nodes of J staged in shared memory per step.  The FP64 pipe
+// bounds it: two FMAs per real node and entry (J is real there), four on the arc
+// (split 0); a column group ends where its exponentials have decayed (group_end).
+// 5 x 5 cylinders on glass: 35.4 ms (complex J, five components, every node) -> 5.2 ms; the
+// spectral values 12.3 -> 2 ms.
 constexpr int CT_I = 8, CT_N = 32;
-__global__ void __launch_bounds__(128) mgf_contract_kernel(const double2* __restrict__ Jm, const double2* __restrict__ F, int nnodes,
-                                                           int nr, int nargs, int per_split, double2* part) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i0 = blockIdx.y * CT_I;
-  const int c = blockIdx.z % 5, split = blockIdx.z / 5;
-  const int order = c >= 3 ? 1 : 0;
-  const double2* J = Jm + int64_t(order) * nr * nnodes;
+__global__ void __launch_bounds__(128) mgf_contract_kernel(const double* __restrict__ J, const double* __restrict__ Jc,
+                                                           const double2* __restrict__ F, int nnodes, int ncomplex, int nr,
+                                                           int nargs, int per_split, const int* __restrict__ group_end,
+                                                           double2* part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = blockIdx.x * CT_J + lane, i0 = blockIdx.y * (4 * CT_I);
+  const int c = blockIdx.z % 4, split = blockIdx.z / 4;
+  const int order = c == 3 ? 1 : 0;
+  const double* Jo = J + int64_t(order) * nr * nnodes;
+  const double* Jco = Jc + int64_t(order) * nr * ncomplex;
   const double2* Fc = F + int64_t(c) * nnodes * nargs;
-  const int n_begin = split * per_split, n_end = min(nnodes, n_begin + per_split);
-  __shared__ double2 Js[CT_I][CT_N];
-  cx acc[CT_I];
+  const int n_begin = split == 0 ? 0 : ncomplex + (split - 1) * per_split;
+  const int n_end = min(group_end[blockIdx.x], split == 0 ? ncomplex : min(nnodes, n_begin + per_split));
+  __shared__ double Js[4 * CT_I][CT_N];
+  __shared__ double Ji[4 * CT_I][CT_N];
+  double ar[CT_I], ai[CT_I];
 #pragma unroll
-  for (int ii = 0; ii < CT_I; ++ii) acc[ii] = mk(0);
-  for (int n0 = n_begin; n0 < n_end; n0 += CT_N) {
-    for (int e = threadIdx.x; e < CT_I * CT_N; e += blockDim.x) {
-      const int ii = e / CT_N, q = e % CT_N;
-      const int gi = i0 + ii, gn = n0 + q;
-      Js[ii][q] = (gi < nr && gn < n_end) ? J[int64_t(gi) * nnodes + gn] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    if (j < nargs) {
+  for (int ii = 0; ii < CT_I; ++ii) ar[ii] = ai[ii] = 0.0;
+  // the arc apart: as a predicate in one loop its FMAs would take pipe slots on every node
+  auto sum = [&](auto arc) {
+    constexpr bool ARC = decltype(arc)::value;
+    for (int n0 = n_begin; n0 < n_end; n0 += CT_N) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < 4 * CT_I * CT_N; e += blockDim.x) {
+        const int ii = e / CT_N, q = e % CT_N, gi = i0 + ii, gn = n0 + q;
+        const bool ok = gi < nr && gn < n_end;
+        Js[ii][q] = ok ? Jo[int64_t(gi) * nnodes + gn] : 0.0;
+        if (ARC) Ji[ii][q] = ok ? Jco[int64_t(gi) * ncomplex + gn] : 0.0;
+      }
+      __syncthreads();
+      if (j >= nargs) continue;
       const int nq = min(CT_N, n_end - n0);
+#pragma unroll 2
       for (int q = 0; q < nq; ++q) {
         const double2 f = Fc[int64_t(n0 + q) * nargs + j];
 #pragma unroll
         for (int ii = 0; ii < CT_I; ++ii) {
-          const double2 a = Js[ii][q];
-          acc[ii].r = fma(a.x, f.x, fma(-a.y, f.y, acc[ii].r));
-          acc[ii].i = fma(a.x, f.y, fma(a.y, f.x, acc[ii].i));
+          const double a = Js[warp * CT_I + ii][q];
+          ar[ii] = fma(a, f.x, ar[ii]);
+          ai[ii] = fma(a, f.y, ai[ii]);
+          if (ARC) {
+            const double b = Ji[warp * CT_I + ii][q];
+            ar[ii] = fma(-b, f.y, ar[ii]);
+            ai[ii] = fma(b, f.x, ai[ii]);
+          }
         }
       }
     }
-    __syncthreads();
-  }
+  };
+  if (split == 0) sum(std::true_type{});
+  else sum(std::false_type{});
   if (j >= nargs) return;
-  for (int ii = 0; ii < CT_I; ++ii)
-    if (i0 + ii < nr) part[((int64_t(split) * 5 + c) * nr + i0 + ii) * nargs + j] = make_double2(acc[ii].r, acc[ii].i);
+  for (int ii = 0; ii < CT_I; ++ii) {
+    const int i = i0 + warp * CT_I + ii;
+    if (i < nr) part[((int64_t(split) * 4 + c) * nr + i) * nargs + j] = make_double2(ar[ii], ai[ii]);
+  }
 }
 
-// table[c][i][j] = sum over splits of part (in split order), times -j for the order-1 components
-__global__ void mgf_sum_splits(const double2* __restrict__ part, int nsplit, int64_t per, int nr, int nargs, double2* table) {
+// table[c][i][j] = sum over splits of part (in split order), times -j for the order-1
+// components; the z-rho component is -(rho-z) in part 0 and equal to it in part 1
+__global__ void mgf_sum_splits(const double2* __restrict__ part, int nsplit, int64_t per, int nr, int nargs, int which,
+                               double2* table) {
   const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= per) return;
   double re = 0, im = 0;
@@ -302,8 +367,14 @@ __global__ void mgf_sum_splits(const double2* __restrict__ part, int nsplit, int
     re += v.x;
     im += v.y;
   }
-  const int c = int(idx / (int64_t(nr) * nargs));
-  table[idx] = c >= 3 ? make_double2(im, -re) : make_double2(re, im);
+  const int64_t plane = int64_t(nr) * nargs;
+  const int c = int(idx / plane);
+  if (c < 3) {
+    table[idx] = make_double2(re, im);
+    return;
+  }
+  table[idx + plane] = make_double2(im, -re);                                          // rho-z
+  table[idx] = which == 0 ? make_double2(-im, re) : make_double2(im, -re);  // z-rho
 }
 
 // ---------------------------------------------------------------- host: nodes and tables
@@ -388,32 +459,63 @@ static void build_one(const MgfStackHost& H, const MgfStatic& Q, double omega, c
   std::vector<double2> nodes, weights;
   sommerfeld_nodes(H, omega, rho.back() / 1.0, zeta_min, nodes, weights);
   const int nn = int(nodes.size()), nr = int(rho.size()), na = int(args.size());
-  DBuf<double2> dn, dw, F, Jm;
-  DBuf<double> dr, da;
+  const int ncomplex = std::min(MGF_N_ELLIPSE, nn);
+  // A column's exponentials fall at least like exp(-kappa zeta), kappa = sqrt(k_rho^2 -
+  // Re k_l^2) on the real axis, zeta its smallest distance to an image: past kappa zeta =
+  // 60 (1e-26; the other factors grow like a power of k_rho) nothing reaches the sum's
+  // rounding, and the group of 32 columns ends there.
+  const double k0 = omega / C0_, kl2 = std::real(k0 * k0 * H.eps[H.l] * H.mu[H.l]);
+  std::vector<int> gend;
+  for (int j0 = 0; j0 < na; j0 += CT_J) {
+    double zeta = 1e300;
+    for (int j = j0; j < std::min(na, j0 + CT_J); ++j) {
+      if (part == 0 && H.top) zeta = std::min(zeta, 2 * H.zu - args[j]);
+      if (part == 0 && H.bot) zeta = std::min(zeta, args[j] - 2 * H.zb);
+      if (part == 1) zeta = std::min(zeta, 2 * (H.zu - H.zb) - args[j]);
+    }
+    int e = nn;
+    if (zeta > 0) {
+      const double kap = 60.0 / zeta, kmax = std::sqrt(std::max(0.0, kl2 + kap * kap));
+      e = ncomplex;
+      while (e < nn && nodes[e].x <= kmax) ++e;
+    }
+    gend.push_back(e);
+  }
+  DBuf<double2> dn, dw, F;
+  DBuf<double> dr, da, J, Jc;
+  DBuf<int> dg;
+  DBuf<SpecNode> sn;
   dn.upload(nodes, s);
   dw.upload(weights, s);
   dr.upload(rho, s);
   da.upload(args, s);
-  F.alloc(size_t(nn) * na * 5);
-  Jm.alloc(size_t(2) * nr * nn);
+  dg.upload(gend, s);
+  F.alloc(size_t(nn) * na * 4);
+  J.alloc(size_t(2) * nr * nn);
+  Jc.alloc(size_t(2) * nr * ncomplex);
+  sn.alloc(nn);
   const DevStack S = dev_stack(H, omega);
   {
     ScopedTimer tm("mgf_tables", s);
+    mgf_nodes_kernel<<<unsigned((nn + 63) / 64), 64, 0, s>>>(S, Q, dn.p, dw.p, nn, part, sn.p), ::sldm::count_launch();
     const int64_t tot = int64_t(nn) * na;
-    mgf_spectral_kernel<<<unsigned((tot + 127) / 128), 128, 0, s>>>(S, Q, dn.p, dw.p, nn, da.p, na, part, F.p), ::sldm::count_launch();
-    const int64_t totb = int64_t(nn) * nr;
-    mgf_bessel_kernel<<<unsigned((totb + 127) / 128), 128, 0, s>>>(dn.p, nn, dr.p, nr, Jm.p), ::sldm::count_launch();
-    // split the nodes so that the product runs ~4 CTAs per SM
-    const int base = ((na + 127) / 128) * ((nr + CT_I - 1) / CT_I) * 5;
-    const int nsplit = std::max(1, std::min(64, (4 * 152 + base - 1) / base));
-    const int per_split = ((nn + nsplit - 1) / nsplit + CT_N - 1) / CT_N * CT_N;
-    const int64_t per = int64_t(5) * nr * na;
-    DBuf<double2> part;
-    part.alloc(size_t(nsplit) * per);
-    mgf_contract_kernel<<<dim3((na + 127) / 128, (nr + CT_I - 1) / CT_I, 5 * nsplit), 128, 0, s>>>(Jm.p, F.p, nn, nr, na,
-                                                                                                   per_split, part.p),
+    mgf_spectral_kernel<<<unsigned((tot + 127) / 128), 128, 0, s>>>(S, sn.p, nn, da.p, na, part, dg.p, F.p),
         ::sldm::count_launch();
-    mgf_sum_splits<<<unsigned((per + 255) / 256), 256, 0, s>>>(part.p, nsplit, per, nr, na, out), ::sldm::count_launch();
+    const int64_t totb = int64_t(nn) * nr;
+    mgf_bessel_kernel<<<unsigned((totb + 127) / 128), 128, 0, s>>>(dn.p, nn, ncomplex, dr.p, nr, J.p, Jc.p),
+        ::sldm::count_launch();
+    // split the real-axis nodes so that the product runs ~16 CTAs per SM (short ones included)
+    const int base = ((na + CT_J - 1) / CT_J) * ((nr + 4 * CT_I - 1) / (4 * CT_I)) * 4;
+    const int want = std::max(1, std::min(63, (16 * 152 + base - 1) / base));
+    const int per_split = std::max(CT_N, ((nn - ncomplex + want - 1) / want + CT_N - 1) / CT_N * CT_N);
+    const int nsplit = 1 + (nn - ncomplex + per_split - 1) / per_split;
+    const int64_t per = int64_t(4) * nr * na;
+    DBuf<double2> sums;
+    sums.alloc(size_t(nsplit) * per);
+    mgf_contract_kernel<<<dim3((na + CT_J - 1) / CT_J, (nr + 4 * CT_I - 1) / (4 * CT_I), 4 * nsplit), 128, 0, s>>>(
+        J.p, Jc.p, F.p, nn, ncomplex, nr, na, per_split, dg.p, sums.p),
+        ::sldm::count_launch();
+    mgf_sum_splits<<<unsigned((per + 255) / 256), 256, 0, s>>>(sums.p, nsplit, per, nr, na, part, out), ::sldm::count_launch();
     SLDM_CUDA(cudaStreamSynchronize(s));
   }
   SLDM_CUDA(cudaGetLastError());
