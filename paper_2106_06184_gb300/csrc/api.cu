@@ -37,26 +37,31 @@ struct ObjInfo {
   bool nested = false;  // Y E by inner solves (nested.h); Y11, Y21 are not formed
 };
 
-// Pinned flag buffers and events of the GMRES convergence polls (one per slot).
+// Pinned flag buffers and events of the GMRES convergence polls (one per slot; the
+// step's kernel writes the flags), and pinned room for what a cycle reads back.
+struct HostBack {
+  double norm[MAX_NRHS];
+  GmresState st[MAX_NRHS];
+  int err[3];
+};
 struct PollRing {
   static constexpr int SLOTS = 2;  // the host runs at most one step ahead of what it knows
   cudaEvent_t ev[SLOTS] = {};
   int32_t* flags[SLOTS] = {};
-  bool ready = false;
-  void init(int n) {
-    if (ready) return;
+  HostBack* back = nullptr;
+  void init() {
     for (int i = 0; i < SLOTS; ++i) {
-      SLDM_CUDA(cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming));
-      SLDM_CUDA(cudaMallocHost(&flags[i], sizeof(int32_t) * n));
+      if (!ev[i]) SLDM_CUDA(cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming));
+      if (!flags[i]) SLDM_CUDA(cudaMallocHost(&flags[i], sizeof(int32_t) * MAX_NRHS));
     }
-    ready = true;
+    if (!back) SLDM_CUDA(cudaMallocHost(&back, sizeof(HostBack)));
   }
   ~PollRing() {
-    if (!ready) return;
     for (int i = 0; i < SLOTS; ++i) {
-      cudaEventDestroy(ev[i]);
-      cudaFreeHost(flags[i]);
+      if (ev[i]) cudaEventDestroy(ev[i]);
+      if (flags[i]) cudaFreeHost(flags[i]);
     }
+    if (back) cudaFreeHost(back);
   }
 };
 
@@ -78,7 +83,7 @@ struct sldm_op {
   sldm::DBuf<double> ix_val;
   // structured product: work vectors for up to WR right-hand sides per pass
   static constexpr int WR = sldm::MAX_NRHS;
-  sldm::DBuf<char> wj, we, wu, wt1, wt2, wa, wc, wbc, wbu, wz1, wz2, ww1, ww2, ww3;
+  sldm::DBuf<char> wj, we, wa, wbc, wbu, wz1, wz2, ww1, ww2, ww3;
   sldm::DBuf<sldm::GemvJob> jobs1, jobs2;
   sldm::DBuf<int64_t> rs1, rs2;
   sldm::DBuf<int2> tl1, tl2;
@@ -100,14 +105,12 @@ struct sldm_op {
   // GMRES workspace
   int ws_m = 0;
   int64_t ldv = 0;  // column stride of the Krylov bases: N rounded up to 64, zero rows beyond N
-  sldm::DBuf<double2> V, wb, wx, wr, wtmp, wtmp2, wacc, wz, dh;
+  sldm::DBuf<double2> V, wb, wx, wr, wtmp, dh;
   int ws_nr = 0;
   sldm::DBuf<double> dnorm;
   // GMRES on the device: Hessenberg, rotations, residual vectors, per right-hand side state
   sldm::DBuf<double2> gH, gcs, gsn, gg;
   sldm::DBuf<sldm::GmresState> gst;
-  sldm::DBuf<double> gscale;
-  sldm::DBuf<int> gon;
   sldm::PollRing polls;
   // large objects: Y E by inner solves (nested.h), and their scratch (n_max x WR)
   int nested_min = 2500;  // order of M_l from which Y is not formed (< 0: never)
@@ -135,7 +138,7 @@ static int64_t op_bytes(const sldm_op* op) {
 static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1, DBuf<int64_t>& drs1, DBuf<int2>& dt1,
                        GemvPlan& p1, DBuf<GemvJob>& dj2, DBuf<int64_t>& drs2, DBuf<int2>& dt2, GemvPlan& p2,
                        TcPlan* tc1 = nullptr, TcPlan* tc2 = nullptr) {
-  const int64_t ne = op->ne, nt = op->nt, nq = op->nq;
+  const int64_t ne = op->ne, nt = op->nt;
   auto P = [&](DBuf<char>& b, int64_t off) { return (void*)(b.p + off * es_v); };
   const char* loc = op->loc.p;
   auto L = [&](int64_t off) { return (const void*)(loc + off * es_m); };
@@ -147,9 +150,9 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
   std::vector<GemvJob> j1, j2;
   for (auto& o : op->obj) {
     if (o.nested) continue;  // Y E by inner solves in apply_dev
-    j1.push_back({L(o.oY11), o.ne, o.ne, o.ne, P(op->we, o.e0), ne, P(op->wt1, o.e0), ne, 1, 0, 0, 0, Lo(o.oY11)});
-    if (o.nq > 0)
-      j1.push_back({L(o.oY21), o.ne, o.nq, o.ne, P(op->we, o.e0), ne, P(op->wt2, o.q0), nq, 1, 0, 0, 0, Lo(o.oY21)});
+    // a = j - Y11 e and bc = B u + B Y21 e (j and B u are there already)
+    j1.push_back({L(o.oY11), o.ne, o.ne, o.ne, P(op->we, o.e0), ne, P(op->wa, o.e0), ne, -1, 0, 1, 0, Lo(o.oY11)});
+    j1.push_back({L(o.oY21), o.ne, o.nt, o.ne, P(op->we, o.e0), ne, P(op->wbc, o.t0), nt, 1, 0, 1, 0, Lo(o.oY21)});
   }
   j2.push_back({op->LAm.p, ne, int32_t(ne), int32_t(ne), P(op->wa, 0), ne, P(op->wz1, 0), ne, 1, 0, 0, 0, LAlo});
   j2.push_back({op->LPm.p, nt, int32_t(nt), int32_t(nt), P(op->wbc, 0), nt, P(op->wz2, 0), nt, 1, 0, 0, 0, LPlo});
@@ -195,12 +198,10 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
 
 template <class C>
 static void build_plans(sldm_op* op, cudaStream_t s) {
-  const int64_t ne = op->ne, nt = op->nt, nq = op->nq;
+  const int64_t ne = op->ne, nt = op->nt;
   const int WR = sldm_op::WR;
   const size_t ev = sizeof(double2);
-  op->wj.alloc(ne * WR * ev); op->we.alloc(ne * WR * ev); op->wu.alloc(std::max<int64_t>(nq, 1) * WR * ev);
-  op->wt1.alloc(ne * WR * ev); op->wt2.alloc(std::max<int64_t>(nq, 1) * WR * ev);
-  op->wa.alloc(ne * WR * ev); op->wc.alloc(std::max<int64_t>(nq, 1) * WR * ev);
+  op->wj.alloc(ne * WR * ev); op->we.alloc(ne * WR * ev); op->wa.alloc(ne * WR * ev);
   op->wbc.alloc(nt * WR * ev); op->wbu.alloc(nt * WR * ev);
   op->wz1.alloc(ne * WR * ev); op->wz2.alloc(nt * WR * ev);
   op->ww1.alloc(ne * WR * ev); op->ww2.alloc(ne * WR * ev); op->ww3.alloc(nt * WR * ev);
@@ -210,8 +211,7 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
   if (c64) {
     // where the tensor cores start to beat passes of 8 on the CUDA cores, measured
     // on this operator's own blocks (finite inputs: the work vectors zeroed)
-    for (DBuf<char>* w : {&op->wj, &op->we, &op->wu, &op->wt1, &op->wt2, &op->wa, &op->wc, &op->wbc, &op->wbu, &op->wz1,
-                          &op->wz2, &op->ww1, &op->ww2, &op->ww3})
+    for (DBuf<char>* w : {&op->wj, &op->we, &op->wa, &op->wbc, &op->wbu, &op->wz1, &op->wz2, &op->ww1, &op->ww2, &op->ww3})
       w->zero(s);
     gemv_autotune(op->plan1, s);
     gemv_autotune(op->plan2, s);
@@ -235,42 +235,57 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
   }
 }
 
-// y = Z x for nrhs columns, x/y complex128 on the device (column stride N)
-// y = Z x: matrix entries CM, vectors and accumulation CV
+static ApplyDims dims_of(const sldm_op* op) {
+  return {int32_t(op->ne), int32_t(op->nt), int32_t(op->nq), int32_t(op->nobj)};
+}
+// The structured product of the columns in the work vectors (apply_in, prec_apply_in):
+// matrix entries CM, vectors and accumulation CV.  First a = j - Y11 e and bc = B (u + Y21 e):
 template <class CM, class CV>
-static void apply_dev(const sldm_op* op_, const double2* x, double2* y, int nrhs, cudaStream_t s, const GemvPlan& p1,
+static void apply_y(sldm_op* op, const GemvPlan& p1, int nr, cudaStream_t s) {
+  if (p1.njobs > 0) gemv_jobs_mixed<CM, CV>(p1, nr, s);
+  if (op->nested.empty()) return;
+  if (sizeof(CV) != sizeof(double2)) throw Error{SLDM_EINVAL, "apply: inner-solve objects need complex128 vectors"};
+  for (const auto& u : op->nested)
+    nested_apply(*u, op->wnt.p, op->wny.p, op->wnr.p, op->ldn, reinterpret_cast<double2*>(op->wa.p), op->ne,
+                 reinterpret_cast<double2*>(op->wbc.p), op->nt, nr, op->mesh->h.ell, s);
+}
+// then the blocks, and the rows of the product (third block scaled by s3) into the columns y
+template <class CM, class CV, class CY>
+static void apply_rest(sldm_op* op, const GemvPlan& p2, double s3, const VecBatch<double2, CY>& y, int nr, cudaStream_t s,
+                       double2* const* zh = nullptr, int nzh = 0, double* nrm = nullptr) {
+  gemv_jobs_mixed<CM, CV>(p2, nr, s);
+  apply_combine<CV, CY>(op->mesh, dims_of(op), op->k0, op->ix_val.p, op->wz1.p, op->wz2.p, op->ww1.p, op->ww2.p, op->ww3.p,
+                        op->we.p, op->wa.p, op->wbc.p, s3, y, nr, s, zh, nzh, nrm);
+}
+
+// y = diag(1, 1, s3) Z x for nrhs columns, x/y complex128 on the device (column stride N)
+template <class CM, class CV>
+static void apply_dev(const sldm_op* op_, const double2* x, double2* y, int nrhs, double s3, cudaStream_t s, const GemvPlan& p1,
                       const GemvPlan& p2) {
   sldm_op* op = const_cast<sldm_op*>(op_);
-  ApplyDims D{int32_t(op->ne), int32_t(op->nt), int32_t(op->nq), int32_t(op->nobj)};
   for (int r0 = 0; r0 < nrhs; r0 += sldm_op::WR) {
-    int nr = std::min(sldm_op::WR, nrhs - r0);
-    const double2* xr = x + int64_t(r0) * op->N;
-    double2* yr = y + int64_t(r0) * op->N;
-    apply_glue_split<CV>(xr, op->N, D, op->wj.p, op->we.p, op->wu.p, nr, s);
-    if (p1.njobs > 0) gemv_jobs_mixed<CM, CV>(p1, nr, s);
-    if (!op->nested.empty()) {
-      if (sizeof(CV) != sizeof(double2)) throw Error{SLDM_EINVAL, "apply: inner-solve objects need complex128 vectors"};
-      for (const auto& u : op->nested)
-        nested_apply(*u, op->wnt.p, op->wny.p, op->wnr.p, op->ldn, reinterpret_cast<double2*>(op->wt1.p), op->ne,
-                     reinterpret_cast<double2*>(op->wt2.p), op->nq, nr, op->mesh->h.ell, s);
+    const int nr = std::min(sldm_op::WR, nrhs - r0);
+    VecBatch<double2, double2> b;
+    for (int c = 0; c < nr; ++c) {
+      b.x[c] = x + int64_t(r0 + c) * op->N;
+      b.y[c] = y + int64_t(r0 + c) * op->N;
     }
-    apply_glue_prep<CV>(op->mesh, D, op->wj.p, op->wu.p, op->wt1.p, op->wt2.p, op->wa.p, op->wc.p, op->wbc.p, op->wbu.p, nr,
-                        s, op->mesh->d.tri_begin.p, op->mesh->d.edge_begin.p);
-    gemv_jobs_mixed<CM, CV>(p2, nr, s);
-    apply_glue_combine<CV>(op->mesh, D, op->k0, op->ix_val.p, op->wz1.p, op->wz2.p, op->ww1.p, op->ww2.p, op->ww3.p,
-                           op->we.p, op->wa.p, op->wc.p, yr, op->N, nr, s);
+    apply_in<double2, CV>(op->mesh, b, 1.0, 1.0, 1.0, dims_of(op), op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
+    apply_y<CM, CV>(op, p1, nr, s);
+    apply_rest<CM, CV, double2>(op, p2, s3, b, nr, s);
   }
 }
 
 // acc64: a complex64 operator's product with complex128 vectors, accumulated to
 // ~48 bits (compensated FP32 sums of exactly split products; iterative refinement)
-static void apply_any(const sldm_op* op, const double2* x, double2* y, int nrhs, cudaStream_t s, bool acc64 = false) {
+static void apply_any(const sldm_op* op, const double2* x, double2* y, int nrhs, cudaStream_t s, bool acc64 = false,
+                      double s3 = 1.0) {
   ScopedTimer tm("apply", s);
   if (op->prec == SLDM_PREC_F32) {
-    if (acc64) apply_dev<float2, double2>(op, x, y, nrhs, s, op->plan1d, op->plan2d);
-    else apply_dev<float2, float2>(op, x, y, nrhs, s, op->plan1, op->plan2);
+    if (acc64) apply_dev<float2, double2>(op, x, y, nrhs, s3, s, op->plan1d, op->plan2d);
+    else apply_dev<float2, float2>(op, x, y, nrhs, s3, s, op->plan1, op->plan2);
   } else {
-    apply_dev<double2, double2>(op, x, y, nrhs, s, op->plan1, op->plan2);
+    apply_dev<double2, double2>(op, x, y, nrhs, s3, s, op->plan1, op->plan2);
   }
 }
 
@@ -519,7 +534,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
     oi.oLP = al(int64_t(oi.nt) * oi.nt);
     oi.oK = al(int64_t(oi.ne) * oi.ne);
     oi.oY11 = al(int64_t(oi.ne) * oi.ne);
-    oi.oY21 = al(int64_t(oi.nq) * oi.ne);
+    oi.oY21 = al(int64_t(oi.nt) * oi.ne);  // B Y21: Y21 and minus its column sums
     op->obj.push_back(oi);
   }
   op->loc.alloc(off * es);
@@ -643,7 +658,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
       u->mat_owner = r;
       u->mat = nmat[r];
       u->e0 = op->obj[o].e0;
-      u->q0 = op->obj[o].q0;
+      u->t0 = op->obj[o].t0;
       op->nested.push_back(std::move(u));
     }
     for (int o = 0; o < op->nobj; ++o) {
@@ -652,6 +667,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
       // undo the length scaling of M_l: Y11 = Yh11 / l, Y21 = l Yh21
       copy_scaled<C>(Rl.p + rl_off[o], int64_t(oi.ne) * oi.ne, 1.0 / h.ell, loc + oi.oY11 * es, s);
       copy_scaled<C>(Rl.p + rl_off[o] + int64_t(oi.ne) * oi.ne, int64_t(oi.nq) * oi.ne, h.ell, loc + oi.oY21 * es, s);
+      neg_colsum<C>(reinterpret_cast<C*>(loc + oi.oY21 * es), oi.nq, oi.ne, s);
     }
     // repeated objects: the first one's L^A, L^phi, K, Y11, Y21 (same layout, same sizes)
     for (int o = 0; o < op->nobj; ++o) {
@@ -665,7 +681,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
       SLDM_CUDA(cudaMemcpyAsync(loc + oi.oK * es, loc + ri.oK * es, n_ee * es, cudaMemcpyDeviceToDevice, s));
       if (oi.nested) continue;  // Y is not formed
       SLDM_CUDA(cudaMemcpyAsync(loc + oi.oY11 * es, loc + ri.oY11 * es, n_ee * es, cudaMemcpyDeviceToDevice, s));
-      SLDM_CUDA(cudaMemcpyAsync(loc + oi.oY21 * es, loc + ri.oY21 * es, int64_t(oi.nq) * oi.ne * es,
+      SLDM_CUDA(cudaMemcpyAsync(loc + oi.oY21 * es, loc + ri.oY21 * es, int64_t(oi.nt) * oi.ne * es,
                                 cudaMemcpyDeviceToDevice, s));
     }
     SLDM_CUDA(cudaStreamSynchronize(s));
@@ -732,9 +748,6 @@ static void ensure_ws(sldm_op* op, int m, int nr) {
   op->wx.alloc(N * W);
   op->wr.alloc(N * W);
   op->wtmp.alloc(N * W);
-  op->wtmp2.alloc(N * W);
-  op->wacc.alloc(N * W);
-  op->wz.alloc(N * W);
   op->dh.alloc(W * 2 * (m + 2));
   op->dnorm.alloc(W);
   // Hessenberg matrices, rotations and residual vectors on the device
@@ -743,19 +756,9 @@ static void ensure_ws(sldm_op* op, int m, int nr) {
   op->gsn.alloc(W * size_t(m));
   op->gg.alloc(W * size_t(m + 1));
   op->gst.alloc(W);
-  op->gscale.alloc(W);
-  op->gon.alloc(W);
-  op->polls.init(int(W));
+  op->polls.init();
   op->ws_m = m;
   op->ws_nr = nr;
-}
-
-static double dnorm(sldm_op* op, const double2* v, cudaStream_t s) {
-  vnorm2(v, op->N, op->dnorm.p, s);
-  double h = 0;
-  SLDM_CUDA(cudaMemcpyAsync(&h, op->dnorm.p, sizeof(double), cudaMemcpyDeviceToHost, s));
-  SLDM_CUDA(cudaStreamSynchronize(s));
-  return std::sqrt(h);
 }
 
 // The Krylov iteration runs on the length-scaled system Dr Z Dc, Dr = diag(1,
@@ -787,36 +790,40 @@ static void gmres_block(sldm_op* op, bool use_p, bool refine, bool x_zero, int m
   const int64_t ldv = op->ldv;
   auto Vr = [&](int r) { return reinterpret_cast<CB*>(op->V.p) + int64_t(r) * ldv * (m + 1); };
   auto dhr = [&](int r) { return op->dh.p + int64_t(r) * 2 * (m + 2); };
-  std::vector<double> bnorm(nr), beta(nr);
-  for (int r = 0; r < nr; ++r) {
-    vscale3(N, ne, 1.0, 1.0, l, col(op->wb, r), col(op->wb, r), s);  // bh = Dr b
-    bnorm[r] = dnorm(op, col(op->wb, r), s);
-    if (bnorm[r] == 0) SLDM_CUDA(cudaMemsetAsync(col(op->wx, r), 0, N * sizeof(double2), s));  // b = 0: x = 0
-  }
-  auto residuals = [&]() {  // wr = Dr (b - Z x), every column
-    tc_check(op->tc1, s);     // a tensor-core pass whose bounded wait ran out: SLDM_ETIMEOUT
-    tc_check(op->tc2, s);
-    tc_check(op->pc.tc, s);
-    if (x_zero) SLDM_CUDA(cudaMemsetAsync(op->wr.p, 0, size_t(nr) * N * sizeof(double2), s));  // Z 0 = 0
-    else apply_any(op, op->wx.p, op->wr.p, nr, s, refine);
-    x_zero = false;
-    for (int r = 0; r < nr; ++r) {
-      vscale3(N, ne, 1.0, 1.0, l, col(op->wr, r), col(op->wr, r), s);
-      vaxpby(N, 1.0, col(op->wb, r), -1.0, col(op->wr, r), s);
-      beta[r] = dnorm(op, col(op->wr, r), s);
-    }
-  };
-  residuals();
-  // Hessenberg matrices, rotations and convergence tests live on the device
-  // (gmres_givens): the host learns which right-hand sides still iterate from
-  // a copy of their flags that it reads without waiting, or after at most
-  // LAG newer steps have been queued, so converged ones run at most LAG extra
-  // (frozen) steps and the host never waits on a step it has just queued.
-  constexpr int LAG = PollRing::SLOTS - 1;
-  std::vector<int> it(nr, 0), kused(nr, 0);
-  std::vector<char> live(nr, 0);
-  std::vector<GmresState> hst(nr);
   PollRing& polls = op->polls;
+  HostBack& back = *polls.back;
+  std::vector<double> bnorm(nr), beta(nr);
+  const ApplyDims D = dims_of(op);
+  auto read_norms = [&](std::vector<double>& out) {
+    SLDM_CUDA(cudaMemcpyAsync(back.norm, op->dnorm.p, nr * sizeof(double), cudaMemcpyDeviceToHost, s));
+    const TcPlan* tcs[3] = {&op->tc1, &op->tc2, &op->pc.tc};
+    for (int i = 0; i < 3; ++i) tc_err_async(*tcs[i], &back.err[i], s);
+    SLDM_CUDA(cudaStreamSynchronize(s));
+    // a tensor-core pass whose bounded wait ran out: SLDM_ETIMEOUT
+    for (int i = 0; i < 3; ++i) tc_err_check(*tcs[i], back.err[i], s);
+    for (int r = 0; r < nr; ++r) out[r] = std::sqrt(back.norm[r]);
+  };
+  SLDM_CUDA(cudaMemsetAsync(op->dnorm.p, 0, op->dnorm.bytes(), s));
+  gmres_rhs(N, 2 * ne, l, op->wb.p, op->wr.p, op->dnorm.p, nr, s);  // bh = Dr b, wr = bh
+  read_norms(bnorm);
+  for (int r = 0; r < nr; ++r)
+    if (bnorm[r] == 0) SLDM_CUDA(cudaMemsetAsync(col(op->wx, r), 0, N * sizeof(double2), s));  // b = 0: x = 0
+  auto residuals = [&]() {  // wr = Dr (b - Z x), every column
+    apply_any(op, op->wx.p, op->wtmp.p, nr, s, refine, l);
+    SLDM_CUDA(cudaMemsetAsync(op->dnorm.p, 0, op->dnorm.bytes(), s));
+    gmres_residual(N, op->wb.p, op->wtmp.p, op->wr.p, op->dnorm.p, nr, s);
+    read_norms(beta);
+  };
+  if (x_zero) beta = bnorm;  // the first residual is b
+  else residuals();
+  // Hessenberg matrices, rotations and convergence tests live on the device
+  // (gmres_orthogonalise): the host learns which right-hand sides still iterate from
+  // flags that the step's kernel writes to pinned memory, read without waiting, or
+  // after at most LAG newer steps have been queued, so converged ones run at most LAG
+  // extra (frozen) steps and the host never waits on a step it has just queued.
+  constexpr int LAG = PollRing::SLOTS - 1;
+  std::vector<int> it(nr, 0);
+  std::vector<char> live(nr, 0);
   for (;;) {
     std::vector<int> act;
     for (int r = 0; r < nr; ++r) {
@@ -825,23 +832,23 @@ static void gmres_block(sldm_op* op, bool use_p, bool refine, bool x_zero, int m
     }
     if (act.empty()) break;
     {
-      std::vector<double2> g0(size_t(nr) * (m + 1), make_double2(0.0, 0.0));
+      CycleStart cs{};
+      for (int r : act) cs.live[r] = live[r] = 1;
       for (int r = 0; r < nr; ++r) {
-        hst[r] = GmresState{it[r], 0, 0, 0, bnorm[r], beta[r]};
-        g0[size_t(r) * (m + 1)] = make_double2(beta[r], 0.0);
+        cs.it[r] = it[r];
+        cs.bnorm[r] = bnorm[r];
+        cs.beta[r] = beta[r];
+        cs.v0[r] = Vr(r);
       }
-      for (int r : act) {
-        vaxpby<double2, CB>(N, 1.0 / beta[r], col(op->wr, r), 0.0, Vr(r), s);
-        hst[r].live = 1;
-        live[r] = 1;
-        kused[r] = 0;
-      }
-      SLDM_CUDA(cudaMemcpyAsync(op->gg.p, g0.data(), g0.size() * sizeof(double2), cudaMemcpyHostToDevice, s));
-      SLDM_CUDA(cudaMemcpyAsync(op->gst.p, hst.data(), nr * sizeof(GmresState), cudaMemcpyHostToDevice, s));
-      SLDM_CUDA(cudaStreamSynchronize(s));  // g0, hst are host temporaries
+      cs.r = op->wr.p;
+      cs.st = op->gst.p;
+      cs.g = op->gg.p;
+      cs.m = m;
+      gmres_cycle_start<CB>(N, cs, nr, s);
     }
-    std::vector<int> on, on_dev;
-    int next_poll = 0, oldest = 0;  // ring of outstanding flag copies [oldest, next_poll)
+    std::vector<int> on;
+    int next_poll = 0, oldest = 0;  // ring of outstanding flags [oldest, next_poll)
+    std::vector<int> asked[PollRing::SLOTS];
     auto consume = [&](bool wait) {
       while (oldest < next_poll) {
         const int sl = oldest % PollRing::SLOTS;
@@ -852,8 +859,8 @@ static void gmres_block(sldm_op* op, bool use_p, bool refine, bool x_zero, int m
         } else {
           SLDM_CUDA(cudaEventSynchronize(polls.ev[sl]));
         }
-        for (int r : act)
-          if (!polls.flags[sl][r]) live[r] = 0;
+        for (int r : asked[sl])
+          if (!static_cast<volatile int32_t*>(polls.flags[sl])[r]) live[r] = 0;
         ++oldest;
         wait = false;  // one forced wait at most
       }
@@ -864,114 +871,94 @@ static void gmres_block(sldm_op* op, bool use_p, bool refine, bool x_zero, int m
         if (live[r]) on.push_back(r);
       if (on.empty()) break;
       const int na = int(on.size());
-      if (on != on_dev) {
-        SLDM_CUDA(cudaMemcpyAsync(op->gon.p, on.data(), na * sizeof(int), cudaMemcpyHostToDevice, s));
-        SLDM_CUDA(cudaStreamSynchronize(s));  // `on` is reused by the host
-        on_dev = on;
-      }
-      // the products of this step, together: w_r = Dr Z P^-1 Dr^-1 v_r (or Dr Z Dc v_r)
+      if (next_poll - oldest == PollRing::SLOTS) consume(true);
+      const int sl = next_poll % PollRing::SLOTS;
+      // the products of this step, together: w_r = Dr Z P^-1 Dr^-1 v_r (or Dr Z Dc v_r), straight
+      // from and into the Krylov bases
       VecBatch<CB, double2> bv;
+      VecBatch<double2, CB> bw;
+      KrylovStep ks;
+      GivensArgs ga{};
+      double2 *h1[MAX_NRHS], *h2[MAX_NRHS];
+      ks.n = N;
+      ks.ldv = ldv;
+      ks.k = k + 1;
+      ks.na = na;
+      ks.nrm = op->dnorm.p;
       for (int j = 0; j < na; ++j) {
         bv.x[j] = Vr(on[j]) + int64_t(k) * ldv;
-        bv.y[j] = col(use_p ? op->wtmp2 : op->wtmp, j);
-        bv.a[j] = 1.0;
+        bw.y[j] = Vr(on[j]) + int64_t(k + 1) * ldv;
+        ks.V[j] = Vr(on[j]);
+        h1[j] = dhr(on[j]);
+        h2[j] = dhr(on[j]) + (m + 2);
+        ga.on[j] = on[j];
       }
-      if (use_p) {
-        vscale3_batch(N, ne, 1.0, 1.0, 1.0 / l, bv, na, s);
-        prec_apply(op->pc, op->mesh, op->wtmp2.p, op->wtmp.p, N, na, s);
-      } else {
-        vscale3_batch(N, ne, 1.0 / l, 1.0, l, bv, na, s);
-      }
-      apply_any(op, op->wtmp.p, op->wz.p, na, s);
+      if (use_p)
+        prec_apply_in<CB, CB>(op->pc, op->mesh, bv, 1.0 / l, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, na, s);
+      else
+        apply_in<CB, CB>(op->mesh, bv, 1.0 / l, 1.0, l, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, na, s);
       {
-        // classical Gram-Schmidt, twice, of every w_r = Dr wz_r against its basis
+        ScopedTimer tm("apply", s);
+        apply_y<CB, CB>(op, op->plan1, na, s);
+        apply_rest<CB, CB, CB>(op, op->plan2, l, bw, na, s, h1, 2 * (m + 2), op->dnorm.p);
+      }
+      {
+        // classical Gram-Schmidt, twice, of every w_r against its basis, the rotations and
+        // convergence tests, v_{k+1} = w / h_{k+1,k}.  Bytes the two passes move: per pass
+        // V[:, :k+1] read by the dots and by the update, w read by both and written by the update
         ScopedTimer tgs("gram_schmidt", s);
-        SLDM_CUDA(cudaMemsetAsync(op->dh.p, 0, op->dh.bytes(), s));
-        SLDM_CUDA(cudaMemsetAsync(op->dnorm.p, 0, op->dnorm.bytes(), s));
-        VecBatch<double2, CB> bw;
-        KrylovStep ks;
-        ks.n = N;
-        ks.ldv = ldv;
-        ks.k = k + 1;
-        ks.na = na;
-        ks.nrm = op->dnorm.p;
-        for (int j = 0; j < na; ++j) {
-          bw.x[j] = col(op->wz, j);
-          bw.y[j] = Vr(on[j]) + int64_t(k + 1) * ldv;
-          bw.a[j] = 1.0;
-          ks.V[j] = Vr(on[j]);
-          ks.h[j] = dhr(on[j]);
-        }
-        vscale3_batch(N, ne, 1.0, 1.0, l, bw, na, s);
-        // bytes the two passes move: per pass V[:, :k+1] read by the dots and by the
-        // update, w read by both and written by the update
         timer_units("gram_schmidt", double(na) * 2.0 * (2.0 * (k + 1) + 3.0) * double(ldv) * sizeof(CB));
-        krylov_dots<CB>(ks, s);
-        krylov_update<CB>(ks, false, s);
-        for (int j = 0; j < na; ++j) ks.h[j] = dhr(on[j]) + (m + 2);
-        krylov_dots<CB>(ks, s);
-        krylov_update<CB>(ks, true, s);
+        ga.k = k;
+        ga.m = m;
+        ga.na = na;
+        ga.refine = refine ? 1 : 0;
+        ga.dh = op->dh.p;
+        ga.ldh = 2 * (m + 2);
+        ga.nrm = op->dnorm.p;
+        ga.H = op->gH.p;
+        ga.cs = op->gcs.p;
+        ga.sn = op->gsn.p;
+        ga.g = op->gg.p;
+        ga.st = op->gst.p;
+        ga.tol = tol;
+        ga.cycle = REFINE_CYCLE;
+        ga.maxit = maxit;
+        ga.flags = polls.flags[sl];
+        gmres_orthogonalise<CB>(ga, ks, h1, h2, s);
       }
-      // rotations and convergence tests on the device; v_{k+1} = w / h_{k+1,k}
-      GivensArgs ga{};
-      ga.k = k;
-      ga.m = m;
-      ga.na = na;
-      ga.refine = refine ? 1 : 0;
-      ga.on = op->gon.p;
-      ga.dh = op->dh.p;
-      ga.ldh = 2 * (m + 2);
-      ga.nrm = op->dnorm.p;
-      ga.H = op->gH.p;
-      ga.cs = op->gcs.p;
-      ga.sn = op->gsn.p;
-      ga.g = op->gg.p;
-      ga.st = op->gst.p;
-      ga.tol = tol;
-      ga.cycle = REFINE_CYCLE;
-      ga.maxit = maxit;
-      ga.scale = op->gscale.p;
-      gmres_givens(ga, s);
-      VecBatch<CB, CB> bn;
-      for (int j = 0; j < na; ++j) bn.x[j] = bn.y[j] = Vr(on[j]) + int64_t(k + 1) * ldv;
-      vscale_dev_batch<CB>(N, bn, op->gscale.p, na, s);
-      // queue a copy of the flags; read the finished copies, waiting only when LAG are pending
-      {
-        if (next_poll - oldest == PollRing::SLOTS) consume(true);
-        const int sl = next_poll % PollRing::SLOTS;
-        SLDM_CUDA(cudaMemcpy2DAsync(polls.flags[sl], sizeof(int32_t), &op->gst.p[0].live, sizeof(GmresState),
-                                    sizeof(int32_t), nr, cudaMemcpyDeviceToHost, s));
-        SLDM_CUDA(cudaEventRecord(polls.ev[sl], s));
-        ++next_poll;
-        consume(next_poll - oldest > LAG);
-      }
+      // the step's flags are complete at its event; read the finished ones, waiting only when LAG are pending
+      SLDM_CUDA(cudaEventRecord(polls.ev[sl], s));
+      asked[sl] = on;
+      ++next_poll;
+      consume(next_poll - oldest > LAG);
     }
     // the cycle's state; y = H^-1 g on the device;  x += (P^-1 Dr^-1 or Dc) V y
-    SLDM_CUDA(cudaMemcpyAsync(hst.data(), op->gst.p, nr * sizeof(GmresState), cudaMemcpyDeviceToHost, s));
+    SLDM_CUDA(cudaMemcpyAsync(back.st, op->gst.p, nr * sizeof(GmresState), cudaMemcpyDeviceToHost, s));
     SLDM_CUDA(cudaStreamSynchronize(s));
+    CycleEnd ce{};
+    VecBatch<double2, double2> bx;
+    int ns = 0;
     for (int r : act) {
-      it[r] = hst[r].it;
-      kused[r] = hst[r].kused;
+      it[r] = back.st[r].it;
+      if (back.st[r].kused <= 0) continue;
+      ce.on[ns] = r;
+      ce.k[ns] = back.st[r].kused;
+      ce.V[ns] = Vr(r);
+      ce.out[ns] = col(op->wtmp, ns);
+      bx.x[ns] = col(op->wtmp, ns);
+      bx.y[ns] = col(op->wx, r);
+      ++ns;
     }
-    std::vector<int> solve;
-    for (int r : act)
-      if (kused[r] > 0) solve.push_back(r);
-    if (!solve.empty()) {
-      SLDM_CUDA(cudaMemcpyAsync(op->gon.p, solve.data(), solve.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-      gmres_backsolve(int(solve.size()), op->gon.p, m, op->gH.p, op->gg.p, op->gst.p, op->dh.p, 2 * (m + 2), s);
-      SLDM_CUDA(cudaStreamSynchronize(s));  // `solve` is a host temporary
-    }
-    for (int r : solve) {
-      const int ku = kused[r];
-      SLDM_CUDA(cudaMemsetAsync(col(op->wacc, r), 0, N * sizeof(double2), s));
-      vmul<CB, double2>(Vr(r), ldv, ku, dhr(r), 1.0, col(op->wacc, r), N, s);
-      if (use_p) {
-        vscale3(N, ne, 1.0, 1.0, 1.0 / l, col(op->wacc, r), col(op->wtmp2, 0), s);
-        prec_apply(op->pc, op->mesh, col(op->wtmp2, 0), col(op->wtmp, 0), N, 1, s);
-      } else {
-        vscale3(N, ne, 1.0 / l, 1.0, l, col(op->wacc, r), col(op->wtmp, 0), s);
-      }
-      vaxpby(N, 1.0, col(op->wtmp, 0), 1.0, col(op->wx, r), s);
+    ce.H = op->gH.p;
+    ce.g = op->gg.p;
+    ce.dh = op->dh.p;
+    ce.ldh = 2 * (m + 2);
+    ce.ldv = ldv;
+    ce.m = m;
+    if (ns > 0) {
+      gmres_cycle_end<CB>(N, ce, ns, s);
+      if (use_p) prec_apply_add(op->pc, op->mesh, bx, 1.0 / l, ns, s);
+      else gmres_add_scaled(N, ne, 1.0 / l, l, bx, ns, s);
     }
     residuals();
   }
@@ -1491,28 +1478,24 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
   DBuf<double2> dx, jd;
   dx.alloc(size_t(op->N) * nr_pass);
   jd.alloc(size_t(op->ne) * nrhs);
-  ApplyDims D{int32_t(op->ne), int32_t(op->nt), int32_t(op->nq), int32_t(op->nobj)};
+  const ApplyDims D = dims_of(op);
   // j_Delta = j - Y11 e (per object), from the first two stages of the structured product
   for (int r0 = 0; r0 < nrhs; r0 += WR) {
     const int nr = std::min(WR, nrhs - r0);
     const size_t bytes = size_t(op->N) * nr * sizeof(double2);
     const char* xs = static_cast<const char*>(x) + size_t(op->N) * r0 * sizeof(double2);
     SLDM_CUDA(cudaMemcpyAsync(dx.p, xs, bytes, where == SLDM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    VecBatch<double2, double2> b;
+    for (int c = 0; c < nr; ++c) b.x[c] = dx.p + int64_t(c) * op->N;
+    double2* jo = jd.p + int64_t(op->ne) * r0;
     if (op->prec == SLDM_PREC_F32) {
-      apply_glue_split<float2>(dx.p, op->N, D, op->wj.p, op->we.p, op->wu.p, nr, s);
-      gemv_jobs<float2>(op->plan1, nr, s);
-      apply_glue_prep<float2>(op->mesh, D, op->wj.p, op->wu.p, op->wt1.p, op->wt2.p, op->wa.p, op->wc.p, op->wbc.p,
-                              op->wbu.p, nr, s, op->mesh->d.tri_begin.p, op->mesh->d.edge_begin.p);
-      to_c128<float2>(op->wa.p, int64_t(op->ne) * nr, jd.p + int64_t(op->ne) * r0, s);
+      apply_in<double2, float2>(op->mesh, b, 1.0, 1.0, 1.0, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
+      apply_y<float2, float2>(op, op->plan1, nr, s);
+      to_c128<float2>(op->wa.p, int64_t(op->ne) * nr, jo, s);
     } else {
-      apply_glue_split<double2>(dx.p, op->N, D, op->wj.p, op->we.p, op->wu.p, nr, s);
-      gemv_jobs<double2>(op->plan1, nr, s);
-      for (const auto& u : op->nested)  // objects whose Y E comes from inner solves
-        nested_apply(*u, op->wnt.p, op->wny.p, op->wnr.p, op->ldn, reinterpret_cast<double2*>(op->wt1.p), op->ne,
-                     reinterpret_cast<double2*>(op->wt2.p), op->nq, nr, op->mesh->h.ell, s);
-      apply_glue_prep<double2>(op->mesh, D, op->wj.p, op->wu.p, op->wt1.p, op->wt2.p, op->wa.p, op->wc.p, op->wbc.p,
-                               op->wbu.p, nr, s, op->mesh->d.tri_begin.p, op->mesh->d.edge_begin.p);
-      to_c128<double2>(op->wa.p, int64_t(op->ne) * nr, jd.p + int64_t(op->ne) * r0, s);
+      apply_in<double2, double2>(op->mesh, b, 1.0, 1.0, 1.0, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
+      apply_y<double2, double2>(op, op->plan1, nr, s);
+      to_c128<double2>(op->wa.p, int64_t(op->ne) * nr, jo, s);
     }
   }
   DBuf<double> da, dr;

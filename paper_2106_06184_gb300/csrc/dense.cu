@@ -16,6 +16,7 @@
 
 #include "dense.h"
 #include "gemm_tc.h"
+#include "widen.cuh"
 
 namespace sldm {
 
@@ -728,8 +729,10 @@ __device__ __forceinline__ void warp_tsum(R (&v)[K], int lane) {
 // join the error sum, so the result is that of the FP64 operator A + Alo.
 template <class CM, class CV, int NR, bool LO = false>
 __global__ void __launch_bounds__(256, LO ? 1 : 2) gemv_tile_kernel(const GemvJob* __restrict__ jobs,
-                                                                   const int2* __restrict__ tiles, int nrhs, int col0) {
+                                                                   const int2* __restrict__ tiles, int nrhs_, int col00) {
   typedef GemvTile<CM, CV> T;
+  // passes of NR right-hand sides side by side (blockIdx.y), the last one possibly fewer
+  const int col0 = col00 + int(blockIdx.y) * NR, nrhs = min(NR, nrhs_ - int(blockIdx.y) * NR);
   typedef typename CT<CV>::R R;
   constexpr int RW = T::RW, CW = T::CW, ST = T::ST;
   constexpr size_t a_all = (LO ? 2 : 1) * T::a_stage;     // matrix bytes per stage
@@ -915,14 +918,19 @@ __global__ void __launch_bounds__(256, LO ? 1 : 2) gemv_tile_kernel(const GemvJo
     for (int i = 0; i < RW * NR * 2; ++i) acc[i] = R(cs[i]) + R(cc[i]);
   }
   cp_wait<0>();
-  constexpr int K = RW * NR * 2;
+  // the exchange takes a power of two of sums: the odd counts' missing ones are zero
+  constexpr int K0 = RW * NR * 2;
+  constexpr int K = K0 <= 4 ? 4 : K0 <= 8 ? 8 : K0 <= 16 ? 16 : K0 <= 32 ? 32 : 64;
+  R sums[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) sums[i] = i < K0 ? acc[i < K0 ? i : 0] : R(0);
   constexpr int V = K >= 32 ? K / 32 : 1;
   constexpr int S = K >= 32 ? 0 : (K == 16 ? 1 : K == 8 ? 2 : K == 4 ? 3 : 4);
-  warp_tsum<K, 16>(acc, lane);
+  warp_tsum<K, 16>(sums, lane);
   CV* y = reinterpret_cast<CV*>(J.y) + int64_t(col0) * J.ldy;
   auto put = [&](int p, R re, R im) {  // p = row-in-warp * NR + rhs
     const int i = p / NR, r = p % NR, row = row0 + i;
-    if (row < J.m && r < nrhs) {
+    if (i < RW && row < J.m && r < nrhs) {
       R vr = R(J.ar) * re - R(J.ai) * im;
       R vi = R(J.ar) * im + R(J.ai) * re;
       CV* yy = y + int64_t(r) * J.ldy + row;
@@ -936,11 +944,11 @@ __global__ void __launch_bounds__(256, LO ? 1 : 2) gemv_tile_kernel(const GemvJo
   };
   if constexpr (V >= 2) {
 #pragma unroll
-    for (int q = 0; q < V / 2; ++q) put((V / 2) * lane + q, acc[2 * q], acc[2 * q + 1]);
+    for (int q = 0; q < V / 2; ++q) put((V / 2) * lane + q, sums[2 * q], sums[2 * q + 1]);
   } else {
-    const R other = __shfl_xor_sync(0xffffffffu, acc[0], 1 << S);
+    const R other = __shfl_xor_sync(0xffffffffu, sums[0], 1 << S);
     const int idx = lane >> S;
-    if ((lane & ((1 << S) - 1)) == 0 && (idx & 1) == 0) put(idx >> 1, acc[0], other);
+    if ((lane & ((1 << S) - 1)) == 0 && (idx & 1) == 0) put(idx >> 1, sums[0], other);
   }
 }
 
@@ -958,7 +966,8 @@ static void launch_tile(const GemvPlan& plan, int nrhs, cudaStream_t s, int col0
                                    int(smem)));
     done.fetch_or(bit);
   }
-  gemv_tile_kernel<CM, CV, NR, LO><<<unsigned(plan.ntiles), 256, smem, s>>>(plan.jobs, plan.tiles, nrhs, col0);
+  gemv_tile_kernel<CM, CV, NR, LO><<<dim3(unsigned(plan.ntiles), unsigned((nrhs + NR - 1) / NR)), 256, smem, s>>>(plan.jobs, plan.tiles,
+                                                                                                              nrhs, col0);
   count_launch();
 }
 
@@ -984,24 +993,39 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s) {
     SLDM_REQUIRE((plan.tiles != nullptr && plan.tile_rows == GemvTile<CM, CV>::ROWS), SLDM_EINVAL,
                  "GEMV plan without row tiles for this vector type");
     if (plan.ntiles == 0) return;
-    // passes of up to 8 right-hand sides on the CUDA cores
-    for (int c0 = 0; c0 < nrhs; c0 += TILE_NRHS) {
-      const int nr = std::min(TILE_NRHS, nrhs - c0);
-      if constexpr (comp) {
-        if (plan.has_lo) {  // the FP64 operator held as a complex64 pair
-          if (nr <= 1) launch_tile<CM, CV, 1, true>(plan, nr, s, c0);
-          else if (nr <= 2) launch_tile<CM, CV, 2, true>(plan, nr, s, c0);
-          else if (nr <= 4) launch_tile<CM, CV, 4, true>(plan, nr, s, c0);
-          else launch_tile<CM, CV, 8, true>(plan, nr, s, c0);
-          continue;
-        }
+    // Passes of 8 right-hand sides on the CUDA cores, all in one launch.  In FP64 and in
+    // the compensated product the arithmetic is the bound (4 DFMA or ~44 FP32 operations per
+    // entry and right-hand side), so the rest takes a kernel of its own width; complex64
+    // passes, bound by launches and L2, take it as one more pass of 8.
+    // (box of 432 triangles, FP64, 5 right-hand sides: 425 us with 8 -> 272 us)
+    const int full = c64 && nrhs > 4 ? nrhs : nrhs / TILE_NRHS * TILE_NRHS, rest = nrhs - full;
+    auto go = [&](auto lo) {
+      constexpr bool LO = decltype(lo)::value;
+      if (full > 0) launch_tile<CM, CV, 8, LO>(plan, full, s, 0);
+      switch (rest) {
+        case 1:
+          if constexpr (comp) launch_tile<CM, CV, 1, LO>(plan, rest, s, full);
+          else launch_tile<CM, CV, 2, LO>(plan, rest, s, full);
+          break;
+        case 2: launch_tile<CM, CV, 2, LO>(plan, rest, s, full); break;
+        case 3:
+          if constexpr (c64) launch_tile<CM, CV, 4, LO>(plan, rest, s, full);
+          else launch_tile<CM, CV, 3, LO>(plan, rest, s, full);
+          break;
+        case 4: launch_tile<CM, CV, 4, LO>(plan, rest, s, full); break;
+        default:
+          if constexpr (!c64) {
+            if (rest == 5) launch_tile<CM, CV, 5, LO>(plan, rest, s, full);
+            else if (rest == 6) launch_tile<CM, CV, 6, LO>(plan, rest, s, full);
+            else if (rest == 7) launch_tile<CM, CV, 7, LO>(plan, rest, s, full);
+          }
       }
-      if (nr <= 1) {
-        if constexpr (comp) launch_tile<CM, CV, 1>(plan, nr, s, c0);  // the only one-column use
-        else launch_tile<CM, CV, 2>(plan, nr, s, c0);
-      } else if (nr <= 2) launch_tile<CM, CV, 2>(plan, nr, s, c0);
-      else if (nr <= 4) launch_tile<CM, CV, 4>(plan, nr, s, c0);
-      else launch_tile<CM, CV, 8>(plan, nr, s, c0);
+    };
+    if constexpr (comp) {
+      if (plan.has_lo) go(std::true_type{});  // the FP64 operator held as a complex64 pair
+      else go(std::false_type{});
+    } else {
+      go(std::false_type{});
     }
   } else {
     gemv_jobs_kernel<CM, CV, 1><<<blocks, 256, 0, s>>>(plan.jobs, plan.rowstart, plan.njobs, plan.total_rows, nrhs);
@@ -1080,156 +1104,232 @@ void gemv_jobs(const GemvPlan& plan, int nrhs, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- structured product glue
-// x (complex128, N x nrhs) -> op precision split vectors j (ne), e (ne), u (nq) per rhs.
-template <class C>
-__global__ void split_in_kernel(const double2* __restrict__ x, int64_t ldx, int ne, int nq, C* j, C* e, C* u, int nrhs) {
-  int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  int r = blockIdx.y;
-  if (i >= 2 * ne + nq) return;
-  double2 v = x[int64_t(r) * ldx + i];
-  C c;
-  c.x = decltype(c.x)(v.x);
-  c.y = decltype(c.y)(v.y);
-  if (i < ne) j[int64_t(r) * ne + i] = c;
-  else if (i < 2 * ne) e[int64_t(r) * ne + (i - ne)] = c;
-  else u[int64_t(r) * nq + (i - 2 * ne)] = c;
-}
-
-// a = j - t1 (ne);  c = u + t2 (nq);  bc = B c, bu = B u (nt), one CTA per (object, rhs)
-template <class C>
-__global__ void prep_kernel(const ApplyDims D, const int32_t* __restrict__ tri_begin, const int32_t* __restrict__ edge_begin,
-                            const C* __restrict__ j, const C* __restrict__ u, const C* __restrict__ t1, const C* __restrict__ t2,
-                            C* a, C* c, C* bc, C* bu) {
-  typedef typename CT<C>::R R;
-  const int o = blockIdx.x, r = blockIdx.y;
-  const int t0 = tri_begin[o], t1e = tri_begin[o + 1];
-  const int q0 = t0 - o, nq_o = t1e - t0 - 1;
-  const int e0 = edge_begin[o], e1 = edge_begin[o + 1];
-  const C* jr = j + int64_t(r) * D.ne;
-  const C* t1r = t1 + int64_t(r) * D.ne;
-  C* ar = a + int64_t(r) * D.ne;
-  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    C v;
-    v.x = jr[e].x - t1r[e].x;
-    v.y = jr[e].y - t1r[e].y;
-    ar[e] = v;
-  }
-  const C* ur = u + int64_t(r) * D.nq;
-  const C* t2r = t2 + int64_t(r) * D.nq;
-  C* cr = c + int64_t(r) * D.nq;
-  C* bcr = bc + int64_t(r) * D.nt;
-  C* bur = bu + int64_t(r) * D.nt;
-  double sc_r = 0, sc_i = 0, su_r = 0, su_i = 0;
-  for (int q = threadIdx.x; q < nq_o; q += blockDim.x) {
-    C uv = ur[q0 + q];
-    C v;
-    v.x = uv.x + t2r[q0 + q].x;
-    v.y = uv.y + t2r[q0 + q].y;
-    cr[q0 + q] = v;
-    bcr[t0 + q] = v;
-    bur[t0 + q] = uv;
-    sc_r += v.x;
-    sc_i += v.y;
-    su_r += uv.x;
-    su_i += uv.y;
-  }
-  __shared__ double red[4][256];
-  red[0][threadIdx.x] = sc_r;
-  red[1][threadIdx.x] = sc_i;
-  red[2][threadIdx.x] = su_r;
-  red[3][threadIdx.x] = su_i;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int k = 0; k < 4; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    C v;
-    v.x = R(-red[0][0]);
-    v.y = R(-red[1][0]);
-    bcr[t1e - 1] = v;
-    v.x = R(-red[2][0]);
-    v.y = R(-red[3][0]);
-    bur[t1e - 1] = v;
-  }
-}
-
-// y1 = z1 + D^T z2 + I_x e;  y2 = w1 - w2 + D^T w3;  y3 = F D a + k0^2 c   (complex128 output)
-template <class C>
-__global__ void combine_kernel(const ApplyDims D, double k0, const int32_t* __restrict__ tplus, const int32_t* __restrict__ tminus,
-                               const int32_t* __restrict__ tri_edge, const int8_t* __restrict__ tri_sign,
-                               const int32_t* __restrict__ q2t, const int32_t* __restrict__ ix_ptr,
-                               const int32_t* __restrict__ ix_col, const double* __restrict__ ix_val, const C* __restrict__ z1,
-                               const C* __restrict__ z2, const C* __restrict__ w1, const C* __restrict__ w2,
-                               const C* __restrict__ w3, const C* __restrict__ e, const C* __restrict__ a,
-                               const C* __restrict__ c, double2* y, int64_t ldy) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+// The columns of a pass into the work vectors: x (blocks scaled by s1, s2, s3) into j,
+// a = j (gemv_y subtracts Y11 e), e, bu = B u and bc = B u (gemv_y adds B Y21 e), in the
+// product's precision.  Blocks below nobj take one object's charges (B u: the last
+// triangle's is minus the sum of the others), the others 256 edge entries.
+template <class CX, class C>
+__global__ void __launch_bounds__(256) apply_in_kernel(VecBatch<CX, double2> xb, double s1, double s2, double s3, const ApplyDims D,
+                                                       const int32_t* __restrict__ tri_begin, C* __restrict__ j, C* __restrict__ a,
+                                                       C* __restrict__ e, C* __restrict__ bu, C* __restrict__ bc) {
   const int r = blockIdx.y;
+  const CX* __restrict__ x = xb.x[r];
+  auto conv = [](const CX v, double sc) {
+    C o;
+    o.x = decltype(o.x)(sc * widen(v.x));
+    o.y = decltype(o.y)(sc * widen(v.y));
+    return o;
+  };
+  if (int(blockIdx.x) >= D.nobj) {
+    const int i = (int(blockIdx.x) - D.nobj) * 256 + threadIdx.x;
+    if (i >= 2 * D.ne) return;
+    const C c = conv(x[i], i < D.ne ? s1 : s2);
+    if (i < D.ne) {
+      j[int64_t(r) * D.ne + i] = c;
+      a[int64_t(r) * D.ne + i] = c;
+    } else {
+      e[int64_t(r) * D.ne + (i - D.ne)] = c;
+    }
+    return;
+  }
+  const int o = blockIdx.x, t0 = tri_begin[o], nq = tri_begin[o + 1] - t0 - 1;
+  const CX* __restrict__ u = x + 2 * int64_t(D.ne) + (t0 - o);
+  C* __restrict__ bur = bu + int64_t(r) * D.nt + t0;
+  C* __restrict__ bcr = bc + int64_t(r) * D.nt + t0;
+  double sr = 0, si = 0;
+  for (int q = threadIdx.x; q < nq; q += 256) {
+    const C c = conv(u[q], s3);
+    bur[q] = c;
+    bcr[q] = c;
+    sr += widen(c.x);
+    si += widen(c.y);
+  }
+  __shared__ double red[2][8];
+  for (int w = 16; w > 0; w >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, w);
+    si += __shfl_xor_sync(0xffffffffu, si, w);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = sr;
+    red[1][threadIdx.x >> 5] = si;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      sr += red[0][w];
+      si += red[1][w];
+    }
+    C c;
+    c.x = decltype(c.x)(-sr);
+    c.y = decltype(c.y)(-si);
+    bur[nq] = c;
+    bcr[nq] = c;
+  }
+}
+
+// y1 = z1 + D^T z2 + I_x e;  y2 = w1 - w2 + D^T w3;  y3 = F D a + k0^2 c (c: bc without each
+// object's last entry), the third block scaled by s3, into the columns yb.y.  A
+// thread takes one row for up to CR right-hand sides, which share its sparse entries: 4
+// where the rows fill the device (32 columns of N = 34,524: 102 -> 63 us), one where it is
+// the chain of loads that counts (N = 1,279, 12 columns: 19 us with 4, 6 with 1).
+// With zh: the step's Gram-Schmidt accumulators are cleared too (nzh complex entries of
+// zh[r] and nrm[r], per column).
+struct CombineClear {
+  double2* h[MAX_NRHS];
+  double* nrm;
+  int n;
+};
+template <class C, class CY, int CR>
+__global__ void __launch_bounds__(128) combine_kernel(const ApplyDims D, double k0, const int32_t* __restrict__ tplus,
+                                                      const int32_t* __restrict__ tminus, const int32_t* __restrict__ tri_edge,
+                                                      const int8_t* __restrict__ tri_sign, const int32_t* __restrict__ q2t,
+                                                      const int32_t* __restrict__ ix_ptr, const int32_t* __restrict__ ix_col,
+                                                      const double* __restrict__ ix_val, const C* __restrict__ z1,
+                                                      const C* __restrict__ z2, const C* __restrict__ w1, const C* __restrict__ w2,
+                                                      const C* __restrict__ w3, const C* __restrict__ e, const C* __restrict__ a,
+                                                      const C* __restrict__ bc, double s3, VecBatch<double2, CY> yb, int nrhs,
+                                                      CombineClear clr) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r0 = blockIdx.y * CR;
   const int ne = D.ne, nt = D.nt, nq = D.nq;
+  if (clr.n > 0)
+    for (int r = r0; r < min(nrhs, r0 + CR); ++r) {
+      if (i < clr.n) clr.h[r][i] = make_double2(0.0, 0.0);
+      if (i == 0) clr.nrm[r] = 0.0;
+    }
   if (i >= 2 * ne + nq) return;
-  double vr, vi;
+  double vr[CR], vi[CR];
   if (i < ne) {
-    const int m = int(i);
-    C a1 = z1[int64_t(r) * ne + m];
-    C p = z2[int64_t(r) * nt + tplus[m]], q = z2[int64_t(r) * nt + tminus[m]];
-    vr = double(a1.x) + double(p.x) - double(q.x);
-    vi = double(a1.y) + double(p.y) - double(q.y);
-    for (int z = ix_ptr[m]; z < ix_ptr[m + 1]; ++z) {
-      C ev = e[int64_t(r) * ne + ix_col[z]];
-      vr += ix_val[z] * double(ev.x);
-      vi += ix_val[z] * double(ev.y);
+    const int m = i, tp = tplus[m], tm = tminus[m];
+#pragma unroll
+    for (int q = 0; q < CR; ++q)
+      if (r0 + q < nrhs) {
+        const int64_t r = r0 + q;
+        const C v = z1[r * ne + m], p = z2[r * nt + tp], g = z2[r * nt + tm];
+        vr[q] = widen(v.x) + widen(p.x) - widen(g.x);
+        vi[q] = widen(v.y) + widen(p.y) - widen(g.y);
+      }
+    const int z1e = ix_ptr[m + 1];
+#pragma unroll 4
+    for (int z = ix_ptr[m]; z < z1e; ++z) {
+      const int col = ix_col[z];
+      const double x = ix_val[z];
+#pragma unroll
+      for (int q = 0; q < CR; ++q)
+        if (r0 + q < nrhs) {
+          const C ev = e[int64_t(r0 + q) * ne + col];
+          vr[q] = fma(x, widen(ev.x), vr[q]);
+          vi[q] = fma(x, widen(ev.y), vi[q]);
+        }
     }
   } else if (i < 2 * ne) {
-    const int m = int(i - ne);
-    C a1 = w1[int64_t(r) * ne + m], b1 = w2[int64_t(r) * ne + m];
-    C p = w3[int64_t(r) * nt + tplus[m]], q = w3[int64_t(r) * nt + tminus[m]];
-    vr = double(a1.x) - double(b1.x) + double(p.x) - double(q.x);
-    vi = double(a1.y) - double(b1.y) + double(p.y) - double(q.y);
+    const int m = i - ne, tp = tplus[m], tm = tminus[m];
+#pragma unroll
+    for (int q = 0; q < CR; ++q)
+      if (r0 + q < nrhs) {
+        const int64_t r = r0 + q;
+        const C v = w1[r * ne + m], b = w2[r * ne + m], p = w3[r * nt + tp], g = w3[r * nt + tm];
+        vr[q] = widen(v.x) - widen(b.x) + widen(p.x) - widen(g.x);
+        vi[q] = widen(v.y) - widen(b.y) + widen(p.y) - widen(g.y);
+      }
   } else {
-    const int qq = int(i - 2 * ne);
-    const int t = q2t[qq];  // triangle of charge unknown qq (each object's last triangle has none)
-    double sr = 0, si = 0;
-    for (int k = 0; k < 3; ++k) {
-      C av = a[int64_t(r) * ne + tri_edge[3 * t + k]];
-      double sg = double(tri_sign[3 * t + k]);
-      sr += sg * double(av.x);
-      si += sg * double(av.y);
-    }
-    C cv = c[int64_t(r) * nq + qq];
-    vr = sr + k0 * k0 * double(cv.x);
-    vi = si + k0 * k0 * double(cv.y);
+    const int t = q2t[i - 2 * ne];  // triangle of the charge unknown (each object's last triangle has none)
+    const double kk = k0 * k0;
+#pragma unroll
+    for (int q = 0; q < CR; ++q)
+      if (r0 + q < nrhs) {
+        const int64_t r = r0 + q;
+        double sr = 0, si = 0;
+        for (int k = 0; k < 3; ++k) {
+          const C av = a[r * ne + tri_edge[3 * t + k]];
+          const bool neg = tri_sign[3 * t + k] < 0;
+          sr += neg ? -widen(av.x) : widen(av.x);
+          si += neg ? -widen(av.y) : widen(av.y);
+        }
+        const C cv = bc[r * nt + t];
+        vr[q] = s3 * fma(kk, widen(cv.x), sr);
+        vi[q] = s3 * fma(kk, widen(cv.y), si);
+      }
   }
-  y[int64_t(r) * ldy + i] = make_double2(vr, vi);
+#pragma unroll
+  for (int q = 0; q < CR; ++q)
+    if (r0 + q < nrhs) {
+      CY o;
+      o.x = decltype(o.x)(vr[q]);
+      o.y = decltype(o.y)(vi[q]);
+      yb.y[r0 + q][i] = o;
+    }
 }
 
-template <class C>
-void apply_glue_split(const double2* x, int64_t ldx, const ApplyDims& D, void* j, void* e, void* u, int nrhs, cudaStream_t s) {
-  int64_t N = 2 * D.ne + D.nq;
-  split_in_kernel<C><<<dim3(unsigned((N + 255) / 256), nrhs), 256, 0, s>>>(x, ldx, D.ne, D.nq, (C*)j, (C*)e, (C*)u, nrhs), ::sldm::count_launch();
+template <class CX, class C>
+void apply_in(const sldm_mesh* m, const VecBatch<CX, double2>& x, double s1, double s2, double s3, const ApplyDims& D, void* j,
+              void* a, void* e, void* bu, void* bc, int nrhs, cudaStream_t s) {
+  apply_in_kernel<CX, C><<<dim3(unsigned(D.nobj + (2 * D.ne + 255) / 256), nrhs), 256, 0, s>>>(
+      x, s1, s2, s3, D, m->d.tri_begin.p, (C*)j, (C*)a, (C*)e, (C*)bu, (C*)bc), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
+template void apply_in<double2, double2>(const sldm_mesh*, const VecBatch<double2, double2>&, double, double, double,
+                                         const ApplyDims&, void*, void*, void*, void*, void*, int, cudaStream_t);
+template void apply_in<double2, float2>(const sldm_mesh*, const VecBatch<double2, double2>&, double, double, double,
+                                        const ApplyDims&, void*, void*, void*, void*, void*, int, cudaStream_t);
+template void apply_in<float2, float2>(const sldm_mesh*, const VecBatch<float2, double2>&, double, double, double,
+                                       const ApplyDims&, void*, void*, void*, void*, void*, int, cudaStream_t);
 
-template <class C>
-void apply_glue_prep(const sldm_mesh* m, const ApplyDims& D, const void* j, const void* u, const void* t1, const void* t2,
-                     void* a, void* c, void* bc, void* bu, int nrhs, cudaStream_t s, const int32_t* tri_begin_dev,
-                     const int32_t* edge_begin_dev) {
-  prep_kernel<C><<<dim3(unsigned(D.nobj), nrhs), 256, 0, s>>>(D, tri_begin_dev, edge_begin_dev, (const C*)j, (const C*)u,
-                                                             (const C*)t1, (const C*)t2, (C*)a, (C*)c, (C*)bc, (C*)bu), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-
-template <class C>
-void apply_glue_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1,
-                        const void* z2, const void* w1, const void* w2, const void* w3, const void* e, const void* a,
-                        const void* c, double2* y, int64_t ldy, int nrhs, cudaStream_t s) {
-  int64_t N = 2 * D.ne + D.nq;
+template <class C, class CY>
+void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1, const void* z2,
+                   const void* w1, const void* w2, const void* w3, const void* e, const void* a, const void* bc, double s3,
+                   const VecBatch<double2, CY>& y, int nrhs, cudaStream_t s, double2* const* zh, int nzh, double* nrm) {
   const DevMesh& d = m->d;
-  combine_kernel<C><<<dim3(unsigned((N + 255) / 256), nrhs), 256, 0, s>>>(
-      D, k0, d.tplus.p, d.tminus.p, d.tri_edge.p, d.tri_sign.p, d.q2t.p, d.ix_ptr.p, d.ix_col.p, ix_val, (const C*)z1,
-      (const C*)z2, (const C*)w1, (const C*)w2, (const C*)w3, (const C*)e, (const C*)a, (const C*)c, y, ldy), ::sldm::count_launch();
+  CombineClear clr{};
+  if (zh) {
+    for (int r = 0; r < nrhs; ++r) clr.h[r] = zh[r];
+    clr.nrm = nrm;
+    clr.n = nzh;
+  }
+  const int rows = std::max(2 * D.ne + D.nq, clr.n);
+  auto go = [&](auto cr) {
+    constexpr int CR = decltype(cr)::value;
+    combine_kernel<C, CY, CR><<<dim3(unsigned((rows + 127) / 128), unsigned((nrhs + CR - 1) / CR)), 128, 0, s>>>(
+        D, k0, d.tplus.p, d.tminus.p, d.tri_edge.p, d.tri_sign.p, d.q2t.p, d.ix_ptr.p, d.ix_col.p, ix_val, (const C*)z1,
+        (const C*)z2, (const C*)w1, (const C*)w2, (const C*)w3, (const C*)e, (const C*)a, (const C*)bc, s3, y, nrhs, clr),
+        ::sldm::count_launch();
+  };
+  if (int64_t(rows) * nrhs > (1 << 17)) go(std::integral_constant<int, 4>{});
+  else go(std::integral_constant<int, 1>{});
   SLDM_CUDA(cudaGetLastError());
 }
+#define SLDM_COMBINE_INST(C, CY)                                                                                               \
+  template void apply_combine<C, CY>(const sldm_mesh*, const ApplyDims&, double, const double*, const void*, const void*,     \
+                                     const void*, const void*, const void*, const void*, const void*, const void*, double,    \
+                                     const VecBatch<double2, CY>&, int, cudaStream_t, double2* const*, int, double*);
+SLDM_COMBINE_INST(double2, double2)
+SLDM_COMBINE_INST(float2, double2)
+SLDM_COMBINE_INST(float2, float2)
+#undef SLDM_COMBINE_INST
+
+// row n of an (n + 1) x nc row-major block: minus the sum of its first n rows (the
+// eliminated charge of each column)
+template <class C>
+__global__ void neg_colsum_kernel(C* A, int n, int nc) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nc) return;
+  double sr = 0, si = 0;
+  for (int i = 0; i < n; ++i) {
+    const C v = A[int64_t(i) * nc + c];
+    sr += double(v.x);
+    si += double(v.y);
+  }
+  A[int64_t(n) * nc + c].x = decltype(A->x)(-sr);
+  A[int64_t(n) * nc + c].y = decltype(A->y)(-si);
+}
+template <class C>
+void neg_colsum(C* A, int n, int nc, cudaStream_t s) {
+  if (nc <= 0) return;
+  neg_colsum_kernel<C><<<(nc + 63) / 64, 64, 0, s>>>(A, n, nc), ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+template void neg_colsum<float2>(float2*, int, int, cudaStream_t);
+template void neg_colsum<double2>(double2*, int, int, cudaStream_t);
 
 // ---------------------------------------------------------------- vector kernels for GMRES
 // Templated on the storage of the Krylov basis and of the vector being
@@ -1244,128 +1344,6 @@ template <>
 __device__ __forceinline__ float2 cmake<float2>(double x, double y) { return make_float2(float(x), float(y)); }
 template <>
 __device__ __forceinline__ double2 cmake<double2>(double x, double y) { return make_double2(x, y); }
-
-// w += sign * V[:, :k] h (arithmetic in w's precision).  A CTA owns 32 rows;
-// its 8 warps take every 8th Krylov column, four columns in flight, and the
-// partial sums meet in shared memory.
-template <class CB, class CW>
-__global__ void __launch_bounds__(256) vmul_kernel(const CB* __restrict__ V, int64_t ldv, int k,
-                                                   const double2* __restrict__ h, double sign, CW* w, int64_t n) {
-  typedef typename CT<CW>::R R;
-  __shared__ R part[8][32][2];
-  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
-  const int64_t t = int64_t(blockIdx.x) * 32 + lane;
-  R sr = 0, si = 0;
-  if (t < n) {
-    int i = slice;
-    for (; i + 24 < k; i += 32) {
-      CB v[4];
-      double2 c[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        v[u] = V[int64_t(i + 8 * u) * ldv + t];
-        c[u] = h[i + 8 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) cfma(sr, si, R(v[u].x), R(v[u].y), R(c[u].x), R(c[u].y));
-    }
-    for (; i < k; i += 8) {
-      const CB v = V[int64_t(i) * ldv + t];
-      const double2 c = h[i];
-      cfma(sr, si, R(v.x), R(v.y), R(c.x), R(c.y));
-    }
-  }
-  part[slice][lane][0] = sr;
-  part[slice][lane][1] = si;
-  __syncthreads();
-  if (slice == 0 && t < n) {
-    R ar = 0, ai = 0;
-    for (int q = 0; q < 8; ++q) {
-      ar += part[q][lane][0];
-      ai += part[q][lane][1];
-    }
-    const CW o = w[t];
-    w[t].x = o.x + R(sign) * ar;
-    w[t].y = o.y + R(sign) * ai;
-  }
-}
-
-template <class C>
-__global__ void norm2_kernel(const C* __restrict__ w, int64_t n, double* out) {
-  double s = 0;
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n; t += int64_t(gridDim.x) * blockDim.x) {
-    const C a = w[t];
-    s += double(a.x) * double(a.x) + double(a.y) * double(a.y);
-  }
-  __shared__ double r[256];
-  r[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) r[threadIdx.x] += r[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(out, r[0]);
-}
-
-// y = alpha * x + beta * y (real alpha, beta; FP64 arithmetic, y stored in its type;
-// beta = 0 ignores the old y)
-template <class CX, class CY>
-__global__ void axpby_kernel(int64_t n, double alpha, const CX* __restrict__ x, double beta, CY* y) {
-  int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const CX a = x[t];
-  double vr = alpha * double(a.x), vi = alpha * double(a.y);
-  if (beta != 0.0) {
-    const CY b = y[t];
-    vr += beta * double(b.x);
-    vi += beta * double(b.y);
-  }
-  y[t] = cmake<CY>(vr, vi);
-}
-
-// y[i] = s_b x[i] with s_b = s1 on [0, ne), s2 on [ne, 2 ne), s3 on [2 ne, n) (in place allowed)
-template <class CX, class CY>
-__global__ void vscale3_kernel(int64_t n, int64_t ne, double s1, double s2, double s3, const CX* __restrict__ x, CY* y) {
-  int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const double s = t < ne ? s1 : (t < 2 * ne ? s2 : s3);
-  const CX a = x[t];
-  y[t] = cmake<CY>(s * double(a.x), s * double(a.y));
-}
-
-template <class CX, class CY>
-void vscale3(int64_t n, int64_t ne, double s1, double s2, double s3, const CX* x, CY* y, cudaStream_t s) {
-  vscale3_kernel<CX, CY><<<unsigned((n + 255) / 256), 256, 0, s>>>(n, ne, s1, s2, s3, x, y), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-template <class CB, class CW>
-void vmul(const CB* V, int64_t ldv, int k, const double2* h, double sign, CW* w, int64_t n, cudaStream_t s) {
-  vmul_kernel<CB, CW><<<unsigned((n + 31) / 32), 256, 0, s>>>(V, ldv, k, h, sign, w, n), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-template <class C>
-void vnorm2(const C* w, int64_t n, double* out, cudaStream_t s) {
-  SLDM_CUDA(cudaMemsetAsync(out, 0, sizeof(double), s));
-  unsigned b = unsigned(std::min<int64_t>((n + 255) / 256, 1024));
-  norm2_kernel<C><<<b, 256, 0, s>>>(w, n, out), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-template <class CX, class CY>
-void vaxpby(int64_t n, double alpha, const CX* x, double beta, CY* y, cudaStream_t s) {
-  axpby_kernel<CX, CY><<<unsigned((n + 255) / 256), 256, 0, s>>>(n, alpha, x, beta, y), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-#define SLDM_VEC_INST(CX, CY)                                                                                   \
-  template void vscale3<CX, CY>(int64_t, int64_t, double, double, double, const CX*, CY*, cudaStream_t);       \
-  template void vmul<CX, CY>(const CX*, int64_t, int, const double2*, double, CY*, int64_t, cudaStream_t);     \
-  template void vaxpby<CX, CY>(int64_t, double, const CX*, double, CY*, cudaStream_t);
-SLDM_VEC_INST(double2, double2)
-SLDM_VEC_INST(float2, float2)
-SLDM_VEC_INST(float2, double2)
-SLDM_VEC_INST(double2, float2)
-#undef SLDM_VEC_INST
-template void vnorm2<double2>(const double2*, int64_t, double*, cudaStream_t);
-template void vnorm2<float2>(const float2*, int64_t, double*, cudaStream_t);
 
 // ---------------------------------------------------------------- batched Gram-Schmidt
 // One launch per pass for every live right-hand side of a lockstep step.  The
@@ -1425,39 +1403,42 @@ __global__ void __launch_bounds__(256) krylov_dots_kernel(KrylovStep ks) {
 
 // V_j[:, k] -= V_j[:, :k] h_j, and with `norm` nrm[j] += |V_j[:, k]|^2 after the
 // update.  Grid (ldv / 512, na): warp = 64 rows (lane = 2), over all k columns
-// with eight column loads in flight and no exchange between warps.
+// with eight column loads in flight and no exchange between warps.  The
+// coefficients are staged in shared memory in the arithmetic's precision: converting
+// them per lane (two per column, on the narrow FP64 pipe) cost as much as the HBM
+// read (N = 34,524, 32 right-hand sides, k ~ 90: 150 us per pass).
 template <class CB>
 __global__ void __launch_bounds__(256) krylov_update_kernel(KrylovStep ks, int norm) {
   typedef typename CT<CB>::R R;
+  extern __shared__ __align__(16) unsigned char ku_raw[];
+  CB* hs = reinterpret_cast<CB*>(ku_raw);
   const int lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5)) * 64;
-  if (r0 >= ks.ldv) return;  // whole warps
   const int j = blockIdx.y;
+  for (int i = threadIdx.x; i < ks.k; i += 256) hs[i] = cmake<CB>(ks.h[j][i].x, ks.h[j][i].y);
+  __syncthreads();
+  if (r0 >= ks.ldv) return;  // whole warps
   CB* V = reinterpret_cast<CB*>(ks.V[j]);
-  const double2* __restrict__ h = ks.h[j];
   const int64_t t = r0 + 2 * lane;
   R s0r = 0, s0i = 0, s1r = 0, s1i = 0;
   int i = 0;
   for (; i + 8 <= ks.k; i += 8) {
     CB a[8], b[8];
-    double2 c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) ld_pair(V + int64_t(i + u) * ks.ldv + t, a[u], b[u]);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      ld_pair(V + int64_t(i + u) * ks.ldv + t, a[u], b[u]);
-      c[u] = h[i + u];
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      cfma(s0r, s0i, R(a[u].x), R(a[u].y), R(c[u].x), R(c[u].y));
-      cfma(s1r, s1i, R(b[u].x), R(b[u].y), R(c[u].x), R(c[u].y));
+      const CB c = hs[i + u];
+      cfma(s0r, s0i, a[u].x, a[u].y, c.x, c.y);
+      cfma(s1r, s1i, b[u].x, b[u].y, c.x, c.y);
     }
   }
   for (; i < ks.k; ++i) {
     CB a, b;
     ld_pair(V + int64_t(i) * ks.ldv + t, a, b);
-    const double2 c = h[i];
-    cfma(s0r, s0i, R(a.x), R(a.y), R(c.x), R(c.y));
-    cfma(s1r, s1i, R(b.x), R(b.y), R(c.x), R(c.y));
+    const CB c = hs[i];
+    cfma(s0r, s0i, a.x, a.y, c.x, c.y);
+    cfma(s1r, s1i, b.x, b.y, c.x, c.y);
   }
   CB* w = V + int64_t(ks.k) * ks.ldv + t;
   CB a, b;
@@ -1484,7 +1465,7 @@ void krylov_dots(const KrylovStep& ks, cudaStream_t s) {
 template <class CB>
 void krylov_update(const KrylovStep& ks, bool norm, cudaStream_t s) {
   if (ks.na <= 0) return;
-  krylov_update_kernel<CB><<<dim3(unsigned((ks.ldv / 64 + 7) / 8), ks.na), 256, 0, s>>>(ks, norm ? 1 : 0),
+  krylov_update_kernel<CB><<<dim3(unsigned((ks.ldv / 64 + 7) / 8), ks.na), 256, size_t(ks.k) * sizeof(CB), s>>>(ks, norm ? 1 : 0),
       ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
@@ -1493,32 +1474,6 @@ template void krylov_dots<double2>(const KrylovStep&, cudaStream_t);
 template void krylov_update<float2>(const KrylovStep&, bool, cudaStream_t);
 template void krylov_update<double2>(const KrylovStep&, bool, cudaStream_t);
 
-// y_j = a_j s(i) x_j[i] for the na column pairs, s = s1, s2, s3 on the three blocks
-template <class CX, class CY>
-__global__ void vscale3_batch_kernel(int64_t n, int64_t ne, double s1, double s2, double s3, VecBatch<CX, CY> b) {
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const int j = blockIdx.y;
-  const double sc = b.a[j] * (t < ne ? s1 : (t < 2 * ne ? s2 : s3));
-  const CX v = b.x[j][t];
-  b.y[j][t] = cmake<CY>(sc * double(v.x), sc * double(v.y));
-}
-template <class CX, class CY>
-void vscale3_batch(int64_t n, int64_t ne, double s1, double s2, double s3, const VecBatch<CX, CY>& b, int na,
-                   cudaStream_t s) {
-  if (na <= 0) return;
-  vscale3_batch_kernel<CX, CY><<<dim3(unsigned((n + 255) / 256), na), 256, 0, s>>>(n, ne, s1, s2, s3, b), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-template void vscale3_batch<double2, double2>(int64_t, int64_t, double, double, double, const VecBatch<double2, double2>&, int,
-                                              cudaStream_t);
-template void vscale3_batch<float2, double2>(int64_t, int64_t, double, double, double, const VecBatch<float2, double2>&, int,
-                                             cudaStream_t);
-template void vscale3_batch<double2, float2>(int64_t, int64_t, double, double, double, const VecBatch<double2, float2>&, int,
-                                             cudaStream_t);
-template void vscale3_batch<float2, float2>(int64_t, int64_t, double, double, double, const VecBatch<float2, float2>&, int,
-                                            cudaStream_t);
-
 // ---------------------------------------------------------------- conversions
 template <class C>
 __global__ void to_c128_kernel(const C* __restrict__ src, int64_t n, double2* dst) {
@@ -1526,24 +1481,10 @@ __global__ void to_c128_kernel(const C* __restrict__ src, int64_t n, double2* ds
   if (t < n) dst[t] = make_double2(double(src[t].x), double(src[t].y));
 }
 template <class C>
-__global__ void from_c128_kernel(const double2* __restrict__ src, int64_t n, C* dst) {
-  int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t < n) {
-    dst[t].x = decltype(dst[t].x)(src[t].x);
-    dst[t].y = decltype(dst[t].y)(src[t].y);
-  }
-}
-template <class C>
 void to_c128(const void* src, int64_t n, double2* dst, cudaStream_t s) {
   to_c128_kernel<C><<<unsigned((n + 255) / 256), 256, 0, s>>>((const C*)src, n, dst), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
-template <class C>
-void from_c128(const double2* src, int64_t n, void* dst, cudaStream_t s) {
-  from_c128_kernel<C><<<unsigned((n + 255) / 256), 256, 0, s>>>(src, n, (C*)dst), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-
 // FP64 operator kept as a complex64 pair: hi = fl32(v), lo = fl32(v - hi)
 __global__ void split_c128_kernel(const double2* __restrict__ src, int64_t n, float2* __restrict__ hi,
                                   float2* __restrict__ lo) {
@@ -1690,168 +1631,11 @@ void copy_scaled(const void* src, int64_t n, double alpha, void* dst, cudaStream
   template void build_Ml<C>(const sldm_mesh*, int, double, const void*, int64_t, const void*, int64_t, const void*,     \
                             int64_t, const double*, C*, C*, cudaStream_t);                                              \
   template void gemv_jobs<C>(const GemvPlan&, int, cudaStream_t);                                                       \
-  template void apply_glue_split<C>(const double2*, int64_t, const ApplyDims&, void*, void*, void*, int, cudaStream_t); \
-  template void apply_glue_prep<C>(const sldm_mesh*, const ApplyDims&, const void*, const void*, const void*,           \
-                                   const void*, void*, void*, void*, void*, int, cudaStream_t, const int32_t*,         \
-                                   const int32_t*);                                                                     \
-  template void apply_glue_combine<C>(const sldm_mesh*, const ApplyDims&, double, const double*, const void*,           \
-                                      const void*, const void*, const void*, const void*, const void*, const void*,     \
-                                      const void*, double2*, int64_t, int, cudaStream_t);                               \
   template void to_c128<C>(const void*, int64_t, double2*, cudaStream_t);                                               \
-  template void from_c128<C>(const double2*, int64_t, void*, cudaStream_t);                                             \
   template void add_ix<C>(const sldm_mesh*, int, double, const double*, void*, int64_t, cudaStream_t);             \
   template void copy_scaled<C>(const void*, int64_t, double, void*, cudaStream_t);
 INST(float2)
 INST(double2)
-
-// ---------------------------------------------------------------- GMRES on the device
-__device__ __forceinline__ double2 zmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-__device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -a.y); }
-__device__ __forceinline__ double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double zabs(double2 a) { return hypot(a.x, a.y); }
-
-// One warp per active right-hand side: the lanes stage column k of H and the
-// earlier rotations in shared memory, lane 0 applies the rotations in order (each
-// depends on the previous one) and the new one, and the lanes write the column back.
-__global__ void gmres_givens_kernel(GivensArgs a) {
-  extern __shared__ __align__(16) unsigned char gv_raw[];
-  double2* gsm = reinterpret_cast<double2*>(gv_raw);  // column (m + 2), cs (m), sn (m)
-  const int j = blockIdx.x;
-  if (j >= a.na) return;
-  const int r = a.on[j];
-  GmresState* st = a.st + r;
-  const int lane = threadIdx.x;
-  if (!st->live) {
-    if (lane == 0) a.scale[j] = 0.0;
-    return;
-  }
-  const int m = a.m, k = a.k;
-  const double2* hr = a.dh + int64_t(r) * a.ldh;
-  double2* H = a.H + int64_t(r) * (m + 1) * m;
-  double2* cs = a.cs + int64_t(r) * m;
-  double2* sn = a.sn + int64_t(r) * m;
-  double2* g = a.g + int64_t(r) * (m + 1);
-  double2* col = gsm;
-  double2* scs = gsm + (m + 2);
-  double2* ssn = scs + m;
-  const double h1 = sqrt(a.nrm[j]);
-  for (int i = lane; i <= k; i += 32) col[i] = zadd(hr[i], hr[(m + 2) + i]);
-  for (int i = lane; i < k; i += 32) {
-    scs[i] = cs[i];
-    ssn[i] = sn[i];
-  }
-  if (lane == 0) col[k + 1] = make_double2(h1, 0.0);
-  __syncwarp();
-  if (lane == 0) {
-    for (int i = 0; i < k; ++i) {  // the earlier rotations
-      const double2 x = col[i], y = col[i + 1];
-      col[i] = zadd(zmul(scs[i], x), zmul(ssn[i], y));
-      const double2 msn = zconj(ssn[i]);
-      col[i + 1] = zadd(make_double2(-(msn.x * x.x - msn.y * x.y), -(msn.x * x.y + msn.y * x.x)), zmul(scs[i], y));
-    }
-    const double2 x = col[k], y = col[k + 1];
-    const double ax = zabs(x);
-    const double t = sqrt(x.x * x.x + x.y * x.y + y.x * y.x + y.y * y.y);
-    double2 c, sv;
-    if (ax == 0) {
-      c = make_double2(0.0, 0.0);
-      sv = make_double2(1.0, 0.0);
-      col[k] = y;
-    } else {
-      const double2 ph = make_double2(x.x / ax, x.y / ax);  // a / |a|
-      c = make_double2(ax / t, 0.0);
-      const double2 p = zmul(ph, zconj(y));
-      sv = make_double2(p.x / t, p.y / t);
-      col[k] = make_double2(ph.x * t, ph.y * t);
-    }
-    col[k + 1] = make_double2(0.0, 0.0);
-    cs[k] = c;
-    sn[k] = sv;
-    const double2 gk = g[k];
-    const double2 msn = zconj(sv);
-    g[k + 1] = make_double2(-(msn.x * gk.x - msn.y * gk.y), -(msn.x * gk.y + msn.y * gk.x));
-    g[k] = zmul(c, gk);
-    st->it += 1;
-    st->kused = k + 1;
-    const double res = zabs(g[k + 1]);
-    if (res / st->bnorm <= a.tol || st->it >= a.maxit || h1 == 0) st->live = 0;
-    if (a.refine && res <= a.cycle * st->beta) st->live = 0;
-    a.scale[j] = h1 > 0 ? 1.0 / h1 : 0.0;
-  }
-  __syncwarp();
-  for (int i = lane; i <= k + 1; i += 32) H[int64_t(i) * m + k] = col[i];
-}
-
-void gmres_givens(const GivensArgs& a, cudaStream_t s) {
-  if (a.na <= 0) return;
-  const size_t smem = size_t(3 * a.m + 2) * sizeof(double2);
-  SLDM_REQUIRE(smem <= 48 * 1024, SLDM_EINVAL, "GMRES: restart length too large for the device rotations");
-  gmres_givens_kernel<<<a.na, 32, smem, s>>>(a), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-
-// one warp per right-hand side: back substitution, row by row from the bottom,
-// the sum over the columns to the right split across the lanes
-__global__ void gmres_backsolve_kernel(int na, const int* __restrict__ on, int m, const double2* __restrict__ H,
-                                       const double2* __restrict__ g, const GmresState* __restrict__ st, double2* dh,
-                                       int64_t ldh) {
-  const int j = blockIdx.x;
-  if (j >= na) return;
-  const int r = on[j];
-  const int ku = st[r].kused;
-  const double2* Hr = H + int64_t(r) * (m + 1) * m;
-  const double2* gr = g + int64_t(r) * (m + 1);
-  double2* y = dh + int64_t(r) * ldh;
-  const int lane = threadIdx.x;
-  for (int i = ku - 1; i >= 0; --i) {
-    double sr = 0, si = 0;
-    for (int c = i + 1 + lane; c < ku; c += 32) {
-      const double2 h = Hr[int64_t(i) * m + c], v = y[c];
-      sr += h.x * v.x - h.y * v.y;
-      si += h.x * v.y + h.y * v.x;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      sr += __shfl_down_sync(0xffffffffu, sr, o);
-      si += __shfl_down_sync(0xffffffffu, si, o);
-    }
-    if (lane == 0) {
-      const double2 acc = make_double2(gr[i].x - sr, gr[i].y - si);
-      const double2 d = Hr[int64_t(i) * m + i];
-      const double dn = d.x * d.x + d.y * d.y;
-      y[i] = make_double2((acc.x * d.x + acc.y * d.y) / dn, (acc.y * d.x - acc.x * d.y) / dn);
-    }
-    __syncwarp();
-  }
-}
-
-void gmres_backsolve(int na, const int* on, int m, const double2* H, const double2* g, const GmresState* st, double2* dh,
-                     int64_t ldh, cudaStream_t s) {
-  if (na <= 0) return;
-  gmres_backsolve_kernel<<<na, 32, 0, s>>>(na, on, m, H, g, st, dh, ldh), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-
-template <class CB>
-__global__ void vscale_dev_kernel(int64_t n, VecBatch<CB, CB> b, const double* __restrict__ scale) {
-  const int j = blockIdx.y;
-  const double a = scale[j];
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    CB v = b.x[j][i];
-    v.x = decltype(v.x)(double(v.x) * a);
-    v.y = decltype(v.y)(double(v.y) * a);
-    b.y[j][i] = v;
-  }
-}
-
-template <class CB>
-void vscale_dev_batch(int64_t n, const VecBatch<CB, CB>& b, const double* scale, int na, cudaStream_t s) {
-  if (na <= 0) return;
-  const unsigned gx = unsigned(std::min<int64_t>((n + 255) / 256, 1024));
-  vscale_dev_kernel<CB><<<dim3(gx, na), 256, 0, s>>>(n, b, scale), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
-}
-template void vscale_dev_batch<double2>(int64_t, const VecBatch<double2, double2>&, const double*, int, cudaStream_t);
-template void vscale_dev_batch<float2>(int64_t, const VecBatch<float2, float2>&, const double*, int, cudaStream_t);
 
 }  // namespace sldm
 

@@ -91,16 +91,27 @@ void gemv_autotune(GemvPlan& plan, cudaStream_t s);
 struct ApplyDims {
   int32_t ne, nt, nq, nobj;
 };
+template <class CX, class CY>
+struct VecBatch {
+  const CX* x[MAX_NRHS] = {};
+  CY* y[MAX_NRHS] = {};
+  double a[MAX_NRHS] = {};
+};
+// columns x (blocks scaled by s1, s2, s3) into the structured product's work vectors:
+// j, a = j, e, bu = B u, bc = B u (C: the product's precision)
+template <class CX, class C>
+void apply_in(const sldm_mesh* m, const VecBatch<CX, double2>& x, double s1, double s2, double s3, const ApplyDims& D, void* j,
+              void* a, void* e, void* bu, void* bc, int nrhs, cudaStream_t s);
+// the product's rows from its work vectors into the columns y (third block scaled by
+// s3); with zh, also clears nzh coefficients of every zh[r] and nrm[r]
+template <class C, class CY>
+void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1, const void* z2,
+                   const void* w1, const void* w2, const void* w3, const void* e, const void* a, const void* bc, double s3,
+                   const VecBatch<double2, CY>& y, int nrhs, cudaStream_t s, double2* const* zh = nullptr, int nzh = 0,
+                   double* nrm = nullptr);
+// row n of an (n + 1) x nc block = minus the sum of rows 0 .. n - 1
 template <class C>
-void apply_glue_split(const double2* x, int64_t ldx, const ApplyDims& D, void* j, void* e, void* u, int nrhs, cudaStream_t s);
-template <class C>
-void apply_glue_prep(const sldm_mesh* m, const ApplyDims& D, const void* j, const void* u, const void* t1, const void* t2,
-                     void* a, void* c, void* bc, void* bu, int nrhs, cudaStream_t s, const int32_t* tri_begin_dev,
-                     const int32_t* edge_begin_dev);
-template <class C>
-void apply_glue_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1,
-                        const void* z2, const void* w1, const void* w2, const void* w3, const void* e, const void* a,
-                        const void* c, double2* y, int64_t ldy, int nrhs, cudaStream_t s);
+void neg_colsum(C* A, int n, int nc, cudaStream_t s);
 
 // One Gram-Schmidt pass over the Krylov bases of the live right-hand sides of a
 // lockstep step: column k of each basis against its columns 0..k-1.  The
@@ -116,36 +127,12 @@ template <class CB>
 void krylov_dots(const KrylovStep& ks, cudaStream_t s);                // h_j += V_j[:, :k]^H V_j[:, k]
 template <class CB>
 void krylov_update(const KrylovStep& ks, bool norm, cudaStream_t s);   // V_j[:, k] -= V_j[:, :k] h_j
-template <class CX, class CY>
-struct VecBatch {
-  const CX* x[MAX_NRHS] = {};
-  CY* y[MAX_NRHS] = {};
-  double a[MAX_NRHS] = {};
-};
-// y_j = a_j s(i) x_j (s = s1 on [0, ne), s2 on [ne, 2 ne), s3 beyond), j < na, in place allowed
-template <class CX, class CY>
-void vscale3_batch(int64_t n, int64_t ne, double s1, double s2, double s3, const VecBatch<CX, CY>& b, int na,
-                   cudaStream_t s);
-
-// complex128 or complex64 storage (instantiated for double2 and float2; mixed
-// pairs for vmul, vaxpby and vscale3)
-template <class CB, class CW>
-void vmul(const CB* V, int64_t ldv, int k, const double2* h, double sign, CW* w, int64_t n, cudaStream_t s);
-template <class C>
-void vnorm2(const C* w, int64_t n, double* out, cudaStream_t s);
-template <class CX, class CY>
-void vaxpby(int64_t n, double alpha, const CX* x, double beta, CY* y, cudaStream_t s);
-template <class CX, class CY>
-void vscale3(int64_t n, int64_t ne, double s1, double s2, double s3, const CX* x, CY* y, cudaStream_t s);
-
 template <class C>
 void to_c128(const void* src, int64_t n, double2* dst, cudaStream_t s);
 // hi = complex64 rounding of src, lo = complex64 rounding of src - hi (src = hi + lo to ~2^-48)
 void split_c128(const double2* src, int64_t n, float2* hi, float2* lo, cudaStream_t s);
 // dst += lo (complex64 low parts onto a complex128 copy of the high parts)
 void add_lo_c128(const float2* lo, int64_t n, double2* dst, cudaStream_t s);
-template <class C>
-void from_c128(const double2* src, int64_t n, void* dst, cudaStream_t s);
 template <class C>
 void copy_scaled(const void* src, int64_t n, double alpha, void* dst, cudaStream_t s);
 // Copies of sub-blocks within one row-major matrix (leading dimension ld):
@@ -173,12 +160,11 @@ struct GmresState {
 // sqrt(nrm[j]); the earlier Givens rotations, a new one annihilating h_{k+1,k},
 // the rotated residual vector g_r; then the convergence tests (|g_{k+1}| <=
 // tol ||b||, it >= maxit, h_{k+1,k} = 0, and with refine |g_{k+1}| <= cycle
-// beta) clear live.  scale[j] = 1 / h_{k+1,k} for the next basis vector (0 once
-// the right-hand side has stopped).  H: (m + 1) x m row-major per right-hand
-// side, cs, sn: m, g: m + 1 (complex).
+// beta) clear live.  flags[r] (pinned host memory) receives whether r still iterates.
+// H: (m + 1) x m row-major per right-hand side, cs, sn: m, g: m + 1 (complex).
 struct GivensArgs {
   int k, m, na, refine;
-  const int* on;
+  int on[MAX_NRHS];
   const double2* dh;
   int64_t ldh;
   const double* nrm;
@@ -186,15 +172,44 @@ struct GivensArgs {
   GmresState* st;
   double tol, cycle;
   int maxit, pad;
-  double* scale;
+  int32_t* flags;
 };
-void gmres_givens(const GivensArgs& a, cudaStream_t s);
-// y_r = H_r^-1 g_r (upper triangular, kused_r columns) into dh + r * ldh, for the na
-// right-hand sides on[j] (one warp each).
-void gmres_backsolve(int na, const int* on, int m, const double2* H, const double2* g, const GmresState* st, double2* dh,
-                     int64_t ldh, cudaStream_t s);
-// y_j = scale[j] x_j (scale on the device), j < na, in place allowed
+// w_j (column ks.k of its basis) orthogonalised twice against columns 0 .. ks.k - 1, column
+// ks.k - 1 = a.k of H, the rotations and tests, and w_j / h_{k+1,k}: one launch of a cluster per
+// right-hand side for small systems, else separate kernels, which add up in h1[j] and
+// h2[j] (a.dh's two parts) and a.nrm (cleared by the caller).
 template <class CB>
-void vscale_dev_batch(int64_t n, const VecBatch<CB, CB>& b, const double* scale, int na, cudaStream_t s);
+void gmres_orthogonalise(const GivensArgs& a, KrylovStep ks, double2* const* h1, double2* const* h2, cudaStream_t s);
+// b = D b, r = b, nrm[c] += |b_c|^2 (D = diag(1, l) with l from entry n2 on; nr columns of n)
+void gmres_rhs(int64_t n, int64_t n2, double l, double2* b, double2* r, double* nrm, int nr, cudaStream_t s);
+// r = b - y, nrm[c] += |r_c|^2
+void gmres_residual(int64_t n, const double2* b, const double2* y, double2* r, double* nrm, int nr, cudaStream_t s);
+// A cycle's state and g of every column; v0 = r / beta of the live ones
+struct CycleStart {
+  int it[MAX_NRHS], live[MAX_NRHS];
+  double bnorm[MAX_NRHS], beta[MAX_NRHS];
+  void* v0[MAX_NRHS];
+  const double2* r;
+  GmresState* st;
+  double2* g;
+  int m;
+};
+template <class CB>
+void gmres_cycle_start(int64_t n, const CycleStart& a, int nr, cudaStream_t s);
+// y_r = H_r^-1 g_r (upper triangular, k[j] columns) into dh + r * ldh and out[j] = V[j] y_r for
+// the na right-hand sides r = on[j]
+struct CycleEnd {
+  int on[MAX_NRHS], k[MAX_NRHS];
+  void* V[MAX_NRHS];
+  double2* out[MAX_NRHS];
+  const double2 *H, *g;
+  double2* dh;
+  int64_t ldh, ldv;
+  int m;
+};
+template <class CB>
+void gmres_cycle_end(int64_t n, const CycleEnd& a, int na, cudaStream_t s);
+// y_j += diag(s1, 1, s3) x_j
+void gmres_add_scaled(int64_t n, int64_t ne, double s1, double s3, const VecBatch<double2, double2>& b, int na, cudaStream_t s);
 
 }  // namespace sldm

@@ -666,15 +666,14 @@ void gemm_tc(const GemvPlan& plan, const TcPlan& tp, int nrhs, cudaStream_t s) {
   SLDM_CUDA(cudaGetLastError());
 }
 
-void tc_check(const TcPlan& tp, cudaStream_t s) {
-  if (!tp.ok) return;
-  int h = 0;
-  SLDM_CUDA(cudaMemcpyAsync(&h, tp.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-  SLDM_CUDA(cudaStreamSynchronize(s));
-  if (h) {
-    SLDM_CUDA(cudaMemsetAsync(tp.err.p, 0, sizeof(int), s));
-    throw Error{SLDM_ETIMEOUT, "tensor-core product: a bounded wait ran out"};
-  }
+void tc_err_async(const TcPlan& tp, int* host, cudaStream_t s) {
+  *host = 0;
+  if (tp.ok) SLDM_CUDA(cudaMemcpyAsync(host, tp.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+}
+void tc_err_check(const TcPlan& tp, int err, cudaStream_t s) {
+  if (!err) return;
+  SLDM_CUDA(cudaMemsetAsync(tp.err.p, 0, sizeof(int), s));
+  throw Error{SLDM_ETIMEOUT, "tensor-core product: a bounded wait ran out"};
 }
 
 }  // namespace sldm

@@ -41,7 +41,10 @@ struct TcPlan {
 void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, cudaStream_t s);
 // One pass over every job of `plan` for nrhs (<= 32) right-hand sides.
 void gemm_tc(const GemvPlan& plan, const TcPlan& tp, int nrhs, cudaStream_t s);
-// SLDM_ETIMEOUT when a tensor-core pass recorded a bounded wait that ran out (reads and clears the flag).
-void tc_check(const TcPlan& tp, cudaStream_t s);
+// Queue a copy of the flag that a tensor-core pass sets when a bounded wait ran out
+// into *host (pinned); once the stream has been waited for, tc_err_check turns a set
+// flag into SLDM_ETIMEOUT and clears it.
+void tc_err_async(const TcPlan& tp, int* host, cudaStream_t s);
+void tc_err_check(const TcPlan& tp, int err, cudaStream_t s);
 
 }  // namespace sldm

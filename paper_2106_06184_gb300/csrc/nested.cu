@@ -17,15 +17,47 @@ static __global__ void identity_kernel(int64_t n, float2* __restrict__ b) {
   if (i < n * n) b[i] = make_float2(i / n == i % n ? 1.f : 0.f, 0.f);
 }
 
-// wt1[e0 + i] = y[i] / ell (i < ne), wt2[q0 + i] = ell y[ne + i] (i < nq), per column
-static __global__ void nested_out_kernel(int ne, int nq, int nr, const double2* __restrict__ y, int64_t ldw, double ell,
-                                  double2* __restrict__ wt1, int64_t ld1, double2* __restrict__ wt2, int64_t ld2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// a[e0 + i] -= y[i] / ell (i < ne), bc[t0 + q] += ell y[ne + q] and bc[t0 + nq] -= their sum, per
+// column; the last CTA of a column (blockIdx.x = gridDim.x - 1) takes the sum
+static __global__ void __launch_bounds__(128) nested_out_kernel(int ne, int nq, int nr, const double2* __restrict__ y, int64_t ldw,
+                                                                double ell, double2* __restrict__ a, int64_t lda,
+                                                                double2* __restrict__ bc, int64_t ldb) {
   const int c = blockIdx.y;
-  if (c >= nr || i >= ne + nq) return;
-  const double2 v = y[int64_t(c) * ldw + i];
-  if (i < ne) wt1[int64_t(c) * ld1 + i] = make_double2(v.x / ell, v.y / ell);
-  else wt2[int64_t(c) * ld2 + (i - ne)] = make_double2(v.x * ell, v.y * ell);
+  y += int64_t(c) * ldw;
+  a += int64_t(c) * lda;
+  bc += int64_t(c) * ldb;
+  if (blockIdx.x + 1 < gridDim.x) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ne + nq) return;
+    const double2 v = y[i];
+    if (i < ne) {
+      a[i].x -= v.x / ell;
+      a[i].y -= v.y / ell;
+    } else {
+      bc[i - ne].x += v.x * ell;
+      bc[i - ne].y += v.y * ell;
+    }
+    return;
+  }
+  double sr = 0, si = 0;
+  for (int q = threadIdx.x; q < nq; q += 128) {
+    sr += y[ne + q].x;
+    si += y[ne + q].y;
+  }
+  __shared__ double red[2][4];
+  for (int w = 16; w > 0; w >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, w);
+    si += __shfl_xor_sync(0xffffffffu, si, w);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = sr;
+    red[1][threadIdx.x >> 5] = si;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bc[nq].x -= ell * ((red[0][0] + red[0][1]) + (red[0][2] + red[0][3]));
+    bc[nq].y -= ell * ((red[1][0] + red[1][1]) + (red[1][2] + red[1][3]));
+  }
 }
 
 // copy nr columns of n entries (column strides ld)
@@ -139,8 +171,8 @@ void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, doubl
                u.tXa, u.pXa);
 }
 
-void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, int64_t ldw, double2* wt1, int64_t ld1,
-                  double2* wt2, int64_t ld2, int nr, double ell, cudaStream_t s) {
+void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, int64_t ldw, double2* a, int64_t lda,
+                  double2* bc, int64_t ldb, int nr, double ell, cudaStream_t s) {
   const NestedMat& m = *u.mat;
   ScopedTimer tm("nested_y", s);
   gemv_jobs_mixed<double2, double2>(u.pR, nr, s);   // t = R e
@@ -150,8 +182,8 @@ void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, 
     gemv_jobs_mixed<double2, double2>(u.pM, nr, s);  // r = t - M y
     gemv_jobs_mixed<float2, double2>(u.pXa, nr, s);  // y += X r
   }
-  nested_out_kernel<<<dim3(unsigned((m.n + 127) / 128), nr), 128, 0, s>>>(m.ne, m.nq, nr, y, ldw, ell, wt1 + u.e0, ld1,
-                                                                        wt2 + u.q0, ld2),
+  nested_out_kernel<<<dim3(unsigned((m.n + 127) / 128 + 1), nr), 128, 0, s>>>(m.ne, m.nq, nr, y, ldw, ell, a + u.e0, lda,
+                                                                            bc + u.t0, ldb),
       count_launch();
   SLDM_CUDA(cudaGetLastError());
 }

@@ -33,7 +33,7 @@ struct NestedMat {
 struct NestedUse {
   int obj = 0, mat_owner = 0;  // this object, the object whose M_l it shares
   std::shared_ptr<NestedMat> mat;
-  int64_t e0 = 0, q0 = 0;
+  int64_t e0 = 0, t0 = 0;
   DBuf<GemvJob> jR, jX0, jXa, jM;
   DBuf<int64_t> rR, rX0, rXa, rM;
   DBuf<int2> tR, tX0, tXa, tM;
@@ -44,14 +44,13 @@ struct NestedUse {
 // reach 1e-13 within 12 steps (the caller then factors M_l in FP64).
 bool nested_setup(NestedMat& mat, cudaStream_t s);
 
-// Plans of object use u against the work vectors: e (edges, column stride lde),
-// wt1 (edges, stride ld1), wt2 (triangles - objects, stride ld2) and the scratch
-// t, y, r (n x WR complex128 each, column stride ldw).
+// Plans of object use u against the work vectors: e (edges, column stride lde) and
+// the scratch t, y, r (n x WR complex128 each, column stride ldw).
 void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, double2* y, double2* r, int64_t ldw);
 
-// wt1 = Y11 e / ell and wt2 = ell Y21 e of object use u for nr columns (ell: the
-// length scaling of M_l), by the refinement above.
-void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, int64_t ldw, double2* wt1, int64_t ld1,
-                  double2* wt2, int64_t ld2, int nr, double ell, cudaStream_t s);
+// a -= Y11 e / ell and bc += B (ell Y21 e) of object use u for nr columns (ell: the length
+// scaling of M_l), by the refinement above; a: edges, stride lda, bc: triangles, stride ldb.
+void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, int64_t ldw, double2* a, int64_t lda,
+                  double2* bc, int64_t ldb, int nr, double ell, cudaStream_t s);
 
 }  // namespace sldm

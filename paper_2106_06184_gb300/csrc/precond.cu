@@ -12,8 +12,11 @@
 //   [x1; x2] = Lambda ([r1; r2] - [P13; P23] x3).
 // S is block diagonal by object (D, B, F are); each block is formed on the
 // device and inverted once per assembly with the batched LU.
+#include <algorithm>
+
 #include "dense.h"
 #include "precond.h"
+#include "widen.cuh"
 
 namespace sldm {
 
@@ -106,76 +109,73 @@ template <>
 __device__ __forceinline__ double2 to_cv<double2>(double2 v) { return v; }
 template <>
 __device__ __forceinline__ float2 to_cv<float2>(double2 v) { return make_float2(float(v.x), float(v.y)); }
+template <class CX>
+__device__ __forceinline__ double2 wide2(const CX v) { return make_double2(widen(v.x), widen(v.y)); }
 
-// t3 = r3 - F D (L11 r1 + L12 r2) (per charge unknown; column blockIdx.y)
-template <class CV>
+// t3 = s3 r3 - F D (L11 r1 + L12 r2) (per charge unknown; column blockIdx.y)
+template <class CX, class CV>
 __global__ void prec_apply1_kernel(int ne, int nq, const int32_t* __restrict__ q2t, const int32_t* __restrict__ tri_edge,
-                                   const int8_t* __restrict__ tri_sign, const double2* __restrict__ lam,
-                                   const double2* __restrict__ r, int64_t ld, CV* t3) {
+                                   const int8_t* __restrict__ tri_sign, const double2* __restrict__ lam, VecBatch<CX, double2> rb,
+                                   double s3, CV* t3) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nq) return;
-  r += int64_t(blockIdx.y) * ld;
+  const CX* __restrict__ r = rb.x[blockIdx.y];
   const int t = q2t[q];
-  double2 acc = r[2 * ne + q];
+  double2 acc = wide2(r[2 * ne + q]);
+  acc.x *= s3;
+  acc.y *= s3;
   for (int i = 0; i < 3; ++i) {
     const int e = tri_edge[3 * t + i];
-    const double s = double(tri_sign[3 * t + i]);
-    const double2 v = c_add(c_mul(lam[4 * e + 0], r[e]), c_mul(lam[4 * e + 1], r[ne + e]));
-    acc.x -= s * v.x;
-    acc.y -= s * v.y;
+    const double2 v = c_add(c_mul(lam[4 * e + 0], wide2(r[e])), c_mul(lam[4 * e + 1], wide2(r[ne + e])));
+    const bool neg = tri_sign[3 * t + i] < 0;
+    acc.x += neg ? v.x : -v.x;
+    acc.y += neg ? v.y : -v.y;
   }
   t3[int64_t(blockIdx.y) * nq + q] = to_cv<CV>(acc);
 }
 
-// full charges bx = B x3 per object (the last triangle carries minus the sum),
-// one CTA per object and column
-template <class CV>
-__global__ void prec_apply3_kernel(const PrecObj* __restrict__ objs, int nq_all, int nt, const CV* __restrict__ x3,
-                                   double2* bx) {
-  const PrecObj O = objs[blockIdx.x];
-  x3 += int64_t(blockIdx.y) * nq_all;
-  bx += int64_t(blockIdx.y) * nt;
-  const int nq = O.nt - 1;
-  double sr = 0, si = 0;
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    const CV v = x3[O.q0 + q];
-    bx[O.t0 + q] = make_double2(double(v.x), double(v.y));
-    sr += double(v.x);
-    si += double(v.y);
-  }
-  __shared__ double rr[256], ri[256];
-  rr[threadIdx.x] = sr;
-  ri[threadIdx.x] = si;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      rr[threadIdx.x] += rr[threadIdx.x + w];
-      ri[threadIdx.x] += ri[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) bx[O.t0 + O.nt - 1] = make_double2(-rr[0], -ri[0]);
-}
-
-// x1, x2 = Lambda (r1 - P13 x3, r2 - P23 x3); x3 copied into the output (column blockIdx.y)
-template <class CV>
-__global__ void prec_apply45_kernel(int ne, int nq, int nt, const int32_t* __restrict__ tplus,
-                                    const int32_t* __restrict__ tminus, const double2* __restrict__ lam,
-                                    const double2* __restrict__ pdiag, const double2* __restrict__ r, int64_t ld,
-                                    const double2* __restrict__ bx, const CV* __restrict__ x3, double2* x) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  r += int64_t(blockIdx.y) * ld;
-  x += int64_t(blockIdx.y) * ld;
-  bx += int64_t(blockIdx.y) * nt;
-  x3 += int64_t(blockIdx.y) * nq;
+// x1, x2 = Lambda (r1 - P13 x3, r2 - P23 x3) and x3, with bx = B x3 (column blockIdx.y).
+// WORK: into the product's work vectors; else added to the columns rb.y.
+struct PrecWork {
+  void *j, *a, *e, *bu, *bc;
+};
+template <class CX, class CV, bool WORK>
+__global__ void __launch_bounds__(128) prec_apply45_kernel(int ne, int nq, int nt, const int32_t* __restrict__ tplus,
+                                                           const int32_t* __restrict__ tminus, const int32_t* __restrict__ q2t,
+                                                           const double2* __restrict__ lam, const double2* __restrict__ pdiag,
+                                                           VecBatch<CX, double2> rb, const CV* __restrict__ bx, PrecWork W) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t c = blockIdx.y;
+  const CX* __restrict__ r = rb.x[c];
+  bx += c * nt;
   if (i < ne) {
     const int tp = tplus[i], tm = tminus[i];
-    const double2 y1 = c_sub(r[i], c_sub(c_mul(pdiag[2 * tp], bx[tp]), c_mul(pdiag[2 * tm], bx[tm])));
-    const double2 y2 = c_sub(r[ne + i], c_sub(c_mul(pdiag[2 * tp + 1], bx[tp]), c_mul(pdiag[2 * tm + 1], bx[tm])));
-    x[i] = c_add(c_mul(lam[4 * i + 0], y1), c_mul(lam[4 * i + 1], y2));
-    x[ne + i] = c_add(c_mul(lam[4 * i + 2], y1), c_mul(lam[4 * i + 3], y2));
+    const double2 bp = wide2(bx[tp]), bm = wide2(bx[tm]);
+    const double2 y1 = c_sub(wide2(r[i]), c_sub(c_mul(pdiag[2 * tp], bp), c_mul(pdiag[2 * tm], bm)));
+    const double2 y2 = c_sub(wide2(r[ne + i]), c_sub(c_mul(pdiag[2 * tp + 1], bp), c_mul(pdiag[2 * tm + 1], bm)));
+    const double2 x1 = c_add(c_mul(lam[4 * i + 0], y1), c_mul(lam[4 * i + 1], y2));
+    const double2 x2 = c_add(c_mul(lam[4 * i + 2], y1), c_mul(lam[4 * i + 3], y2));
+    if (WORK) {
+      const CV v = to_cv<CV>(x1);
+      reinterpret_cast<CV*>(W.j)[c * ne + i] = v;
+      reinterpret_cast<CV*>(W.a)[c * ne + i] = v;
+      reinterpret_cast<CV*>(W.e)[c * ne + i] = to_cv<CV>(x2);
+    } else {
+      double2* xc = rb.y[c];
+      xc[i] = c_add(xc[i], x1);
+      xc[ne + i] = c_add(xc[ne + i], x2);
+    }
   }
-  if (i < nq) x[2 * ne + i] = make_double2(double(x3[i].x), double(x3[i].y));
+  if (WORK) {
+    if (i < nt) {
+      const CV v = bx[i];
+      reinterpret_cast<CV*>(W.bu)[c * nt + i] = v;
+      reinterpret_cast<CV*>(W.bc)[c * nt + i] = v;
+    }
+  } else if (i < nq) {
+    double2* xc = rb.y[c] + 2 * ne;
+    xc[i] = c_add(xc[i], wide2(bx[q2t[i]]));
+  }
 }
 
 __global__ void to_c64_kernel(int64_t n, const double2* __restrict__ a, float2* b) {
@@ -200,7 +200,7 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   std::vector<int64_t> off;
   for (auto& o : objs) {
     off.push_back(tot);
-    tot += int64_t(o.nt - 1) * (o.nt - 1);
+    tot += int64_t(o.nt) * (o.nt - 1);
   }
   DBuf<double2> Sm;
   Sm.alloc(tot);
@@ -215,6 +215,7 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   }
   SLDM_CUDA(cudaGetLastError());
   lu_solve_batched(sys, s);  // sinv <- S^-1
+  for (size_t i = 0; i < objs.size(); ++i) neg_colsum(P.sinv.p + off[i], objs[i].nt - 1, objs[i].nt - 1, s);
   // a complex64 operator takes an FP32 preconditioner: S^-1 (inverted in FP64)
   // rounded to complex64, applied with FP32 arithmetic
   P.f32 = sizeof(C) == sizeof(float2);
@@ -225,12 +226,11 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
     SLDM_CUDA(cudaStreamSynchronize(s));
     P.sinv.release();
   }
-  // GEMV plan: x3_o = S_o^-1 t3_o, WR columns of nq
+  // GEMV plan: (B x3)_o = B_o S_o^-1 t3_o, WR columns
   const size_t ev = P.f32 ? sizeof(float2) : sizeof(double2);
   P.nq = h.nt - h.nobj;
   const int64_t nq1 = std::max<int64_t>(P.nq, 1);
   P.t3.alloc(nq1 * MAX_NRHS);
-  P.x3.alloc(nq1 * MAX_NRHS);
   P.bx.alloc(h.nt * MAX_NRHS);
   std::vector<GemvJob> jobs;
   std::vector<int64_t> rs;
@@ -240,11 +240,11 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   for (size_t i = 0; i < objs.size(); ++i) {
     const int nq = objs[i].nt - 1;
     if (nq <= 0) continue;
-    for (int r0 = 0; r0 < nq; r0 += gemv_tile_rows(ev)) tiles.push_back(make_int2(int(jobs.size()), r0));
-    jobs.push_back({A0 + off[i] * ev, nq, nq, nq, (char*)P.t3.p + objs[i].q0 * ev, P.nq, (char*)P.x3.p + objs[i].q0 * ev,
-                    P.nq, 1, 0, 0, 0});
+    for (int r0 = 0; r0 < nq + 1; r0 += gemv_tile_rows(ev)) tiles.push_back(make_int2(int(jobs.size()), r0));
+    jobs.push_back({A0 + off[i] * ev, nq, nq + 1, nq, (char*)P.t3.p + objs[i].q0 * ev, P.nq, (char*)P.bx.p + objs[i].t0 * ev,
+                    h.nt, 1, 0, 0, 0});
     rs.push_back(acc);
-    acc += nq;
+    acc += nq + 1;
   }
   P.jobs.upload(jobs, s);
   P.rs.upload(rs, s);
@@ -267,31 +267,51 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   SLDM_CUDA(cudaStreamSynchronize(s));
 }
 
-template <class CV>
-static void prec_apply_t(const Precond& P, const sldm_mesh* m, const double2* r, double2* x, int64_t ld, int nr,
+// B x3 of every column: the right-hand side of the Schur complement and its inverse
+template <class CX, class CV>
+static void prec_charges(const Precond& P, const sldm_mesh* m, const VecBatch<CX, double2>& r, double s3, int nr,
                          cudaStream_t s) {
-  const HostMesh& h = m->h;
+  SLDM_REQUIRE((nr >= 1 && nr <= MAX_NRHS), SLDM_EINVAL, "preconditioner: 1 to 32 columns");
   const DevMesh& d = m->d;
-  const int ne = int(h.ne), nq = int(P.nq), nt = int(h.nt);
-  CV* t3 = reinterpret_cast<CV*>(P.t3.p);
-  CV* x3 = reinterpret_cast<CV*>(P.x3.p);
-  if (nq > 0) {
-    prec_apply1_kernel<CV><<<dim3((nq + 255) / 256, nr), 256, 0, s>>>(ne, nq, d.q2t.p, d.tri_edge.p, d.tri_sign.p, P.lam.p,
-                                                                       r, ld, t3), ::sldm::count_launch();
-    gemv_jobs<CV>(P.plan, nr, s);
-  }
-  prec_apply3_kernel<CV><<<dim3(unsigned(h.nobj), nr), 256, 0, s>>>(P.objs.p, nq, nt, x3, P.bx.p), ::sldm::count_launch();
-  const int n = std::max(ne, nq);
-  prec_apply45_kernel<CV><<<dim3((n + 255) / 256, nr), 256, 0, s>>>(ne, nq, nt, d.tplus.p, d.tminus.p, P.lam.p, P.pdiag.p,
-                                                                     r, ld, P.bx.p, x3, x), ::sldm::count_launch();
-  SLDM_CUDA(cudaGetLastError());
+  const int ne = int(m->h.ne), nq = int(P.nq);
+  prec_apply1_kernel<CX, CV><<<dim3((nq + 127) / 128, nr), 128, 0, s>>>(ne, nq, d.q2t.p, d.tri_edge.p, d.tri_sign.p, P.lam.p, r,
+                                                                      s3, reinterpret_cast<CV*>(P.t3.p)), ::sldm::count_launch();
+  gemv_jobs<CV>(P.plan, nr, s);
 }
 
-void prec_apply(const Precond& P, const sldm_mesh* m, const double2* r, double2* x, int64_t ld, int nr, cudaStream_t s) {
+template <class CX, class C>
+void prec_apply_in(const Precond& P, const sldm_mesh* m, const VecBatch<CX, double2>& r, double s3, void* j, void* a, void* e,
+                   void* bu, void* bc, int nr, cudaStream_t s) {
   ScopedTimer tm("precond", s);
-  SLDM_REQUIRE((nr >= 1 && nr <= MAX_NRHS), SLDM_EINVAL, "preconditioner: 1 to 32 columns");
-  if (P.f32) prec_apply_t<float2>(P, m, r, x, ld, nr, s);
-  else prec_apply_t<double2>(P, m, r, x, ld, nr, s);
+  const DevMesh& d = m->d;
+  const int ne = int(m->h.ne), nq = int(P.nq), nt = int(m->h.nt);
+  prec_charges<CX, C>(P, m, r, s3, nr, s);
+  prec_apply45_kernel<CX, C, true><<<dim3((std::max(ne, nt) + 127) / 128, nr), 128, 0, s>>>(
+      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, r, reinterpret_cast<const C*>(P.bx.p),
+      PrecWork{j, a, e, bu, bc}), ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+template void prec_apply_in<float2, float2>(const Precond&, const sldm_mesh*, const VecBatch<float2, double2>&, double, void*,
+                                            void*, void*, void*, void*, int, cudaStream_t);
+template void prec_apply_in<double2, double2>(const Precond&, const sldm_mesh*, const VecBatch<double2, double2>&, double, void*,
+                                              void*, void*, void*, void*, int, cudaStream_t);
+
+template <class CV>
+static void prec_add_t(const Precond& P, const sldm_mesh* m, const VecBatch<double2, double2>& r, double s3, int nr,
+                       cudaStream_t s) {
+  const DevMesh& d = m->d;
+  const int ne = int(m->h.ne), nq = int(P.nq), nt = int(m->h.nt);
+  prec_charges<double2, CV>(P, m, r, s3, nr, s);
+  prec_apply45_kernel<double2, CV, false><<<dim3((std::max(ne, nt) + 127) / 128, nr), 128, 0, s>>>(
+      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, r, reinterpret_cast<const CV*>(P.bx.p), PrecWork{}),
+      ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+void prec_apply_add(const Precond& P, const sldm_mesh* m, const VecBatch<double2, double2>& r, double s3, int nr,
+                    cudaStream_t s) {
+  ScopedTimer tm("precond", s);
+  if (P.f32) prec_add_t<float2>(P, m, r, s3, nr, s);
+  else prec_add_t<double2>(P, m, r, s3, nr, s);
 }
 
 template void prec_setup<float2>(Precond&, const sldm_mesh*, const std::vector<PrecObj>&, double, const void*, const void*,

@@ -15,11 +15,13 @@ struct Precond {
   DBuf<PrecObj> objs;
   DBuf<double2> lam;    // 4 per edge: Lambda11, Lambda12, Lambda21, Lambda22
   DBuf<double2> pdiag;  // 2 per triangle: diag L^phi_m, diag of the object's L^phi/eps
-  DBuf<double2> sinv;   // per object (nt_o - 1)^2: S_o^-1, row-major (complex128 operators)
+  // per object nt_o x (nt_o - 1): B_o S_o^-1 = [S_o^-1; minus its column sums], row-major, so
+  // that the product gives the full charges B x3 (complex128 operators)
+  DBuf<double2> sinv;
   DBuf<float2> sinv32;  // the same in complex64 (complex64 operators: an FP32 preconditioner)
   bool f32 = false;
-  // WR columns each: t3, x3 of nq (entries of the preconditioner's precision), bx of nt
-  DBuf<double2> t3, x3, bx;
+  // WR columns each, entries of the preconditioner's precision: t3 of nq, bx = B x3 of nt
+  DBuf<double2> t3, bx;
   int64_t nq = 0;
   DBuf<GemvJob> jobs;
   DBuf<int64_t> rs;
@@ -32,7 +34,13 @@ struct Precond {
 template <class C>
 void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs, double k0, const void* LAm,
                 const void* LPm, const char* loc, const double* ix_val, cudaStream_t s);
-// x = P^-1 r for nr <= WR columns (complex128 vectors of length N, column stride ld)
-void prec_apply(const Precond& P, const sldm_mesh* m, const double2* r, double2* x, int64_t ld, int nr, cudaStream_t s);
+// Columns of x = P^-1 D r, D = diag(1, 1, s3), for nr <= MAX_NRHS columns r.x (CX), either
+// into the work vectors of the structured product (C: its precision; j, a = j, e, bu =
+// B u, bc = B u) or added to the columns r.y (complex128).
+template <class CX, class C>
+void prec_apply_in(const Precond& P, const sldm_mesh* m, const VecBatch<CX, double2>& r, double s3, void* j, void* a, void* e,
+                   void* bu, void* bc, int nr, cudaStream_t s);
+void prec_apply_add(const Precond& P, const sldm_mesh* m, const VecBatch<double2, double2>& r, double s3, int nr,
+                    cudaStream_t s);
 
 }  // namespace sldm
