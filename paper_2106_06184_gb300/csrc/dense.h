@@ -18,6 +18,9 @@ void lu_solve_batched(const std::vector<LUSysT<C>>& systems, cudaStream_t s);
 // every system of order LU_BLOCKED_MIN or more (below that the look-ahead
 // kernel, whose steps need no grid barrier, is faster).
 constexpr int LU_BLOCKED_MIN = 1024;
+// One or two systems go there from this order on: the look-ahead kernel's chain of
+// published columns costs ~18 us a column whatever the order.
+constexpr int LU_BLOCKED_FEW = 160;
 template <class C>
 void lu_solve_blocked(const LUSysT<C>& S, cudaStream_t s);
 inline void lu_solve_batched(const std::vector<LUSys>& systems, cudaStream_t s) { lu_solve_batched<double2>(systems, s); }

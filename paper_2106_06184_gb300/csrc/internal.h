@@ -62,6 +62,7 @@ void budget_take(size_t bytes);
 void budget_give(size_t bytes);
 // Test injection (sldm_test_inject): consumes one pending LU stall, if any.
 bool take_lu_stall();
+bool lu_stall_pending();
 
 // ---------------------------------------------------------------- device buffers
 template <class T>
