@@ -294,13 +294,34 @@ __global__ void lu_moves_kernel(const int* __restrict__ piv, int j0, int nb, Mov
     reinterpret_cast<int*>(out)[i] = reinterpret_cast<const int*>(&m)[i];
 }
 
+// A pivot candidate as one integer: |Re| + |Im| (32 leading bits: the choice is within 2^-20
+// of the largest) above the complement of the row, so the maximum is the largest value
+// and, on ties, the smallest row.  Non-finite values order last, 0 is no candidate.
+__device__ __forceinline__ unsigned long long pivot_key(float2 a, int row) {
+  const unsigned v = __float_as_uint(fabsf(a.x) + fabsf(a.y));
+  return ((unsigned long long)v << 32) | unsigned(~row);
+}
+__device__ __forceinline__ unsigned long long pivot_key(double2 a, int row) {
+  const unsigned v = unsigned(__double2hiint(fabs(a.x) + fabs(a.y)));
+  return ((unsigned long long)v << 32) | unsigned(~row);
+}
+__device__ __forceinline__ bool pivot_ok(unsigned long long key, float) { return (key >> 32) - 1 < 0x7f800000u - 1; }
+__device__ __forceinline__ bool pivot_ok(unsigned long long key, double) { return (key >> 32) - 1 < 0x7ff00000u - 1; }
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = w > v ? w : v;
+  }
+  return v;
+}
+
 // CTA of rank c holds rows [j0 + c chunk, ..) in shared memory.  Per column: the largest
-// |a|^2 of its rows (compared as integers: no FP64 compares), candidate and rows
+// candidate of its rows (integer compares), candidate and rows
 // published, one cluster barrier, then every CTA picks the winner, takes the pivot row and
 // updates its rows.  Publication buffers alternate: a CTA writes buffer b again only
 // after the next column's barrier, which all reach having read b.
-// Measured per 64-column complex64 panel (n = 3,199): 482 us with two grid barriers through
-// global memory -> 234 us.
+// The 50 panels of a complex64 system of n = 3,199: 24.1 ms with two grid barriers through
+// global memory -> 10.8 ms in a cluster -> 8.4 ms with integer keys and four barriers of the CTA per column.
 constexpr int PC_THREADS = 512;
 template <class C, int CS>
 __global__ void __launch_bounds__(PC_THREADS) lu_panel_cluster(C* A, int n, int j0, int nb, int chunk, Moves* moves, int* err) {
@@ -309,8 +330,8 @@ __global__ void __launch_bounds__(PC_THREADS) lu_panel_cluster(C* A, int n, int 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* P = reinterpret_cast<C*>(smem_raw);  // chunk x LD
   __shared__ __align__(16) C crow[2][NB_MAX], orow[2][NB_MAX], U[NB_MAX];
-  __shared__ unsigned long long cand_v[2], cand_i[2], wv[PC_THREADS / 32];
-  __shared__ int wi[PC_THREADS / 32], s_win, s_p, piv[NB_MAX];
+  __shared__ unsigned long long cand[2], wv[PC_THREADS / 32];
+  __shared__ int s_win, s_p, piv[NB_MAX];
   __shared__ C s_inv;
   __shared__ Moves mv;
   if (*(volatile int*)err) return;  // an earlier panel failed (uniform across the grid)
@@ -325,75 +346,27 @@ __global__ void __launch_bounds__(PC_THREADS) lu_panel_cluster(C* A, int n, int 
   bool failed = false;
   for (int j = 0; j < nb; ++j) {
     const int J = j0 + j, buf = j & 1;
-    // largest |a|^2 over rows >= J, smallest row on ties; non-finite values order last
     unsigned long long best = 0;
-    int bi = n;
-    for (int i = threadIdx.x; i < nr; i += PC_THREADS) {
-      if (r0 + i < J) continue;
-      const double x = widen(P[i * LD + j].x), y = widen(P[i * LD + j].y);
-      const unsigned long long v = __double_as_longlong(x * x + y * y) & 0x7fffffffffffffffull;
-      if (bi == n || v > best) {
-        best = v;
-        bi = r0 + i;
+    for (int i = threadIdx.x; i < nr; i += PC_THREADS)
+      if (r0 + i >= J) {
+        const unsigned long long v = pivot_key(P[i * LD + j], r0 + i);
+        best = v > best ? v : best;
       }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (oi < n && (bi == n || ob > best || (ob == best && oi < bi))) {
-        best = ob;
-        bi = oi;
-      }
-    }
-    if (lane == 0) {
-      wv[warp] = best;
-      wi[warp] = bi;
-    }
+    best = warp_max(best);
+    if (lane == 0) wv[warp] = best;
     __syncthreads();
-    if (warp == 0) {
-      best = lane < PC_THREADS / 32 ? wv[lane] : 0;
-      bi = lane < PC_THREADS / 32 ? wi[lane] : n;
-      for (int o = 8; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (oi < n && (bi == n || ob > best || (ob == best && oi < bi))) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (lane == 0) {
-        cand_v[buf] = best;
-        cand_i[buf] = (unsigned long long)(unsigned)bi;
-        s_p = bi;
-      }
-    }
-    __syncthreads();
-    {
-      const int ci = s_p;
-      if (ci < n)
-        for (int t = threadIdx.x; t < nb; t += PC_THREADS) crow[buf][t] = P[(ci - r0) * LD + t];
-      if (J >= r0 && J < r0 + nr)
-        for (int t = threadIdx.x; t < nb; t += PC_THREADS) orow[buf][t] = P[(J - r0) * LD + t];
-    }
+    best = warp_max(lane < PC_THREADS / 32 ? wv[lane] : 0);  // every warp for itself
+    if (threadIdx.x == 0) cand[buf] = best;
+    if (best != 0)
+      for (int t = threadIdx.x; t < nb; t += PC_THREADS) crow[buf][t] = P[(int(~unsigned(best)) - r0) * LD + t];
+    if (J >= r0 && J < r0 + nr)
+      for (int t = threadIdx.x; t < nb; t += PC_THREADS) orow[buf][t] = P[(J - r0) * LD + t];
     cluster_sync();
     if (warp == 0) {
-      unsigned long long v = 0;
-      int p = n, w = 0;
-      if (lane < CS) {
-        v = ld_cta_u64(in_cta(&cand_v[buf], lane));
-        p = int(ld_cta_u64(in_cta(&cand_i[buf], lane)));
-        w = lane;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int op = __shfl_xor_sync(0xffffffffu, p, o), ow = __shfl_xor_sync(0xffffffffu, w, o);
-        if (op < n && (p >= n || ov > v || (ov == v && op < p))) {
-          v = ov;
-          p = op;
-          w = ow;
-        }
-      }
-      const bool ok = p < n && v != 0 && v < 0x7ff0000000000000ull;
+      const unsigned long long mine = lane < CS ? ld_cta_u64(in_cta(&cand[buf], lane)) : 0;
+      const unsigned long long v = warp_max(mine);
+      const int w = __ffs(__ballot_sync(0xffffffffu, mine == v && lane < CS)) - 1;
+      const bool ok = pivot_ok(v, R());
       for (int t = lane; t < nb && ok; t += 32) {  // the pivot row, from its CTA
         C u;
         ld_cta(in_cta(&crow[buf][t], w), u);
@@ -402,9 +375,9 @@ __global__ void __launch_bounds__(PC_THREADS) lu_panel_cluster(C* A, int n, int 
       __syncwarp();
       if (lane == 0) {
         s_win = w;
-        s_p = ok ? p : -1;
+        s_p = ok ? int(~unsigned(v)) : -1;
         if (ok) {
-          piv[j] = p;
+          piv[j] = int(~unsigned(v));
           C one;
           one.x = R(1);
           one.y = R(0);
@@ -436,13 +409,27 @@ __global__ void __launch_bounds__(PC_THREADS) lu_panel_cluster(C* A, int n, int 
     const int lo = max(0, J + 1 - r0);  // first row below J
     for (int i = lo + threadIdx.x; i < nr; i += PC_THREADS) P[i * LD + j] = cmul_(P[i * LD + j], inv);
     __syncthreads();
-    const int w = nb - j - 1, work = (nr - lo) * w;
-    for (int t = threadIdx.x; t < work; t += PC_THREADS) {
-      const int i = lo + t / w, cc = j + 1 + t % w;
-      const C l = P[i * LD + j], u = U[cc];
-      C a = P[i * LD + cc];
-      cfms(a.x, a.y, l.x, l.y, u.x, u.y);
-      P[i * LD + cc] = a;
+    if constexpr (sizeof(C) == 16) {
+      // FP64: full warps whatever the column count (an instruction costs 16 clocks however many lanes it serves)
+      const int w = nb - j - 1, work = (nr - lo) * w;
+      for (int t = threadIdx.x; t < work; t += PC_THREADS) {
+        const int i = lo + t / w, cc = j + 1 + t % w;
+        const C l = P[i * LD + j], u = U[cc];
+        C a = P[i * LD + cc];
+        cfms(a.x, a.y, l.x, l.y, u.x, u.y);
+        P[i * LD + cc] = a;
+      }
+    } else for (int c0 = j + 1; c0 < nb; c0 += 32) {  // a warp takes a row, its lanes the columns
+      const int cc = c0 + lane;
+      if (cc >= nb) continue;
+      const C u = U[cc];
+#pragma unroll 4
+      for (int i = lo + warp; i < nr; i += PC_THREADS / 32) {
+        const C l = P[i * LD + j];
+        C a = P[i * LD + cc];
+        cfms(a.x, a.y, l.x, l.y, u.x, u.y);
+        P[i * LD + cc] = a;
+      }
     }
     __syncthreads();
   }
