@@ -80,6 +80,7 @@ struct sldm_op {
   sldm::DBuf<char> LAm, LPm, loc;
   sldm::DBuf<char> LAm_lo, LPm_lo, loc_lo;  // SLDM_PREC_F32X2: FP64 value - complex64 value, in complex64
   std::vector<sldm::ObjInfo> obj;
+  std::vector<int> ref;  // the first object that each repeats, or itself
   sldm::DBuf<double> ix_val;
   // structured product: work vectors for up to WR right-hand sides per pass
   static constexpr int WR = sldm::MAX_NRHS;
@@ -347,6 +348,32 @@ static std::vector<int> repeated_objects(const HostMesh& h, const sldm_material*
   return ref;
 }
 
+// The first object with the same preconditioner block as each: a repeat (repeated_objects'
+// ref) whose own global blocks repeat too (in a stack: at the same height).
+static std::vector<PrecObj> prec_objects(const sldm_op* op) {
+  const HostMesh& h = op->mesh->h;
+  std::vector<PrecObj> po;
+  auto z0 = [&](int o) { return h.xyz[3 * size_t(h.tri[3 * size_t(h.tri_begin[o])]) + 2]; };
+  double lo = 1e300, hi = -1e300;
+  for (int64_t v = 0; v < h.nv; ++v) {
+    lo = std::min(lo, h.xyz[3 * v]);
+    hi = std::max(hi, h.xyz[3 * v]);
+  }
+  std::map<int, std::vector<int>> firsts;  // by ref: the objects that start a block
+  for (int o = 0; o < op->nobj; ++o) {
+    const ObjInfo& oi = op->obj[o];
+    int same = o;
+    for (int f : firsts[op->ref[o]])
+      if (!op->layered || std::fabs(z0(f) - z0(o)) <= 1e-12 * (hi - lo)) {
+        same = f;
+        break;
+      }
+    if (same == o) firsts[op->ref[o]].push_back(o);
+    po.push_back({oi.e0, oi.ne, oi.t0, oi.nt, oi.q0, same, oi.oLA, oi.oK, oi.oLP});
+  }
+  return po;
+}
+
 // Reuse of the global blocks L^A_m, L^phi_m.  The block of object pair (i, j)
 // (rows: i's edges or triangles, columns: j's) integrates G(r, r') over i's test
 // and j's source triangles.  In a homogeneous background G depends on r - r'
@@ -541,7 +568,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
   op->loc.zero(s);
   char* loc = op->loc.p;
   // ---- objects that repeat an earlier one take its interior blocks and Y
-  const std::vector<int> ref = repeated_objects(h, mats);
+  const std::vector<int>& ref = op->ref = repeated_objects(h, mats);
   // ---- internal L^A, L^phi with each object's wavenumber
   {
     std::vector<LTask> tasks;
@@ -698,9 +725,7 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
   build_plans<C>(op, s);
   // ---- preconditioner P (Eq. pcext): diagonals and the per-object Schur complement inverses
   {
-    std::vector<PrecObj> po;
-    for (auto& oi : op->obj) po.push_back({oi.e0, oi.ne, oi.t0, oi.nt, oi.q0, 0, oi.oLA, oi.oK, oi.oLP});
-    prec_setup<C>(op->pc, m, po, op->k0, op->LAm.p, op->LPm.p, op->loc.p, op->ix_val.p, s);
+    prec_setup<C>(op->pc, m, prec_objects(op), op->k0, op->LAm.p, op->LPm.p, op->loc.p, op->ix_val.p, s);
     op->pc.ready = true;
   }
   SLDM_CUDA(cudaStreamSynchronize(s));
@@ -729,9 +754,7 @@ static void split_to_x2(sldm_op* op, cudaStream_t s) {
   op->esz = sizeof(float2);
   op->x2 = true;
   build_plans<float2>(op, s);
-  std::vector<PrecObj> po;
-  for (auto& oi : op->obj) po.push_back({oi.e0, oi.ne, oi.t0, oi.nt, oi.q0, 0, oi.oLA, oi.oK, oi.oLP});
-  prec_setup<float2>(op->pc, op->mesh, po, op->k0, op->LAm.p, op->LPm.p, op->loc.p, op->ix_val.p, s);
+  prec_setup<float2>(op->pc, op->mesh, prec_objects(op), op->k0, op->LAm.p, op->LPm.p, op->loc.p, op->ix_val.p, s);
   op->pc.ready = true;
   SLDM_CUDA(cudaStreamSynchronize(s));
 }

@@ -23,6 +23,8 @@ constexpr int LU_BLOCKED_MIN = 1024;
 constexpr int LU_BLOCKED_FEW = 160;
 template <class C>
 void lu_solve_blocked(const LUSysT<C>& S, cudaStream_t s);
+// C += A B, n x n row-major, the product in FP32
+void square_gemm_add(int n, const float2* A, const float2* B, double2* C, cudaStream_t s);
 inline void lu_solve_batched(const std::vector<LUSys>& systems, cudaStream_t s) { lu_solve_batched<double2>(systems, s); }
 
 template <class C>

@@ -661,6 +661,75 @@ __global__ void __launch_bounds__(256) lu_gemm_kernel(Cols<C> S, const C* __rest
   }
 }
 
+// ---------------------------------------------------------------- C += A B, complex64, C complex128, n x n
+// 64 x 64 tiles of 256 threads, 16 columns of A and rows of B per step, the next step's
+// entries loaded into registers while this one's are multiplied; packed FP32 pairs.
+__global__ void __launch_bounds__(256) square_gemm_kernel(int n, const float2* __restrict__ A, const float2* __restrict__ B,
+                                                          double2* __restrict__ C) {
+  constexpr int TK = 16;
+  __shared__ __align__(16) float2 As[64][TK + 2], Bs[TK][64];
+  const int rt = blockIdx.y * 64, qt = blockIdx.x * 64;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  unsigned long long acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0ull;
+  float2 ra[4], rb[4];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = threadIdx.x + 256 * u;
+      const int i = e / TK, k = e % TK, kb = e / 64, q = e % 64;
+      ra[u] = rt + i < n && k0 + k < n ? A[int64_t(rt + i) * n + k0 + k] : make_float2(0.f, 0.f);
+      rb[u] = k0 + kb < n && qt + q < n ? B[int64_t(k0 + kb) * n + qt + q] : make_float2(0.f, 0.f);
+    }
+  };
+  load(0);
+  for (int k0 = 0; k0 < n; k0 += TK) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = threadIdx.x + 256 * u;
+      As[e / TK][e % TK] = ra[u];
+      Bs[e / 64][e % 64] = rb[u];
+    }
+    __syncthreads();
+    if (k0 + TK < n) load(k0 + TK);
+#pragma unroll
+    for (int k = 0; k < TK; k += 2) {
+      float4 p[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) p[a] = *reinterpret_cast<const float4*>(&As[ty * 4 + a][k]);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float2 q0 = Bs[k][tx + 16 * b], q1 = Bs[k + 1][tx + 16 * b];
+        const unsigned long long x0 = pk(q0.x, q0.y), y0 = pk(-q0.y, q0.x), x1 = pk(q1.x, q1.y), y1 = pk(-q1.y, q1.x);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          fma2(acc[a][b], pk(p[a].x, p[a].x), x0);
+          fma2(acc[a][b], pk(p[a].y, p[a].y), y0);
+          fma2(acc[a][b], pk(p[a].z, p[a].z), x1);
+          fma2(acc[a][b], pk(p[a].w, p[a].w), y1);
+        }
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int i = rt + ty * 4 + a, q = qt + tx + 16 * b;
+      if (i >= n || q >= n) continue;
+      float lo, hi;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[a][b]));
+      double2 v = C[int64_t(i) * n + q];
+      v.x += widen(lo);
+      v.y += widen(hi);
+      C[int64_t(i) * n + q] = v;
+    }
+}
+
 // ---------------------------------------------------------------- launches
 // per function and context, shared by every launching thread: set once to the
 // largest size a launch may ask for, never to one call's size
@@ -732,6 +801,11 @@ bool panel_cluster(C* A, int n, int j0, int nb, Moves* mv, int* err, int dev, cu
 }
 
 }  // namespace
+
+void square_gemm_add(int n, const float2* A, const float2* B, double2* C, cudaStream_t s) {
+  square_gemm_kernel<<<dim3((n + 63) / 64, (n + 63) / 64), 256, 0, s>>>(n, A, B, C), count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
 
 template <class C>
 void lu_solve_blocked(const LUSysT<C>& S, cudaStream_t s) {

@@ -7,7 +7,8 @@ namespace sldm {
 
 // Object description for the preconditioner (offsets are elements of the op's local block storage).
 struct PrecObj {
-  int32_t e0, ne, t0, nt, q0, pad;
+  int32_t e0, ne, t0, nt, q0;
+  int32_t same;  // the first object with the same Schur complement (a repeat of this one's blocks), or itself
   int64_t oLA, oK, oLP;
 };
 
