@@ -95,6 +95,12 @@ struct sldm_op {
   sldm::DBuf<int64_t> rs1d, rs2d;
   sldm::DBuf<int2> tl1d, tl2d;
   sldm::GemvPlan plan1d, plan2d;
+  // SLDM_PREC_F32X2: Y11 e, Y21 e of the far field
+  sldm::DBuf<sldm::GemvJob> jobsf;
+  sldm::DBuf<int64_t> rsf;
+  sldm::DBuf<int2> tlf;
+  sldm::GemvPlan planf;
+  sldm::TcPlan tcf;
   // layered background (external problem with the multilayer kernel)
   bool layered = false;
   sldm::MgfStackHost H;
@@ -163,7 +169,7 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
     j2.push_back({L(o.oLP), o.nt, o.nt, o.nt, P(op->wbu, o.t0), nt, P(op->ww3, o.t0), nt, 1, 0, 0, 0, Lo(o.oLP)});
   }
   auto mk = [&](std::vector<GemvJob>& j, DBuf<GemvJob>& dj, DBuf<int64_t>& drs, DBuf<int2>& dt, GemvPlan& plan,
-                TcPlan* tc) {
+                TcPlan* tc, bool f16 = true) {
     std::vector<int64_t> rs(j.size());
     std::vector<int2> tiles;
     int64_t acc = 0;
@@ -187,12 +193,27 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
     for (auto& jb : j) plan.bytes += double(jb.m) * jb.n * es_m * (lo ? 2 : 1);
     plan.tc = nullptr;
     if (tc) {  // complex64 blocks and vectors: tensor-core passes of 9 to 32 right-hand sides
-      tc_plan_build(j, *tc, 0);
+      tc_plan_build(j, *tc, f16, 0);
       if (tc->ok) plan.tc = tc;
     }
   };
   mk(j1, dj1, drs1, dt1, p1, tc1);
   mk(j2, dj2, drs2, dt2, p2, tc2);
+  // The far field of an FP64 system held as pairs goes through a complex64 product with Y: complex128
+  // numbers that show its rounding, so it keeps the TF32 form and the products by themselves
+  if (op->x2 && es_v == sizeof(float2)) {
+    std::vector<GemvJob> jf;
+    for (auto& o : op->obj) {
+      jf.push_back({L(o.oY11), o.ne, o.ne, o.ne, P(op->we, o.e0), ne, P(op->wz1, o.e0), ne, 1, 0, 0, 0, nullptr});
+      if (o.nt > 1) jf.push_back({L(o.oY21), o.ne, o.nt - 1, o.ne, P(op->we, o.e0), ne, P(op->wz2, o.q0), op->nq, 1, 0, 0, 0, nullptr});
+    }
+    mk(jf, op->jobsf, op->rsf, op->tlf, op->planf, &op->tcf, false);
+    op->planf.name = "gemv_y";
+    // not measured: its kernel, and so the far field's last digits, should not hang on a timing.  16 right-hand
+    // sides: 4 x 4 metasurface 34 us against 26 on the CUDA cores, one sphere of 1,280 triangles 53 / 42; 32: 36 / 42
+    // and 55 / 60
+    op->planf.tc_from = tc_policy() ? tc_policy() : (op->planf.total_rows >= 4096 ? TILE_NRHS + 1 : 2 * TILE_NRHS + 1);
+  }
   p1.name = "gemv_y";     // Y11, Y21 (per object)
   p2.name = "gemv_main";  // L^A_m, L^phi_m and the internal blocks
 }
@@ -1513,8 +1534,13 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
     double2* jo = jd.p + int64_t(op->ne) * r0;
     if (op->prec == SLDM_PREC_F32) {
       apply_in<double2, float2>(op->mesh, b, 1.0, 1.0, 1.0, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
-      apply_y<float2, float2>(op, op->plan1, nr, s);
-      to_c128<float2>(op->wa.p, int64_t(op->ne) * nr, jo, s);
+      if (op->x2) {
+        gemv_jobs<float2>(op->planf, nr, s);
+        sub_c64(reinterpret_cast<const float2*>(op->wj.p), reinterpret_cast<const float2*>(op->wz1.p), int64_t(op->ne) * nr, jo, s);
+      } else {
+        apply_y<float2, float2>(op, op->plan1, nr, s);
+        to_c128<float2>(op->wa.p, int64_t(op->ne) * nr, jo, s);
+      }
     } else {
       apply_in<double2, double2>(op->mesh, b, 1.0, 1.0, 1.0, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
       apply_y<double2, double2>(op, op->plan1, nr, s);

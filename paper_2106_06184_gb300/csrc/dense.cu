@@ -9,9 +9,9 @@
 //    Krylov basis' precision, batched over the lockstep right-hand sides.
 #include <algorithm>
 #include <atomic>
-#include <tuple>
 #include <mutex>
 #include <map>
+#include <tuple>
 #include <type_traits>
 
 #include "dense.h"
@@ -1002,7 +1002,7 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s) {
     // the compensated product the arithmetic is the bound (4 DFMA or ~44 FP32 operations per
     // entry and right-hand side), so the rest takes a kernel of its own width; complex64
     // passes, bound by launches and L2, take it as one more pass of 8.
-    // (box of 432 triangles, FP64, 5 right-hand sides: 425 us with 8 -> 272 us)
+    // (box of 432 triangles, FP64, 5 right-hand sides, the whole product: 453 us with 8 -> 303 us)
     const int full = c64 && nrhs > 4 ? nrhs : nrhs / TILE_NRHS * TILE_NRHS, rest = nrhs - full;
     auto go = [&](auto lo) {
       constexpr bool LO = decltype(lo)::value;
@@ -1043,10 +1043,11 @@ template void gemv_jobs_mixed<float2, float2>(const GemvPlan&, int, cudaStream_t
 template void gemv_jobs_mixed<double2, double2>(const GemvPlan&, int, cudaStream_t);
 
 static std::atomic<int> g_tc_force{0};  // sldm_set_tc_policy: 0 = measure, else the width to use
+int tc_policy() { return g_tc_force.load(); }
 
 // decisions by plan shape (jobs, rows, bytes streamed per pass): a shape is timed once per process
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int64_t, double>, int> g_tuned;
+static std::map<std::tuple<int, int64_t, double, bool>, int> g_tuned;
 
 void gemv_autotune(GemvPlan& plan, cudaStream_t s) {
   if (plan.njobs == 0 || plan.tc == nullptr || !plan.tc->ok) return;
@@ -1054,7 +1055,7 @@ void gemv_autotune(GemvPlan& plan, cudaStream_t s) {
     plan.tc_from = f;
     return;
   }
-  const auto key = std::make_tuple(plan.njobs, plan.total_rows, plan.bytes);
+  const auto key = std::make_tuple(plan.njobs, plan.total_rows, plan.bytes, plan.tc->f16);
   {
     std::lock_guard<std::mutex> l(g_tune_mu);
     auto it = g_tuned.find(key);
@@ -1488,6 +1489,15 @@ __global__ void to_c128_kernel(const C* __restrict__ src, int64_t n, double2* ds
 template <class C>
 void to_c128(const void* src, int64_t n, double2* dst, cudaStream_t s) {
   to_c128_kernel<C><<<unsigned((n + 255) / 256), 256, 0, s>>>((const C*)src, n, dst), ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+__global__ void sub_c64_kernel(const float2* __restrict__ a, const float2* __restrict__ b, int64_t n, double2* dst) {
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t < n) dst[t] = make_double2(widen(a[t].x - b[t].x), widen(a[t].y - b[t].y));
+}
+void sub_c64(const float2* a, const float2* b, int64_t n, double2* dst, cudaStream_t s) {
+  if (n <= 0) return;
+  sub_c64_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(a, b, n, dst), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
 // FP64 operator kept as a complex64 pair: hi = fl32(v), lo = fl32(v - hi)

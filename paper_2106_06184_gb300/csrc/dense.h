@@ -93,6 +93,9 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s);
 // finite values (the caller zeroes them).
 void gemv_autotune(GemvPlan& plan, cudaStream_t s);
 
+// the width forced by sldm_set_tc_policy, 0 = measured
+int tc_policy();
+
 struct ApplyDims {
   int32_t ne, nt, nq, nobj;
 };
@@ -134,6 +137,8 @@ template <class CB>
 void krylov_update(const KrylovStep& ks, bool norm, cudaStream_t s);   // V_j[:, k] -= V_j[:, :k] h_j
 template <class C>
 void to_c128(const void* src, int64_t n, double2* dst, cudaStream_t s);
+// dst = a - b, the difference in FP32
+void sub_c64(const float2* a, const float2* b, int64_t n, double2* dst, cudaStream_t s);
 // hi = complex64 rounding of src, lo = complex64 rounding of src - hi (src = hi + lo to ~2^-48)
 void split_c128(const double2* src, int64_t n, float2* hi, float2* lo, cudaStream_t s);
 // dst += lo (complex64 low parts onto a complex128 copy of the high parts)

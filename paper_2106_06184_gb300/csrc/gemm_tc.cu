@@ -13,13 +13,20 @@
 // tc_bprime_kernel into global memory and streamed by TMA as well (it is the same
 // for all row tiles of a job, so building it in each tile would repeat the work).
 //
-// Near-FP32 accuracy from TF32 operands (three products): with hi(v) = v rounded
-// to TF32 (10 stored mantissa bits: |v - hi| <= 2^-11 |v|) and lo(v) = v - hi
-// rounded to TF32 (error <= 2^-11 |v - hi| <= 2^-22 |v|),
+// Near-FP32 accuracy from FP16 operands (three products): every 128-column segment of a
+// row of A, and of every column of B', is scaled by a power of two that puts its largest
+// entry into [2^14, 2^15) (A's exponents are worked out once with the plan, B''s with
+// each pass).  With hi(v) = v rounded to FP16 (11 bits: |v - hi| <= 2^-11 |v|) and lo(v) =
+// v - hi rounded to FP16 (error <= 2^-11 |v - hi| <= 2^-22 |v|),
 //     D = hi(A) hi(B) + lo(A) hi(B) + hi(A) lo(B)        (FP32 accumulation),
 // the dropped lo(A) lo(B) (<= 2^-22 |A||B|) and the two roundings of lo leave
 // each product term within 3 x 2^-22 of |A||B| (about 2^-22 for typical data),
-// against 2^-24 for an FP32 product; the sums are compensated (below).
+// against 2^-24 for an FP32 product; entries below 2^-17 of their segment's largest
+// lose lo's last bits, an absolute error of 2^-39 of that largest.  FP16 has TF32's
+// precision at twice its rate and half its bytes: four MMAs per 32 columns instead of
+// eight, whose issue (~75 cycles each) bound the TF32 form, and half the B' traffic.  The
+// sums are compensated (below).  The TF32 form of the operands (hi and lo rounded to TF32, no
+// scales, the same error) is kept for the far field of FP64 operators held as pairs (gemm_tc.h).
 //
 // Per CTA (one per SM, persistent over its tiles, longest first), 128-row
 // tiles streamed in stages of 4 TMA boxes (128 rows x 4 x 128 B, 128-byte
@@ -27,44 +34,43 @@
 // ~0.98 of the copy rate, against ~0.65 for 128-byte runs.  Each stage is
 // split into four K sub-chunks of 32 FP32 columns.  Warp-specialised,
 // synchronised by mbarriers only:
-//   warp 0   TMA: a ring of 2 stages (128 KB in flight per SM);
-//   warp 18  TMA: B' hi/lo of each sub-chunk (one 128-row x 128 B box) into the
-//            operand buffer of that sub-chunk once the MMAs that read it before
-//            have completed;
-//   warps 2-9 split (two per TMEM lane quarter, half the K columns each):
-//            thread = row; for each sub-chunk reads its row, splits it
-//            into hi and lo and stores both into a TMEM operand buffer (A of
-//            the MMA in tensor memory: lane = row, column = K); the ring stage is
-//            freed after its fourth sub-chunk;
-//   warp 1   MMA: one thread issues 8 MMAs per sub-chunk, per K step of 8:
+//   warp 0   TMA: a ring of stages;
+//   warp 18  TMA of B' (hi and lo; a box of two sub-chunks, one in TF32) into its shared operand buffers;
+//   warps 2-9 split: thread = row, the two warps of 32 rows take the sub-chunks in turn: scaled,
+//            rounded to FP16 hi and lo and stored as pairs into one of the TMEM
+//            operand buffers (A of tcgen05.mma in tensor memory).  Whole sub-chunks per warp
+//            halve the barrier round trips of this chain, which is its length (1,415 -> 1,363 us);
+//   warp 1   MMA: one thread issues, per K step of 16 (TF32: 8),
 //            hi(A) x [hi(B') | lo(B')] (M 128, N 128: B' hi and lo are the two
 //            halves of one 128-row operand) and lo(A) x hi(B') (N 64) into the
 //            first half, into one of two 128-column TMEM accumulators, a fresh
 //            one for every stage (a segment of 128 K columns), and commits them
-//            to the operand buffer's barrier.  Two products per K step instead
-//            of three N = 64 ones: the tensor pipe spends ~70 cycles on an
-//            M 128 N 64 K 8 TF32 product, so three of them per K step took more
-//            of its time than the stage's HBM transfer leaves;
+//            to the operand buffer's barrier;
 //   warps 10-17 epilogue: fold each segment's accumulator (the sum of its two
-//            halves) into compensated FP32 sums in registers (warp w: TMEM
+//            halves, scaled back) into compensated FP32 sums in registers (warp w: TMEM
 //            lanes 32 (w % 4) .., 32 of the 64 output columns), and at the end
 //            of a tile write Y.
 // The tensor core rounds its FP32 accumulator at every MMA: a tile's ~10^4
-// MMAs into one accumulator would lose ~2^-17 of the result; segments of 32
+// MMAs into one accumulator would lose ~2^-17 of the result; segments of 16
 // MMAs and compensated sums across them keep the product as accurate as an
 // FP32 CUDA-core product.
-// Operand buffers: 4 for A (TMEM, the most that fits beside the two 128-column
-// accumulators), 6 for B' (shared memory), so that the B' loads, whose latency
-// from L2 under the streaming load is ~10^3 cycles, are issued well ahead.
 // Tiles are padded to whole stages (zero columns from TMA and zero B').
+//
+// 8 x 8 metasurface, 32 right-hand sides (6.47 GB): 1,745 us in TF32 -> 1,363 us, 0.71 of the
+// HBM copy rate.  The stream of A alone takes 982 us through this ring; the rest is the latency of the split
+// and epilogue warps, which share the four schedulers.
 #include <cuda.h>
 
 #include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <queue>
+#include <type_traits>
+
+#include <cuda_fp16.h>
 
 #include "gemm_tc.h"
+#include "tc_ptx.cuh"
 
 namespace sldm {
 
@@ -76,90 +82,51 @@ constexpr int TC_KC = 32;              // FP32 columns of A per chunk: one 128-b
 constexpr int TC_BPS = 4;              // TMA boxes (sub-chunks) per stage
 constexpr int TC_R = 2;                // stages in the ring
 constexpr int TC_THREADS = 608;        // 19 warps: TMA (A), MMA, 8 split, 8 epilogue, TMA (B')
-constexpr int TC_NA = 4;               // A operand buffers (TMEM, hi/lo)
 constexpr int TC_NBB = 6;              // B' operand buffers (shared, hi/lo)
+// the two forms of the operands (F: scaled FP16, else TF32)
+template <bool F>
+struct TcForm {
+  static constexpr int AW = F ? 32 : 64;   // TMEM columns of an A operand buffer: hi, lo
+  static constexpr int NA = 256 / AW;      // A operand buffers
+  static constexpr int BPB = F ? 2 : 1;    // sub-chunks per B' buffer (one box of 128-byte rows)
+  static constexpr int KS = F ? 16 : 8;    // K of an MMA
+};
 constexpr uint32_t TC_A_BYTES = TC_M * TC_KC * 4;  // 16 KB: one box, one sub-chunk
 constexpr uint32_t TC_STAGE_BYTES = TC_BPS * TC_A_BYTES;
-constexpr uint32_t TC_B_BYTES = TC_N * TC_KC * 4;  // 8 KB
+constexpr int TC_BK = 2 * TC_KC;                    // K columns of a B' box in FP16: one 128-byte swizzle row
+constexpr uint32_t TC_B_BYTES = TC_N * 128;         // 8 KB
 constexpr uint32_t TC_BBUF = 2 * TC_B_BYTES;       // B' hi, lo
 constexpr uint32_t TC_RING = TC_R * TC_STAGE_BYTES;
 // TMEM: two accumulators of 128 columns (hi(A) hi(B') in 0-63, hi(A) lo(B') in
-// 64-127) at columns 0 and 128, A operand buffers (hi 32 + lo 32 columns each) from 256
+// 64-127) at columns 0 and 128, A operand buffers (hi and lo: 16 columns of FP16 pairs or 32 of TF32 each) from 256
 constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr uint32_t TC_ACC_COLS = 2 * TC_N;
 constexpr uint32_t TC_ACC_COL = 0, TC_AOP_COL = 2 * TC_ACC_COLS;
-static_assert(TC_AOP_COL + TC_NA * 64 <= TC_TMEM_COLS, "accumulators and operand buffers exceed the TMEM allocation");
-constexpr int TC_NBARS = 2 * TC_R + 2 * TC_NA + 4 + 2 * TC_NBB;
-constexpr size_t TC_SMEM = size_t(TC_RING) + TC_NBB * size_t(TC_BBUF) + 1024 + 256;
-static_assert(8 * TC_NBARS + 4 <= 256, "barriers and the TMEM slot exceed their shared-memory space");
-constexpr uint32_t TC_SPIN = 1u << 21;  // try_wait rounds before a wait is declared failed
+static_assert(TC_AOP_COL + 256 <= TC_TMEM_COLS, "accumulators and operand buffers exceed the TMEM allocation");
+constexpr int TC_NBARS = 2 * TC_R + 2 * 8 + 4 + 2 * TC_NBB;
+constexpr size_t TC_BAR_BYTES = 512;
+constexpr size_t TC_SMEM = size_t(TC_RING) + TC_NBB * size_t(TC_BBUF) + 1024 + TC_BAR_BYTES;
+static_assert(8 * TC_NBARS + 4 <= TC_BAR_BYTES, "barriers and the TMEM slot exceed their shared-memory space");
 
 static_assert(TC_BBUF % 1024 == 0 && TC_A_BYTES % 1024 == 0 && TC_B_BYTES % 1024 == 0, "swizzle atoms are 1 KB aligned");
 static_assert(TC_SMEM <= 227 * 1024, "ring and operand buffers exceed the shared memory of a CTA");
 
-// instruction descriptor, kind::tf32: D FP32 (bits 4-5 = 1), A and B TF32 (bits
-// 7-9, 10-12 = 2), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at 24-28
-constexpr uint32_t tc_idesc(int n) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(n >> 3) << 17) | (uint32_t(TC_M >> 4) << 24);
-}
-constexpr uint32_t TC_IDESC_N64 = tc_idesc(TC_N), TC_IDESC_N128 = tc_idesc(2 * TC_N);
-
-// shared-memory matrix descriptor of a K-major operand in the 128-byte swizzled
-// layout: start address >> 4 (bits 0-13), leading byte offset 16 B (unused for
-// this layout, bits 16-29), stride byte offset 1024 B between 8-row groups
-// (bits 32-45), descriptor version 1 (bit 46), swizzle mode 2 = 128 B (bits 61-63)
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  return uint64_t((saddr & 0x3FFFFu) >> 4) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) | (uint64_t(1) << 46) |
-         (uint64_t(2) << 61);
+// instruction descriptor: D FP32 (bits 4-5 = 1), A and B FP16 or TF32 (bits
+// 7-9, 10-12 = 0 or 2), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at 24-28
+__host__ __device__ constexpr uint32_t tc_idesc(bool f16, int n) {
+  return (1u << 4) | (f16 ? 0u : (2u << 7) | (2u << 10)) | (uint32_t(n >> 3) << 17) | (uint32_t(TC_M >> 4) << 24);
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// bounded wait for the phase of parity `parity` to complete; gives up early
-// when another warp recorded a failure in *fail (shared memory)
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const volatile int* fail = nullptr) {
-  for (uint32_t it = 0; it < TC_SPIN; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (fail && (it & 63) == 63 && *fail) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
 // D (TMEM) (+)= A (TMEM: lane = row, one TF32 per column) x B (shared memory descriptor)
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void tc_mma_tf32(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
       "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // 8 consecutive accumulator columns of this warp's 32 TMEM lanes, at two column offsets
-__device__ __forceinline__ void tmem_ld8x2(uint32_t taddr, uint32_t off, float (&v)[8], float (&w)[8]) {
+__device__ __forceinline__ void tmem_ld8x2(uint32_t taddr, uint32_t off, f2 (&v)[4], f2 (&w)[4]) {
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n"
@@ -170,21 +137,16 @@ __device__ __forceinline__ void tmem_ld8x2(uint32_t taddr, uint32_t off, float (
       : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    v[i] = __uint_as_float(r[i]);
-    w[i] = __uint_as_float(r[8 + i]);
+  for (int i = 0; i < 4; ++i) {
+    v[i] = f2_pack(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+    w[i] = f2_pack(__uint_as_float(r[8 + 2 * i]), __uint_as_float(r[9 + 2 * i]));
   }
 }
-// 16 consecutive TMEM columns of this warp's 32 lanes from registers
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16};\n" ::"r"(taddr),
-      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-      "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-      "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-      "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
-      : "memory");
+// 8 consecutive TMEM columns of this warp's 32 lanes from registers
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"r"(taddr), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
 }
 
 // FP32 -> TF32 (10 mantissa bits), round to nearest, ties away from zero: the
@@ -201,15 +163,39 @@ __device__ __forceinline__ void tf32_split(float v, float& hi, float& lo) {
   hi = tf32_rn(v);
   lo = tf32_rn(v - hi);
 }
-
-
+// 16 consecutive TMEM columns of this warp's 32 lanes from registers
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16};\n" ::"r"(taddr),
+      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+      "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
+      "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
+      "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
+      : "memory");
+}
+// v = hi + lo, both FP16 pairs (the first number in the lower half), rounded to nearest
+__device__ __forceinline__ void f16_split(f2 v, uint32_t& hi, uint32_t& lo) {
+  float a, b;
+  f2_unpack(v, a, b);
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  f2_unpack(f2_sub(v, f2_pack(f.x, f.y)), a, b);
+  const __half2 l = __floats2half2_rn(a, b);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
 }  // namespace
 
 // 19 warps over the 4 SM sub-partitions (5, 5, 5, 4) x 32 threads x 96 registers <= 16,384 each
+template <bool F>
 __global__ void __maxnreg__(96)
     gemm_tc_kernel(const GemvJob* __restrict__ jobs, const unsigned char* __restrict__ maps, const TcTile* __restrict__ tiles,
                    const int32_t* __restrict__ cta_begin, const unsigned char* __restrict__ bmap,
-                   const int32_t* __restrict__ job_base, int nrhs, int* err) {
+                   const TcJob* __restrict__ tj, const signed char* __restrict__ aexp, const float* __restrict__ bscale,
+                   int nrhs, int* err) {
+  constexpr int TC_NA = TcForm<F>::NA, AW = TcForm<F>::AW, BPB = TcForm<F>::BPB, KS = TcForm<F>::KS;
+  constexpr uint32_t IDESC_N64 = tc_idesc(F, TC_N), IDESC_N128 = tc_idesc(F, 2 * TC_N);
   extern __shared__ unsigned char tc_raw[];
   const int t_begin = cta_begin[blockIdx.x], t_end = cta_begin[blockIdx.x + 1];
   if (t_begin >= t_end) return;
@@ -238,7 +224,7 @@ __global__ void __maxnreg__(96)
       mbar_init(empty(q), 8);
     }
     for (int b = 0; b < TC_NA; ++b) {
-      mbar_init(ready(b), 8);
+      mbar_init(ready(b), 4);
       mbar_init(wfree(b), 1);
     }
     for (int a = 0; a < 2; ++a) {
@@ -299,30 +285,36 @@ __global__ void __maxnreg__(96)
     if (lane == 0) {
       int tile_i = 0, k = 0, nk = nk_of(t_begin), last = -1;
       for (int g = 0; g < total; ++g) {
-        const int b = g % TC_NA, bb = g % TC_NBB, seg = g / TC_BPS, j = g % TC_BPS;
+        const int b = g % TC_NA, gb = g / BPB, bb = gb % TC_NBB, seg = g / TC_BPS, j = g % TC_BPS;
         bool ok = true;
         if (j == 0 && seg >= 2) ok = mbar_wait(accempty(seg & 1), uint32_t(((seg >> 1) - 1) & 1), vfail);
+        if (ok && g % BPB == 0) ok = mbar_wait(bfull(bb), uint32_t((gb / TC_NBB) & 1), vfail);
         if (ok) ok = mbar_wait(ready(b), uint32_t((g / TC_NA) & 1), vfail);
-        if (ok) ok = mbar_wait(bfull(bb), uint32_t((g / TC_NBB) & 1), vfail);
         if (!ok) {
           *vfail = 1;
           break;
         }
         tc_fence_after();
         const uint32_t acc = tmem + TC_ACC_COL + uint32_t(seg & 1) * TC_ACC_COLS;
-        const uint32_t aop = tmem + TC_AOP_COL + uint32_t(b) * 64u;  // hi at +0, lo at +32
-        const uint32_t bh = bbuf0 + uint32_t(bb) * TC_BBUF;           // B' hi rows 0-63, lo rows 64-127
+        const uint32_t aop = tmem + TC_AOP_COL + uint32_t(b) * AW;  // hi, then lo
+        // B' hi rows 0-63, lo rows 64-127; this sub-chunk's half of the 128-byte rows
+        const uint32_t bh = bbuf0 + uint32_t(bb) * TC_BBUF + uint32_t(g % BPB) * 64u;
 #pragma unroll
-        for (int ks = 0; ks < TC_KC / 8; ++ks) {
-          const uint32_t o = uint32_t(ks) * 32u;  // 8 TF32 = 32 bytes along K in the swizzle row of B'
+        for (int ks = 0; ks < TC_KC / KS; ++ks) {
+          const uint32_t o = uint32_t(ks) * 32u;  // 16 FP16 or 8 TF32 = 32 bytes along K in the swizzle row of B'
           const uint32_t ac = uint32_t(ks) * 8u;  // 8 TMEM columns of A
           const uint32_t acc0 = (j > 0 || ks > 0) ? 1u : 0u;  // a fresh accumulator per segment
           // hi(A) [hi(B') | lo(B')] in one N = 128 product, then lo(A) hi(B') into columns 0-63
-          tc_mma_ts(acc, aop + ac, sw128_desc(bh + o), TC_IDESC_N128, acc0);
-          tc_mma_ts(acc, aop + 32u + ac, sw128_desc(bh + o), TC_IDESC_N64, 1u);
+          if constexpr (F) {
+            tc_mma_f16(acc, aop + ac, sw128_desc(bh + o), IDESC_N128, acc0);
+            tc_mma_f16(acc, aop + AW / 2 + ac, sw128_desc(bh + o), IDESC_N64, 1u);
+          } else {
+            tc_mma_tf32(acc, aop + ac, sw128_desc(bh + o), IDESC_N128, acc0);
+            tc_mma_tf32(acc, aop + AW / 2 + ac, sw128_desc(bh + o), IDESC_N64, 1u);
+          }
         }
         tc_commit(wfree(b));
-        tc_commit(bfree(bb));
+        if (g % BPB == BPB - 1) tc_commit(bfree(bb));
         if (j == TC_BPS - 1) tc_commit(accfull(seg & 1));
         last = g;
         if (++k == nk) {
@@ -334,16 +326,40 @@ __global__ void __maxnreg__(96)
       // the MMAs in flight (they complete in order) finish before the CTA leaves
       if (last >= 0) {
         mbar_wait(wfree(last % TC_NA), uint32_t((last / TC_NA) & 1));
-        mbar_wait(bfree(last % TC_NBB), uint32_t((last / TC_NBB) & 1));
+        if (last % BPB == BPB - 1) mbar_wait(bfree(last / BPB % TC_NBB), uint32_t((last / BPB / TC_NBB) & 1));
       }
     }
     __syncwarp();
   } else if (warp < 10) {
     // ---------------- split warps: thread = row of the tile (TMEM lane quarter warp % 4); the
-    // two warps of a lane quarter take the K columns 16 kh .. 16 kh + 15 of each sub-chunk
+    // two warps of a lane quarter take the sub-chunks in turn
     const int q4 = warp & 3, kh = (warp - 2) >> 2, row = 32 * q4 + lane;
-    for (int g = 0; g < total; ++g) {
+    // scale exponents of this row, one stage ahead of their use
+    int tile = t_begin, k = 0, nk = 0, mpad = 0;
+    const signed char* ea = nullptr;
+    auto next_exp = [&]() {
+      if (k == nk) {
+        if (tile == t_end) return 0;
+        const TcTile T = tiles[tile++];
+        const TcJob J = tj[T.job];
+        k = 0;
+        nk = T.nk;
+        mpad = J.mpad;
+        ea = aexp + J.aexp + int64_t(T.k0 / TC_BPS) * mpad + T.row0 + row;
+      }
+      const int e = *ea;
+      ea += mpad;
+      k += TC_BPS;
+      return e;
+    };
+    int enext = F ? next_exp() : 0;
+    f2 sc2 = f2_pack(1.f, 1.f);
+    for (int g = kh; g < total; g += 2) {
       const int st = g / TC_BPS, j = g % TC_BPS, q = st % TC_R, b = g % TC_NA;
+      if (F && j == kh) {  // this row's scale for the stage
+        sc2 = f2_pack(pow2f(enext), pow2f(enext));
+        enext = next_exp();
+      }
       bool ok = mbar_wait(full(q), uint32_t((st / TC_R) & 1), vfail);
       if (ok && g >= TC_NA) ok = mbar_wait(wfree(b), uint32_t(((g / TC_NA) - 1) & 1), vfail);
       ok = __all_sync(0xffffffffu, ok);  // the TMEM stores below need the whole warp
@@ -351,43 +367,61 @@ __global__ void __maxnreg__(96)
         *vfail = 1;
         break;
       }
-      // this row's half of box j of the landed stage: 4 x 16 B, swizzled
+      // this row of box j of the landed stage: 8 x 16 B, swizzled
       const unsigned char* rp = gb + size_t(q) * TC_STAGE_BYTES + size_t(j) * TC_A_BYTES + size_t(row) * 128;
-      float h[16], l[16];
+      const uint32_t ta = tmem + (uint32_t(32 * q4) << 16) + TC_AOP_COL + uint32_t(b) * AW;
+      float4 a[8];
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        const float4 a = *reinterpret_cast<const float4*>(rp + (((4 * kh + jj) ^ (row & 7)) * 16));
-        tf32_split(a.x, h[4 * jj], l[4 * jj]);
-        tf32_split(a.y, h[4 * jj + 1], l[4 * jj + 1]);
-        tf32_split(a.z, h[4 * jj + 2], l[4 * jj + 2]);
-        tf32_split(a.w, h[4 * jj + 3], l[4 * jj + 3]);
+      for (int jj = 0; jj < 8; ++jj) a[jj] = *reinterpret_cast<const float4*>(rp + ((jj ^ (row & 7)) * 16));
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        if constexpr (!F) {
+          float h[16], l[16];
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            const float4 v = a[4 * hf + jj];
+            tf32_split(v.x, h[4 * jj], l[4 * jj]);
+            tf32_split(v.y, h[4 * jj + 1], l[4 * jj + 1]);
+            tf32_split(v.z, h[4 * jj + 2], l[4 * jj + 2]);
+            tf32_split(v.w, h[4 * jj + 3], l[4 * jj + 3]);
+          }
+          tmem_st16(ta + uint32_t(16 * hf), h);
+          tmem_st16(ta + AW / 2 + uint32_t(16 * hf), l);
+          continue;
+        }
+        uint32_t h[8], l[8];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          const float4 v = a[4 * hf + jj];
+          f16_split(f2_mul(f2_pack(v.x, v.y), sc2), h[2 * jj], l[2 * jj]);
+          f16_split(f2_mul(f2_pack(v.z, v.w), sc2), h[2 * jj + 1], l[2 * jj + 1]);
+        }
+        tmem_st8(ta + uint32_t(8 * hf), h);
+        tmem_st8(ta + AW / 2 + uint32_t(8 * hf), l);
       }
-      const uint32_t ta = tmem + (uint32_t(32 * q4) << 16) + TC_AOP_COL + uint32_t(b) * 64u + uint32_t(16 * kh);
-      tmem_st16(ta, h);
-      tmem_st16(ta + 32u, l);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        if (j == TC_BPS - 1) mbar_arrive(empty(q));  // the stage's last sub-chunk: it may be refilled
+        if (j >= TC_BPS - 2) mbar_arrive(empty(q));  // this warp's last sub-chunk of the stage
         mbar_arrive(ready(b));                        // A of this sub-chunk is in TMEM
       }
     }
   } else if (warp == 18) {
-    // ---------------- TMA producer of B' (hi rows 0-63, lo rows 64-127 of one box per
-    // sub-chunk, built for the pass by tc_bprime_kernel) into the operand buffers
+    // ---------------- TMA producer of B' (hi rows 0-63, lo rows 64-127 of one box per two
+    // sub-chunks, built for the pass by tc_bprime_kernel) into the operand buffers
     if (lane == 0) {
       int tile = t_begin, k = 0, nk = nk_of(t_begin), g = 0;
-      for (; g < total; ++g) {
+      for (; g < total / BPB; ++g) {
         const int b = g % TC_NBB;
         if (g >= TC_NBB && !mbar_wait(bfree(b), uint32_t(((g / TC_NBB) - 1) & 1), vfail)) {
           *vfail = 1;
           break;
         }
         mbar_expect_tx(bfull(b), TC_BBUF);
-        tma_load_2d(bbuf0 + uint32_t(b) * TC_BBUF, bmap, 0, 2 * TC_N * (job_base[tiles[tile].job] + tiles[tile].k0 + k),
+        tma_load_2d(bbuf0 + uint32_t(b) * TC_BBUF, bmap, 0, 2 * TC_N * (tj[tiles[tile].job].base * (2 / BPB) + (tiles[tile].k0 + k) / BPB),
                     bfull(b));
-        if (++k == nk) {
+        if ((k += BPB) == nk) {
           k = 0;
           if (++tile < t_end) nk = nk_of(tile);
         }
@@ -399,31 +433,55 @@ __global__ void __maxnreg__(96)
   } else {
     // ---------------- epilogue warps: TMEM lane quarter warp % 4, accumulator columns 32 half ..
     const int q4 = warp & 3, half = (warp - 10) >> 2;
-    float cs[32], cc[32];  // compensated sums of this row's 32 columns over the tile's segments
+    // compensated sums of this row's 32 columns over the tile's segments, as the pairs
+    // (re, im) of 16 right-hand sides: packed FP32 operations, half the issue slots (these warps and
+    // the split warps share them; with single ones this kernel was bound there)
+    f2 cs[16], cc[16];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) cs[i] = cc[i] = 0.f;
+    for (int i = 0; i < 16; ++i) cs[i] = cc[i] = 0ull;
     int seg = 0;
     for (int t = t_begin; t < t_end; ++t) {
       const int nseg = nk_of(t) / TC_BPS;
       bool ok = true;
+      // the scales of the tile's segments: this row's of A, and in lane i the one of right-hand side 16 half + i
+      const signed char* ea;
+      const float* eb;
+      int mpad;
+      {
+        const TcTile T = tiles[t];
+        const TcJob TJ = tj[T.job];
+        mpad = TJ.mpad;
+        ea = aexp + TJ.aexp + int64_t(T.k0 / TC_BPS) * mpad + T.row0 + 32 * q4 + lane;
+        eb = bscale + (TJ.base / 2 + T.k0 / TC_BPS) * TC_MAX_NRHS + half * 16 + (lane & 15);
+      }
       for (int sg = 0; sg < nseg; ++sg, ++seg) {
+        float sa = 1.f, sbl = 1.f;
+        if (F) {  // before the wait for the segment
+          sa = pow2f(-*ea);
+          sbl = __ldg(eb);
+          ea += mpad;
+          eb += TC_MAX_NRHS;
+        }
         ok = __all_sync(0xffffffffu, mbar_wait(accfull(seg & 1), uint32_t((seg >> 1) & 1), vfail));
         if (!ok) break;  // the TMEM loads below need the whole warp
         tc_fence_after();
 #pragma unroll
         for (int hq = 0; hq < 4; ++hq) {
-          float v[8], w[8];  // hi(A) hi(B') + lo(A) hi(B'), and hi(A) lo(B')
+          f2 v[4], w[4];  // hi(A) hi(B') + lo(A) hi(B'), and hi(A) lo(B')
           tmem_ld8x2(tmem + (uint32_t(32 * q4) << 16) + TC_ACC_COL + uint32_t(seg & 1) * TC_ACC_COLS +
                          uint32_t(half * 32 + 8 * hq),
                      TC_N, v, w);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] = __fadd_rn(v[i], w[i]);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {  // TwoSum (Knuth): cs + cc carries the running sum
-            const int c = 8 * hq + i;
-            const float sum = __fadd_rn(cs[c], v[i]);
-            const float bp = __fsub_rn(sum, cs[c]);
-            cc[c] = __fadd_rn(cc[c], __fadd_rn(__fsub_rn(cs[c], __fsub_rn(sum, bp)), __fsub_rn(v[i], bp)));
+          for (int i = 0; i < 4; ++i) {  // 8 columns = 4 right-hand sides
+            const int c = 4 * hq + i;
+            f2 u = f2_add(v[i], w[i]);
+            if (F) {
+              const float sb = __shfl_sync(0xffffffffu, sbl, c);
+              u = f2_mul(f2_mul(u, f2_pack(sa, sa)), f2_pack(sb, sb));
+            }
+            // TwoSum (Knuth): cs + cc carries the running sum
+            const f2 sum = f2_add(cs[c], u), bp = f2_sub(sum, cs[c]);
+            cc[c] = f2_add(cc[c], f2_add(f2_sub(cs[c], f2_sub(sum, bp)), f2_sub(u, bp)));
             cs[c] = sum;
           }
         }
@@ -436,7 +494,7 @@ __global__ void __maxnreg__(96)
         break;
       }
       const TcTile T = tiles[t];
-      const GemvJob J = jobs[T.job];
+      const GemvJob& J = jobs[T.job];
       const int row = T.row0 + 32 * q4 + lane;
       if (row < J.m) {
         float2* y = reinterpret_cast<float2*>(J.y);
@@ -445,7 +503,8 @@ __global__ void __maxnreg__(96)
         for (int c = 0; c < 16; ++c) {
           const int r = half * 16 + c;
           if (r < nrhs) {
-            const float re = cs[2 * c] + cc[2 * c], im = cs[2 * c + 1] + cc[2 * c + 1];
+            float re, im;
+            f2_unpack(f2_add(cs[c], cc[c]), re, im);
             float2 o = make_float2(ar * re - ai * im, ar * im + ai * re);
             float2* yy = y + int64_t(r) * J.ldy + row;
             if (T.split) {
@@ -462,7 +521,7 @@ __global__ void __maxnreg__(96)
         }
       }
 #pragma unroll
-      for (int i = 0; i < 32; ++i) cs[i] = cc[i] = 0.f;
+      for (int i = 0; i < 16; ++i) cs[i] = cc[i] = 0ull;
     }
   }
   tc_fence_before();
@@ -473,14 +532,93 @@ __global__ void __maxnreg__(96)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
 }
 
+// B' of one stage (64 complex columns, two boxes of 64 K columns) per block: for
+// right-hand side r and complex column c row 2r holds (Re x_r[c], -Im x_r[c]) and row 2r + 1
+// (Im x_r[c], Re x_r[c]) at K columns 2c, 2c + 1, scaled by the power of two of the right-hand
+// side's largest entry in the stage, FP16 hi (rows 0-63) and lo (64-127) parts, row-major (TMA
+// applies the 128-byte swizzle); zero for r >= nrhs and beyond the job's columns.
+// bscale[stage][r] undoes the scale.  8 threads per right-hand side, 8 columns each.
+// Blocks nstage and above zero the Y rows of the tiles split along K.
+__global__ void __launch_bounds__(256) tc_bprime_kernel(const GemvJob* __restrict__ jobs, const int32_t* __restrict__ gjob,
+                                                        const int32_t* __restrict__ gst, int nstage,
+                                                        const TcTile* __restrict__ ztiles, int nrhs, __half* __restrict__ bp,
+                                                        float* __restrict__ bscale) {
+  const int gidx = blockIdx.x;
+  if (gidx >= nstage) {  // Y rows of a tile split along K: zeroed, the two halves add into them
+    const TcTile T = ztiles[gidx - nstage];
+    const GemvJob& J = jobs[T.job];
+    float2* y = reinterpret_cast<float2*>(J.y);
+    for (int e = threadIdx.x; e < TC_M * nrhs; e += blockDim.x) {
+      const int row = T.row0 + e % TC_M, r = e / TC_M;
+      if (row < J.m) y[int64_t(r) * J.ldy + row] = make_float2(0.f, 0.f);
+    }
+    return;
+  }
+  const GemvJob& J = jobs[gjob[gidx]];
+  const int r = threadIdx.x >> 3, sub = threadIdx.x & 7;
+  const int c0 = gst[gidx] * (2 * TC_KC) + sub * 8;  // 64 complex columns per stage
+  const float2* x = reinterpret_cast<const float2*>(J.x) + int64_t(r) * J.ldx;
+  float2 v[8];
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[i] = r < nrhs && c0 + i < J.n ? x[c0 + i] : make_float2(0.f, 0.f);
+    m = fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
+  }
+  for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int e = tc_scale_exp(m);
+  const float sc = pow2f(e);
+  if (sub == 0) bscale[int64_t(gidx) * TC_MAX_NRHS + r] = pow2f(-e);
+  uint32_t h0[8], l0[8], h1[8], l1[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float re = sc * v[i].x, im = sc * v[i].y;
+    f16_split(f2_pack(re, -im), h0[i], l0[i]);
+    f16_split(f2_pack(im, re), h1[i], l1[i]);
+  }
+  // box 2 gidx + (sub / 4), row, 8 pairs from K column 16 (sub % 4)
+  __half* box = bp + (size_t(2 * gidx + (sub >> 2)) * 2 * TC_N) * TC_BK + 16 * (sub & 3);
+  auto put = [&](int row, const uint32_t (&w)[8]) {
+    uint4* d = reinterpret_cast<uint4*>(box + size_t(row) * TC_BK);
+    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    d[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  };
+  put(2 * r, h0);
+  put(2 * r + 1, h1);
+  put(TC_N + 2 * r, l0);
+  put(TC_N + 2 * r + 1, l1);
+}
+
+// Scale exponents of A: one per row and stage (128 FP32 columns = 512 bytes of the row),
+// one warp each; aexp[stage][row] per job, rows padded to whole tiles.
+__global__ void __launch_bounds__(256) tc_aexp_kernel(const GemvJob* __restrict__ jobs, const TcJob* __restrict__ tj, int job,
+                                                      signed char* __restrict__ aexp) {
+  const GemvJob& J = jobs[job];
+  const TcJob T = tj[job];
+  const int64_t w = (int64_t(blockIdx.x) * 256 + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, nst = (2 * J.n + TC_KC * TC_BPS - 1) / (TC_KC * TC_BPS);
+  const int64_t row = w / nst;
+  const int st = int(w % nst);
+  if (row >= J.m) return;
+  const float2* a = reinterpret_cast<const float2*>(J.A) + row * J.lda;
+  float m = 0.f;
+  for (int c = st * (TC_KC * TC_BPS / 2) + lane, i = 0; i < 2; ++i, c += 32)
+    if (c < J.n) {
+      const float2 v = a[c];
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) aexp[T.aexp + int64_t(st) * T.mpad + row] = static_cast<signed char>(tc_scale_exp(m));
+}
+
 // B' of every sub-chunk of the pass (hi rows 0-63, lo rows 64-127, 32 FP32 columns
 // each, row-major; TMA applies the 128-byte swizzle): for right-hand side r and
 // complex column c = 16 kc + u / 2 of the sub-chunk's job, row 2r holds
 // (Re x_r[c], -Im x_r[c]) and row 2r + 1 (Im x_r[c], Re x_r[c]) at columns u, u + 1
 // (u even), TF32 hi and lo parts; zero for r >= nrhs and beyond the job's columns.
 // Blocks nsub and above zero the Y rows of the tiles split along K.
-__global__ void tc_bprime_kernel(const GemvJob* __restrict__ jobs, const int32_t* __restrict__ gjob,
-                                 const int32_t* __restrict__ gkc, int nsub, const TcTile* __restrict__ ztiles, int nrhs,
+__global__ void tf32_bprime_kernel(const GemvJob* __restrict__ jobs, const int32_t* __restrict__ gjob,
+                                 const int32_t* __restrict__ gst, int nsub, const TcTile* __restrict__ ztiles, int nrhs,
                                  float* __restrict__ bp) {
   const int gidx = blockIdx.x;
   if (gidx >= nsub) {  // Y rows of a tile split along K: zeroed, the two halves add into them
@@ -493,8 +631,8 @@ __global__ void tc_bprime_kernel(const GemvJob* __restrict__ jobs, const int32_t
     }
     return;
   }
-  const GemvJob& J = jobs[gjob[gidx]];
-  const int kc = gkc[gidx];
+  const GemvJob& J = jobs[gjob[gidx / TC_BPS]];
+  const int kc = gst[gidx / TC_BPS] * TC_BPS + gidx % TC_BPS;
   const float2* x = reinterpret_cast<const float2*>(J.x);
   for (int e = threadIdx.x; e < TC_N * TC_KC / 2; e += blockDim.x) {  // (row, complex column) pairs
     const int brow = e / (TC_KC / 2), cl = e % (TC_KC / 2);
@@ -530,35 +668,47 @@ static EncodeTiledFn encoder() {
   return fn;
 }
 
-void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, cudaStream_t s) {
-  tp.ok = false;
-  EncodeTiledFn enc = encoder();
-  if (!enc || jobs.empty()) return;
+bool tc_map_2d(int type, const void* p, uint64_t nx, uint64_t ny, uint64_t pitch, int bx, int by, unsigned char* out) {
   static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
+  const EncodeTiledFn enc = encoder();
+  if (!enc || pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(p) & 15) != 0) return false;
+  alignas(64) CUtensorMap map;
+  const cuuint64_t dims[2] = {nx, ny};
+  const cuuint64_t strides[1] = {pitch};
+  const cuuint32_t box[2] = {cuuint32_t(bx), cuuint32_t(by)};
+  const cuuint32_t estr[2] = {1, 1};
+  if (enc(&map, CUtensorMapDataType(type), 2, const_cast<void*>(p), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return false;
+  std::memcpy(out, &map, 128);
+  return true;
+}
+bool tc_block_map(const void* A, int64_t lda, int m, int n, unsigned char* out) {
+  return m > 0 && n > 0 && tc_map_2d(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, A, uint64_t(2) * n, m, uint64_t(lda) * 8, TC_KC, TC_M, out);
+}
+
+void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, bool f16, cudaStream_t s) {
+  tp.ok = false;
+  tp.f16 = f16;
+  tp.longest = 0;
+  if (jobs.empty()) return;
   std::vector<unsigned char> maps(jobs.size() * 128);
   std::vector<TcTile> tl;
   std::vector<int> cost;
-  std::vector<int32_t> job_base, gjob, gkc;
+  std::vector<int32_t> gjob, gst;
+  std::vector<TcJob> tjobs;
+  int64_t aexp_n = 0;
   std::vector<TcTile> tp_zero;  // tiles split along K: their Y rows are zeroed before each pass
   for (size_t i = 0; i < jobs.size(); ++i) {
     const GemvJob& J = jobs[i];
-    const uint64_t pitch = uint64_t(J.lda) * 8;
-    if (J.m <= 0 || J.n <= 0 || pitch % 16 != 0 || (reinterpret_cast<uintptr_t>(J.A) & 15) != 0) return;
-    alignas(64) CUtensorMap map;
-    const cuuint64_t dims[2] = {cuuint64_t(2) * J.n, cuuint64_t(J.m)};
-    const cuuint64_t strides[1] = {pitch};
-    const cuuint32_t box[2] = {cuuint32_t(TC_KC), cuuint32_t(TC_M)};
-    const cuuint32_t estr[2] = {1, 1};
-    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(J.A), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return;
-    std::memcpy(&maps[i * 128], &map, 128);
+    if (!tc_block_map(J.A, J.lda, J.m, J.n, &maps[i * 128])) return;
     const int nk = ((2 * J.n + TC_KC - 1) / TC_KC + TC_BPS - 1) / TC_BPS * TC_BPS;
-    job_base.push_back(int32_t(gjob.size()));
-    for (int kc = 0; kc < nk; ++kc) {
+    const int nst = nk / TC_BPS, mpad = (J.m + TC_M - 1) / TC_M * TC_M;
+    tjobs.push_back({aexp_n, mpad, 2 * int32_t(gjob.size())});
+    aexp_n += int64_t(nst) * mpad;
+    for (int st = 0; st < nst; ++st) {
       gjob.push_back(int32_t(i));
-      gkc.push_back(kc);
+      gst.push_back(st);
     }
     for (int r0 = 0; r0 < J.m; r0 += TC_M) {
       tl.push_back({int32_t(i), r0, 0, nk, 0});
@@ -608,6 +758,7 @@ void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, cudaStream_t s)
     pq.pop();
     per[lc.second].push_back(tl[i]);
     pq.push({lc.first + cost[i], lc.second});
+    tp.longest = std::max(tp.longest, int((lc.first + cost[i]) / TC_BPS));
   }
   std::vector<TcTile> flat;
   std::vector<int32_t> begin(1, 0);
@@ -615,27 +766,34 @@ void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, cudaStream_t s)
     flat.insert(flat.end(), v.begin(), v.end());
     begin.push_back(int32_t(flat.size()));
   }
-  // B' for every sub-chunk and its tensor map (boxes of 128 rows x 128 B, swizzled like the A boxes)
-  tp.nsub = int(gjob.size());
-  tp.bprime.alloc(size_t(tp.nsub) * 2 * TC_N * TC_KC);
-  {
-    alignas(64) CUtensorMap bm;
-    const cuuint64_t dims[2] = {cuuint64_t(TC_KC), cuuint64_t(tp.nsub) * 2 * TC_N};
-    const cuuint64_t strides[1] = {cuuint64_t(TC_KC) * 4};
-    const cuuint32_t box[2] = {cuuint32_t(TC_KC), cuuint32_t(2 * TC_N)};
-    const cuuint32_t estr[2] = {1, 1};
-    if (enc(&bm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, tp.bprime.p, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return;
-    std::vector<unsigned char> bmv(128);
-    std::memcpy(bmv.data(), &bm, 128);
-    tp.bmap.upload(bmv, s);
-  }
+  // B' for every stage and its tensor map (boxes of 128 rows x 128 B, swizzled like the A boxes)
+  tp.nstage = int(gjob.size());
+  const uint64_t brows = uint64_t(tp.nstage) * (f16 ? 2 : 4) * 2 * TC_N;  // of 128 bytes
+  tp.bprime.alloc(size_t(brows) * 128);
+  tp.bscale.alloc(size_t(tp.nstage) * TC_MAX_NRHS);
+  std::vector<unsigned char> bmv(128);
+  const int bx = f16 ? TC_BK : TC_KC;
+  if (!tc_map_2d(f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, tp.bprime.p, bx, brows, 128, bx, 2 * TC_N,
+                 bmv.data()))
+    return;
+  tp.bmap.upload(bmv, s);
   tp.nzero = int(tp_zero.size());
   if (tp.nzero > 0) tp.ztiles.upload(tp_zero, s);
-  tp.job_base.upload(job_base, s);
+  tp.tj.upload(tjobs, s);
   tp.gjob.upload(gjob, s);
-  tp.gkc.upload(gkc, s);
+  tp.gst.upload(gst, s);
+  tp.aexp.alloc(size_t(aexp_n));
+  tp.aexp.zero(s);
+  {
+    DBuf<GemvJob> dj;
+    dj.upload(jobs, s);
+    for (size_t i = 0; i < jobs.size(); ++i) {
+      const int64_t warps = int64_t(jobs[i].m) * ((2 * jobs[i].n + TC_KC * TC_BPS - 1) / (TC_KC * TC_BPS));
+      tc_aexp_kernel<<<unsigned((warps * 32 + 255) / 256), 256, 0, s>>>(dj.p, tp.tj.p, int(i), tp.aexp.p), count_launch();
+    }
+    SLDM_CUDA(cudaGetLastError());
+    SLDM_CUDA(cudaStreamSynchronize(s));
+  }
   tp.maps.upload(maps, s);
   tp.tiles.upload(flat, s);
   tp.cta_begin.upload(begin, s);
@@ -648,21 +806,34 @@ void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, cudaStream_t s)
 
 void gemm_tc(const GemvPlan& plan, const TcPlan& tp, int nrhs, cudaStream_t s) {
   SLDM_REQUIRE(tp.ok && nrhs >= 1 && nrhs <= TC_MAX_NRHS, SLDM_EINVAL, "tensor-core product: invalid plan or nrhs");
-  static std::atomic<uint64_t> attr_set{0};  // devices whose attribute is set
+  static std::atomic<uint64_t> attr_set{0};  // devices whose attributes are set
   int dev = 0;
   SLDM_CUDA(cudaGetDevice(&dev));
   const uint64_t bit = uint64_t(1) << (dev & 63);
   if (!(attr_set.load() & bit)) {
-    SLDM_CUDA(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TC_SMEM)));
+    SLDM_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TC_SMEM)));
+    SLDM_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(TC_SMEM)));
     attr_set.fetch_or(bit);
   }
   ScopedTimer tm("gemm_tc", s);
-  tc_bprime_kernel<<<unsigned(tp.nsub + tp.nzero), 256, 0, s>>>(plan.jobs, tp.gjob.p, tp.gkc.p, tp.nsub, tp.ztiles.p, nrhs,
-                                                                tp.bprime.p);
-  count_launch();
-  gemm_tc_kernel<<<unsigned(tp.nctas), TC_THREADS, TC_SMEM, s>>>(plan.jobs, tp.maps.p, tp.tiles.p, tp.cta_begin.p,
-                                                                  tp.bmap.p, tp.job_base.p, nrhs, tp.err.p);
-  count_launch();
+  auto go = [&](auto f) {
+    gemm_tc_kernel<decltype(f)::value><<<unsigned(tp.nctas), TC_THREADS, TC_SMEM, s>>>(plan.jobs, tp.maps.p, tp.tiles.p, tp.cta_begin.p,
+                                                                                       tp.bmap.p, tp.tj.p, tp.aexp.p, tp.bscale.p, nrhs,
+                                                                                       tp.err.p);
+    count_launch();
+  };
+  if (tp.f16) {
+    tc_bprime_kernel<<<unsigned(tp.nstage + tp.nzero), 256, 0, s>>>(plan.jobs, tp.gjob.p, tp.gst.p, tp.nstage, tp.ztiles.p, nrhs,
+                                                                    reinterpret_cast<__half*>(tp.bprime.p), tp.bscale.p);
+    count_launch();
+    go(std::true_type{});
+  } else {
+    const int nsub = tp.nstage * TC_BPS;
+    tf32_bprime_kernel<<<unsigned(nsub + tp.nzero), 256, 0, s>>>(plan.jobs, tp.gjob.p, tp.gst.p, nsub, tp.ztiles.p, nrhs,
+                                                                 reinterpret_cast<float*>(tp.bprime.p));
+    count_launch();
+    go(std::false_type{});
+  }
   SLDM_CUDA(cudaGetLastError());
 }
 

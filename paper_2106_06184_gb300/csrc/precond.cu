@@ -428,7 +428,7 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   for (auto& jb : jobs) P.plan.bytes += double(jb.m) * jb.n * ev;
   P.plan.tc = nullptr;
   if (P.f32) {
-    tc_plan_build(jobs, P.tc, s);
+    tc_plan_build(jobs, P.tc, true, s);
     if (P.tc.ok) P.plan.tc = &P.tc;
   }
   SLDM_CUDA(cudaStreamSynchronize(s));
