@@ -12,6 +12,7 @@
 
 #include "dense.h"
 #include "gemm_tc.h"
+#include "gemm_x2.h"
 #include "internal.h"
 #include "mgf.h"
 #include "nested.h"
@@ -95,7 +96,8 @@ struct sldm_op {
   sldm::DBuf<int64_t> rs1d, rs2d;
   sldm::DBuf<int2> tl1d, tl2d;
   sldm::GemvPlan plan1d, plan2d;
-  // SLDM_PREC_F32X2: Y11 e, Y21 e of the far field
+  sldm::X2Plan x2p1, x2p2;  // SLDM_PREC_F32X2: the same on the tensor cores
+  // and Y11 e, Y21 e of its far field
   sldm::DBuf<sldm::GemvJob> jobsf;
   sldm::DBuf<int64_t> rsf;
   sldm::DBuf<int2> tlf;
@@ -144,7 +146,7 @@ static int64_t op_bytes(const sldm_op* op) {
 // operator's precision and FP64 fit).
 static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1, DBuf<int64_t>& drs1, DBuf<int2>& dt1,
                        GemvPlan& p1, DBuf<GemvJob>& dj2, DBuf<int64_t>& drs2, DBuf<int2>& dt2, GemvPlan& p2,
-                       TcPlan* tc1 = nullptr, TcPlan* tc2 = nullptr) {
+                       TcPlan* tc1 = nullptr, TcPlan* tc2 = nullptr, X2Plan* x1 = nullptr, X2Plan* x2 = nullptr) {
   const int64_t ne = op->ne, nt = op->nt;
   auto P = [&](DBuf<char>& b, int64_t off) { return (void*)(b.p + off * es_v); };
   const char* loc = op->loc.p;
@@ -169,7 +171,7 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
     j2.push_back({L(o.oLP), o.nt, o.nt, o.nt, P(op->wbu, o.t0), nt, P(op->ww3, o.t0), nt, 1, 0, 0, 0, Lo(o.oLP)});
   }
   auto mk = [&](std::vector<GemvJob>& j, DBuf<GemvJob>& dj, DBuf<int64_t>& drs, DBuf<int2>& dt, GemvPlan& plan,
-                TcPlan* tc, bool f16 = true) {
+                TcPlan* tc, X2Plan* xp, const TcPlan& like, bool f16 = true) {
     std::vector<int64_t> rs(j.size());
     std::vector<int2> tiles;
     int64_t acc = 0;
@@ -196,9 +198,14 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
       tc_plan_build(j, *tc, f16, 0);
       if (tc->ok) plan.tc = tc;
     }
+    plan.x2 = nullptr;
+    if (xp && lo && tc_policy() <= MAX_NRHS) {
+      x2_plan_build(j, like, *xp, 0);
+      if (xp->ok) plan.x2 = xp;
+    }
   };
-  mk(j1, dj1, drs1, dt1, p1, tc1);
-  mk(j2, dj2, drs2, dt2, p2, tc2);
+  mk(j1, dj1, drs1, dt1, p1, tc1, x1, op->tc1);
+  mk(j2, dj2, drs2, dt2, p2, tc2, x2, op->tc2);
   // The far field of an FP64 system held as pairs goes through a complex64 product with Y: complex128
   // numbers that show its rounding, so it keeps the TF32 form and the products by themselves
   if (op->x2 && es_v == sizeof(float2)) {
@@ -207,7 +214,7 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
       jf.push_back({L(o.oY11), o.ne, o.ne, o.ne, P(op->we, o.e0), ne, P(op->wz1, o.e0), ne, 1, 0, 0, 0, nullptr});
       if (o.nt > 1) jf.push_back({L(o.oY21), o.ne, o.nt - 1, o.ne, P(op->we, o.e0), ne, P(op->wz2, o.q0), op->nq, 1, 0, 0, 0, nullptr});
     }
-    mk(jf, op->jobsf, op->rsf, op->tlf, op->planf, &op->tcf, false);
+    mk(jf, op->jobsf, op->rsf, op->tlf, op->planf, &op->tcf, nullptr, op->tcf, false);
     op->planf.name = "gemv_y";
     // not measured: its kernel, and so the far field's last digits, should not hang on a timing.  16 right-hand
     // sides: 4 x 4 metasurface 34 us against 26 on the CUDA cores, one sphere of 1,280 triangles 53 / 42; 32: 36 / 42
@@ -241,7 +248,7 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
   }
   if (sizeof(C) == sizeof(float2)) {
     make_plans(op, sizeof(C), sizeof(double2), op->jobs1d, op->rs1d, op->tl1d, op->plan1d, op->jobs2d, op->rs2d, op->tl2d,
-               op->plan2d);
+               op->plan2d, nullptr, nullptr, &op->x2p1, &op->x2p2);
     op->plan1d.name = "gemv_y_f64acc";
     op->plan2d.name = "gemv_main_f64acc";
   }

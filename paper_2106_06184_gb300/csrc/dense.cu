@@ -16,6 +16,7 @@
 
 #include "dense.h"
 #include "gemm_tc.h"
+#include "gemm_x2.h"
 #include "widen.cuh"
 
 namespace sldm {
@@ -993,7 +994,17 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s) {
     }
   }
   ScopedTimer tm(plan.name, s);
-  timer_units(plan.name, plan.bytes * double((nrhs + TILE_NRHS - 1) / TILE_NRHS));
+  int c0 = 0;
+  if constexpr (comp) {
+    if (plan.x2 != nullptr && plan.x2->ok) {  // tensor-core passes of up to 16, as long as they are worth it
+      for (int nr; (nr = std::min(X2_NRHS, nrhs - c0)) >= plan.x2->from; c0 += nr) {
+        timer_units(plan.name, plan.bytes);
+        gemm_x2(plan, *plan.x2, nr, c0, s);
+      }
+      if (c0 == nrhs) return;
+    }
+  }
+  timer_units(plan.name, plan.bytes * double((nrhs - c0 + TILE_NRHS - 1) / TILE_NRHS));
   if (nrhs >= 2 || comp) {
     SLDM_REQUIRE((plan.tiles != nullptr && plan.tile_rows == GemvTile<CM, CV>::ROWS), SLDM_EINVAL,
                  "GEMV plan without row tiles for this vector type");
@@ -1003,26 +1014,26 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s) {
     // entry and right-hand side), so the rest takes a kernel of its own width; complex64
     // passes, bound by launches and L2, take it as one more pass of 8.
     // (box of 432 triangles, FP64, 5 right-hand sides, the whole product: 453 us with 8 -> 303 us)
-    const int full = c64 && nrhs > 4 ? nrhs : nrhs / TILE_NRHS * TILE_NRHS, rest = nrhs - full;
+    const int left = nrhs - c0, full = c64 && left > 4 ? left : left / TILE_NRHS * TILE_NRHS, rest = left - full, c1 = c0 + full;
     auto go = [&](auto lo) {
       constexpr bool LO = decltype(lo)::value;
-      if (full > 0) launch_tile<CM, CV, 8, LO>(plan, full, s, 0);
+      if (full > 0) launch_tile<CM, CV, 8, LO>(plan, full, s, c0);
       switch (rest) {
         case 1:
-          if constexpr (comp) launch_tile<CM, CV, 1, LO>(plan, rest, s, full);
-          else launch_tile<CM, CV, 2, LO>(plan, rest, s, full);
+          if constexpr (comp) launch_tile<CM, CV, 1, LO>(plan, rest, s, c1);
+          else launch_tile<CM, CV, 2, LO>(plan, rest, s, c1);
           break;
-        case 2: launch_tile<CM, CV, 2, LO>(plan, rest, s, full); break;
+        case 2: launch_tile<CM, CV, 2, LO>(plan, rest, s, c1); break;
         case 3:
-          if constexpr (c64) launch_tile<CM, CV, 4, LO>(plan, rest, s, full);
-          else launch_tile<CM, CV, 3, LO>(plan, rest, s, full);
+          if constexpr (c64) launch_tile<CM, CV, 4, LO>(plan, rest, s, c1);
+          else launch_tile<CM, CV, 3, LO>(plan, rest, s, c1);
           break;
-        case 4: launch_tile<CM, CV, 4, LO>(plan, rest, s, full); break;
+        case 4: launch_tile<CM, CV, 4, LO>(plan, rest, s, c1); break;
         default:
           if constexpr (!c64) {
-            if (rest == 5) launch_tile<CM, CV, 5, LO>(plan, rest, s, full);
-            else if (rest == 6) launch_tile<CM, CV, 6, LO>(plan, rest, s, full);
-            else if (rest == 7) launch_tile<CM, CV, 7, LO>(plan, rest, s, full);
+            if (rest == 5) launch_tile<CM, CV, 5, LO>(plan, rest, s, c1);
+            else if (rest == 6) launch_tile<CM, CV, 6, LO>(plan, rest, s, c1);
+            else if (rest == 7) launch_tile<CM, CV, 7, LO>(plan, rest, s, c1);
           }
       }
     };

@@ -48,6 +48,7 @@ struct GemvJob {
   const void* Alo;
 };
 struct TcPlan;
+struct X2Plan;
 // right-hand sides in lockstep (GMRES) and per pass of the structured product
 // and the preconditioner: up to 32 (tensor cores for complex64 operators; the
 // CUDA-core kernels take 8 per launch)
@@ -71,6 +72,8 @@ struct GemvPlan {
   // complex64 blocks and vectors: the tensor-core plan for 9 to 32 right-hand
   // sides per pass (gemm_tc.h), or null / not ok for passes of 8 on the CUDA cores
   const TcPlan* tc = nullptr;
+  // FP64-accurate products (has_lo): their tensor-core plan (gemm_x2.h), or null
+  const X2Plan* x2 = nullptr;
   // smallest lockstep width sent to the tensor cores (set by gemv_autotune;
   // 33 = never): below it, passes of 8 on the CUDA cores
   int tc_from = TILE_NRHS + 1;
