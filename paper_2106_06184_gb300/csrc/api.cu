@@ -1526,19 +1526,37 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
   ScopedTimer tm("farfield", s);
   const int WR = sldm_op::WR;
   const int nr_pass = std::min(nrhs, WR);
-  DBuf<double2> dx, jd;
-  dx.alloc(size_t(op->N) * nr_pass);
-  jd.alloc(size_t(op->ne) * nrhs);
+  // one allocation: the angles' records, the currents, the result, and x or the far field's
+  // workspace, which is cut down where memory is short
+  const size_t nx = size_t(op->N) * nr_pass, nj = size_t(op->ne) * nrhs, nrcs = (size_t(n) * nrhs + 1) / 2;
+  const size_t nrec = op->layered ? size_t(n) * PW_REC : size_t(n);
+  DBuf<double2> buf;
+  int chunk = farfield_chunk(op->mesh, nrhs, n);
+  for (;; chunk /= 2) {
+    const size_t nm = size_t(chunk) * 6 * op->nt;
+    try {
+      buf.alloc(nrec + nj + nrcs + std::max(nx, nm));
+      break;
+    } catch (const Error& e) {
+      if (e.code != SLDM_ENOMEM || nm <= nx) throw;
+    }
+  }
+  double* const dr = reinterpret_cast<double*>(buf.p + nrec + nj);
+  double2 *const jd = buf.p + nrec, *const dx = buf.p + nrec + nj + nrcs;
+  auto upload = [&](const std::vector<double>& v) {
+    SLDM_CUDA(cudaMemcpyAsync(buf.p, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+    return reinterpret_cast<const double*>(buf.p);
+  };
   const ApplyDims D = dims_of(op);
   // j_Delta = j - Y11 e (per object), from the first two stages of the structured product
   for (int r0 = 0; r0 < nrhs; r0 += WR) {
     const int nr = std::min(WR, nrhs - r0);
     const size_t bytes = size_t(op->N) * nr * sizeof(double2);
     const char* xs = static_cast<const char*>(x) + size_t(op->N) * r0 * sizeof(double2);
-    SLDM_CUDA(cudaMemcpyAsync(dx.p, xs, bytes, where == SLDM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    SLDM_CUDA(cudaMemcpyAsync(dx, xs, bytes, where == SLDM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     VecBatch<double2, double2> b;
-    for (int c = 0; c < nr; ++c) b.x[c] = dx.p + int64_t(c) * op->N;
-    double2* jo = jd.p + int64_t(op->ne) * r0;
+    for (int c = 0; c < nr; ++c) b.x[c] = dx + int64_t(c) * op->N;
+    double2* jo = jd + int64_t(op->ne) * r0;
     if (op->prec == SLDM_PREC_F32) {
       apply_in<double2, float2>(op->mesh, b, 1.0, 1.0, 1.0, D, op->wj.p, op->wa.p, op->we.p, op->wbu.p, op->wbc.p, nr, s);
       if (op->x2) {
@@ -1554,8 +1572,6 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
       to_c128<double2>(op->wa.p, int64_t(op->ne) * nr, jo, s);
     }
   }
-  DBuf<double> da, dr;
-  dr.alloc(size_t(n) * nrhs);
   if (op->layered) {
     // reciprocity: the stack's theta- and phi-polarised waves arriving from each direction
     std::vector<double> rec(size_t(2) * n * PW_REC);
@@ -1566,18 +1582,16 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
       mgf_plane_wave(op->H, op->thick, op->z_top, 2 * PI_ * op->freq, khat, pt, rec.data() + size_t(2 * i) * PW_REC);
       mgf_plane_wave(op->H, op->thick, op->z_top, 2 * PI_ * op->freq, khat, pp, rec.data() + size_t(2 * i + 1) * PW_REC);
     }
-    da.upload(rec, s);
-    farfield_layered(op->mesh, jd.p, op->ne, nrhs, da.p, n, dr.p, s);
+    farfield_layered(op->mesh, jd, op->ne, nrhs, upload(rec), n, dx, chunk, dr, s);
   } else {
     std::vector<double> ang(2 * size_t(n));
     for (int i = 0; i < n; ++i) {
       ang[2 * i] = theta[i];
       ang[2 * i + 1] = phi[i];
     }
-    da.upload(ang, s);
-    farfield(op->mesh, op->k0, jd.p, op->ne, nrhs, da.p, n, dr.p, s);
+    farfield(op->mesh, op->k0, jd, op->ne, nrhs, upload(ang), n, dx, chunk, dr, s);
   }
-  SLDM_CUDA(cudaMemcpyAsync(rcs, dr.p, size_t(n) * nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
+  SLDM_CUDA(cudaMemcpyAsync(rcs, dr, size_t(n) * nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
   SLDM_CUDA(cudaStreamSynchronize(s));
   API_END
 }

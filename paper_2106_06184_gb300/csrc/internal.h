@@ -251,11 +251,13 @@ void rhs_planewave_layered(const sldm_mesh* m, const double* rec_dev, int nrhs, 
 // RCS above a stack: per angle the theta- and phi-polarised plane-wave records
 // (2n records of PW_REC doubles, device) of waves arriving from the observation
 // direction; jd: nr columns of complex128 RWG coefficients (stride ldj), rcs:
-// n x nr (stride n), device
-void farfield_layered(const sldm_mesh* m, const double2* jd, int64_t ldj, int nr, const double* rec_dev, int n, double* rcs,
-                      cudaStream_t s);
+// n x nr (stride n), device; M: workspace of chunk x 6 x triangles (chunk: farfield_chunk's, or less down to 0,
+// without it)
+int farfield_chunk(const sldm_mesh* m, int nr, int n);
+void farfield_layered(const sldm_mesh* m, const double2* jd, int64_t ldj, int nr, const double* rec_dev, int n, double2* M, int chunk,
+                      double* rcs, cudaStream_t s);
 // far field in free space: angles (theta, phi) pairs, device; jd, rcs as above
-void farfield(const sldm_mesh* m, double k0, const double2* jd, int64_t ldj, int nr, const double* ang_dev, int n,
+void farfield(const sldm_mesh* m, double k0, const double2* jd, int64_t ldj, int nr, const double* ang_dev, int n, double2* M, int chunk,
               double* rcs, cudaStream_t s);
 
 }  // namespace sldm
