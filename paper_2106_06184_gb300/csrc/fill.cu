@@ -501,9 +501,11 @@ __global__ void __launch_bounds__(TILE_SRC, sizeof(R) == 4 ? 4 : 2) fill_K_bulk(
 }
 
 // ---------------------------------------------------------------- FP64 touching Kbar pairs
-// Same lane layout as the L kernel: lane q < 6 takes outer point q.
+// Same lane layout as the L kernel: lane q < 6 takes outer point q.  Tasks by object (obj_task), or
+// task 0 for the object `only`.  A sphere of 320 triangles: 418 us
+// with a thread per pair, 271 so.
 template <class R>
-__global__ void fill_K_touch(const KTask* __restrict__ tasks, const int32_t* __restrict__ obj_task,
+__global__ void fill_K_touch(const KTask* __restrict__ tasks, const int32_t* __restrict__ obj_task, int only,
                              const int32_t* __restrict__ tri_obj, const int32_t* __restrict__ pa,
                              const int32_t* __restrict__ pc, int npairs, const double* __restrict__ geo,
                              const double* __restrict__ bgeo, const double* __restrict__ xyz,
@@ -515,7 +517,7 @@ __global__ void fill_K_touch(const KTask* __restrict__ tasks, const int32_t* __r
   if (p < npairs) {
     t = pa[p];
     cg = pc[p];
-    task = obj_task[tri_obj[t]];
+    task = obj_task != nullptr ? obj_task[tri_obj[t]] : (tri_obj[t] == only ? 0 : -1);
   }
   const bool act = task >= 0 && q < 6;
   KTask tk;
@@ -765,7 +767,7 @@ void fill_K(const sldm_mesh* m, const std::vector<KTask>& tasks, cudaStream_t s)
   dot.upload(unsplit_object_tasks(m->h, tasks, split), s);
   if (np > 0) {
     ScopedTimer tm("fill_K_touch", s);
-    fill_K_touch<R><<<unsigned((int64_t(np) * 8 + 255) / 256), 256, 0, s>>>(dt.p, dot.p, d.obj.p, d.touchK_a.p, d.touchK_c.p, np,
+    fill_K_touch<R><<<unsigned((int64_t(np) * 8 + 255) / 256), 256, 0, s>>>(dt.p, dot.p, -1, d.obj.p, d.touchK_a.p, d.touchK_c.p, np,
                                                                             d.geo.p, d.bgeo.p, d.xyz.p, d.tri.p, d.tri_edge.p,
                                                                             d.btri_edge.p), ::sldm::count_launch();
   }
@@ -1176,112 +1178,6 @@ template void contract_bc<double>(const sldm_mesh*, int, const void*, int64_t, v
 
 }  // namespace sldm
 
-namespace sldm {
-
-// ---------------------------------------------------------------- FP64 touching Kbar pairs, one task by value
-// One thread per pair (used by the allocation-free entry point).
-__global__ void fill_K_touch_one(KTask tk, const int32_t* __restrict__ pa, const int32_t* __restrict__ pc, int npairs,
-                             const double* __restrict__ geo, const double* __restrict__ bgeo,
-                             const double* __restrict__ xyz, const int32_t* __restrict__ tri,
-                             const int32_t* __restrict__ tri_edge, const int32_t* __restrict__ btri_edge) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= npairs) return;
-  const int t = pa[p], cg = pc[p];
-  if (t < tk.t0 || t >= tk.t0 + tk.ntest || cg < tk.c0 || cg >= tk.c0 + tk.nsrc) return;
-  const double* gt = geo + size_t(t) * GEO_STRIDE;
-  const double* gs = bgeo + size_t(cg) * GEO_STRIDE;
-  // child vertices: rebuild from the parent (a, m_ab, g) ... pattern
-  const int par = cg / 6, kk = cg % 6;
-  const double* a = xyz + 3 * tri[3 * par];
-  const double* b = xyz + 3 * tri[3 * par + 1];
-  const double* c = xyz + 3 * tri[3 * par + 2];
-  double V[7][3];  // a, b, c, m_ab, m_bc, m_ca, g
-  for (int d = 0; d < 3; ++d) {
-    V[0][d] = a[d]; V[1][d] = b[d]; V[2][d] = c[d];
-    V[3][d] = 0.5 * (a[d] + b[d]); V[4][d] = 0.5 * (b[d] + c[d]); V[5][d] = 0.5 * (c[d] + a[d]);
-    V[6][d] = (a[d] + b[d] + c[d]) / 3.0;
-  }
-  const int cv[6][3] = {{0, 3, 6}, {3, 1, 6}, {1, 4, 6}, {4, 2, 6}, {2, 5, 6}, {5, 0, 6}};
-  const double* p1 = V[cv[kk][0]];
-  const double* p2 = V[cv[kk][1]];
-  const double* p3 = V[cv[kk][2]];
-  const cd k = {tk.kr, tk.ki};
-  cd P1 = {0, 0}, P2[3] = {{0, 0}, {0, 0}, {0, 0}}, X[3] = {{0, 0}, {0, 0}, {0, 0}}, S[3] = {{0, 0}, {0, 0}, {0, 0}};
-  for (int q = 0; q < 6; ++q) {
-    double r[3], rq[3];
-    for (int d = 0; d < 3; ++d) {
-      rq[d] = gt[GEO_RHO + 3 * q + d];
-      r[d] = gt[GEO_C + d] + rq[d];
-    }
-    cd U[3] = {{0, 0}, {0, 0}, {0, 0}}, Vv[3] = {{0, 0}, {0, 0}, {0, 0}};
-    for (int j = 0; j < 6; ++j) {
-      const double* rs = gs + GEO_RHO + 3 * j;
-      double D[3] = {r[0] - gs[GEO_C] - rs[0], r[1] - gs[GEO_C + 1] - rs[1], r[2] - gs[GEO_C + 2] - rs[2]};
-      double Rr = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
-      cd g1 = grad_smooth(k, Rr);
-      double w = gs[GEO_W + j];
-      g1.r *= w;
-      g1.i *= w;
-      double cr[3] = {D[1] * rs[2] - D[2] * rs[1], D[2] * rs[0] - D[0] * rs[2], D[0] * rs[1] - D[1] * rs[0]};
-      for (int d = 0; d < 3; ++d) {
-        U[d].r += g1.r * cr[d];
-        U[d].i += g1.i * cr[d];
-        Vv[d].r += g1.r * D[d];
-        Vv[d].i += g1.i * D[d];
-      }
-    }
-    // static part: V_s = int grad 1/(4 pi R) dS', U_s = V_s x (r - c')
-    Pot P;
-    potentials(r, p1, p2, p3, P);
-    double vs[3], rc[3];
-    for (int d = 0; d < 3; ++d) {
-      vs[d] = INV4PI * P.grad[d];
-      rc[d] = r[d] - gs[GEO_C + d];
-    }
-    double us[3] = {vs[1] * rc[2] - vs[2] * rc[1], vs[2] * rc[0] - vs[0] * rc[2], vs[0] * rc[1] - vs[1] * rc[0]};
-    for (int d = 0; d < 3; ++d) {
-      U[d].r += us[d];
-      Vv[d].r += vs[d];
-    }
-    double w = gt[GEO_W + q];
-    for (int d = 0; d < 3; ++d) {
-      P1.r += w * rq[d] * U[d].r;
-      P1.i += w * rq[d] * U[d].i;
-      P2[d].r += w * U[d].r;
-      P2[d].i += w * U[d].i;
-      S[d].r += w * Vv[d].r;
-      S[d].i += w * Vv[d].i;
-    }
-    X[0].r += w * (rq[1] * Vv[2].r - rq[2] * Vv[1].r); X[0].i += w * (rq[1] * Vv[2].i - rq[2] * Vv[1].i);
-    X[1].r += w * (rq[2] * Vv[0].r - rq[0] * Vv[2].r); X[1].i += w * (rq[2] * Vv[0].i - rq[0] * Vv[2].i);
-    X[2].r += w * (rq[0] * Vv[1].r - rq[1] * Vv[0].r); X[2].i += w * (rq[0] * Vv[1].i - rq[1] * Vv[0].i);
-  }
-  for (int i = 0; i < 3; ++i) {
-    const double* av = gt + GEO_AV + 3 * i;
-    cd base = P1;
-    for (int d = 0; d < 3; ++d) {
-      base.r += av[d] * P2[d].r;
-      base.i += av[d] * P2[d].i;
-    }
-    cd axs[3] = {{av[1] * S[2].r - av[2] * S[1].r, av[1] * S[2].i - av[2] * S[1].i},
-                 {av[2] * S[0].r - av[0] * S[2].r, av[2] * S[0].i - av[0] * S[2].i},
-                 {av[0] * S[1].r - av[1] * S[0].r, av[0] * S[1].i - av[1] * S[0].i}};
-    for (int j = 0; j < 3; ++j) {
-      const double* bv = gs + GEO_AV + 3 * j;
-      cd v = base;
-      for (int d = 0; d < 3; ++d) {
-        v.r += bv[d] * (X[d].r + axs[d].r);
-        v.i += bv[d] * (X[d].i + axs[d].i);
-      }
-      double sc = gt[GEO_SIG + i] * gs[GEO_SIG + j];
-      add_d<double>(tk.Kb, int64_t(tri_edge[3 * t + i] - tk.e_row0) * tk.ld + (btri_edge[3 * cg + j] - tk.b_col0), v.r * sc,
-               v.i * sc);
-    }
-  }
-}
-
-}  // namespace sldm
-
 // ---------------------------------------------------------------- allocation-free Kbar
 // sldm_kbar_noalloc: the barycentric Kbar fill of one object and its contraction
 // with the BC coefficients, with every temporary (task record, tile list and the
@@ -1377,8 +1273,10 @@ extern "C" int sldm_kbar_noalloc(const sldm_mesh* m, int32_t obj, double k_re, d
     SLDM_CUDA(cudaGetLastError());
     const int np = int(h.touchK_a.size());
     if (np > 0)
-      fill_K_touch_one<<<(np + 127) / 128, 128, 0, s>>>(t, d.touchK_a.p, d.touchK_c.p, np, d.geo.p, d.bgeo.p, d.xyz.p,
-                                                        d.tri.p, d.tri_edge.p, d.btri_edge.p), ::sldm::count_launch();
+      fill_K_touch<double><<<unsigned((int64_t(np) * 8 + 255) / 256), 256, 0, s>>>(dtask, nullptr, obj, d.obj.p, d.touchK_a.p,
+                                                                                d.touchK_c.p, np, d.geo.p, d.bgeo.p, d.xyz.p,
+                                                                                d.tri.p, d.tri_edge.p, d.btri_edge.p),
+          ::sldm::count_launch();
     SLDM_CUDA(cudaGetLastError());
     contract_bc<double>(m, obj, Kb, nbe_o, K_out, ne_o, s);
   } catch (const sldm::Error& e) {
