@@ -83,6 +83,7 @@ struct sldm_op {
   std::vector<sldm::ObjInfo> obj;
   std::vector<int> ref;  // the first object that each repeats, or itself
   sldm::DBuf<double> ix_val;
+  sldm::DBuf<float2> ix32;  // the same as pairs (complex64 operators)
   // structured product: work vectors for up to WR right-hand sides per pass
   static constexpr int WR = sldm::MAX_NRHS;
   sldm::DBuf<char> wj, we, wa, wbc, wbu, wz1, wz2, ww1, ww2, ww3;
@@ -137,7 +138,7 @@ static int64_t op_bytes(const sldm_op* op) {
   for (const auto& u : op->nested)
     if (u->mat && u->obj == u->mat_owner) nb += int64_t(u->mat->M.bytes() + u->mat->R.bytes() + u->mat->X.bytes());
   return nb + int64_t(op->LAm.bytes() + op->LPm.bytes() + op->loc.bytes() + op->LAm_lo.bytes() + op->LPm_lo.bytes() +
-                 op->loc_lo.bytes() + op->ix_val.bytes() + op->V.bytes() +
+                 op->loc_lo.bytes() + op->ix_val.bytes() + op->ix32.bytes() + op->V.bytes() +
                  op->pc.sinv.bytes() + op->pc.sinv32.bytes() + op->pc.lam.bytes() + op->pc.pdiag.bytes());
 }
 
@@ -238,6 +239,8 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
   make_plans(op, sizeof(C), sizeof(C), op->jobs1, op->rs1, op->tl1, op->plan1, op->jobs2, op->rs2, op->tl2, op->plan2,
              c64 ? &op->tc1 : nullptr, c64 ? &op->tc2 : nullptr);
   if (c64) {
+    op->ix32.alloc(op->ix_val.n);
+    split_pairs(op->ix_val.p, int64_t(op->ix_val.n), op->ix32.p, s);
     // where the tensor cores start to beat passes of 8 on the CUDA cores, measured
     // on this operator's own blocks (finite inputs: the work vectors zeroed)
     for (DBuf<char>* w : {&op->wj, &op->we, &op->wa, &op->wbc, &op->wbu, &op->wz1, &op->wz2, &op->ww1, &op->ww2, &op->ww3})
@@ -283,7 +286,7 @@ template <class CM, class CV, class CY>
 static void apply_rest(sldm_op* op, const GemvPlan& p2, double s3, const VecBatch<double2, CY>& y, int nr, cudaStream_t s,
                        double2* const* zh = nullptr, int nzh = 0, double* nrm = nullptr) {
   gemv_jobs_mixed<CM, CV>(p2, nr, s);
-  apply_combine<CV, CY>(op->mesh, dims_of(op), op->k0, op->ix_val.p, op->wz1.p, op->wz2.p, op->ww1.p, op->ww2.p, op->ww3.p,
+  apply_combine<CV, CY>(op->mesh, dims_of(op), op->k0, op->ix_val.p, op->ix32.p, op->wz1.p, op->wz2.p, op->ww1.p, op->ww2.p, op->ww3.p,
                         op->we.p, op->wa.p, op->wbc.p, s3, y, nr, s, zh, nzh, nrm);
 }
 

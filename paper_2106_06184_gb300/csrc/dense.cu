@@ -17,6 +17,7 @@
 #include "dense.h"
 #include "gemm_tc.h"
 #include "gemm_x2.h"
+#include "pair32.cuh"
 #include "widen.cuh"
 
 namespace sldm {
@@ -1188,7 +1189,9 @@ __global__ void __launch_bounds__(256) apply_in_kernel(VecBatch<CX, double2> xb,
 // object's last entry), the third block scaled by s3, into the columns yb.y.  A
 // thread takes one row for up to CR right-hand sides, which share its sparse entries: 4
 // where the rows fill the device (32 columns of N = 34,524: 102 -> 63 us), one where it is
-// the chain of loads that counts (N = 1,279, 12 columns: 19 us with 4, 6 with 1).
+// the chain of loads that counts (N = 1,279, 12 columns: 19 us with 4, 9 with 1).  In
+// complex64 the sums are pairs of FP32 numbers (pair32.cuh), which carry 48 bits of terms that have 24: in
+// FP64 its pipe was the bound (63 -> 31 us; 8 x 8, 32 columns of complex128 results: 95 -> 48).
 // With zh: the step's Gram-Schmidt accumulators are cleared too (nzh complex entries of
 // zh[r] and nrm[r], per column).
 struct CombineClear {
@@ -1201,8 +1204,8 @@ __global__ void __launch_bounds__(128) combine_kernel(const ApplyDims D, double 
                                                       const int32_t* __restrict__ tminus, const int32_t* __restrict__ tri_edge,
                                                       const int8_t* __restrict__ tri_sign, const int32_t* __restrict__ q2t,
                                                       const int32_t* __restrict__ ix_ptr, const int32_t* __restrict__ ix_col,
-                                                      const double* __restrict__ ix_val, const C* __restrict__ z1,
-                                                      const C* __restrict__ z2, const C* __restrict__ w1, const C* __restrict__ w2,
+                                                      const double* __restrict__ ix_val, const float2* __restrict__ ix32,
+                                                      float4 kf, const C* __restrict__ z1, const C* __restrict__ z2, const C* __restrict__ w1, const C* __restrict__ w2,
                                                       const C* __restrict__ w3, const C* __restrict__ e, const C* __restrict__ a,
                                                       const C* __restrict__ bc, double s3, VecBatch<double2, CY> yb, int nrhs,
                                                       CombineClear clr) {
@@ -1215,6 +1218,71 @@ __global__ void __launch_bounds__(128) combine_kernel(const ApplyDims D, double 
       if (i == 0) clr.nrm[r] = 0.0;
     }
   if (i >= 2 * ne + nq) return;
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    P32 vr[CR], vi[CR];
+    if (i < ne) {
+      const int m = i, tp = tplus[m], tm = tminus[m];
+#pragma unroll
+      for (int q = 0; q < CR; ++q)
+        if (r0 + q < nrhs) {
+          const int64_t r = r0 + q;
+          const C v = z1[r * ne + m], p = z2[r * nt + tp], g = z2[r * nt + tm];
+          vr[q].add(v.x), vr[q].add(p.x), vr[q].add(-g.x);
+          vi[q].add(v.y), vi[q].add(p.y), vi[q].add(-g.y);
+        }
+      const int z1e = ix_ptr[m + 1];
+#pragma unroll 4
+      for (int z = ix_ptr[m]; z < z1e; ++z) {
+        const int col = ix_col[z];
+        const float2 x = ix32[z];
+#pragma unroll
+        for (int q = 0; q < CR; ++q)
+          if (r0 + q < nrhs) {
+            const C ev = e[int64_t(r0 + q) * ne + col];
+            vr[q].fma(x.x, x.y, ev.x);
+            vi[q].fma(x.x, x.y, ev.y);
+          }
+      }
+    } else if (i < 2 * ne) {
+      const int m = i - ne, tp = tplus[m], tm = tminus[m];
+#pragma unroll
+      for (int q = 0; q < CR; ++q)
+        if (r0 + q < nrhs) {
+          const int64_t r = r0 + q;
+          const C v = w1[r * ne + m], b = w2[r * ne + m], p = w3[r * nt + tp], g = w3[r * nt + tm];
+          vr[q].add(v.x), vr[q].add(-b.x), vr[q].add(p.x), vr[q].add(-g.x);
+          vi[q].add(v.y), vi[q].add(-b.y), vi[q].add(p.y), vi[q].add(-g.y);
+        }
+    } else {
+      const int t = q2t[i - 2 * ne];
+#pragma unroll
+      for (int q = 0; q < CR; ++q)
+        if (r0 + q < nrhs) {
+          const int64_t r = r0 + q;
+          P32 sr, si;
+          for (int k = 0; k < 3; ++k) {
+            const C av = a[r * ne + tri_edge[3 * t + k]];
+            const bool neg = tri_sign[3 * t + k] < 0;
+            sr.add(neg ? -av.x : av.x);
+            si.add(neg ? -av.y : av.y);
+          }
+          const C cv = bc[r * nt + t];
+          sr.fma(kf.x, kf.y, cv.x);
+          si.fma(kf.x, kf.y, cv.y);
+          vr[q] = sr.scaled(kf.z, kf.w);
+          vi[q] = si.scaled(kf.z, kf.w);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < CR; ++q)
+      if (r0 + q < nrhs) {
+        CY o;
+        vr[q].get(o.x);
+        vi[q].get(o.y);
+        yb.y[r0 + q][i] = o;
+      }
+    return;
+  }
   double vr[CR], vi[CR];
   if (i < ne) {
     const int m = i, tp = tplus[m], tm = tminus[m];
@@ -1293,7 +1361,7 @@ template void apply_in<float2, float2>(const sldm_mesh*, const VecBatch<float2, 
                                        const ApplyDims&, void*, void*, void*, void*, void*, int, cudaStream_t);
 
 template <class C, class CY>
-void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1, const void* z2,
+void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const float2* ix32, const void* z1, const void* z2,
                    const void* w1, const void* w2, const void* w3, const void* e, const void* a, const void* bc, double s3,
                    const VecBatch<double2, CY>& y, int nrhs, cudaStream_t s, double2* const* zh, int nzh, double* nrm) {
   const DevMesh& d = m->d;
@@ -1304,10 +1372,17 @@ void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const doub
     clr.n = nzh;
   }
   const int rows = std::max(2 * D.ne + D.nq, clr.n);
+  auto hl = [](double v, float& h, float& l) {
+    h = float(v);
+    l = float(v - double(h));
+  };
+  float4 kf;  // k0^2 and s3 as pairs
+  hl(k0 * k0, kf.x, kf.y);
+  hl(s3, kf.z, kf.w);
   auto go = [&](auto cr) {
     constexpr int CR = decltype(cr)::value;
     combine_kernel<C, CY, CR><<<dim3(unsigned((rows + 127) / 128), unsigned((nrhs + CR - 1) / CR)), 128, 0, s>>>(
-        D, k0, d.tplus.p, d.tminus.p, d.tri_edge.p, d.tri_sign.p, d.q2t.p, d.ix_ptr.p, d.ix_col.p, ix_val, (const C*)z1,
+        D, k0, d.tplus.p, d.tminus.p, d.tri_edge.p, d.tri_sign.p, d.q2t.p, d.ix_ptr.p, d.ix_col.p, ix_val, ix32, kf, (const C*)z1,
         (const C*)z2, (const C*)w1, (const C*)w2, (const C*)w3, (const C*)e, (const C*)a, (const C*)bc, s3, y, nrhs, clr),
         ::sldm::count_launch();
   };
@@ -1316,7 +1391,7 @@ void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const doub
   SLDM_CUDA(cudaGetLastError());
 }
 #define SLDM_COMBINE_INST(C, CY)                                                                                               \
-  template void apply_combine<C, CY>(const sldm_mesh*, const ApplyDims&, double, const double*, const void*, const void*,     \
+  template void apply_combine<C, CY>(const sldm_mesh*, const ApplyDims&, double, const double*, const float2*, const void*, const void*,     \
                                      const void*, const void*, const void*, const void*, const void*, const void*, double,    \
                                      const VecBatch<double2, CY>&, int, cudaStream_t, double2* const*, int, double*);
 SLDM_COMBINE_INST(double2, double2)
@@ -1423,7 +1498,7 @@ __global__ void __launch_bounds__(256) krylov_dots_kernel(KrylovStep ks) {
 // with eight column loads in flight and no exchange between warps.  The
 // coefficients are staged in shared memory in the arithmetic's precision: converting
 // them per lane (two per column, on the narrow FP64 pipe) cost as much as the HBM
-// read (N = 34,524, 32 right-hand sides, k ~ 90: 150 us per pass).
+// read (N = 34,524, 32 right-hand sides, k = 55 on average: 150 -> 106 us per pass).
 template <class CB>
 __global__ void __launch_bounds__(256) krylov_update_kernel(KrylovStep ks, int norm) {
   typedef typename CT<CB>::R R;
@@ -1509,6 +1584,17 @@ __global__ void sub_c64_kernel(const float2* __restrict__ a, const float2* __res
 void sub_c64(const float2* a, const float2* b, int64_t n, double2* dst, cudaStream_t s) {
   if (n <= 0) return;
   sub_c64_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(a, b, n, dst), ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+__global__ void split_pairs_kernel(const double* __restrict__ src, int64_t n, float2* dst) {
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const float h = __double2float_rn(src[t]);
+  dst[t] = make_float2(h, __double2float_rn(src[t] - double(h)));
+}
+void split_pairs(const double* src, int64_t n, float2* dst, cudaStream_t s) {
+  if (n <= 0) return;
+  split_pairs_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(src, n, dst), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
 // FP64 operator kept as a complex64 pair: hi = fl32(v), lo = fl32(v - hi)

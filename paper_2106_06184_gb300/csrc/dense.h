@@ -116,7 +116,7 @@ void apply_in(const sldm_mesh* m, const VecBatch<CX, double2>& x, double s1, dou
 // the product's rows from its work vectors into the columns y (third block scaled by
 // s3); with zh, also clears nzh coefficients of every zh[r] and nrm[r]
 template <class C, class CY>
-void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const void* z1, const void* z2,
+void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const double* ix_val, const float2* ix32, const void* z1, const void* z2,
                    const void* w1, const void* w2, const void* w3, const void* e, const void* a, const void* bc, double s3,
                    const VecBatch<double2, CY>& y, int nrhs, cudaStream_t s, double2* const* zh = nullptr, int nzh = 0,
                    double* nrm = nullptr);
@@ -142,6 +142,8 @@ template <class C>
 void to_c128(const void* src, int64_t n, double2* dst, cudaStream_t s);
 // dst = a - b, the difference in FP32
 void sub_c64(const float2* a, const float2* b, int64_t n, double2* dst, cudaStream_t s);
+// dst = (fl32(src), fl32(src - fl32(src)))
+void split_pairs(const double* src, int64_t n, float2* dst, cudaStream_t s);
 // hi = complex64 rounding of src, lo = complex64 rounding of src - hi (src = hi + lo to ~2^-48)
 void split_c128(const double2* src, int64_t n, float2* hi, float2* lo, cudaStream_t s);
 // dst += lo (complex64 low parts onto a complex128 copy of the high parts)

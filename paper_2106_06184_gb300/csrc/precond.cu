@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "dense.h"
+#include "pair32.cuh"
 #include "precond.h"
 #include "widen.cuh"
 
@@ -112,15 +113,35 @@ __device__ __forceinline__ float2 to_cv<float2>(double2 v) { return make_float2(
 template <class CX>
 __device__ __forceinline__ double2 wide2(const CX v) { return make_double2(widen(v.x), widen(v.y)); }
 
-// t3 = s3 r3 - F D (L11 r1 + L12 r2) (per charge unknown; column blockIdx.y)
+// t3 = s3 r3 - F D (L11 r1 + L12 r2) (per charge unknown; column blockIdx.y).  Complex64 columns in
+// pairs of FP32 (pair32.cuh), the coefficients held as pairs; in FP64 this kernel and the next were bound by its pipe
+// (N = 34,524, 32 columns: 26 -> 8 us and 39 -> 9 us).
 template <class CX, class CV>
 __global__ void prec_apply1_kernel(int ne, int nq, const int32_t* __restrict__ q2t, const int32_t* __restrict__ tri_edge,
-                                   const int8_t* __restrict__ tri_sign, const double2* __restrict__ lam, VecBatch<CX, double2> rb,
-                                   double s3, CV* t3) {
+                                   const int8_t* __restrict__ tri_sign, const double2* __restrict__ lam,
+                                   const float4* __restrict__ lam32, VecBatch<CX, double2> rb, double s3, float2 s3f, CV* t3) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nq) return;
   const CX* __restrict__ r = rb.x[blockIdx.y];
   const int t = q2t[q];
+  if constexpr (sizeof(CX) == sizeof(float2)) {  // in pairs of FP32
+    P32 re, im;
+    const CX r3 = r[2 * ne + q];
+    re.fma(s3f.x, s3f.y, r3.x);
+    im.fma(s3f.x, s3f.y, r3.y);
+    for (int i = 0; i < 3; ++i) {
+      const int e = tri_edge[3 * t + i];
+      const float sg = tri_sign[3 * t + i] < 0 ? 1.f : -1.f;
+      const CX u = r[e], v = r[ne + e];
+      cfma_pair(re, im, lam32[4 * e], sg * u.x, sg * u.y);
+      cfma_pair(re, im, lam32[4 * e + 1], sg * v.x, sg * v.y);
+    }
+    CV o;
+    re.get(o.x);
+    im.get(o.y);
+    t3[int64_t(blockIdx.y) * nq + q] = o;
+    return;
+  }
   double2 acc = wide2(r[2 * ne + q]);
   acc.x *= s3;
   acc.y *= s3;
@@ -143,12 +164,42 @@ template <class CX, class CV, bool WORK>
 __global__ void __launch_bounds__(128) prec_apply45_kernel(int ne, int nq, int nt, const int32_t* __restrict__ tplus,
                                                            const int32_t* __restrict__ tminus, const int32_t* __restrict__ q2t,
                                                            const double2* __restrict__ lam, const double2* __restrict__ pdiag,
+                                                           const float4* __restrict__ lam32, const float4* __restrict__ pdiag32,
                                                            VecBatch<CX, double2> rb, const CV* __restrict__ bx, PrecWork W) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t c = blockIdx.y;
   const CX* __restrict__ r = rb.x[c];
   bx += c * nt;
-  if (i < ne) {
+  if constexpr (WORK && sizeof(CX) == sizeof(float2)) {  // in pairs of FP32
+    if (i < ne) {
+      const int tp = tplus[i], tm = tminus[i];
+      const CV bp = bx[tp], bm = bx[tm];
+      P32 yr[2], yi[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const CX rk = r[k * ne + i];
+        yr[k].add(rk.x);
+        yi[k].add(rk.y);
+        cfma_pair(yr[k], yi[k], pdiag32[2 * tp + k], -bp.x, -bp.y);
+        cfma_pair(yr[k], yi[k], pdiag32[2 * tm + k], bm.x, bm.y);
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        P32 xr, xi;
+        cfma_pair(xr, xi, lam32[4 * i + 2 * k], yr[0], yi[0]);
+        cfma_pair(xr, xi, lam32[4 * i + 2 * k + 1], yr[1], yi[1]);
+        CV v;
+        xr.get(v.x);
+        xi.get(v.y);
+        if (k == 0) {
+          reinterpret_cast<CV*>(W.j)[c * ne + i] = v;
+          reinterpret_cast<CV*>(W.a)[c * ne + i] = v;
+        } else {
+          reinterpret_cast<CV*>(W.e)[c * ne + i] = v;
+        }
+      }
+    }
+  } else if (i < ne) {
     const int tp = tplus[i], tm = tminus[i];
     const double2 bp = wide2(bx[tp]), bm = wide2(bx[tm]);
     const double2 y1 = c_sub(wide2(r[i]), c_sub(c_mul(pdiag[2 * tp], bp), c_mul(pdiag[2 * tm], bm)));
@@ -178,6 +229,12 @@ __global__ void __launch_bounds__(128) prec_apply45_kernel(int ne, int nq, int n
   }
 }
 
+__global__ void split_c_kernel(int64_t n, const double2* __restrict__ a, float4* b) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float x = float(a[i].x), y = float(a[i].y);
+  b[i] = make_float4(x, y, float(a[i].x - double(x)), float(a[i].y - double(y)));
+}
 __global__ void to_c64_kernel(int64_t n, const double2* __restrict__ a, float2* b) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     b[i] = make_float2(float(a[i].x), float(a[i].y));
@@ -386,6 +443,12 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   // a complex64 operator takes an FP32 preconditioner: S^-1 (inverted in FP64)
   // rounded to complex64, applied with FP32 arithmetic
   P.f32 = sizeof(C) == sizeof(float2);
+  if (P.f32) {
+    P.lam32.alloc(size_t(4) * ne);
+    P.pdiag32.alloc(size_t(2) * nt);
+    split_c_kernel<<<(4 * ne + 255) / 256, 256, 0, s>>>(4 * ne, P.lam.p, P.lam32.p), ::sldm::count_launch();
+    split_c_kernel<<<(2 * nt + 255) / 256, 256, 0, s>>>(2 * nt, P.pdiag.p, P.pdiag32.p), ::sldm::count_launch();
+  }
   if (P.f32 && tot > 0) {
     P.sinv32.alloc(tot);
     to_c64_kernel<<<std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, s>>>(tot, P.sinv.p, P.sinv32.p), ::sldm::count_launch();
@@ -441,8 +504,9 @@ static void prec_charges(const Precond& P, const sldm_mesh* m, const VecBatch<CX
   SLDM_REQUIRE((nr >= 1 && nr <= MAX_NRHS), SLDM_EINVAL, "preconditioner: 1 to 32 columns");
   const DevMesh& d = m->d;
   const int ne = int(m->h.ne), nq = int(P.nq);
-  prec_apply1_kernel<CX, CV><<<dim3((nq + 127) / 128, nr), 128, 0, s>>>(ne, nq, d.q2t.p, d.tri_edge.p, d.tri_sign.p, P.lam.p, r,
-                                                                      s3, reinterpret_cast<CV*>(P.t3.p)), ::sldm::count_launch();
+  prec_apply1_kernel<CX, CV><<<dim3((nq + 127) / 128, nr), 128, 0, s>>>(ne, nq, d.q2t.p, d.tri_edge.p, d.tri_sign.p, P.lam.p,
+                                                                      P.lam32.p, r, s3, make_float2(float(s3), float(s3 - double(float(s3)))),
+                                                                      reinterpret_cast<CV*>(P.t3.p)), ::sldm::count_launch();
   gemv_jobs<CV>(P.plan, nr, s);
 }
 
@@ -454,7 +518,7 @@ void prec_apply_in(const Precond& P, const sldm_mesh* m, const VecBatch<CX, doub
   const int ne = int(m->h.ne), nq = int(P.nq), nt = int(m->h.nt);
   prec_charges<CX, C>(P, m, r, s3, nr, s);
   prec_apply45_kernel<CX, C, true><<<dim3((std::max(ne, nt) + 127) / 128, nr), 128, 0, s>>>(
-      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, r, reinterpret_cast<const C*>(P.bx.p),
+      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, P.lam32.p, P.pdiag32.p, r, reinterpret_cast<const C*>(P.bx.p),
       PrecWork{j, a, e, bu, bc}), ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }
@@ -470,7 +534,7 @@ static void prec_add_t(const Precond& P, const sldm_mesh* m, const VecBatch<doub
   const int ne = int(m->h.ne), nq = int(P.nq), nt = int(m->h.nt);
   prec_charges<double2, CV>(P, m, r, s3, nr, s);
   prec_apply45_kernel<double2, CV, false><<<dim3((std::max(ne, nt) + 127) / 128, nr), 128, 0, s>>>(
-      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, r, reinterpret_cast<const CV*>(P.bx.p), PrecWork{}),
+      ne, nq, nt, d.tplus.p, d.tminus.p, d.q2t.p, P.lam.p, P.pdiag.p, P.lam32.p, P.pdiag32.p, r, reinterpret_cast<const CV*>(P.bx.p), PrecWork{}),
       ::sldm::count_launch();
   SLDM_CUDA(cudaGetLastError());
 }

@@ -15,6 +15,7 @@ struct PrecObj {
 struct Precond {
   DBuf<PrecObj> objs;
   DBuf<double2> lam;    // 4 per edge: Lambda11, Lambda12, Lambda21, Lambda22
+  DBuf<float4> lam32, pdiag32;  // complex64 operators: both as pairs (hi.x, hi.y, lo.x, lo.y)
   DBuf<double2> pdiag;  // 2 per triangle: diag L^phi_m, diag of the object's L^phi/eps
   // per object nt_o x (nt_o - 1): B_o S_o^-1 = [S_o^-1; minus its column sums], row-major, so
   // that the product gives the full charges B x3 (complex128 operators)
