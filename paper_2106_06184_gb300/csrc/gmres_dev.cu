@@ -505,8 +505,11 @@ void gmres_cycle_start(int64_t n, const CycleStart& a, int nr, cudaStream_t s) {
 }
 
 // The one-launch step where its cluster's work is less than what the launches of the
-// separate kernels cost: four passes over N (k + 1) entries per right-hand side.
-constexpr double GS_MAX_C128 = 1.0e5, GS_MAX_C64 = 4.0e5;
+// separate kernels cost: four passes over N (k + 1) entries per right-hand side.  Separate kernels
+// against the cluster, us per step over a whole solve: complex128, N = 319 (28 steps) 41 / 25, 1,279 (40) 68 / 31, 5,119
+// (54 steps, up to 2.8e5) 89 / 63; complex64, N = 1,279, 12 columns (51 steps) 38 / 21, 5,119 (69 steps, up to
+// 3.5e5) 51 / 31, 8,631, 32 columns (up to 5e5 and more) 83 / 87.
+constexpr double GS_MAX_C128 = 3.0e5, GS_MAX_C64 = 4.0e5;
 
 template <class CB>
 void gmres_orthogonalise(const GivensArgs& a, KrylovStep ks, double2* const* h1, double2* const* h2, cudaStream_t s) {
