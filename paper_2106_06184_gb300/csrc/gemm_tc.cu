@@ -590,25 +590,26 @@ __global__ void __launch_bounds__(256) tc_bprime_kernel(const GemvJob* __restric
 }
 
 // Scale exponents of A: one per row and stage (128 FP32 columns = 512 bytes of the row),
-// one warp each; aexp[stage][row] per job, rows padded to whole tiles.
-__global__ void __launch_bounds__(256) tc_aexp_kernel(const GemvJob* __restrict__ jobs, const TcJob* __restrict__ tj, int job,
+// one warp each; aexp[stage][row] per job (blockIdx.y), rows padded to whole tiles.
+__global__ void __launch_bounds__(256) tc_aexp_kernel(const GemvJob* __restrict__ jobs, const TcJob* __restrict__ tj, int job0,
                                                       signed char* __restrict__ aexp) {
-  const GemvJob& J = jobs[job];
-  const TcJob T = tj[job];
-  const int64_t w = (int64_t(blockIdx.x) * 256 + threadIdx.x) >> 5;
+  const GemvJob& J = jobs[job0 + blockIdx.y];
+  const TcJob T = tj[job0 + blockIdx.y];
   const int lane = threadIdx.x & 31, nst = (2 * J.n + TC_KC * TC_BPS - 1) / (TC_KC * TC_BPS);
-  const int64_t row = w / nst;
-  const int st = int(w % nst);
-  if (row >= J.m) return;
-  const float2* a = reinterpret_cast<const float2*>(J.A) + row * J.lda;
-  float m = 0.f;
-  for (int c = st * (TC_KC * TC_BPS / 2) + lane, i = 0; i < 2; ++i, c += 32)
-    if (c < J.n) {
-      const float2 v = a[c];
-      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
-    }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) aexp[T.aexp + int64_t(st) * T.mpad + row] = static_cast<signed char>(tc_scale_exp(m));
+  const int64_t total = int64_t(J.m) * nst;
+  for (int64_t w = (int64_t(blockIdx.x) * 256 + threadIdx.x) >> 5; w < total; w += int64_t(gridDim.x) * 8) {
+    const int64_t row = w / nst;
+    const int st = int(w % nst);
+    const float2* a = reinterpret_cast<const float2*>(J.A) + row * J.lda;
+    float m = 0.f;
+    for (int c = st * (TC_KC * TC_BPS / 2) + lane, i = 0; i < 2; ++i, c += 32)
+      if (c < J.n) {
+        const float2 v = a[c];
+        m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+      }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) aexp[T.aexp + int64_t(st) * T.mpad + row] = static_cast<signed char>(tc_scale_exp(m));
+  }
 }
 
 // B' of every sub-chunk of the pass (hi rows 0-63, lo rows 64-127, 32 FP32 columns
@@ -787,10 +788,10 @@ void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, bool f16, cudaS
   {
     DBuf<GemvJob> dj;
     dj.upload(jobs, s);
-    for (size_t i = 0; i < jobs.size(); ++i) {
-      const int64_t warps = int64_t(jobs[i].m) * ((2 * jobs[i].n + TC_KC * TC_BPS - 1) / (TC_KC * TC_BPS));
-      tc_aexp_kernel<<<unsigned((warps * 32 + 255) / 256), 256, 0, s>>>(dj.p, tp.tj.p, int(i), tp.aexp.p), count_launch();
-    }
+    for (size_t i = 0; i < jobs.size(); i += 65535)  // two waves of CTAs per job: small jobs leave most of theirs idle
+      tc_aexp_kernel<<<dim3(152 * 16, unsigned(std::min<size_t>(65535, jobs.size() - i))), 256, 0, s>>>(dj.p, tp.tj.p, int(i),
+                                                                                                  tp.aexp.p),
+          count_launch();
     SLDM_CUDA(cudaGetLastError());
     SLDM_CUDA(cudaStreamSynchronize(s));
   }
