@@ -87,6 +87,7 @@ struct DBuf {
     budget_take(count * sizeof(T));
     cudaError_t e = cudaMalloc(&p, count * sizeof(T));
     if (e != cudaSuccess) {
+      cudaGetLastError();  // the runtime keeps it: a caller that goes on without this buffer would meet it at its next launch
       p = nullptr;
       budget_give(count * sizeof(T));
       throw Error{SLDM_ENOMEM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed"};
