@@ -246,7 +246,11 @@ int sldm_op_table(const sldm_op* op, int32_t which, void* dst, int64_t* dims, do
  * complex128 with leading dimension N.  Z is applied in its structured form:
  * global L^A_m, L^phi_m products plus per-object blocks, never a dense Z.
  * SLDM_PREC_F32 operators multiply in FP32; SLDM_PREC_F32X2 operators apply
- * hi + lo with ~48-bit compensated sums (the FP64 operator). */
+ * hi + lo with ~48-bit compensated sums (the FP64 operator).
+ * Complex64 blocks with several right-hand sides go to the tensor cores, whose waits are
+ * bounded.  One that runs out is reported as SLDM_ETIMEOUT by the call whose product it was where
+ * that call waits for its result (host memory, sldm_solve, sldm_farfield); with device memory
+ * this call only queues its product, and the next of those calls on the operator reports it. */
 int sldm_apply(const sldm_op* op, const void* x, void* y, int32_t nrhs, int32_t where, void* stream);
 
 /* Right-hand sides for plane waves (Eq. finalsystem right-hand side):
@@ -442,8 +446,12 @@ int sldm_device_bytes(int64_t* in_use);
  * CTA records the failure, every other CTA leaves at its next wait, and the call
  * that launched the solver (sldm_assemble) returns SLDM_ETIMEOUT.  No fault is
  * raised and the CUDA context stays usable.  count = 0 clears the injection.
+ * SLDM_INJECT_TC_WAIT: the next `count` tensor-core products record, once they have run, the
+ * flag that a product whose bounded wait ran out leaves; the call that reads it returns
+ * SLDM_ETIMEOUT (see sldm_apply).
  * SLDM_EINVAL for an unknown `what` or a negative count. */
 #define SLDM_INJECT_LU_STALL 1
+#define SLDM_INJECT_TC_WAIT 2
 int sldm_test_inject(int32_t what, int32_t count);
 
 /* ---------------------------------------------------------------------------

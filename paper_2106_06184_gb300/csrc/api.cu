@@ -43,7 +43,7 @@ struct ObjInfo {
 struct HostBack {
   double norm[MAX_NRHS];
   GmresState st[MAX_NRHS];
-  int err[3];
+  int err[4];  // TC_PLANS
 };
 struct PollRing {
   static constexpr int SLOTS = 2;  // the host runs at most one step ahead of what it knows
@@ -265,6 +265,21 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
     for (auto& u : op->nested)
       nested_plans(*u, reinterpret_cast<const double2*>(op->we.p), ne, op->wnt.p, op->wny.p, op->wnr.p, op->ldn);
   }
+}
+
+// The flags that a tensor-core pass sets when a bounded wait ran out, of every plan of the operator's
+// products: queued behind them on s (host: room for TC_PLANS flags), and, once s has been
+// waited for, turned into SLDM_ETIMEOUT and cleared, all of them.
+constexpr int TC_PLANS = 4;
+static void tc_flags_async(const sldm_op* op, int* host, cudaStream_t s) {
+  const TcPlan* tcs[TC_PLANS] = {&op->tc1, &op->tc2, &op->pc.tc, &op->tcf};
+  for (int i = 0; i < TC_PLANS; ++i) tc_err_async(*tcs[i], &host[i], s);
+}
+static void tc_flags_check(const sldm_op* op, const int* host, cudaStream_t s) {
+  const TcPlan* tcs[TC_PLANS] = {&op->tc1, &op->tc2, &op->pc.tc, &op->tcf};
+  bool lost = false;
+  for (int i = 0; i < TC_PLANS; ++i) lost |= tc_err_clear(*tcs[i], host[i], s);
+  SLDM_REQUIRE(!lost, SLDM_ETIMEOUT, "tensor-core product: a bounded wait ran out");
 }
 
 static ApplyDims dims_of(const sldm_op* op) {
@@ -850,11 +865,9 @@ static void gmres_block(sldm_op* op, bool use_p, bool refine, bool x_zero, int m
   const ApplyDims D = dims_of(op);
   auto read_norms = [&](std::vector<double>& out) {
     SLDM_CUDA(cudaMemcpyAsync(back.norm, op->dnorm.p, nr * sizeof(double), cudaMemcpyDeviceToHost, s));
-    const TcPlan* tcs[3] = {&op->tc1, &op->tc2, &op->pc.tc};
-    for (int i = 0; i < 3; ++i) tc_err_async(*tcs[i], &back.err[i], s);
+    tc_flags_async(op, back.err, s);
     SLDM_CUDA(cudaStreamSynchronize(s));
-    // a tensor-core pass whose bounded wait ran out: SLDM_ETIMEOUT
-    for (int i = 0; i < 3; ++i) tc_err_check(*tcs[i], back.err[i], s);
+    tc_flags_check(op, back.err, s);
     for (int r = 0; r < nr; ++r) out[r] = std::sqrt(back.norm[r]);
   };
   SLDM_CUDA(cudaMemsetAsync(op->dnorm.p, 0, op->dnorm.bytes(), s));
@@ -1381,7 +1394,10 @@ int sldm_apply(const sldm_op* op, const void* x, void* y, int32_t nrhs, int32_t 
     SLDM_CUDA(cudaMemcpyAsync(dx.p, x, bytes, cudaMemcpyHostToDevice, s));
     apply_any(op, dx.p, dy.p, nrhs, s, op->x2);
     SLDM_CUDA(cudaMemcpyAsync(y, dy.p, bytes, cudaMemcpyDeviceToHost, s));
+    int err[TC_PLANS];
+    tc_flags_async(op, err, s);
     SLDM_CUDA(cudaStreamSynchronize(s));
+    tc_flags_check(op, err, s);
   }
   API_END
 }
@@ -1595,7 +1611,10 @@ int sldm_farfield_n(const sldm_op* op_, const void* x, int32_t nrhs, int32_t whe
     farfield(op->mesh, op->k0, jd, op->ne, nrhs, upload(ang), n, dx, chunk, dr, s);
   }
   SLDM_CUDA(cudaMemcpyAsync(rcs, dr, size_t(n) * nrhs * sizeof(double), cudaMemcpyDeviceToHost, s));
+  int err[TC_PLANS];
+  tc_flags_async(op, err, s);
   SLDM_CUDA(cudaStreamSynchronize(s));
+  tc_flags_check(op, err, s);
   API_END
 }
 

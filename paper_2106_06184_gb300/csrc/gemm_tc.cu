@@ -836,16 +836,18 @@ void gemm_tc(const GemvPlan& plan, const TcPlan& tp, int nrhs, cudaStream_t s) {
     go(std::false_type{});
   }
   SLDM_CUDA(cudaGetLastError());
+  tp.ran = true;
+  if (take_tc_wait()) SLDM_CUDA(cudaMemsetAsync(tp.err.p, 1, sizeof(int), s));
 }
 
 void tc_err_async(const TcPlan& tp, int* host, cudaStream_t s) {
   *host = 0;
-  if (tp.ok) SLDM_CUDA(cudaMemcpyAsync(host, tp.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+  if (tp.ran) SLDM_CUDA(cudaMemcpyAsync(host, tp.err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+  tp.ran = false;
 }
-void tc_err_check(const TcPlan& tp, int err, cudaStream_t s) {
-  if (!err) return;
-  SLDM_CUDA(cudaMemsetAsync(tp.err.p, 0, sizeof(int), s));
-  throw Error{SLDM_ETIMEOUT, "tensor-core product: a bounded wait ran out"};
+bool tc_err_clear(const TcPlan& tp, int err, cudaStream_t s) {
+  if (err) SLDM_CUDA(cudaMemsetAsync(tp.err.p, 0, sizeof(int), s));
+  return err != 0;
 }
 
 }  // namespace sldm

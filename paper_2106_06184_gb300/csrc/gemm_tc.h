@@ -29,6 +29,7 @@ struct TcPlan {
   DBuf<TcTile> tiles;
   DBuf<int32_t> cta_begin;   // CTA c takes tiles [cta_begin[c], cta_begin[c + 1])
   DBuf<int> err;             // set to 1 by a CTA whose bounded wait ran out
+  mutable bool ran = false;  // passes launched since err was last read
   // B' of the pass (built from the vectors before each pass): stage g of the plan is
   // (job gjob[g], its stage gst[g]); boxes of 128 rows (hi, lo) x 128 bytes, two per stage in FP16,
   // four in TF32, read by TMA through bmap, and (FP16) the factor that undoes each right-hand side's scale
@@ -63,9 +64,9 @@ bool tc_block_map(const void* A, int64_t lda, int m, int n, unsigned char* out);
 // One pass over every job of `plan` for nrhs (<= 32) right-hand sides.
 void gemm_tc(const GemvPlan& plan, const TcPlan& tp, int nrhs, cudaStream_t s);
 // Queue a copy of the flag that a tensor-core pass sets when a bounded wait ran out
-// into *host (pinned); once the stream has been waited for, tc_err_check turns a set
-// flag into SLDM_ETIMEOUT and clears it.
+// into *host (0 at once where none was launched since the last reading); once the stream has been waited for, tc_err_clear says whether it was set
+// and clears it.
 void tc_err_async(const TcPlan& tp, int* host, cudaStream_t s);
-void tc_err_check(const TcPlan& tp, int err, cudaStream_t s);
+bool tc_err_clear(const TcPlan& tp, int err, cudaStream_t s);
 
 }  // namespace sldm

@@ -537,6 +537,8 @@ void gemm_x2(const GemvPlan& plan, const X2Plan& xp, int nrhs, int col0, cudaStr
                                                                xp.bmap.p, tc.tj.p, tc.aexp.p, xp.bscale.p, nrhs, col0, tc.err.p),
       count_launch();
   SLDM_CUDA(cudaGetLastError());
+  tc.ran = true;
+  if (take_tc_wait()) SLDM_CUDA(cudaMemsetAsync(tc.err.p, 1, sizeof(int), s));
 }
 
 }  // namespace sldm

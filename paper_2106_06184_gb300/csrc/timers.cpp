@@ -34,6 +34,13 @@ bool take_lu_stall() {
     if (g_lu_stall.compare_exchange_weak(v, v - 1)) return true;
   return false;
 }
+static std::atomic<int> g_tc_wait{0};
+bool take_tc_wait() {
+  int v = g_tc_wait.load();
+  while (v > 0)
+    if (g_tc_wait.compare_exchange_weak(v, v - 1)) return true;
+  return false;
+}
 
 namespace {
 struct Pending {
@@ -208,10 +215,10 @@ extern "C" int sldm_device_bytes(int64_t* in_use) {
 }
 
 extern "C" int sldm_test_inject(int32_t what, int32_t count) {
-  if (what != SLDM_INJECT_LU_STALL || count < 0) {
+  if ((what != SLDM_INJECT_LU_STALL && what != SLDM_INJECT_TC_WAIT) || count < 0) {
     sldm::set_error("test_inject: unknown injection or negative count");
     return SLDM_EINVAL;
   }
-  sldm::g_lu_stall.store(count);
+  (what == SLDM_INJECT_LU_STALL ? sldm::g_lu_stall : sldm::g_tc_wait).store(count);
   return SLDM_OK;
 }
