@@ -689,6 +689,18 @@ static void assemble_impl(sldm_op* op, const sldm_material* mats, cudaStream_t s
     auto inner = [&](const ObjInfo& oi) {
       return sizeof(C) == sizeof(double2) && !op->want_x2 && op->nested_min >= 0 && oi.ne + oi.nq >= op->nested_min;
     };
+    // In a stack the repeated blocks are copied once the reflected part is in, but M_l takes each object's
+    // own block as it is now: objects that repeat a shape in a material of their own get theirs here
+    if (op->layered) {
+      std::vector<BlockCopy> ca, cp;
+      for (size_t i = 0; i < gr.copyA.size(); ++i)
+        if (gr.copyA[i].dr == gr.copyA[i].dc && ref[h.obj[gr.copyP[i].dr]] == h.obj[gr.copyP[i].dr]) {
+          ca.push_back(gr.copyA[i]);
+          cp.push_back(gr.copyP[i]);
+        }
+      copy_blocks(ca, es, op->LAm.p, op->ne, s);
+      copy_blocks(cp, es, op->LPm.p, op->nt, s);
+    }
     std::vector<int> cand;
     for (int o = 0; o < op->nobj; ++o) {
       if (ref[o] != o) continue;
