@@ -16,7 +16,7 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libsldm.so")
 SOURCES = ["mesh.cpp", "timers.cpp", "fill.cu", "fill_sub.cu", "dense.cu", "gmres_dev.cu", "gemm_tc.cu", "gemm_x2.cu", "lu_blocked.cu", "precond.cu",
            "mgf.cu", "nested.cu", "ports.cu", "api.cu", "serve.cpp"]
-HEADERS = ["internal.h", "fill_dev.cuh", "widen.cuh", "dense.h", "gemm_tc.h", "gemm_x2.h", "tc_ptx.cuh", "pair32.cuh", "precond.h", "mgf.h", "nested.h", os.path.join("..", "..", "include", "sldm.h")]
+HEADERS = ["internal.h", "fill_dev.cuh", "widen.cuh", "cluster.h", "dense.h", "gemm_tc.h", "gemm_x2.h", "tc_ptx.cuh", "pair32.cuh", "precond.h", "mgf.h", "nested.h", os.path.join("..", "..", "include", "sldm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

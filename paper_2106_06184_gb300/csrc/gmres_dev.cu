@@ -2,8 +2,8 @@
 // Gram-Schmidt step of a small system in one launch, Givens rotations and
 // convergence tests, the cycle's back substitution and update (Sec. IV).
 #include <algorithm>
-#include <atomic>
 
+#include "cluster.h"
 #include "dense.h"
 #include "widen.cuh"
 
@@ -436,34 +436,7 @@ __global__ void __launch_bounds__(256) add_scaled_kernel(int64_t n, int64_t ne, 
 // ---------------------------------------------------------------- choice of the Gram-Schmidt form
 // Cluster size: 8 is portable; complex128 steps, which the FP64 pipes of the
 // cluster's SMs bound, take 16 where the device schedules them.
-template <class CB, int CS>
-bool cluster_fits(int dev, size_t smem) {
-  static std::atomic<uint64_t> yes{0}, no{0};
-  const uint64_t bit = uint64_t(1) << (dev & 63);
-  if (yes.load() & bit) return true;
-  if (no.load() & bit) return false;
-  bool ok = cudaFuncSetAttribute(gs_cluster_kernel<CB, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) == cudaSuccess;
-  if (ok && CS > 8)
-    ok = cudaFuncSetAttribute(gs_cluster_kernel<CB, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-  if (ok) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(CS);
-    cfg.blockDim = dim3(GS_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    ok = cudaOccupancyMaxActiveClusters(&n, gs_cluster_kernel<CB, CS>, &cfg) == cudaSuccess && n > 0;
-  }
-  if (!ok) cudaGetLastError();
-  (ok ? yes : no).fetch_or(bit);
-  return ok;
-}
-
+constexpr size_t GS_SMEM_MAX = 128 * 1024;
 template <class CB, int CS>
 bool launch_cluster(const GivensArgs& a, const KrylovStep& ks, cudaStream_t s) {
   const int rs = int((ks.ldv + CS * 32 - 1) / (CS * 32)) * 32;
@@ -471,19 +444,11 @@ bool launch_cluster(const GivensArgs& a, const KrylovStep& ks, cudaStream_t s) {
   const size_t smem = (3 * K + 1) * sizeof(double2) + (K + (K & 1) + rs + GS_THREADS) * sizeof(CB) + K * sizeof(Rot);
   int dev = 0;
   SLDM_CUDA(cudaGetDevice(&dev));
-  if (smem > 128 * 1024 || !cluster_fits<CB, CS>(dev, smem)) return false;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(unsigned(CS * ks.na));
-  cfg.blockDim = dim3(GS_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CS;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  SLDM_CUDA(cudaLaunchKernelEx(&cfg, gs_cluster_kernel<CB, CS>, a, ks, rs));
+  static ClusterFit fit;
+  if (smem > GS_SMEM_MAX || !cluster_fits(fit, dev, reinterpret_cast<const void*>(gs_cluster_kernel<CB, CS>), CS, GS_THREADS, GS_SMEM_MAX))
+    return false;
+  ClusterLaunch c(CS, unsigned(CS * ks.na), GS_THREADS, smem, s);
+  SLDM_CUDA(cudaLaunchKernelEx(&c.cfg, gs_cluster_kernel<CB, CS>, a, ks, rs));
   count_launch();
   return true;
 }

@@ -19,6 +19,7 @@
 #include <atomic>
 #include <type_traits>
 
+#include "cluster.h"
 #include "dense.h"
 #include "widen.cuh"
 
@@ -769,33 +770,10 @@ bool panel_cluster(C* A, int n, int j0, int nb, Moves* mv, int* err, int dev, cu
   const int chunk = (n - j0 + CS - 1) / CS;
   const size_t smem = size_t(chunk) * (panel_width<C>() + 1) * sizeof(C);
   if (smem > LIMIT) return false;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(CS);
-  cfg.blockDim = dim3(PC_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CS;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  static std::atomic<uint64_t> yes{0}, no{0};
-  const uint64_t bit = uint64_t(1) << (dev & 63);
-  if (no.load() & bit) return false;
-  if (!(yes.load() & bit)) {  // does this device schedule such a cluster
-    bool ok = cudaFuncSetAttribute(lu_panel_cluster<C, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LIMIT)) == cudaSuccess;
-    if (ok && CS > 8)
-      ok = cudaFuncSetAttribute(lu_panel_cluster<C, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-    int nc = 0;
-    cfg.dynamicSmemBytes = LIMIT;
-    ok = ok && cudaOccupancyMaxActiveClusters(&nc, lu_panel_cluster<C, CS>, &cfg) == cudaSuccess && nc > 0;
-    cfg.dynamicSmemBytes = smem;
-    if (!ok) cudaGetLastError();
-    (ok ? yes : no).fetch_or(bit);
-    if (!ok) return false;
-  }
-  SLDM_CUDA(cudaLaunchKernelEx(&cfg, lu_panel_cluster<C, CS>, A, n, j0, nb, chunk, mv, err));
+  static ClusterFit fit;
+  if (!cluster_fits(fit, dev, reinterpret_cast<const void*>(lu_panel_cluster<C, CS>), CS, PC_THREADS, LIMIT)) return false;
+  ClusterLaunch c(CS, CS, PC_THREADS, smem, s);
+  SLDM_CUDA(cudaLaunchKernelEx(&c.cfg, lu_panel_cluster<C, CS>, A, n, j0, nb, chunk, mv, err));
   count_launch();
   return true;
 }
