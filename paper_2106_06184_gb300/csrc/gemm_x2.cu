@@ -7,12 +7,15 @@
 // matrix units): every 128-column segment of a row of A, and of every column of the
 // real-form right-hand side B' (gemm_tc.cu), is scaled by a power of two that takes its
 // largest entry into [2^6, 2^7) and cut into seven signed 8-bit digits,
-//     a = sum_i a_i 2^-8i,  |a_i| <= 128 (a_i an integer),  i = 0 .. 6.
-// Integers of 8 bits are exact in FP16, their products in FP32, and a sum over 128
-// columns of at most seven digit products of one weight stays below 7 x 128 x 2^14 < 2^24:
-// the tensor core's FP32 accumulators hold exact integers.  The products with i + j <= 6
+//     a = sum_i a_i 2^-8i,  i = 0 .. 6,  |a_i| <= 128 (an integer; the fourth and fifth, which the
+//     pair's second number joins, at most 192).
+// Such integers are exact in FP16, their products in FP32, and the sums over 128 columns of the digit
+// products of one weight stay within 2^24 for the weights 0 .. 5 (i + j): the tensor core's FP32
+// accumulators hold exact integers.  Weight 6 can reach 1.2 x 2^24 if every digit is at its bound; an
+// addition beyond 2^24 loses at most a unit of 2^-48, together below 2^-54 of the largest entries' product
+// (tests/test_x2_bounds.py).  The products with i + j <= 6
 // are kept (28 of 49), level l = i + j in an accumulator of its own; what is left out and
-// the digits' tails are below 2^-54 of the segments' largest entries.  The levels of a
+// the digits' tails are below 2^-50 of the segments' largest entries' product, term by term.  The levels of a
 // segment are scaled back and added into a compensated pair of FP32 sums (TwoSum for the
 // levels 0-3, which carry bits above the pair's first number's last place).  Six digits
 // are not enough: rows whose entries lie mostly 10^-2 below their segment's largest lost 2^-42.
@@ -73,7 +76,7 @@ __host__ __device__ constexpr uint32_t x_idesc(int n) {  // kind::f16, D FP32, A
 
 // the seven digits of (hi + lo) sc of two entries, sc24 = 2^24 sc: rounding to the nearest
 // integer by adding and subtracting 1.5 2^23, remainders exact; the low part's integer joins
-// the fourth digit (which may reach 192), its fraction the remainder
+// the fourth digit and its fraction the remainder, so the fourth and fifth may reach 192
 __device__ __forceinline__ void digits(float h0, float h1, float l0, float l1, float sc, float sc24, f2 (&d)[X_D]) {
   const f2 MG = f2_pack(12582912.f, 12582912.f), NM = f2_pack(-12582912.f, -12582912.f), K = f2_pack(256.f, 256.f);
   f2 t = f2_mul(f2_pack(h0, h1), f2_pack(sc, sc));
