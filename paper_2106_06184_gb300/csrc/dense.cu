@@ -1399,6 +1399,34 @@ SLDM_COMBINE_INST(float2, double2)
 SLDM_COMBINE_INST(float2, float2)
 #undef SLDM_COMBINE_INST
 
+// One CTA per object and column.
+__global__ void __launch_bounds__(128) close_charges_kernel(const ApplyDims D, const int32_t* __restrict__ tri_begin,
+                                                            double2* __restrict__ bc) {
+  const int o = blockIdx.x, t0 = tri_begin[o], nq = tri_begin[o + 1] - t0 - 1;
+  double2* __restrict__ b = bc + int64_t(blockIdx.y) * D.nt + t0;
+  double sr = 0, si = 0;
+  for (int q = threadIdx.x; q < nq; q += 128) {
+    sr += b[q].x;
+    si += b[q].y;
+  }
+  __shared__ double red[2][4];
+  for (int w = 16; w > 0; w >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, w);
+    si += __shfl_xor_sync(0xffffffffu, si, w);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = sr;
+    red[1][threadIdx.x >> 5] = si;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    b[nq] = make_double2(-((red[0][0] + red[0][1]) + (red[0][2] + red[0][3])), -((red[1][0] + red[1][1]) + (red[1][2] + red[1][3])));
+}
+void close_charges(const sldm_mesh* m, const ApplyDims& D, void* bc, int nrhs, cudaStream_t s) {
+  close_charges_kernel<<<dim3(unsigned(D.nobj), unsigned(nrhs)), 128, 0, s>>>(D, m->d.tri_begin.p, (double2*)bc), ::sldm::count_launch();
+  SLDM_CUDA(cudaGetLastError());
+}
+
 // row n of an (n + 1) x nc row-major block: minus the sum of its first n rows (the
 // eliminated charge of each column)
 template <class C>

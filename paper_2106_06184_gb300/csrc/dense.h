@@ -120,6 +120,8 @@ void apply_combine(const sldm_mesh* m, const ApplyDims& D, double k0, const doub
                    const void* w1, const void* w2, const void* w3, const void* e, const void* a, const void* bc, double s3,
                    const VecBatch<double2, CY>& y, int nrhs, cudaStream_t s, double2* const* zh = nullptr, int nzh = 0,
                    double* nrm = nullptr);
+// each object's last charge of the columns bc (complex128): minus the sum of its others
+void close_charges(const sldm_mesh* m, const ApplyDims& D, void* bc, int nrhs, cudaStream_t s);
 // row n of an (n + 1) x nc block = minus the sum of rows 0 .. n - 1
 template <class C>
 void neg_colsum(C* A, int n, int nc, cudaStream_t s);
