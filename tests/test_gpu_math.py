@@ -1,5 +1,5 @@
-"""The functions of one argument that the fills evaluate by tables and series instead of CUDA's (fill_dev.cuh), over
-the ranges they are used on, against long double (at least 64 bits).
+"""The functions of one argument that the fills evaluate by tables and series instead of CUDA's (fill_dev.cuh, widen.cuh), over
+the ranges they are used on, against long double (at least 64 bits) and, where it is exact, the conversion itself.
 
 Bounds, from the operations: wave_cis one table entry (CUDA's sincospi: 1 ulp below 1, 1.1e-16), two
 roundings of 0.56e-16, series 1e-17: 2.5e-16 absolute whatever the phase.  wave_exp2 the same relative to
@@ -19,6 +19,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SRC = r"""
 #include "internal.h"
 #include "fill_dev.cuh"
+#include "widen.cuh"
 using namespace sldm;
 __global__ void fn(int which, int n, const double* x, double* a, double* b) {
   __shared__ WaveTab T;
@@ -33,6 +34,7 @@ __global__ void fn(int which, int n, const double* x, double* a, double* b) {
   if (which == 2) a[i] = rsqrt_pos(x[i]);
   if (which == 3) a[i] = recip_pos(x[i]);
   if (which == 4) a[i] = log2_pos(L, x[i]);
+  if (which == 5) a[i] = widen(__int_as_float(int(unsigned(x[i]))));
 }
 extern "C" int run(int which, int n, const double* x, double* a, double* b) {
   fn<<<(n + 255) / 256, 256>>>(which, n, x, a, b);
@@ -102,3 +104,15 @@ def test_log2(call):
     v, _ = call(4, x)
     ref = np.log2(x.astype(np.longdouble))
     assert np.all(np.abs(v - ref) <= 1.3e-16 + 2.3e-16 * np.abs(ref))
+
+
+def test_widen_is_the_conversion(call):
+    """Every class of FP32 number: zeros, denormals, normals, infinities, NaN."""
+    rng = np.random.default_rng(5)
+    bits = np.concatenate([rng.integers(0, 2 ** 32, 20000), rng.integers(0, 2 ** 23, 4000), 2 ** 31 + rng.integers(0, 2 ** 23, 4000),
+                           [0, 1, 2 ** 31, 2 ** 31 + 1, 0x007fffff, 0x00800000, 0x7f7fffff, 0x7f800000, 0xff800000, 0x7f800001, 0x7fc00000]])
+    v, _ = call(5, bits.astype(np.float64))
+    with np.errstate(invalid="ignore"):
+        ref = bits.astype(np.uint32).view(np.float32).astype(np.float64)
+    nan = np.isnan(ref)
+    assert np.all(np.isnan(v[nan])) and np.array_equal(v[~nan].view(np.uint64), ref[~nan].view(np.uint64))
