@@ -17,12 +17,13 @@
 // row of A, and of every column of B', is scaled by a power of two that puts its largest
 // entry into [2^14, 2^15) (A's exponents are worked out once with the plan, B''s with
 // each pass).  With hi(v) = v rounded to FP16 (11 bits: |v - hi| <= 2^-11 |v|) and lo(v) =
-// v - hi rounded to FP16 (error <= 2^-11 |v - hi| <= 2^-22 |v|),
-//     D = hi(A) hi(B) + lo(A) hi(B) + hi(A) lo(B)        (FP32 accumulation),
+// 2^11 (v - hi) rounded to FP16 (error <= 2^-11 |v - hi| <= 2^-22 |v|; scaled into hi's range, or its last bits
+// would fall below FP16's smallest number for small v),
+//     D = hi(A) hi(B) + 2^-11 (lo(A) hi(B) + hi(A) lo(B))        (FP32 accumulation of either sum),
 // the dropped lo(A) lo(B) (<= 2^-22 |A||B|) and the two roundings of lo leave
 // each product term within 3 x 2^-22 of |A||B| (about 2^-22 for typical data),
-// against 2^-24 for an FP32 product; entries below 2^-17 of their segment's largest
-// lose lo's last bits, an absolute error of 2^-39 of that largest.  FP16 has TF32's
+// against 2^-24 for an FP32 product.  Entries below 2^-29 of their segment's largest keep fewer bits, an
+// absolute error of 2^-51 of that largest (TF32 keeps them; FP32 sums of the segment do not).  FP16 has TF32's
 // precision at twice its rate and half its bytes: four MMAs per 32 columns instead of
 // eight, whose issue (~75 cycles each) bound the TF32 form, and half the B' traffic.  The
 // sums are compensated (below).  The TF32 form of the operands (hi and lo rounded to TF32, no
@@ -43,7 +44,7 @@
 //   warp 1   MMA: one thread issues, per K step of 16 (TF32: 8),
 //            hi(A) x [hi(B') | lo(B')] (M 128, N 128: B' hi and lo are the two
 //            halves of one 128-row operand) and lo(A) x hi(B') (N 64) into the
-//            first half, into one of two 128-column TMEM accumulators, a fresh
+//            second half (unscaled TF32: the first), into one of two 128-column TMEM accumulators, a fresh
 //            one for every stage (a segment of 128 K columns), and commits them
 //            to the operand buffer's barrier;
 //   warps 10-17 epilogue: fold each segment's accumulator (the sum of its two
@@ -97,8 +98,8 @@ constexpr int TC_BK = 2 * TC_KC;                    // K columns of a B' box in 
 constexpr uint32_t TC_B_BYTES = TC_N * 128;         // 8 KB
 constexpr uint32_t TC_BBUF = 2 * TC_B_BYTES;       // B' hi, lo
 constexpr uint32_t TC_RING = TC_R * TC_STAGE_BYTES;
-// TMEM: two accumulators of 128 columns (hi(A) hi(B') in 0-63, hi(A) lo(B') in
-// 64-127) at columns 0 and 128, A operand buffers (hi and lo: 16 columns of FP16 pairs or 32 of TF32 each) from 256
+// TMEM: two accumulators of 128 columns (hi(A) hi(B') in 0-63, hi(A) lo(B') + lo(A) hi(B') in
+// 64-127; TF32: lo(A) hi(B') in 0-63) at columns 0 and 128, A operand buffers (hi and lo: 16 columns of FP16 pairs or 32 of TF32 each) from 256
 constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr uint32_t TC_ACC_COLS = 2 * TC_N;
 constexpr uint32_t TC_ACC_COL = 0, TC_AOP_COL = 2 * TC_ACC_COLS;
@@ -174,13 +175,14 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
       "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
       : "memory");
 }
-// v = hi + lo, both FP16 pairs (the first number in the lower half), rounded to nearest
+// v = hi + 2^-11 lo, both FP16 pairs (the first number in the lower half), rounded to nearest
+constexpr float LO_UP = 0x1p11f, LO_DOWN = 0x1p-11f;
 __device__ __forceinline__ void f16_split(f2 v, uint32_t& hi, uint32_t& lo) {
   float a, b;
   f2_unpack(v, a, b);
   const __half2 h = __floats2half2_rn(a, b);
   const float2 f = __half22float2(h);
-  f2_unpack(f2_sub(v, f2_pack(f.x, f.y)), a, b);
+  f2_unpack(f2_mul(f2_sub(v, f2_pack(f.x, f.y)), f2_pack(LO_UP, LO_UP)), a, b);
   const __half2 l = __floats2half2_rn(a, b);
   hi = *reinterpret_cast<const uint32_t*>(&h);
   lo = *reinterpret_cast<const uint32_t*>(&l);
@@ -304,10 +306,10 @@ __global__ void __maxnreg__(96)
           const uint32_t o = uint32_t(ks) * 32u;  // 16 FP16 or 8 TF32 = 32 bytes along K in the swizzle row of B'
           const uint32_t ac = uint32_t(ks) * 8u;  // 8 TMEM columns of A
           const uint32_t acc0 = (j > 0 || ks > 0) ? 1u : 0u;  // a fresh accumulator per segment
-          // hi(A) [hi(B') | lo(B')] in one N = 128 product, then lo(A) hi(B') into columns 0-63
+          // hi(A) [hi(B') | lo(B')] in one N = 128 product, then lo(A) hi(B') into columns 64-127 (TF32: 0-63)
           if constexpr (F) {
             tc_mma_f16(acc, aop + ac, sw128_desc(bh + o), IDESC_N128, acc0);
-            tc_mma_f16(acc, aop + AW / 2 + ac, sw128_desc(bh + o), IDESC_N64, 1u);
+            tc_mma_f16(acc + TC_N, aop + AW / 2 + ac, sw128_desc(bh + o), IDESC_N64, 1u);
           } else {
             tc_mma_tf32(acc, aop + ac, sw128_desc(bh + o), IDESC_N128, acc0);
             tc_mma_tf32(acc, aop + AW / 2 + ac, sw128_desc(bh + o), IDESC_N64, 1u);
@@ -467,14 +469,14 @@ __global__ void __maxnreg__(96)
         tc_fence_after();
 #pragma unroll
         for (int hq = 0; hq < 4; ++hq) {
-          f2 v[4], w[4];  // hi(A) hi(B') + lo(A) hi(B'), and hi(A) lo(B')
+          f2 v[4], w[4];  // hi(A) hi(B'), and hi(A) lo(B') + lo(A) hi(B') (TF32: lo(A) hi(B') in the first)
           tmem_ld8x2(tmem + (uint32_t(32 * q4) << 16) + TC_ACC_COL + uint32_t(seg & 1) * TC_ACC_COLS +
                          uint32_t(half * 32 + 8 * hq),
                      TC_N, v, w);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {  // 8 columns = 4 right-hand sides
             const int c = 4 * hq + i;
-            f2 u = f2_add(v[i], w[i]);
+            f2 u = F ? f2_fma(w[i], f2_pack(LO_DOWN, LO_DOWN), v[i]) : f2_add(v[i], w[i]);
             if (F) {
               const float sb = __shfl_sync(0xffffffffu, sbl, c);
               u = f2_mul(f2_mul(u, f2_pack(sa, sa)), f2_pack(sb, sb));
