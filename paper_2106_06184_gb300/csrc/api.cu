@@ -98,7 +98,7 @@ struct sldm_op {
   sldm::DBuf<int2> tl1d, tl2d;
   sldm::GemvPlan plan1d, plan2d;
   sldm::X2Plan x2p1, x2p2;  // SLDM_PREC_F32X2: the same on the tensor cores
-  // and Y11 e, Y21 e of its far field
+  // and Y11 e of its far field
   sldm::DBuf<sldm::GemvJob> jobsf;
   sldm::DBuf<int64_t> rsf;
   sldm::DBuf<int2> tlf;
@@ -211,16 +211,16 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
   // numbers that show its rounding, so it keeps the TF32 form and the products by themselves
   if (op->x2 && es_v == sizeof(float2)) {
     std::vector<GemvJob> jf;
-    for (auto& o : op->obj) {
+    for (auto& o : op->obj)  // the far field takes j - Y11 e alone
       jf.push_back({L(o.oY11), o.ne, o.ne, o.ne, P(op->we, o.e0), ne, P(op->wz1, o.e0), ne, 1, 0, 0, 0, nullptr});
-      if (o.nt > 1) jf.push_back({L(o.oY21), o.ne, o.nt - 1, o.ne, P(op->we, o.e0), ne, P(op->wz2, o.q0), op->nq, 1, 0, 0, 0, nullptr});
-    }
     mk(jf, op->jobsf, op->rsf, op->tlf, op->planf, &op->tcf, nullptr, op->tcf, false);
     op->planf.name = "gemv_y";
-    // not measured: its kernel, and so the far field's last digits, should not hang on a timing.  16 right-hand
-    // sides: 4 x 4 metasurface 34 us against 26 on the CUDA cores, one sphere of 1,280 triangles 53 / 42; 32: 36 / 42
-    // and 55 / 60
-    op->planf.tc_from = tc_policy() ? tc_policy() : (op->planf.total_rows >= 4096 ? TILE_NRHS + 1 : 2 * TILE_NRHS + 1);
+    // Fixed lines, not measured ones: the form, and with it the far field's eighth digit, should not hang on a timing.
+    // us by columns 9-16 / 17 / 32, tensor against CUDA cores: 4 x 4 cylinders 26 / 26 / 27 against 18 / 22 / 29, 6 x 6
+    // 35 / 36 / 40 against 29 / 41 / 53, one sphere of 1,280 triangles 52 / 52 / 54 against 26 / 42 / 42, a box of 1,356
+    // 71 / 72 / 72 against 62 / 62 / 87.  Moving a line to where the two
+    // cross would save up to 27 us of a call of 0.3 ms and more and change those digits of the calls between: it stays.
+    op->planf.tc_from = tc_policy() ? tc_policy() : (ne + op->nq >= 4096 ? TILE_NRHS + 1 : 2 * TILE_NRHS + 1);
   }
   p1.name = "gemv_y";     // Y11, Y21 (per object)
   p2.name = "gemv_main";  // L^A_m, L^phi_m and the internal blocks
