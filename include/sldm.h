@@ -143,7 +143,8 @@ typedef struct {
 
 typedef struct {
   int64_t n_unknowns, ne, nt, nobj;
-  int64_t device_bytes; /* device memory held by the operator */
+  int64_t device_bytes; /* device memory held by the operator: blocks, plans, work vectors and,
+                           after the first solve, the Krylov bases */
   int32_t precision;
   int32_t tc_from;      /* complex64 operators: the smallest lockstep width whose
                            products run on the tensor cores (9, 17, or 33 = never),

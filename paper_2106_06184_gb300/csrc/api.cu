@@ -133,13 +133,20 @@ struct sldm_op {
 
 namespace sldm {
 
+// Device memory that the operator holds, every buffer of it.
 static int64_t op_bytes(const sldm_op* op) {
-  int64_t nb = int64_t(op->wnt.bytes() + op->wny.bytes() + op->wnr.bytes());
-  for (const auto& u : op->nested)
-    if (u->mat && u->obj == u->mat_owner) nb += int64_t(u->mat->M.bytes() + u->mat->R.bytes() + u->mat->X.bytes());
-  return nb + int64_t(op->LAm.bytes() + op->LPm.bytes() + op->loc.bytes() + op->LAm_lo.bytes() + op->LPm_lo.bytes() +
-                 op->loc_lo.bytes() + op->ix_val.bytes() + op->ix32.bytes() + op->V.bytes() +
-                 op->pc.sinv.bytes() + op->pc.sinv32.bytes() + op->pc.lam.bytes() + op->pc.pdiag.bytes());
+  size_t nb = bytes_of(op->LAm, op->LPm, op->loc, op->LAm_lo, op->LPm_lo, op->loc_lo, op->ix_val, op->ix32, op->pc, op->T.A, op->T.B);
+  nb += bytes_of(op->wj, op->we, op->wa, op->wbc, op->wbu, op->wz1, op->wz2, op->ww1, op->ww2, op->ww3);
+  nb += bytes_of(op->jobs1, op->jobs2, op->rs1, op->rs2, op->tl1, op->tl2, op->tc1, op->tc2);
+  nb += bytes_of(op->jobs1d, op->jobs2d, op->rs1d, op->rs2d, op->tl1d, op->tl2d, op->x2p1, op->x2p2);
+  nb += bytes_of(op->jobsf, op->rsf, op->tlf, op->tcf);
+  nb += bytes_of(op->V, op->wb, op->wx, op->wr, op->wtmp, op->dh, op->dnorm, op->gH, op->gcs, op->gsn, op->gg, op->gst);
+  nb += bytes_of(op->wnt, op->wny, op->wnr);
+  for (const auto& u : op->nested) {
+    nb += u->bytes();
+    if (u->mat && u->obj == u->mat_owner) nb += u->mat->bytes();
+  }
+  return int64_t(nb);
 }
 
 // GEMV plans of the structured product with matrix entries of es_m bytes and

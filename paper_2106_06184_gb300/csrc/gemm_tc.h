@@ -46,6 +46,7 @@ struct TcPlan {
   int nctas = 0;
   int longest = 0;           // stages of the CTA with the most
   bool ok = false;           // every job fits the tensor-core path
+  size_t bytes() const { return bytes_of(maps, tiles, cta_begin, err, bprime, bscale, bmap, gjob, gst, tj, aexp, ztiles); }
 };
 
 // Builds tp for the jobs of a complex64 plan (host copies of the jobs), whose blocks

@@ -17,6 +17,7 @@ struct X2Plan {
   DBuf<float> bscale;
   int from = X2_NRHS + 1;  // right-hand sides a pass is worth it for
   bool ok = false;
+  size_t bytes() const { return bytes_of(lomaps, bmap, bprime, bscale); }
 };
 void x2_plan_build(const std::vector<GemvJob>& jobs, const TcPlan& tc, X2Plan& xp, cudaStream_t s);
 // Y = alpha (A + Alo) X (+ Y) for nrhs <= 16 complex128 columns from col0

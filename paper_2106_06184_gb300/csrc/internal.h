@@ -106,6 +106,11 @@ struct DBuf {
   size_t bytes() const { return n * sizeof(T); }
 };
 
+template <class... B>
+size_t bytes_of(const B&... b) {
+  return (size_t(0) + ... + b.bytes());
+}
+
 // ---------------------------------------------------------------- mesh
 // Host topology and its device copy.  Triangle-local index i names the vertex
 // tri[t][i] and the edge opposite to it.

@@ -26,6 +26,7 @@ struct NestedMat {
   DBuf<float2> X;                  // complex64 approximation of M_l^-1 (n x n)
   int steps = 0;                   // refinement steps of every application
   double contraction = 0;          // measured ||r_{k+1}|| / ||r_k|| at assembly
+  size_t bytes() const { return bytes_of(M, R, X); }
 };
 
 // One object's use of a NestedMat: its slices of the structured product's work
@@ -38,6 +39,7 @@ struct NestedUse {
   DBuf<int64_t> rR, rX0, rXa, rM;
   DBuf<int2> tR, tX0, tXa, tM;
   GemvPlan pR, pX0, pXa, pM;
+  size_t bytes() const { return bytes_of(jR, jX0, jXa, jM, rR, rX0, rXa, rM, tR, tX0, tXa, tM); }
 };
 
 // Builds X from mat.M and measures mat.steps; false when refinement would not

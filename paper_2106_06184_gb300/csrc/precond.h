@@ -31,6 +31,7 @@ struct Precond {
   GemvPlan plan;
   TcPlan tc;  // complex64: the Schur-inverse products on the tensor cores (9 to 32 columns)
   bool ready = false;
+  size_t bytes() const { return bytes_of(objs, lam, lam32, pdiag32, pdiag, sinv, sinv32, t3, bx, jobs, rs, tiles, tc); }
 };
 
 template <class C>
