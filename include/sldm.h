@@ -440,12 +440,12 @@ int sldm_set_tc_policy(int32_t tc_from);
 int sldm_device_bytes(int64_t* in_use);
 
 /* Fault injection for tests of the failure paths (no counterpart in the paper).
- * SLDM_INJECT_LU_STALL: the next `count` launches of the batched direct solver
- * (the cooperative LU of M_l and of the preconditioner's Schur complements) make
- * their first CTA wait first on a device flag that nothing sets.  That wait is
- * bounded like every wait of the solver (a few hundred ms); when it runs out the
- * CTA records the failure, every other CTA leaves at its next wait, and the call
- * that launched the solver (sldm_assemble) returns SLDM_ETIMEOUT.  No fault is
+ * SLDM_INJECT_LU_STALL: the next `count` runs of the direct solver, in whichever
+ * form the sizes choose (the batched LU, or the blocked one of a single system: of M_l
+ * and of the preconditioner's Schur complements), wait first on a device flag that
+ * nothing sets.  That wait is bounded like every wait of the solver (a few hundred ms);
+ * when it runs out the failure is recorded, every CTA leaves at its next wait or
+ * launch, and the call that ran the solver (sldm_assemble) returns SLDM_ETIMEOUT.  No fault is
  * raised and the CUDA context stays usable.  count = 0 clears the injection.
  * SLDM_INJECT_TC_WAIT: the next `count` tensor-core products record, once they have run, the
  * flag that a product whose bounded wait ran out leaves; the call that reads it returns

@@ -432,10 +432,10 @@ __global__ void __launch_bounds__(LU_THREADS) lu_coop_kernel(const LUSysT<C>* __
 template <class C>
 void lu_solve_batched(const std::vector<LUSysT<C>>& all, cudaStream_t s) {
   // a few systems of medium order one after the other in blocked form; many, or small
-  // ones, side by side (an injected stall belongs to the side-by-side kernel)
+  // ones, side by side
   int medium = 0;
   for (auto& S : all) medium += S.n >= LU_BLOCKED_FEW;
-  const int from = medium <= 2 && !lu_stall_pending() ? LU_BLOCKED_FEW : LU_BLOCKED_MIN;
+  const int from = medium <= 2 ? LU_BLOCKED_FEW : LU_BLOCKED_MIN;
   std::vector<LUSysT<C>> systems;
   for (auto& S : all) {
     if (S.n >= from) lu_solve_blocked<C>(S, s);

@@ -62,7 +62,6 @@ void budget_take(size_t bytes);
 void budget_give(size_t bytes);
 // Test injection (sldm_test_inject): consumes one pending LU stall, if any.
 bool take_lu_stall();
-bool lu_stall_pending();
 // consumes one pending tensor-core wait that runs out, if any
 bool take_tc_wait();
 

@@ -110,6 +110,16 @@ __device__ bool grid_barrier(unsigned* ctr, unsigned target, int* err) {
   return s_ok != 0;
 }
 
+// Injected failure (sldm_test_inject): a bounded wait for a flag that nothing sets, on the solver's own error
+// record; every kernel after it leaves at once, as after a panel's barrier that ran out.
+__global__ void lu_stall_kernel(const unsigned* flag, int* err) {
+  for (unsigned it = 0; it < SPIN_LIMIT / 8; ++it) {
+    if (ld_acq(flag)) return;
+    __nanosleep(32);
+  }
+  atomicExch(err, 2);
+}
+
 // ---------------------------------------------------------------- 1. panel
 // CTA c holds rows [j0 + c*chunk, min(n, j0 + (c+1)*chunk)) of columns
 // [j0, j0 + nb) in shared memory.  Pivot candidates go to slot_v/slot_i[c];
@@ -814,7 +824,7 @@ void lu_solve_blocked(const LUSysT<C>& S, cudaStream_t s) {
       orow.alloc(NB);
       slot_v.alloc(nsm);
       slot_i.alloc(nsm);
-      bar.alloc(1);
+      if (!bar.p) bar.alloc(1);
       const int max_chunk = (n + nsm - 1) / nsm > PANEL_MIN_ROWS ? (n + nsm - 1) / nsm : PANEL_MIN_ROWS;
       const size_t panel_smem = (size_t(max_chunk) * NB + NB) * sizeof(C);
       SLDM_REQUIRE(panel_smem <= 200 * 1024, SLDM_ENOTSUP, "LU: panel too large for shared memory");
@@ -843,6 +853,11 @@ void lu_solve_blocked(const LUSysT<C>& S, cudaStream_t s) {
     lu_moves_kernel<<<1, 32, 0, s>>>(piv.p, j0, nb, mv.p, err.p), count_launch();
   };
   ScopedTimer tm("lu_blocked", s);
+  if (take_lu_stall()) {
+    bar.alloc(1);
+    bar.zero(s);
+    lu_stall_kernel<<<1, 1, 0, s>>>(bar.p, err.p), count_launch();
+  }
   for (int j0 = 0; j0 < n; j0 += NB) {
     const int nb = std::min(NB, n - j0);
     if (!panel_cluster<C, 16>(S.A, n, j0, nb, mv.p, err.p, dev, s) && !panel_cluster<C, 8>(S.A, n, j0, nb, mv.p, err.p, dev, s))

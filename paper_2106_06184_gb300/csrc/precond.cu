@@ -422,7 +422,7 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
     const int nq = o.nt - 1;
     prec_schur_kernel<<<dim3((nq + 127) / 128, nq), 128, 0, s>>>(o, k0, d.tri_edge.p, d.tri_sign.p, d.tplus.p, d.tminus.p,
                                                                 P.lam.p, P.pdiag.p, Sm.p + soff[i], P.sinv.p + off[i]), ::sldm::count_launch();
-    if (nq >= SCHUR_REFINE_MIN && !lu_stall_pending()) {
+    if (nq >= SCHUR_REFINE_MIN) {
       bool done = false;
       try {
         done = schur_inverse(o, d, P, k0, Sm.p + soff[i], P.sinv.p + off[i], goal, s);

@@ -27,7 +27,6 @@ void budget_take(size_t bytes) {
 void budget_give(size_t bytes) { g_bytes.fetch_sub(int64_t(bytes)); }
 
 static std::atomic<int> g_lu_stall{0};
-bool lu_stall_pending() { return g_lu_stall.load() > 0; }
 bool take_lu_stall() {
   int v = g_lu_stall.load();
   while (v > 0)
