@@ -450,9 +450,13 @@ int sldm_device_bytes(int64_t* in_use);
  * SLDM_INJECT_TC_WAIT: the next `count` tensor-core products record, once they have run, the
  * flag that a product whose bounded wait ran out leaves; the call that reads it returns
  * SLDM_ETIMEOUT (see sldm_apply).
+ * SLDM_INJECT_ALLOC: the count-th device allocation from now fails as one for which there is no
+ * memory: the call that made it returns SLDM_ENOMEM having released what it took, or goes
+ * another way where it has one.
  * SLDM_EINVAL for an unknown `what` or a negative count. */
 #define SLDM_INJECT_LU_STALL 1
 #define SLDM_INJECT_TC_WAIT 2
+#define SLDM_INJECT_ALLOC 3
 int sldm_test_inject(int32_t what, int32_t count);
 
 /* ---------------------------------------------------------------------------

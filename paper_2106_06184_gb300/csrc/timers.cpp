@@ -14,7 +14,10 @@ namespace sldm {
 static std::atomic<int64_t> g_bytes{0};
 static std::atomic<int64_t> g_budget{0};
 
+static std::atomic<int> g_alloc_fail{0};  // the allocation, counted from the next, that fails (0: none)
+
 void budget_take(size_t bytes) {
+  if (g_alloc_fail.load() > 0 && g_alloc_fail.fetch_sub(1) == 1) throw Error{SLDM_ENOMEM, "device allocation: injected failure"};
   const int64_t b = int64_t(bytes);
   const int64_t now = g_bytes.fetch_add(b) + b;
   const int64_t lim = g_budget.load();
@@ -214,10 +217,13 @@ extern "C" int sldm_device_bytes(int64_t* in_use) {
 }
 
 extern "C" int sldm_test_inject(int32_t what, int32_t count) {
-  if ((what != SLDM_INJECT_LU_STALL && what != SLDM_INJECT_TC_WAIT) || count < 0) {
+  if (what < SLDM_INJECT_LU_STALL || what > SLDM_INJECT_ALLOC || count < 0) {
     sldm::set_error("test_inject: unknown injection or negative count");
     return SLDM_EINVAL;
   }
-  (what == SLDM_INJECT_LU_STALL ? sldm::g_lu_stall : sldm::g_tc_wait).store(count);
+  (what == SLDM_INJECT_LU_STALL  ? sldm::g_lu_stall
+   : what == SLDM_INJECT_TC_WAIT ? sldm::g_tc_wait
+                                 : sldm::g_alloc_fail)
+      .store(count);
   return SLDM_OK;
 }

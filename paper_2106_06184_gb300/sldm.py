@@ -18,6 +18,7 @@ LIB_PATH = os.path.join(HERE, "_build", "libsldm.so")
 OK, EINVAL, ENOMEM, ENOTCONV, ENUMERIC, ECUDA, EBUSY, ENOTSUP, ETIMEOUT = 0, -1, -2, -3, -4, -5, -6, -7, -8
 INJECT_LU_STALL = 1
 INJECT_TC_WAIT = 2
+INJECT_ALLOC = 3
 HOST, DEVICE = 0, 1
 PREC_F64, PREC_F32, PREC_F32X2 = 0, 1, 2
 BOTTOM_HALFSPACE, BOTTOM_PEC = 0, 1
