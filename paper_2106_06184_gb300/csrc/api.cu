@@ -152,7 +152,7 @@ static int64_t op_bytes(const sldm_op* op) {
 // GEMV plans of the structured product with matrix entries of es_m bytes and
 // vector entries of es_v bytes (the work vectors hold complex128, so both the
 // operator's precision and FP64 fit).
-static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1, DBuf<int64_t>& drs1, DBuf<int2>& dt1,
+static void make_plans(sldm_op* op, cudaStream_t s, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1, DBuf<int64_t>& drs1, DBuf<int2>& dt1,
                        GemvPlan& p1, DBuf<GemvJob>& dj2, DBuf<int64_t>& drs2, DBuf<int2>& dt2, GemvPlan& p2,
                        TcPlan* tc1 = nullptr, TcPlan* tc2 = nullptr, X2Plan* x1 = nullptr, X2Plan* x2 = nullptr) {
   const int64_t ne = op->ne, nt = op->nt;
@@ -188,9 +188,9 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
       acc += j[i].m;
       for (int r0 = 0; r0 < j[i].m; r0 += gemv_tile_rows(es_v)) tiles.push_back(make_int2(int(i), r0));
     }
-    dj.upload(j);
-    drs.upload(rs);
-    dt.upload(tiles);
+    dj.upload(j, s);
+    drs.upload(rs, s);
+    dt.upload(tiles, s);
     plan.jobs = dj.p;
     plan.rowstart = drs.p;
     plan.njobs = int(j.size());
@@ -203,12 +203,12 @@ static void make_plans(sldm_op* op, size_t es_m, size_t es_v, DBuf<GemvJob>& dj1
     for (auto& jb : j) plan.bytes += double(jb.m) * jb.n * es_m * (lo ? 2 : 1);
     plan.tc = nullptr;
     if (tc) {  // complex64 blocks and vectors: tensor-core passes of 9 to 32 right-hand sides
-      tc_plan_build(j, *tc, f16, 0);
+      tc_plan_build(j, *tc, f16, s);
       if (tc->ok) plan.tc = tc;
     }
     plan.x2 = nullptr;
     if (xp && lo && tc_policy() <= MAX_NRHS) {
-      x2_plan_build(j, like, *xp, 0);
+      x2_plan_build(j, like, *xp, s);
       if (xp->ok) plan.x2 = xp;
     }
   };
@@ -243,7 +243,7 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
   op->wz1.alloc(ne * WR * ev); op->wz2.alloc(nt * WR * ev);
   op->ww1.alloc(ne * WR * ev); op->ww2.alloc(ne * WR * ev); op->ww3.alloc(nt * WR * ev);
   const bool c64 = sizeof(C) == sizeof(float2);
-  make_plans(op, sizeof(C), sizeof(C), op->jobs1, op->rs1, op->tl1, op->plan1, op->jobs2, op->rs2, op->tl2, op->plan2,
+  make_plans(op, s, sizeof(C), sizeof(C), op->jobs1, op->rs1, op->tl1, op->plan1, op->jobs2, op->rs2, op->tl2, op->plan2,
              c64 ? &op->tc1 : nullptr, c64 ? &op->tc2 : nullptr);
   if (c64) {
     op->ix32.alloc(op->ix_val.n);
@@ -257,7 +257,7 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
     SLDM_CUDA(cudaStreamSynchronize(s));
   }
   if (sizeof(C) == sizeof(float2)) {
-    make_plans(op, sizeof(C), sizeof(double2), op->jobs1d, op->rs1d, op->tl1d, op->plan1d, op->jobs2d, op->rs2d, op->tl2d,
+    make_plans(op, s, sizeof(C), sizeof(double2), op->jobs1d, op->rs1d, op->tl1d, op->plan1d, op->jobs2d, op->rs2d, op->tl2d,
                op->plan2d, nullptr, nullptr, &op->x2p1, &op->x2p2);
     op->plan1d.name = "gemv_y_f64acc";
     op->plan2d.name = "gemv_main_f64acc";
@@ -270,7 +270,7 @@ static void build_plans(sldm_op* op, cudaStream_t s) {
     op->wny.alloc(size_t(op->ldn) * WR);
     op->wnr.alloc(size_t(op->ldn) * WR);
     for (auto& u : op->nested)
-      nested_plans(*u, reinterpret_cast<const double2*>(op->we.p), ne, op->wnt.p, op->wny.p, op->wnr.p, op->ldn);
+      nested_plans(*u, reinterpret_cast<const double2*>(op->we.p), ne, op->wnt.p, op->wny.p, op->wnr.p, op->ldn, s);
   }
 }
 
@@ -829,12 +829,12 @@ static void split_to_x2(sldm_op* op, cudaStream_t s) {
 
 // ---------------------------------------------------------------- GMRES
 // GMRES workspace for nr right-hand sides in lockstep (Krylov bases N x (m+1) each)
-static void ensure_ws(sldm_op* op, int m, int nr) {
+static void ensure_ws(sldm_op* op, int m, int nr, cudaStream_t s) {
   if (op->ws_m == m && op->ws_nr >= nr && op->V.p) return;
   const size_t N = size_t(op->N), W = size_t(sldm_op::WR);
   op->ldv = (op->N + 63) / 64 * 64;
   op->V.alloc(size_t(op->ldv) * (m + 1) * nr);
-  op->V.zero();  // the padding rows stay zero
+  op->V.zero(s);  // the padding rows stay zero
   op->wb.alloc(N * W);
   op->wx.alloc(N * W);
   op->wr.alloc(N * W);
@@ -1479,7 +1479,7 @@ int sldm_solve(const sldm_op* op_, const void* b, void* x, int32_t nrhs, const s
   bool refine = op->prec == SLDM_PREC_F32 && !(opts && opts->refine == SLDM_REFINE_OFF);
   cudaStream_t s = (cudaStream_t)stream;
   const int W = sldm_op::WR;
-  ensure_ws(op, m, std::min<int>(nrhs, W));
+  ensure_ws(op, m, std::min<int>(nrhs, W), s);
   const size_t vb = size_t(op->N) * sizeof(double2);
   int iters = 0;
   double worst = 0;

@@ -70,14 +70,14 @@ static __global__ void copy_cols_kernel(int64_t n, int nr, const double2* __rest
 // A plan of one GEMV job (the tiles of the several-right-hand-side kernel
 // included), uploaded to the given buffers.
 static void one_job_plan(const GemvJob& j, size_t es_m, size_t es_v, const char* name, DBuf<GemvJob>& dj,
-                         DBuf<int64_t>& drs, DBuf<int2>& dt, GemvPlan& p) {
+                         DBuf<int64_t>& drs, DBuf<int2>& dt, GemvPlan& p, cudaStream_t s) {
   std::vector<GemvJob> jobs{j};
   std::vector<int64_t> rs{0};
   std::vector<int2> tiles;
   for (int r0 = 0; r0 < j.m; r0 += gemv_tile_rows(es_v)) tiles.push_back(make_int2(0, r0));
-  dj.upload(jobs);
-  drs.upload(rs);
-  dt.upload(tiles);
+  dj.upload(jobs, s);
+  drs.upload(rs, s);
+  dt.upload(tiles, s);
   p.name = name;
   p.jobs = dj.p;
   p.rowstart = drs.p;
@@ -125,10 +125,10 @@ bool nested_setup(NestedMat& mat, cudaStream_t s) {
   DBuf<int2> t1, t2, t3, t4;
   GemvPlan pR, pX0, pM, pXa;
   one_job_plan({mat.R.p, mat.ne, int32_t(n), mat.ne, de.p, mat.ne, t.p, n, 1, 0, 0, 0, nullptr}, 16, 16, "nested_R", j1, r1,
-               t1, pR);
-  one_job_plan({mat.X.p, n, int32_t(n), int32_t(n), t.p, n, y.p, n, 1, 0, 0, 0, nullptr}, 8, 16, "nested_X", j2, r2, t2, pX0);
-  one_job_plan({mat.M.p, n, int32_t(n), int32_t(n), y.p, n, r.p, n, -1, 0, 1, 0, nullptr}, 16, 16, "nested_M", j3, r3, t3, pM);
-  one_job_plan({mat.X.p, n, int32_t(n), int32_t(n), r.p, n, y.p, n, 1, 0, 1, 0, nullptr}, 8, 16, "nested_X", j4, r4, t4, pXa);
+               t1, pR, s);
+  one_job_plan({mat.X.p, n, int32_t(n), int32_t(n), t.p, n, y.p, n, 1, 0, 0, 0, nullptr}, 8, 16, "nested_X", j2, r2, t2, pX0, s);
+  one_job_plan({mat.M.p, n, int32_t(n), int32_t(n), y.p, n, r.p, n, -1, 0, 1, 0, nullptr}, 16, 16, "nested_M", j3, r3, t3, pM, s);
+  one_job_plan({mat.X.p, n, int32_t(n), int32_t(n), r.p, n, y.p, n, 1, 0, 1, 0, nullptr}, 8, 16, "nested_X", j4, r4, t4, pXa, s);
   gemv_jobs_mixed<double2, double2>(pR, 1, s);
   gemv_jobs_mixed<float2, double2>(pX0, 1, s);
   std::vector<double2> h(n);
@@ -158,17 +158,18 @@ bool nested_setup(NestedMat& mat, cudaStream_t s) {
   return false;
 }
 
-void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, double2* y, double2* r, int64_t ldw) {
+void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, double2* y, double2* r, int64_t ldw,
+                  cudaStream_t s) {
   NestedMat& m = *u.mat;
   const int64_t n = m.n;
   one_job_plan({m.R.p, m.ne, int32_t(n), m.ne, e + u.e0, lde, t, ldw, 1, 0, 0, 0, nullptr}, 16, 16, "nested_R", u.jR, u.rR,
-               u.tR, u.pR);
+               u.tR, u.pR, s);
   one_job_plan({m.X.p, n, int32_t(n), int32_t(n), t, ldw, y, ldw, 1, 0, 0, 0, nullptr}, 8, 16, "nested_X", u.jX0, u.rX0,
-               u.tX0, u.pX0);
+               u.tX0, u.pX0, s);
   one_job_plan({m.M.p, n, int32_t(n), int32_t(n), y, ldw, r, ldw, -1, 0, 1, 0, nullptr}, 16, 16, "nested_M", u.jM, u.rM, u.tM,
-               u.pM);
+               u.pM, s);
   one_job_plan({m.X.p, n, int32_t(n), int32_t(n), r, ldw, y, ldw, 1, 0, 1, 0, nullptr}, 8, 16, "nested_X", u.jXa, u.rXa,
-               u.tXa, u.pXa);
+               u.tXa, u.pXa, s);
 }
 
 void nested_apply(const NestedUse& u, const double2* t, double2* y, double2* r, int64_t ldw, double2* a, int64_t lda,

@@ -47,8 +47,9 @@ struct NestedUse {
 bool nested_setup(NestedMat& mat, cudaStream_t s);
 
 // Plans of object use u against the work vectors: e (edges, column stride lde) and
-// the scratch t, y, r (n x WR complex128 each, column stride ldw).
-void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, double2* y, double2* r, int64_t ldw);
+// the scratch t, y, r (n x WR complex128 each, column stride ldw), uploaded on s.
+void nested_plans(NestedUse& u, const double2* e, int64_t lde, double2* t, double2* y, double2* r, int64_t ldw,
+                  cudaStream_t s);
 
 // a -= Y11 e / ell and bc += B (ell Y21 e) of object use u for nr columns (ell: the length
 // scaling of M_l), by the refinement above; a: edges, stride lda, bc: triangles, stride ldb.
