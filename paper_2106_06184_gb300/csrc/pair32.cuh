@@ -1,6 +1,9 @@
 // Sums of products in pairs of FP32 numbers: ~48 bits without the FP64 pipe, whose instructions cost 64
 // FP32 ones on this part.  For the sparse parts of complex64 products, whose terms are FP32
-// numbers times FP64 coefficients held as hi + lo (split_pairs).
+// numbers times FP64 coefficients held as hi + lo (split_pairs).  Below 2^-101 a product's own
+// rounding error falls under FP32's smallest number: an error of 2^-149 per operation then, the spacing of
+// the terms themselves.  A sum that overflows or holds an infinity is that infinity (its error
+// would be Inf - Inf), a NaN stays NaN.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -32,8 +35,9 @@ struct P32 {
     r.fma(h, l, *this);
     return r;
   }
-  __device__ __forceinline__ void get(float& o) const { o = __fadd_rn(s, c); }
-  __device__ __forceinline__ void get(double& o) const { o = widen(s) + widen(c); }
+  __device__ __forceinline__ float err() const { return fabsf(s) < __int_as_float(0x7f800000) ? c : 0.f; }
+  __device__ __forceinline__ void get(float& o) const { o = __fadd_rn(s, err()); }
+  __device__ __forceinline__ void get(double& o) const { o = widen(s) + widen(err()); }
 };
 // complex += a v, a = (hi.x + lo.x) + j (hi.y + lo.y) as (hi.x, hi.y, lo.x, lo.y)
 template <class V>
