@@ -325,10 +325,11 @@ __global__ void __maxnreg__(96)
           if (t_begin + tile_i < t_end) nk = nk_of(t_begin + tile_i);
         }
       }
-      // the MMAs in flight (they complete in order) finish before the CTA leaves
+      // the MMAs in flight (they complete in order) finish, and their commits arrive, before the CTA leaves
       if (last >= 0) {
         mbar_wait(wfree(last % TC_NA), uint32_t((last / TC_NA) & 1));
         if (last % BPB == BPB - 1) mbar_wait(bfree(last / BPB % TC_NBB), uint32_t((last / BPB / TC_NBB) & 1));
+        if (last % TC_BPS == TC_BPS - 1) mbar_wait(accfull(last / TC_BPS & 1), uint32_t((last / TC_BPS >> 1) & 1));
       }
     }
     __syncwarp();

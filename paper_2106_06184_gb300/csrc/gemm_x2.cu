@@ -247,6 +247,7 @@ __global__ void __maxnreg__(96)
       if (last >= 0) {
         mbar_wait(wfree(last % X_NA), uint32_t((last / X_NA) & 1));
         if ((last & 3) == 3) mbar_wait(bfree(last / 4 % X_NBB), uint32_t((last / 4 / X_NBB) & 1));
+        if ((last & 7) == 7) mbar_wait(accfull, uint32_t((last / 8) & 1));
       }
     }
     __syncwarp();
