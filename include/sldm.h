@@ -76,7 +76,8 @@ extern "C" {
  * Y11, Y21 factored) in FP64, then kept as two complex64 parts hi = fl32(v) and
  * lo = fl32(v - hi), so v = hi + lo to ~2^-48 relative.  GMRES cycles apply hi in
  * FP32 arithmetic; the residual of iterative refinement, and sldm_apply, apply
- * hi + lo with compensated FP32 sums (~48 bits), so refined solutions converge to
+ * hi + lo to ~48 bits (compensated FP32 sums, or exact slices on the tensor cores for
+ * several right-hand sides of large operators), so refined solutions converge to
  * those of the FP64 discrete system.  Twice the operator memory of SLDM_PREC_F32
  * (the same as SLDM_PREC_F64). */
 #define SLDM_PREC_F32X2 2

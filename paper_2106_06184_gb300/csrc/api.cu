@@ -225,8 +225,8 @@ static void make_plans(sldm_op* op, cudaStream_t s, size_t es_m, size_t es_v, DB
     // Fixed lines, not measured ones: the form, and with it the far field's eighth digit, should not hang on a timing.
     // us by columns 9-16 / 17 / 32, tensor against CUDA cores: 4 x 4 cylinders 26 / 26 / 27 against 18 / 22 / 29, 6 x 6
     // 35 / 36 / 40 against 29 / 41 / 53, one sphere of 1,280 triangles 52 / 52 / 54 against 26 / 42 / 42, a box of 1,356
-    // 71 / 72 / 72 against 62 / 62 / 87.  Moving a line to where the two
-    // cross would save up to 27 us of a call of 0.3 ms and more and change those digits of the calls between: it stays.
+    // 71 / 72 / 72 against 62 / 62 / 87.  The lines are not where the two cross: the tensor cores lose up to 16 us of a call
+    // of 0.3 ms and more beside theirs and win up to 15.  Moving one changes those digits of the calls between, so they stay.
     op->planf.tc_from = tc_policy() ? tc_policy() : (ne + op->nq >= 4096 ? TILE_NRHS + 1 : 2 * TILE_NRHS + 1);
   }
   p1.name = "gemv_y";     // Y11, Y21 (per object)

@@ -1014,7 +1014,7 @@ void gemv_jobs_mixed(const GemvPlan& plan, int nrhs, cudaStream_t s) {
     // the compensated product the arithmetic is the bound (4 DFMA or ~44 FP32 operations per
     // entry and right-hand side), so the rest takes a kernel of its own width; complex64
     // passes, bound by launches and L2, take it as one more pass of 8.
-    // (box of 432 triangles, FP64, 5 right-hand sides, the whole product: 453 us with 8 -> 303 us)
+    // (box of 696 triangles, FP64, 5 right-hand sides, the whole product: 453 us with 8 -> 303 us)
     const int left = nrhs - c0, full = c64 && left > 4 ? left : left / TILE_NRHS * TILE_NRHS, rest = left - full, c1 = c0 + full;
     auto go = [&](auto lo) {
       constexpr bool LO = decltype(lo)::value;

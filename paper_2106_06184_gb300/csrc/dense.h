@@ -78,9 +78,6 @@ struct GemvPlan {
   // 33 = never): below it, passes of 8 on the CUDA cores
   int tc_from = TILE_NRHS + 1;
 };
-// right-hand sides in lockstep (GMRES) and per pass of the structured product
-// and the preconditioner: up to 32 (tensor cores for complex64 operators; the
-// CUDA-core kernels take 8 per launch)
 
 // rows per tile of the several-right-hand-side kernel for vectors of es_v bytes
 inline int gemv_tile_rows(size_t es_v) { return es_v == 8 ? 32 : 16; }

@@ -54,8 +54,8 @@ struct TcPlan {
 // false (and the plan keeps the CUDA-core kernels) when a job's row pitch is
 // not a multiple of 16 bytes or the driver's tensor-map encoder is unavailable.
 //
-// f16: the FP16 form; else TF32, as accurate and slower (8 x 8 metasurface, 32 right-hand
-// sides: 1,363 against 1,610 us), for products whose rounding shows in complex128 results.
+// f16: the FP16 form; else TF32, no more accurate and slower (8 x 8 metasurface, 32 right-hand
+// sides: 1,390 against 1,610 us), for products whose rounding shows in complex128 results.
 void tc_plan_build(const std::vector<GemvJob>& jobs, TcPlan& tp, bool f16, cudaStream_t s);
 // 128-byte TMA map of a 2-D array (CUtensorMapDataType type, nx x ny, row pitch in bytes,
 // boxes bx x by, 128-byte swizzle), and of a complex64 block read as FP32 in boxes of

@@ -307,7 +307,8 @@ __global__ void lu_moves_kernel(const int* __restrict__ piv, int j0, int nb, Mov
 
 // A pivot candidate as one integer: |Re| + |Im| (32 leading bits: the choice is within 2^-20
 // of the largest) above the complement of the row, so the maximum is the largest value
-// and, on ties, the smallest row.  Non-finite values order last, 0 is no candidate.
+// and, on ties, the smallest row.  A non-finite value is above every finite one: the
+// maximum finds it and pivot_ok refuses it.  0 is no candidate.
 __device__ __forceinline__ unsigned long long pivot_key(float2 a, int row) {
   const unsigned v = __float_as_uint(fabsf(a.x) + fabsf(a.y));
   return ((unsigned long long)v << 32) | unsigned(~row);

@@ -10,8 +10,9 @@
 // P x = r is solved by
 //   S x3 = r3 - F D (L11 r1 + L12 r2),  S = k0^2 I - F D (L11 P13 + L12 P23),
 //   [x1; x2] = Lambda ([r1; r2] - [P13; P23] x3).
-// S is block diagonal by object (D, B, F are); each block is formed on the
-// device and inverted once per assembly with the batched LU.
+// S is block diagonal by object (D, B, F are); each distinct block is formed on the
+// device and inverted once per assembly: by the FP64 LU, from order SCHUR_REFINE_MIN on by a
+// complex64 LU refined with FP64 residuals.
 #include <algorithm>
 
 #include "dense.h"
@@ -440,8 +441,8 @@ void prec_setup(Precond& P, const sldm_mesh* m, const std::vector<PrecObj>& objs
   for (size_t i = 0; i < objs.size(); ++i)
     if (objs[i].same == int(i) && objs[i].nt > 1)
       last_row_kernel<<<(objs[i].nt + 30) / 32, 1024, 0, s>>>(objs[i].nt - 1, P.sinv.p + off[i]), ::sldm::count_launch();
-  // a complex64 operator takes an FP32 preconditioner: S^-1 (inverted in FP64)
-  // rounded to complex64, applied with FP32 arithmetic
+  // a complex64 operator takes an FP32 preconditioner: S^-1 (accurate beyond
+  // that rounding) in complex64, applied with FP32 arithmetic
   P.f32 = sizeof(C) == sizeof(float2);
   if (P.f32) {
     P.lam32.alloc(size_t(4) * ne);
