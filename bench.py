@@ -212,8 +212,8 @@ FP64_OPS_PER_EVAL_REFL = 167.0
 # text in csrc/<file>); for any other source the line reports traffic null.
 GEMV_TRAFFIC = {
     # main-stage launch of the 4 x 4 metasurface, 32 right-hand sides (profiles/gemm_tc_metasurface-4x4-32angles-c64x2.md)
-    "gemm_tc_kernel": dict(sha="0af134201f2d86b2", file="gemm_tc.cu",
-                           per_alg_byte=(442.374485e6 + 2.653184e6) / 423.936e6),
+    "gemm_tc_kernel": dict(sha="2cd48464c10c9c9b", file="gemm_tc.cu",
+                           per_alg_byte=(442.328064e6 + 2.817707e6) / 423.936e6),
 }
 
 
